@@ -150,7 +150,10 @@ __global__ void __launch_bounds__(32 * FWARPS) k_force(ForceArgs a) {
   float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   double ek = 0;
   if (k < a.n) {
-    const int nn = a.nnei[k];
+    // ghost centres (rows from row_end on) are not evaluated: their gradients
+    // are zeros, taken without a load; they keep their places in the sums
+    const int nn = k < a.nlocal ? a.nnei[k] : 0;
+    const int row_end = a.nlocal * NP;
     int cnt = a.rev_cnt[k];
     for (int s = lane; s < nn; s += 32) {
       const size_t row = (size_t)k * NP + s;
@@ -180,7 +183,9 @@ __global__ void __launch_bounds__(32 * FWARPS) k_force(ForceArgs a) {
         __syncwarp();
       }
     for (int t = lane; t < cnt; t += 32) {
-      const float4 g = reinterpret_cast<const float4*>(a.g)[rows[t]];
+      const int row = rows[t];
+      if (row >= row_end) continue;
+      const float4 g = reinterpret_cast<const float4*>(a.g)[row];
       f0 -= g.x; f1 -= g.y; f2 -= g.z;
     }
     f0 = warp_sum(f0); f1 = warp_sum(f1); f2 = warp_sum(f2);
