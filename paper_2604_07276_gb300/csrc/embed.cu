@@ -1,0 +1,285 @@
+// The FP32 SIMT embedding net (stages a5, a13) over live neighbour rows:
+// net_s = 1 -> E0 -> E1 -> E2 (tanh, residual rule), G0 = net_s * (1 + Gt),
+// and its adjoint dR[:, 0] += d net_s / dx . (dG0 * (1 + Gt)).
+//
+// A thread owns one live row; the rows come from the list of all atoms' live
+// rows, so no lane works on padding.  The row's layer-1 and layer-2 units stay
+// in its registers (and, where an index runs, in its own shared-memory column),
+// the weights are read from shared memory as 16-byte broadcasts: 2 loads for 8
+// FMAs.  The bound is the FMA pipe and, for about a third of the time, tanhf
+// (E0 + E1 + E2 per row and direction).  Every product sums in the order of a
+// plain loop over its inputs.
+#include <algorithm>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace dpa1 {
+
+namespace {
+
+constexpr int ER_T = 128;  // threads (rows) per tile
+constexpr int ER_B = 8;    // outputs per weight pass
+
+template <int E0, int E1, int E2>
+struct RowNet {
+  static constexpr int P1 = (E1 + ER_B - 1) / ER_B * ER_B, P2 = (E2 + ER_B - 1) / ER_B * ER_B;  // padded row strides
+  // packed global weights
+  static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2;
+  // shared memory (floats)
+  static constexpr int W1 = 0, W2 = W1 + E0 * P1, B1 = W2 + E1 * P2, B2 = B1 + P1, W0 = B2 + P2, B0 = W0 + E0,
+                       H1 = (B0 + E0 + 3) / 4 * 4, H2 = H1 + E0 * ER_T, TOTAL = H2 + E1 * ER_T;
+  // CTAs per SM that registers and shared memory allow (227 KB)
+  static constexpr int MIN_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 3 : 2);
+  static_assert(MIN_CTAS * (TOTAL * 4 + 1024) <= 228 * 1024, "shared memory");
+};
+
+template <int IN, int OUT>
+__host__ __device__ constexpr bool doubles() {
+  return OUT == 2 * IN;
+}
+
+template <int E0, int E1, int E2>
+__device__ __forceinline__ void row_weights(float* sm, const float* __restrict__ w) {
+  using N = RowNet<E0, E1, E2>;
+  for (int t = threadIdx.x; t < E0 * N::P1; t += ER_T) {
+    const int p = t / N::P1, b = t % N::P1;
+    sm[N::W1 + t] = b < E1 ? w[N::gW1 + p * E1 + b] : 0.f;
+  }
+  for (int t = threadIdx.x; t < E1 * N::P2; t += ER_T) {
+    const int b = t / N::P2, c = t % N::P2;
+    sm[N::W2 + t] = c < E2 ? w[N::gW2 + b * E2 + c] : 0.f;
+  }
+  for (int t = threadIdx.x; t < N::P1; t += ER_T) sm[N::B1 + t] = t < E1 ? w[N::gB1 + t] : 0.f;
+  for (int t = threadIdx.x; t < N::P2; t += ER_T) sm[N::B2 + t] = t < E2 ? w[N::gB2 + t] : 0.f;
+  for (int t = threadIdx.x; t < E0; t += ER_T) {
+    sm[N::W0 + t] = w[t];
+    sm[N::B0 + t] = w[N::gB0 + t];
+  }
+  __syncthreads();
+}
+
+// z[u] = bias[c + u] + sum_k in[k] W[k][c + u], u < 8 (W with row stride LD)
+template <int K, int LD>
+__device__ __forceinline__ void row_block(const float* in, const float* W, const float* bias, int c, float* z) {
+  const float4 b0 = *reinterpret_cast<const float4*>(bias + c), b1 = *reinterpret_cast<const float4*>(bias + c + 4);
+  z[0] = b0.x; z[1] = b0.y; z[2] = b0.z; z[3] = b0.w;
+  z[4] = b1.x; z[5] = b1.y; z[6] = b1.z; z[7] = b1.w;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const float4 w0 = *reinterpret_cast<const float4*>(W + k * LD + c);
+    const float4 w1 = *reinterpret_cast<const float4*>(W + k * LD + c + 4);
+    z[0] = fmaf(in[k], w0.x, z[0]); z[1] = fmaf(in[k], w0.y, z[1]);
+    z[2] = fmaf(in[k], w0.z, z[2]); z[3] = fmaf(in[k], w0.w, z[3]);
+    z[4] = fmaf(in[k], w1.x, z[4]); z[5] = fmaf(in[k], w1.y, z[5]);
+    z[6] = fmaf(in[k], w1.z, z[6]); z[7] = fmaf(in[k], w1.w, z[7]);
+  }
+}
+
+// Layers 1 and 2 of this thread's row: its shared columns H1 and H2 and the
+// layer-2 units in h2.
+template <int E0, int E1, int E2>
+__device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, float* h2) {
+  using N = RowNet<E0, E1, E2>;
+  float* c1 = sm + N::H1 + threadIdx.x;
+  float* c2 = sm + N::H2 + threadIdx.x;
+  float h1[E0];
+#pragma unroll
+  for (int p = 0; p < E0; ++p) {
+    h1[p] = tanhf(fmaf(x, sm[N::W0 + p], b0t ? b0t[p] : sm[N::B0 + p]));
+    c1[p * ER_T] = h1[p];
+  }
+#pragma unroll 1
+  for (int b = 0; b < E1; b += ER_B) {
+    float z[ER_B];
+    row_block<E0, N::P1>(h1, sm + N::W1, sm + N::B1, b, z);
+#pragma unroll
+    for (int u = 0; u < ER_B; ++u)
+      if (b + u < E1) {
+        const int s = b + u < E0 ? b + u : b + u - E0;  // the skip input of a doubling layer
+        c2[(b + u) * ER_T] = (doubles<E0, E1>() ? c1[s * ER_T] : 0.f) + tanhf(z[u]);
+      }
+  }
+#pragma unroll
+  for (int b = 0; b < E1; ++b) h2[b] = c2[b * ER_T];
+}
+
+// Where a list row's data lie: row rg = atom * NP + slot of the per-row
+// arrays, and G0 / dE/dG0 as stored (four columns c .. c + 3, c % 4 == 0).
+struct RowPos {
+  int rg, ti, tj;
+  size_t g0;  // of column 0
+  int gs;     // distance of consecutive column quads
+  __device__ RowPos(const EmbedArgs& a, int p, int nrows) : rg(-1), ti(0), tj(0), g0(0), gs(4) {
+    if (p >= nrows) return;
+    rg = a.rowmap[p];
+    const int atom = rg / NP;
+    ti = a.atype[atom];
+    tj = a.atype[a.nlist[rg]];
+    g0 = (size_t)atom * NP * a.m1 + (size_t)(rg % NP) * 4;
+    gs = NP * 4;
+  }
+  __device__ size_t quad(int c) const { return g0 + (size_t)(c >> 2) * gs; }
+};
+
+template <int E0, int E1, int E2>
+__global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_rows_fwd(EmbedArgs a) {
+  using N = RowNet<E0, E1, E2>;
+  extern __shared__ __align__(16) float sm[];
+  row_weights<E0, E1, E2>(sm, a.w);
+  const int nrows = *a.nrows;
+  for (int p0 = blockIdx.x * ER_T; p0 < nrows; p0 += gridDim.x * ER_T) {
+    const RowPos r(a, p0 + threadIdx.x, nrows);
+    const size_t pair = (size_t)r.ti * a.ntypes + r.tj;
+    float h2[E1];
+    row_front<E0, E1, E2>(sm, r.rg >= 0 ? a.R[(size_t)r.rg * 4] : 0.f, a.b0t ? a.b0t + pair * E0 : nullptr, h2);
+    const float4* gt4 = reinterpret_cast<const float4*>(a.Gt + pair * E2);
+    const float* c2 = sm + N::H2 + threadIdx.x;
+#pragma unroll 1
+    for (int c = 0; c < E2; c += ER_B) {
+      float z[ER_B];
+      row_block<E1, N::P2>(h2, sm + N::W2, sm + N::B2, c, z);
+#pragma unroll
+      for (int q = 0; q < ER_B; q += 4) {
+        if (c + q >= E2) continue;
+        const float4 gt = gt4[(c + q) >> 2];
+        const float gg[4] = {gt.x, gt.y, gt.z, gt.w};
+        float o[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = c + q + u;
+          const float h3 = (doubles<E1, E2>() ? c2[(k < E1 ? k : k - E1) * ER_T] : 0.f) + tanhf(z[q + u]);
+          o[u] = h3 * (1.f + gg[u]);
+        }
+        if (r.rg >= 0) *reinterpret_cast<float4*>(a.G0 + r.quad(c + q)) = make_float4(o[0], o[1], o[2], o[3]);
+      }
+    }
+  }
+}
+
+template <int E0, int E1, int E2>
+__global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_rows_bwd(EmbedArgs a) {
+  using N = RowNet<E0, E1, E2>;
+  extern __shared__ __align__(16) float sm[];
+  row_weights<E0, E1, E2>(sm, a.w);
+  const int nrows = *a.nrows;
+  // W2 under a second name (an offset of zero that the compiler does not know):
+  // the weights of a column block are loaded again for the adjoint's pass over
+  // them instead of being kept, 8 E1 registers, from the forward's
+  const float* W2b = sm + N::W2 + (nrows >> 31);
+  for (int p0 = blockIdx.x * ER_T; p0 < nrows; p0 += gridDim.x * ER_T) {
+    const RowPos r(a, p0 + threadIdx.x, nrows);
+    const bool live = r.rg >= 0;
+    const size_t pair = (size_t)r.ti * a.ntypes + r.tj;
+    float h2[E1];
+    row_front<E0, E1, E2>(sm, live ? a.R[(size_t)r.rg * 4] : 0.f, a.b0t ? a.b0t + pair * E0 : nullptr, h2);
+    const float4* gt4 = reinterpret_cast<const float4*>(a.Gt + pair * E2);
+    // dH2[b] = sum_c W2[b][c] dZ3[c], dZ3 = g (1 - t3^2), g = dG0 (1 + Gt)
+    float s[E1];
+#pragma unroll
+    for (int b = 0; b < E1; ++b) s[b] = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < E2; c += ER_B) {
+      float z[ER_B];
+      row_block<E1, N::P2>(h2, sm + N::W2, sm + N::B2, c, z);
+#pragma unroll
+      for (int q = 0; q < ER_B; q += 4) {
+        float4 dg = make_float4(0.f, 0.f, 0.f, 0.f), gt = dg;
+        if (c + q < E2) {
+          gt = gt4[(c + q) >> 2];
+          if (live) dg = *reinterpret_cast<const float4*>(a.dG0 + r.quad(c + q));
+        }
+        const float dd[4] = {dg.x, dg.y, dg.z, dg.w}, gg[4] = {gt.x, gt.y, gt.z, gt.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float g = dd[u] * (1.f + gg[u]);
+          const float t = tanhf(z[q + u]);
+          z[q + u] = g * (1.f - t * t);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < E1; ++b) {
+        const float4 w0 = *reinterpret_cast<const float4*>(W2b + b * N::P2 + c);
+        const float4 w1 = *reinterpret_cast<const float4*>(W2b + b * N::P2 + c + 4);
+        s[b] = fmaf(w0.x, z[0], s[b]); s[b] = fmaf(w0.y, z[1], s[b]);
+        s[b] = fmaf(w0.z, z[2], s[b]); s[b] = fmaf(w0.w, z[3], s[b]);
+        s[b] = fmaf(w1.x, z[4], s[b]); s[b] = fmaf(w1.y, z[5], s[b]);
+        s[b] = fmaf(w1.z, z[6], s[b]); s[b] = fmaf(w1.w, z[7], s[b]);
+      }
+    }
+    // the skip part of dH2 (a doubling layer: columns b and b + E1), then
+    // dZ2 = dH2 (1 - t2^2) with t2 = H2 - skip(H1), over the units in h2
+    const float* c1 = sm + N::H1 + threadIdx.x;
+    if (doubles<E1, E2>()) {
+#pragma unroll
+      for (int c = 0; c < E2; c += 4) {
+        const float4 g4 = gt4[c >> 2];
+        float4 dg = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (live) dg = *reinterpret_cast<const float4*>(a.dG0 + r.quad(c));
+        s[c % E1] += dg.x * (1.f + g4.x);
+        s[(c + 1) % E1] += dg.y * (1.f + g4.y);
+        s[(c + 2) % E1] += dg.z * (1.f + g4.z);
+        s[(c + 3) % E1] += dg.w * (1.f + g4.w);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < E1; ++b) {
+      const float t = h2[b] - (doubles<E0, E1>() ? c1[(b % E0) * ER_T] : 0.f);
+      h2[b] = s[b] * (1.f - t * t);
+    }
+    // dH1[p] = skip^T(dH2)[p] + sum_b W1[p][b] dZ2[b]; dx = sum_p W0[p] dH1 (1 - H1^2)
+    float dx = 0.f;
+#pragma unroll
+    for (int p = 0; p < E0; ++p) {
+      float v = 0.f;
+#pragma unroll
+      for (int b = 0; b < N::P1; b += 4) {
+        if (b >= E1) continue;
+        const float4 w = *reinterpret_cast<const float4*>(sm + N::W1 + p * N::P1 + b);
+        v = fmaf(w.x, h2[b], v);
+        if (b + 1 < E1) v = fmaf(w.y, h2[b + 1 < E1 ? b + 1 : 0], v);
+        if (b + 2 < E1) v = fmaf(w.z, h2[b + 2 < E1 ? b + 2 : 0], v);
+        if (b + 3 < E1) v = fmaf(w.w, h2[b + 3 < E1 ? b + 3 : 0], v);
+      }
+      if (doubles<E0, E1>()) {
+        v += s[p];
+        v += s[p + E0 < E1 ? p + E0 : 0];
+      }
+      const float h1 = c1[p * ER_T];
+      dx = __fadd_rn(dx, __fmul_rn(v * (1.f - h1 * h1), sm[N::W0 + p]));
+    }
+    if (live) a.dR[(size_t)r.rg * 4] += dx;
+  }
+}
+
+template <int E0, int E1, int E2>
+void rows_launch(const EmbedArgs& a, bool bwd, cudaStream_t st) {
+  using N = RowNet<E0, E1, E2>;
+  const size_t smem = sizeof(float) * N::TOTAL;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // at most n * NP rows in tiles of ER_T = NP
+  const int grid = std::min(a.n, N::MIN_CTAS * std::max(1, sms));
+  if (!bwd) {
+    cudaFuncSetAttribute(k_embed_rows_fwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_embed_rows_fwd<E0, E1, E2><<<grid, ER_T, smem, st>>>(a);
+  } else {
+    cudaFuncSetAttribute(k_embed_rows_bwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_embed_rows_bwd<E0, E1, E2><<<grid, ER_T, smem, st>>>(a);
+  }
+  note_launch();
+}
+
+}  // namespace
+
+bool launch_embed_rows(const EmbedArgs& a, const int* w, bool bwd, cudaStream_t st) {
+  static_assert(ER_T == NP, "n tiles hold every live row");
+  if (a.n == 0) return true;
+  if (w[0] == 25 && w[1] == 50 && w[2] == 100) { rows_launch<25, 50, 100>(a, bwd, st); return true; }
+  if (w[0] == 16 && w[1] == 32 && w[2] == 64) { rows_launch<16, 32, 64>(a, bwd, st); return true; }
+  if (w[0] == 32 && w[1] == 64 && w[2] == 128) { rows_launch<32, 64, 128>(a, bwd, st); return true; }
+  return false;
+}
+
+}  // namespace dpa1

@@ -120,7 +120,13 @@ struct EmbedArgs {
   float* G0;        // [rows][m1]
   const float* dG0;  // backward only
   float* dR;         // backward only: dR[:,0] +=
+  // row kernels: the list of live rows (atom * NP + slot) and its length (device)
+  const int* rowmap = nullptr;
+  const int* nrows = nullptr;
 };
+// The net over a list of live rows, G0 and dG0 column-quad interleaved per atom
+// (embed.cu): forward, or adjoint.
+bool launch_embed_rows(const EmbedArgs& a, const int* widths, bool bwd, cudaStream_t st);
 bool launch_embed_fwd(const EmbedArgs& a, const int* widths, cudaStream_t st);
 bool launch_embed_bwd(const EmbedArgs& a, const int* widths, cudaStream_t st);
 

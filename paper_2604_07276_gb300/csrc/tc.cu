@@ -759,32 +759,6 @@ __global__ void __launch_bounds__(NT, 1) k_layer_bwd_tc(const __grid_constant__ 
   if (warp == 0) tmem_dealloc(tm, 512);
 }
 
-// Row-major [rows][m1] <-> column-quad interleaved per atom (to_cq = 1: row-major
-// src to interleaved dst), one float4 per thread in the interleaved order.
-__global__ void k_relayout(const float4* __restrict__ src, float4* __restrict__ dst, long long total4, int m1,
-                           int to_cq) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total4) return;
-  const int q4 = m1 / 4;
-  const long long per_atom = (long long)NP * q4;
-  const long long atom = i / per_atom;
-  const int rem = (int)(i % per_atom), q = rem / NP, r = rem % NP;
-  const long long rm = atom * per_atom + (long long)r * q4 + q;
-  if (to_cq)
-    dst[i] = src[rm];
-  else
-    dst[rm] = src[i];
-}
-
-void relayout(const float* src, float* dst, int n, int m1, bool to_cq, cudaStream_t st) {
-  const long long total4 = (long long)n * NP * (m1 / 4);
-  if (total4 == 0) return;
-  k_relayout<<<(unsigned)((total4 + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float4*>(src),
-                                                               reinterpret_cast<float4*>(dst), total4, m1,
-                                                               to_cq ? 1 : 0);
-  note_launch();
-}
-
 int sm_count_dev(int dev) {
   int c = 0;
   cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
@@ -908,13 +882,11 @@ void tc_plan_buffers(dp_model* m, Arena& a, int cap) {
   ws.tc.p[1] = a.take<float>(rows * (size_t)std::max(1, m->nattn));                // rstd per layer
   ws.tc.p[4] = a.take<float2>(rows * (size_t)std::max(1, m->nattn));               // softmax stats per layer
   ws.tc.p[2] = nullptr;
-  // row-major staging of G0 / dE/dG0 for the SIMT embedding net (nets other than 25-50-100)
-  ws.tc.p[3] = m->tcw.emb_W1_t ? nullptr : a.take<float>(rows * m->m1);
   // layers 1 and 2 of the tensor-core embedding net, for its adjoint
   ws.tc.p[5] = m->tcw.emb_W1_t ? a.take<float>(rows * (size_t)(m->emb[0] + m->emb[1])) : nullptr;
-  // the live neighbour rows the tensor-core embedding net runs over, and their number
-  ws.tc.p[6] = m->tcw.emb_W1_t ? a.take<int>(rows) : nullptr;
-  ws.tc.p[7] = m->tcw.emb_W1_t ? a.take<int>(64) : nullptr;
+  // the live neighbour rows the embedding net runs over, and their number
+  ws.tc.p[6] = a.take<int>(rows);
+  ws.tc.p[7] = a.take<int>(64);
 }
 
 
@@ -949,19 +921,20 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
     la.err = m->d_err;
     return la;
   };
-  // embedding, then the attention layers forward
+  // embedding (nets without tensor-core tiles: FP32 SIMT), then the attention
+  // layers forward
   EmbedArgs ea{};
-  float* rm_stage = reinterpret_cast<float*>(ws.tc.p[3]);
   ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m->m1;
-  ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = rm_stage;
+  ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0]; ea.dG0 = ws.dG;
+  ea.dR = ws.dR;
+  ea.rowmap = reinterpret_cast<const int*>(ws.tc.p[6]);
+  ea.nrows = reinterpret_cast<const int*>(ws.tc.p[7]);
   const bool emb_tc = m->tcw.emb_W1_t != nullptr;
-  if (emb_tc) {
-    tc_live_rows(m, n, st);
+  tc_live_rows(m, n, st);
+  if (emb_tc)
     tc_embed_fused(m, n, atype, false, st);
-  } else {
-    launch_embed_fwd(ea, m->emb, st);
-    relayout(rm_stage, ws.G[0], n, m->m1, true, st);
-  }
+  else
+    launch_embed_rows(ea, m->emb, false, st);
   prof_mark(m, "embed_fwd", st);
   for (int l = 0; l < L && n > 0; ++l) {
     if (f16)
@@ -981,14 +954,10 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
     note_launch();
     prof_mark(m, "attn_bwd_tc", st);
   }
-  if (emb_tc) {
+  if (emb_tc)
     tc_embed_fused(m, n, atype, true, st);
-  } else {
-    relayout(ws.dG, rm_stage, n, m->m1, false, st);
-    ea.dG0 = rm_stage;
-    ea.dR = ws.dR;
-    launch_embed_bwd(ea, m->emb, st);
-  }
+  else
+    launch_embed_rows(ea, m->emb, true, st);
   prof_mark(m, "embed_bwd", st);
 }
 
