@@ -5,10 +5,12 @@
 // A thread owns one live row; the rows come from the list of all atoms' live
 // rows, so no lane works on padding.  The row's layer-1 and layer-2 units stay
 // in its registers (and, where an index runs, in its own shared-memory column),
-// the weights are read from shared memory as 16-byte broadcasts: 2 loads for 8
-// FMAs.  The bound is the FMA pipe and, for about a third of the time, tanhf
-// (E0 + E1 + E2 per row and direction).  Every product sums in the order of a
-// plain loop over its inputs.
+// the weights are read from shared memory as 16-byte broadcasts.  The products
+// run on pairs of outputs (fma.rn.f32x2: two FP32 FMAs, each rounded as fmaf):
+// the bound is the issue of FMAs, weight loads and tanhf (E0 + E1 + E2 per row
+// and direction), so 6 instructions for 8 FMAs instead of 10 count.  Two rows
+// per thread, which halve the weight loads, measured no gain.  Every product
+// sums in the order of a plain loop over its inputs.
 #include <algorithm>
 
 #include "common.cuh"
@@ -21,6 +23,18 @@ namespace {
 constexpr int ER_T = 128;  // threads (rows) per tile
 constexpr int ER_B = 8;    // outputs per weight pass
 
+// A pair of FP32 values in one 64-bit register, and its FMA.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(float x, float y) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ void f2_fma(f2& acc, f2 a, f2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b)); }
+// four consecutive floats of shared memory as two pairs
+__device__ __forceinline__ ulonglong2 f2_ld4(const float* p) { return *reinterpret_cast<const ulonglong2*>(p); }
+
 template <int E0, int E1, int E2>
 struct RowNet {
   static constexpr int P1 = (E1 + ER_B - 1) / ER_B * ER_B, P2 = (E2 + ER_B - 1) / ER_B * ER_B;  // padded row strides
@@ -28,10 +42,13 @@ struct RowNet {
   static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2;
   // shared memory (floats)
   static constexpr int W1 = 0, W2 = W1 + E0 * P1, B1 = W2 + E1 * P2, B2 = B1 + P1, W0 = B2 + P2, B0 = W0 + E0,
-                       H1 = (B0 + E0 + 3) / 4 * 4, H2 = H1 + E0 * ER_T, TOTAL = H2 + E1 * ER_T;
-  // CTAs per SM that registers and shared memory allow (227 KB)
-  static constexpr int MIN_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 3 : 2);
-  static_assert(MIN_CTAS * (TOTAL * 4 + 1024) <= 228 * 1024, "shared memory");
+                       H1 = (B0 + E0 + 3) / 4 * 4, H2 = H1 + E0 * ER_T, FWD = H2 + E1 * ER_T;
+  // the adjoint also holds the transposes, rows padded to 4: W2^T [E2][Q1], W1^T [E1][Q0]
+  static constexpr int Q1 = (E1 + 3) / 4 * 4, Q0 = (E0 + 3) / 4 * 4;
+  static constexpr int W2T = FWD, W1T = W2T + P2 * Q1, BWD = W1T + E1 * Q0;
+  // CTAs per SM that registers and shared memory (228 KB) allow
+  static constexpr int F_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 3 : 2), B_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 2 : 1);
+  static_assert(F_CTAS * (FWD * 4 + 1024) <= 228 * 1024 && B_CTAS * (BWD * 4 + 1024) <= 228 * 1024, "shared memory");
 };
 
 template <int IN, int OUT>
@@ -59,35 +76,37 @@ __device__ __forceinline__ void row_weights(float* sm, const float* __restrict__
   __syncthreads();
 }
 
-// z[u] = bias[c + u] + sum_k in[k] W[k][c + u], u < 8 (W with row stride LD)
+// z[u] = bias[c + u] + sum_k in[k] W[k][c + u], u < 8 (W with row stride LD;
+// in[k] as the pair (in[k], in[k]))
 template <int K, int LD>
-__device__ __forceinline__ void row_block(const float* in, const float* W, const float* bias, int c, float* z) {
-  const float4 b0 = *reinterpret_cast<const float4*>(bias + c), b1 = *reinterpret_cast<const float4*>(bias + c + 4);
-  z[0] = b0.x; z[1] = b0.y; z[2] = b0.z; z[3] = b0.w;
-  z[4] = b1.x; z[5] = b1.y; z[6] = b1.z; z[7] = b1.w;
+__device__ __forceinline__ void row_block(const f2* in, const float* W, const float* bias, int c, float* z) {
+  const ulonglong2 b0 = f2_ld4(bias + c), b1 = f2_ld4(bias + c + 4);
+  f2 acc[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const float4 w0 = *reinterpret_cast<const float4*>(W + k * LD + c);
-    const float4 w1 = *reinterpret_cast<const float4*>(W + k * LD + c + 4);
-    z[0] = fmaf(in[k], w0.x, z[0]); z[1] = fmaf(in[k], w0.y, z[1]);
-    z[2] = fmaf(in[k], w0.z, z[2]); z[3] = fmaf(in[k], w0.w, z[3]);
-    z[4] = fmaf(in[k], w1.x, z[4]); z[5] = fmaf(in[k], w1.y, z[5]);
-    z[6] = fmaf(in[k], w1.z, z[6]); z[7] = fmaf(in[k], w1.w, z[7]);
+    const ulonglong2 w0 = f2_ld4(W + k * LD + c), w1 = f2_ld4(W + k * LD + c + 4);
+    f2_fma(acc[0], in[k], w0.x);
+    f2_fma(acc[1], in[k], w0.y);
+    f2_fma(acc[2], in[k], w1.x);
+    f2_fma(acc[3], in[k], w1.y);
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) f2_unpack(acc[q], z[2 * q], z[2 * q + 1]);
 }
 
 // Layers 1 and 2 of this thread's row: its shared columns H1 and H2 and the
-// layer-2 units in h2.
+// layer-2 units in h2 (each as a pair of itself).
 template <int E0, int E1, int E2>
-__device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, float* h2) {
+__device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, f2* h2) {
   using N = RowNet<E0, E1, E2>;
   float* c1 = sm + N::H1 + threadIdx.x;
   float* c2 = sm + N::H2 + threadIdx.x;
-  float h1[E0];
+  f2 h1[E0];
 #pragma unroll
   for (int p = 0; p < E0; ++p) {
-    h1[p] = tanhf(fmaf(x, sm[N::W0 + p], b0t ? b0t[p] : sm[N::B0 + p]));
-    c1[p * ER_T] = h1[p];
+    const float h = tanhf(fmaf(x, sm[N::W0 + p], b0t ? b0t[p] : sm[N::B0 + p]));
+    h1[p] = f2_pack(h, h);
+    c1[p * ER_T] = h;
   }
 #pragma unroll 1
   for (int b = 0; b < E1; b += ER_B) {
@@ -101,7 +120,10 @@ __device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, 
       }
   }
 #pragma unroll
-  for (int b = 0; b < E1; ++b) h2[b] = c2[b * ER_T];
+  for (int b = 0; b < E1; ++b) {
+    const float h = c2[b * ER_T];
+    h2[b] = f2_pack(h, h);
+  }
 }
 
 // Where a list row's data lie: row rg = atom * NP + slot of the per-row
@@ -123,7 +145,7 @@ struct RowPos {
 };
 
 template <int E0, int E1, int E2>
-__global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_rows_fwd(EmbedArgs a) {
+__global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::F_CTAS) k_embed_rows_fwd(EmbedArgs a) {
   using N = RowNet<E0, E1, E2>;
   extern __shared__ __align__(16) float sm[];
   row_weights<E0, E1, E2>(sm, a.w);
@@ -131,7 +153,7 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_ro
   for (int p0 = blockIdx.x * ER_T; p0 < nrows; p0 += gridDim.x * ER_T) {
     const RowPos r(a, p0 + threadIdx.x, nrows);
     const size_t pair = (size_t)r.ti * a.ntypes + r.tj;
-    float h2[E1];
+    f2 h2[E1];
     row_front<E0, E1, E2>(sm, r.rg >= 0 ? a.R[(size_t)r.rg * 4] : 0.f, a.b0t ? a.b0t + pair * E0 : nullptr, h2);
     const float4* gt4 = reinterpret_cast<const float4*>(a.Gt + pair * E2);
     const float* c2 = sm + N::H2 + threadIdx.x;
@@ -158,26 +180,31 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_ro
 }
 
 template <int E0, int E1, int E2>
-__global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_rows_bwd(EmbedArgs a) {
+__global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::B_CTAS) k_embed_rows_bwd(EmbedArgs a) {
   using N = RowNet<E0, E1, E2>;
   extern __shared__ __align__(16) float sm[];
   row_weights<E0, E1, E2>(sm, a.w);
+  for (int t = threadIdx.x; t < N::P2 * N::Q1; t += ER_T) {
+    const int c = t / N::Q1, b = t % N::Q1;
+    sm[N::W2T + t] = b < E1 ? sm[N::W2 + b * N::P2 + c] : 0.f;
+  }
+  for (int t = threadIdx.x; t < E1 * N::Q0; t += ER_T) {
+    const int b = t / N::Q0, p = t % N::Q0;
+    sm[N::W1T + t] = p < E0 ? sm[N::W1 + p * N::P1 + b] : 0.f;
+  }
+  __syncthreads();
   const int nrows = *a.nrows;
-  // W2 under a second name (an offset of zero that the compiler does not know):
-  // the weights of a column block are loaded again for the adjoint's pass over
-  // them instead of being kept, 8 E1 registers, from the forward's
-  const float* W2b = sm + N::W2 + (nrows >> 31);
   for (int p0 = blockIdx.x * ER_T; p0 < nrows; p0 += gridDim.x * ER_T) {
     const RowPos r(a, p0 + threadIdx.x, nrows);
     const bool live = r.rg >= 0;
     const size_t pair = (size_t)r.ti * a.ntypes + r.tj;
-    float h2[E1];
+    f2 h2[E1];
     row_front<E0, E1, E2>(sm, live ? a.R[(size_t)r.rg * 4] : 0.f, a.b0t ? a.b0t + pair * E0 : nullptr, h2);
     const float4* gt4 = reinterpret_cast<const float4*>(a.Gt + pair * E2);
     // dH2[b] = sum_c W2[b][c] dZ3[c], dZ3 = g (1 - t3^2), g = dG0 (1 + Gt)
-    float s[E1];
+    f2 s2[N::Q1 / 2];
 #pragma unroll
-    for (int b = 0; b < E1; ++b) s[b] = 0.f;
+    for (int b = 0; b < N::Q1 / 2; ++b) s2[b] = 0ull;
 #pragma unroll 1
     for (int c = 0; c < E2; c += ER_B) {
       float z[ER_B];
@@ -198,17 +225,22 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_ro
         }
       }
 #pragma unroll
-      for (int b = 0; b < E1; ++b) {
-        const float4 w0 = *reinterpret_cast<const float4*>(W2b + b * N::P2 + c);
-        const float4 w1 = *reinterpret_cast<const float4*>(W2b + b * N::P2 + c + 4);
-        s[b] = fmaf(w0.x, z[0], s[b]); s[b] = fmaf(w0.y, z[1], s[b]);
-        s[b] = fmaf(w0.z, z[2], s[b]); s[b] = fmaf(w0.w, z[3], s[b]);
-        s[b] = fmaf(w1.x, z[4], s[b]); s[b] = fmaf(w1.y, z[5], s[b]);
-        s[b] = fmaf(w1.z, z[6], s[b]); s[b] = fmaf(w1.w, z[7], s[b]);
+      for (int u = 0; u < ER_B; ++u) {
+        const f2 zz = f2_pack(z[u], z[u]);
+        const float* wt = sm + N::W2T + (c + u) * N::Q1;
+#pragma unroll
+        for (int b = 0; b < N::Q1; b += 4) {
+          const ulonglong2 w = f2_ld4(wt + b);
+          f2_fma(s2[b / 2], w.x, zz);
+          f2_fma(s2[b / 2 + 1], w.y, zz);
+        }
       }
     }
+    float s[N::Q1];
+#pragma unroll
+    for (int b = 0; b < N::Q1 / 2; ++b) f2_unpack(s2[b], s[2 * b], s[2 * b + 1]);
     // the skip part of dH2 (a doubling layer: columns b and b + E1), then
-    // dZ2 = dH2 (1 - t2^2) with t2 = H2 - skip(H1), over the units in h2
+    // dZ2 = dH2 (1 - t2^2) with t2 = H2 - skip(H1)
     const float* c1 = sm + N::H1 + threadIdx.x;
     if (doubles<E1, E2>()) {
 #pragma unroll
@@ -222,31 +254,34 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_ro
         s[(c + 3) % E1] += dg.w * (1.f + g4.w);
       }
     }
+    // dH1[p] = skip^T(dH2)[p] + sum_b W1[p][b] dZ2[b]; dx = sum_p W0[p] dH1 (1 - H1^2)
+    f2 v2[N::Q0 / 2];
+#pragma unroll
+    for (int p = 0; p < N::Q0 / 2; ++p) v2[p] = 0ull;
+    const float* c2 = sm + N::H2 + threadIdx.x;
 #pragma unroll
     for (int b = 0; b < E1; ++b) {
-      const float t = h2[b] - (doubles<E0, E1>() ? c1[(b % E0) * ER_T] : 0.f);
-      h2[b] = s[b] * (1.f - t * t);
+      const float t = c2[b * ER_T] - (doubles<E0, E1>() ? c1[(b % E0) * ER_T] : 0.f);
+      const float dz = s[b] * (1.f - t * t);
+      const f2 zz = f2_pack(dz, dz);
+#pragma unroll
+      for (int p = 0; p < N::Q0; p += 4) {
+        const ulonglong2 w = f2_ld4(sm + N::W1T + b * N::Q0 + p);
+        f2_fma(v2[p / 2], w.x, zz);
+        f2_fma(v2[p / 2 + 1], w.y, zz);
+      }
     }
-    // dH1[p] = skip^T(dH2)[p] + sum_b W1[p][b] dZ2[b]; dx = sum_p W0[p] dH1 (1 - H1^2)
-    float dx = 0.f;
+    float v[N::Q0], dx = 0.f;
+#pragma unroll
+    for (int p = 0; p < N::Q0 / 2; ++p) f2_unpack(v2[p], v[2 * p], v[2 * p + 1]);
 #pragma unroll
     for (int p = 0; p < E0; ++p) {
-      float v = 0.f;
-#pragma unroll
-      for (int b = 0; b < N::P1; b += 4) {
-        if (b >= E1) continue;
-        const float4 w = *reinterpret_cast<const float4*>(sm + N::W1 + p * N::P1 + b);
-        v = fmaf(w.x, h2[b], v);
-        if (b + 1 < E1) v = fmaf(w.y, h2[b + 1 < E1 ? b + 1 : 0], v);
-        if (b + 2 < E1) v = fmaf(w.z, h2[b + 2 < E1 ? b + 2 : 0], v);
-        if (b + 3 < E1) v = fmaf(w.w, h2[b + 3 < E1 ? b + 3 : 0], v);
-      }
       if (doubles<E0, E1>()) {
-        v += s[p];
-        v += s[p + E0 < E1 ? p + E0 : 0];
+        v[p] += s[p];
+        v[p] += s[p + E0 < E1 ? p + E0 : 0];
       }
       const float h1 = c1[p * ER_T];
-      dx = __fadd_rn(dx, __fmul_rn(v * (1.f - h1 * h1), sm[N::W0 + p]));
+      dx = __fadd_rn(dx, __fmul_rn(v[p] * (1.f - h1 * h1), sm[N::W0 + p]));
     }
     if (live) a.dR[(size_t)r.rg * 4] += dx;
   }
@@ -255,12 +290,12 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::MIN_CTAS) k_embed_ro
 template <int E0, int E1, int E2>
 void rows_launch(const EmbedArgs& a, bool bwd, cudaStream_t st) {
   using N = RowNet<E0, E1, E2>;
-  const size_t smem = sizeof(float) * N::TOTAL;
+  const size_t smem = sizeof(float) * (bwd ? N::BWD : N::FWD);
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // at most n * NP rows in tiles of ER_T = NP
-  const int grid = std::min(a.n, N::MIN_CTAS * std::max(1, sms));
+  const int grid = std::min(a.n, (bwd ? N::B_CTAS : N::F_CTAS) * std::max(1, sms));
   if (!bwd) {
     cudaFuncSetAttribute(k_embed_rows_fwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_embed_rows_fwd<E0, E1, E2><<<grid, ER_T, smem, st>>>(a);
