@@ -256,6 +256,9 @@ int alloc_workspace(dp_model* m, int cap) {
     ws.nnei = a.take<int>(cap);
     ws.ncand = a.take<int>(cap);
     ws.atype_c = a.take<int>(cap);
+    ws.row_off = a.take<int>(cap + 1);
+    ws.rowmap = a.take<int>(rows);
+    ws.row_seg = a.take<int>(cap / ROW_SEG + 1);
     ws.rev_cnt = a.take<int>(cap);
     ws.rev_rows = a.take<int>((size_t)cap * REV_CAP);
     ws.R = a.take<float>(rows * 4);
@@ -400,6 +403,7 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
   da.n = n; da.m1 = m1; da.axis = m->axis; da.tebd_dim = m->td; da.sel = m->sel; da.fit_in = m->fit_in;
   da.T = ws.T; da.X = ws.X; da.dX = ws.dX; da.dG = ws.dG; da.dR = ws.dR;
   da.cq = fused_tc_precision(m->precision) ? 1 : 0;  // the fused layer kernels' layout
+  da.row_off = ws.row_off;
   launch_desc_fwd(da, st);
   prof_mark(m, "desc_fwd", st);
   // a8: fitting forward
@@ -470,27 +474,31 @@ namespace {
 void run_network_f32(dp_model* m, int n, const int* atype, cudaStream_t st) {
   Workspace& ws = m->ws;
   const int rows = n * NP, L = m->nattn, A = m->A, m1 = m->m1;
+  const int* nrows = ws.row_off + n;  // the live rows (device)
   // a5: embedding
   EmbedArgs ea{};
   ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0];
-  launch_embed_fwd(ea, m->emb, st);
+  ea.dG0 = ws.dG; ea.dR = ws.dR; ea.rowmap = ws.rowmap; ea.nrows = ws.row_off + n; ea.packed = 1;
+  launch_embed_rows(ea, m->emb, false, st);
   prof_mark(m, "embed_fwd", st);
   // a6: attention layers
   for (int l = 0; l < L; ++l) {
     const AttnLayerW& w = m->attn[l];
     // [Q K] = G [Wq Wk] + [bq bk] (V only enters through [Wv Wo; bv Wo])
-    gemm_f32(ws.G[l], m1, w.Wqk, 2 * A, w.bqk, nullptr, 0, ws.QK[l], 2 * A, rows, 2 * A, m1, EPI_BIAS, st);
+    gemm_f32(ws.G[l], m1, w.Wqk, 2 * A, w.bqk, nullptr, 0, ws.QK[l], 2 * A, rows, 2 * A, m1, EPI_BIAS, st,
+             nrows);
     prof_mark(m, "qkv_gemm", st);
     AttnArgs aa{};
-    aa.QK = ws.QK[l]; aa.ldq = 2 * A; aa.rw = ws.rw; aa.w64 = ws.w64; aa.nnei = ws.nnei; aa.n = n; aa.A = A;
+    aa.QK = ws.QK[l]; aa.ldq = 2 * A; aa.rw = ws.rw; aa.w64 = ws.w64; aa.nnei = ws.nnei; aa.row_off = ws.row_off; aa.n = n; aa.A = A;
     aa.shift = (float)m->shift;
     aa.G = ws.G[l]; aa.m1 = m1; aa.ldpg = pg_ld(m1); aa.PG = ws.PG[l];
     launch_attn_fwd_f32(aa, st);
     prof_mark(m, "attn_fwd", st);
     // Y = O Wo + bo = [P G, rowsum(P)] [Wv Wo; bv Wo] + bo
-    gemm_f32(ws.PG[l], pg_ld(m1), w.Wvo, m1, w.bo, nullptr, 0, ws.Y[l], m1, rows, m1, pg_ld(m1), EPI_BIAS, st);
-    launch_ln_res_fwd(ws.Y[l], ws.G[l], ws.nlist, w.ln_g, w.ln_b, (float)m->ln_eps, ws.G[l + 1], ws.stats[l], rows,
+    gemm_f32(ws.PG[l], pg_ld(m1), w.Wvo, m1, w.bo, nullptr, 0, ws.Y[l], m1, rows, m1, pg_ld(m1), EPI_BIAS, st,
+             nrows);
+    launch_ln_res_fwd(ws.Y[l], ws.G[l], nrows, w.ln_g, w.ln_b, (float)m->ln_eps, ws.G[l + 1], ws.stats[l], rows,
                       m1, st);
     prof_mark(m, "wo_gemm_ln", st);
   }
@@ -499,23 +507,23 @@ void run_network_f32(dp_model* m, int n, const int* atype, cudaStream_t st) {
   cudaMemsetAsync(ws.dgeo, 0, sizeof(float) * (size_t)rows * 4, st);
   for (int l = L - 1; l >= 0; --l) {
     const AttnLayerW& w = m->attn[l];
-    launch_ln_bwd(ws.dG, ws.Y[l], ws.stats[l], ws.nlist, w.ln_g, ws.dY, rows, m1, st);
+    launch_ln_bwd(ws.dG, ws.Y[l], ws.stats[l], nrows, w.ln_g, ws.dY, rows, m1, st);
     // dE/d[P G, rowsum P] = dY [Wv Wo; bv Wo]^T
-    gemm_f32(ws.dY, m1, w.WvoT, pg_ld(m1), nullptr, nullptr, 0, ws.dPG, pg_ld(m1), rows, pg_ld(m1), m1, EPI_BIAS, st);
+    gemm_f32(ws.dY, m1, w.WvoT, pg_ld(m1), nullptr, nullptr, 0, ws.dPG, pg_ld(m1), rows, pg_ld(m1), m1, EPI_BIAS, st,
+             nrows);
     prof_mark(m, "ln_wo_bwd", st);
     AttnArgs aa{};
-    aa.QK = ws.QK[l]; aa.ldq = 2 * A; aa.rw = ws.rw; aa.w64 = ws.w64; aa.nnei = ws.nnei; aa.n = n; aa.A = A;
+    aa.QK = ws.QK[l]; aa.ldq = 2 * A; aa.rw = ws.rw; aa.w64 = ws.w64; aa.nnei = ws.nnei; aa.row_off = ws.row_off; aa.n = n; aa.A = A;
     aa.shift = (float)m->shift; aa.G = ws.G[l]; aa.m1 = m1; aa.ldpg = pg_ld(m1);
     aa.dPG = ws.dPG; aa.dQK = ws.dQK; aa.dG = ws.dG; aa.dgeo = ws.dgeo;
     launch_attn_bwd_f32(aa, st);  // dQ, dK; dE/dG += P^T dPG
     prof_mark(m, "attn_bwd", st);
     // dE/dG += [dQ dK] [Wq Wk]^T
-    gemm_f32(ws.dQK, 2 * A, w.WqkT, m1, nullptr, nullptr, 0, ws.dG, m1, rows, m1, 2 * A, EPI_ACCUM, st);
+    gemm_f32(ws.dQK, 2 * A, w.WqkT, m1, nullptr, nullptr, 0, ws.dG, m1, rows, m1, 2 * A, EPI_ACCUM, st, nrows);
     prof_mark(m, "qkv_bwd_gemm", st);
   }
   // a13: embedding backward -> dR[:,0]
-  ea.dG0 = ws.dG; ea.dR = ws.dR;
-  launch_embed_bwd(ea, m->emb, st);
+  launch_embed_rows(ea, m->emb, true, st);
   if (m->grad_scale) launch_embed_wgrad(ea, m->emb, m->grad, m->grad_scale, st);
   prof_mark(m, "embed_bwd", st);
 }
@@ -527,27 +535,28 @@ void run_network_f32(dp_model* m, int n, const int* atype, cudaStream_t st) {
 void run_network_bf16x(dp_model* m, int n, const int* atype, cudaStream_t st) {
   Workspace& ws = m->ws;
   const int rows = n * NP, L = m->nattn, A = m->A, m1 = m->m1;
+  const int* nrows = ws.row_off + n;  // the live rows (device)
   // the 25-50-100 embedding net on the tensor cores (BF16 two-term splits),
   // other nets, and any net while its weight gradient is wanted, in FP32
   const bool emb_tc = m->tcw.emb_W2_t != nullptr && !m->grad_scale;
-  float* H12 = reinterpret_cast<float*>(ws.tc.p[5]);
   EmbedArgs ea{};
   ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0];
+  ea.dG0 = ws.dG; ea.dR = ws.dR; ea.rowmap = ws.rowmap; ea.nrows = ws.row_off + n; ea.packed = 1;
   if (emb_tc)
-    tc_embed_bf16(m, n, atype, false, ws.G[0], nullptr, nullptr, H12, st);
+    tc_embed(m, n, atype, false, st);
   else
-    launch_embed_fwd(ea, m->emb, st);
+    launch_embed_rows(ea, m->emb, false, st);
   prof_mark(m, "embed_fwd", st);
   for (int l = 0; l < L; ++l) {
     const AttnLayerW& w = m->attn[l];
     const XWeights::Layer& x = m->xw.layers[l];
-    gemm_bf16x(m, x.qk, ws.G[l], m1, w.bqk, nullptr, 0, ws.QK[l], 2 * A, rows, EPI_BIAS, st);
+    gemm_bf16x(m, x.qk, ws.G[l], m1, w.bqk, nullptr, 0, ws.QK[l], 2 * A, rows, EPI_BIAS, st, nrows);
     prof_mark(m, "qkv_gemm", st);
     attn_core_fwd_bf16x(m, n, l, st);
     prof_mark(m, "attn_fwd", st);
-    gemm_bf16x(m, x.vo, ws.PG[l], pg_ld(m1), w.bo, nullptr, 0, ws.Y[l], m1, rows, EPI_BIAS, st);
-    launch_ln_res_fwd(ws.Y[l], ws.G[l], ws.nlist, w.ln_g, w.ln_b, (float)m->ln_eps, ws.G[l + 1], ws.stats[l], rows,
+    gemm_bf16x(m, x.vo, ws.PG[l], pg_ld(m1), w.bo, nullptr, 0, ws.Y[l], m1, rows, EPI_BIAS, st, nrows);
+    launch_ln_res_fwd(ws.Y[l], ws.G[l], nrows, w.ln_g, w.ln_b, (float)m->ln_eps, ws.G[l + 1], ws.stats[l], rows,
                       m1, st);
     prof_mark(m, "wo_gemm_ln", st);
   }
@@ -556,20 +565,19 @@ void run_network_bf16x(dp_model* m, int n, const int* atype, cudaStream_t st) {
   for (int l = L - 1; l >= 0; --l) {
     const AttnLayerW& w = m->attn[l];
     const XWeights::Layer& x = m->xw.layers[l];
-    launch_ln_bwd(ws.dG, ws.Y[l], ws.stats[l], ws.nlist, w.ln_g, ws.dY, rows, m1, st);
+    launch_ln_bwd(ws.dG, ws.Y[l], ws.stats[l], nrows, w.ln_g, ws.dY, rows, m1, st);
     // dE/d[P G, rowsum P] = dY [Wv Wo; bv Wo]^T
-    gemm_bf16x(m, x.voT, ws.dY, m1, nullptr, nullptr, 0, ws.dPG, pg_ld(m1), rows, EPI_BIAS, st);
+    gemm_bf16x(m, x.voT, ws.dY, m1, nullptr, nullptr, 0, ws.dPG, pg_ld(m1), rows, EPI_BIAS, st, nrows);
     prof_mark(m, "ln_wo_bwd", st);
     attn_core_bwd_bf16x(m, n, l, st);  // dQ, dK; dE/dG += P^T dPG
     prof_mark(m, "attn_bwd", st);
-    gemm_bf16x(m, x.qkT, ws.dQK, 2 * A, nullptr, nullptr, 0, ws.dG, m1, rows, EPI_ACCUM, st);
+    gemm_bf16x(m, x.qkT, ws.dQK, 2 * A, nullptr, nullptr, 0, ws.dG, m1, rows, EPI_ACCUM, st, nrows);
     prof_mark(m, "qkv_bwd_gemm", st);
   }
-  ea.dG0 = ws.dG; ea.dR = ws.dR;
   if (emb_tc) {
-    tc_embed_bf16(m, n, atype, true, nullptr, ws.dG, ws.dR, H12, st);
+    tc_embed(m, n, atype, true, st);
   } else {
-    launch_embed_bwd(ea, m->emb, st);
+    launch_embed_rows(ea, m->emb, true, st);
     if (m->grad_scale) launch_embed_wgrad(ea, m->emb, m->grad, m->grad_scale, st);
   }
   prof_mark(m, "embed_bwd", st);
@@ -599,6 +607,8 @@ int run_after_neighbors(dp_model* m, int n, const double* coord, const CellGrid*
   ea.fp64 = m->precision == DP_PREC_FP32 ? 1 : 0;
   ea.w64 = ea.fp64 ? ws.w64 : nullptr;
   launch_env(ea, st);
+  // the list of the centres' live rows, which the network runs over
+  launch_row_list(ws.nnei, nc, ws.row_off, ws.rowmap, ws.row_seg, st);
   prof_mark(m, "env", st);
   if (nc == 0) {
     // ghosts only: no centre to evaluate
@@ -650,6 +660,7 @@ void run_force_tangent(dp_model* m, int n, const double* coord, const double* v,
                        float* const* dHd, float* dZ, float* dZd, float* Zd, const float* scale, cudaStream_t st) {
   Workspace& ws = m->ws;
   JvpArgs a{};
+  a.row_off = ws.row_off; a.rowmap = ws.rowmap;
   a.coord = coord; a.grid = ws.grid; a.nlist = ws.nlist; a.nnei = ws.nnei; a.atype = ws.atype_c;
   a.n = n; a.ntypes = m->nt; a.m1 = m->m1; a.axis = m->axis; a.fit_in = m->fit_in; a.sel = m->sel;
   a.dstd = m->dstd; a.rcs = (float)m->rcs; a.rc = (float)m->rcut;
@@ -1293,16 +1304,29 @@ long long dp_debug_copy(dp_model* m, const char* name, void* host_dst, size_t by
   };
   sz = std::min(sz, bytes);
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(DP_ERR_CUDA, "sync failed");
-  if (s[0] == 'G' && fused_tc_precision(m->precision)) {
-    // the tensor-core path keeps G column-quad interleaved per atom: return it row-major
+  if (s[0] == 'G') {
+    // the fused paths keep G column-quad interleaved per atom, the others packed
+    // over the live rows: return it row-major per atom, packed layouts with zeros
+    // past the last neighbour
     const size_t m1 = (size_t)m->m1, full = rows * m1;
-    std::vector<float> raw(full), out(full);
-    if (cudaMemcpy(raw.data(), src, full * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
+    const bool cq = fused_tc_precision(m->precision);
+    std::vector<float> raw(full), out(full, 0.f);
+    std::vector<int> off((size_t)m->call_nlocal + 1, 0);
+    if (cudaMemcpy(raw.data(), src, full * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess ||
+        (m->call_nlocal > 0 &&
+         cudaMemcpy(off.data(), ws.row_off, off.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess))
       return fail(DP_ERR_CUDA, "copy failed");
-    for (size_t atom = 0; atom < n; ++atom)
-      for (int r = 0; r < NP; ++r)
-        for (size_t c = 0; c < m1; ++c)
-          out[(atom * NP + r) * m1 + c] = raw[atom * NP * m1 + cq_off(r, (int)c)];
+    for (size_t atom = 0; atom < (size_t)m->call_nlocal; ++atom) {
+      if (cq) {
+        for (int r = 0; r < NP; ++r)
+          for (size_t c = 0; c < m1; ++c)
+            out[(atom * NP + r) * m1 + c] = raw[atom * NP * m1 + cq_off(r, (int)c)];
+      } else {
+        const int o = off[atom], k = off[atom + 1] - o;
+        if (o < 0 || k < 0 || k > NP || (size_t)(o + k) > rows) continue;  // no evaluation has run
+        memcpy(&out[atom * NP * m1], &raw[(size_t)o * m1], sizeof(float) * k * m1);
+      }
+    }
     memcpy(host_dst, out.data(), sz);
     clear_ghosts(sz);
     return (long long)sz;

@@ -78,7 +78,8 @@ struct XGemmArgs {
   const float* R;       // residual [M][ldr] or null
   float* C;             // [M][ldc]
   int ldr, ldc;
-  int M, N, nkb, bn_max, epi, mtiles;
+  int M, N, nkb, bn_max, epi;
+  const int* m_dev;  // non-null: the rows are *m_dev (device, <= M)
   int* err;
 };
 
@@ -155,7 +156,9 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (ok) ok = mbar_wait(bar, parity, a.err);
   };
-  const int ntile = a.mtiles > (int)blockIdx.x ? (a.mtiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int M = a.m_dev ? *a.m_dev : a.M;
+  const int mtiles = (M + XBM - 1) / XBM;
+  const int ntile = mtiles > (int)blockIdx.x ? (mtiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (warp == 0 && lane == 0) {
     const uint8_t* img = a.bimg + (size_t)nb * a.nkb * 2 * b_tile;
@@ -263,7 +266,7 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
               const int rr = 4 * (k0 + k) + (lane >> 3);
               const long long m = m0 + rr;
               o[k] = *reinterpret_cast<const float4*>(stg + rr * XSLD + q);
-              if (m < a.M && (res || acc)) {
+              if (m < M && (res || acc)) {
                 const float4 e = res ? *reinterpret_cast<const float4*>(a.R + m * a.ldr + n)
                                      : *reinterpret_cast<const float4*>(a.C + m * a.ldc + n);
                 o[k].x += e.x; o[k].y += e.y; o[k].z += e.z; o[k].w += e.w;
@@ -272,7 +275,7 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const long long m = m0 + 4 * (k0 + k) + (lane >> 3);
-              if (m < a.M) *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o[k];
+              if (m < M) *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o[k];
             }
           }
         }
@@ -336,6 +339,8 @@ int x_sm_count(int dev) {
 constexpr int XC_NT = 512;
 constexpr int XT = 32768;
 
+// Rows of QK, G, PG, dPG, dQK and dG are packed (atom i's at row_off[i]), those of
+// rw and dgeo at i * NP.
 struct XCoreArgs {
   const float* QK;   // [rows][ldq]: Q | K (attention width each)
   const float* G;    // [rows][m1] layer input
@@ -346,6 +351,7 @@ struct XCoreArgs {
   float* dgeo;       // bwd: [rows][4] += (d rhat, d w)
   const float* rw;   // [rows][4] (rhat, w)
   const int* nnei;
+  const int* row_off;
   int n, m1, ldpg, npg, ldq;  // npg: MMA width of P G (m1 rounded up to 16)
   float scale, shift;
   int* err;
@@ -480,13 +486,14 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_fwd_bf16x(const __grid_c
   const int ld = a.ldq;  // Q | K, 128 NH columns each
   for (int atom = blockIdx.x; atom < a.n && sy.ok; atom += gridDim.x) {
     const int nn = a.nnei[atom];
-    const size_t base = (size_t)atom * NP;
+    const size_t base = a.row_off[atom], gbase = (size_t)atom * NP;
     const bool rv = row < nn;
     // the next atom's Q and K rows and its layer input into L2
     if (atom + (int)gridDim.x < a.n) {
-      const size_t nb = (size_t)(atom + gridDim.x) * NP;
-      if (tid < NP) prefetch_l2(a.QK + (nb + tid) * ld, (uint32_t)(2 * NH * 128 * sizeof(float)));
-      if (issuer) prefetch_l2(a.G + nb * a.m1, (uint32_t)(NP * a.m1 * sizeof(float)));
+      const size_t nb = a.row_off[atom + gridDim.x];
+      const int rows = a.row_off[atom + gridDim.x + 1] - (int)nb;
+      if (tid < rows) prefetch_l2(a.QK + (nb + tid) * ld, (uint32_t)(2 * NH * 128 * sizeof(float)));
+      if (issuer && rows > 0) prefetch_l2(a.G + nb * a.m1, (uint32_t)(rows * a.m1 * sizeof(float)));
     }
     float v[32];
     // two blocks in flight: each block's loads are issued before the
@@ -495,7 +502,7 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_fwd_bf16x(const __grid_c
     load_blk(a.G + base * a.m1, a.m1, nn, a.m1, v);
     load_blk(a.QK + base * ld, ld, nn, 128, w);  // Q, first half
     store_blk_split(sGh, sGl, v);
-    if (tid < 128) s_key[tid] = tid < nn ? reinterpret_cast<const float4*>(a.rw)[base + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < 128) s_key[tid] = tid < nn ? reinterpret_cast<const float4*>(a.rw)[gbase + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
     // S = sum over the halves of Q_h K_h^T (three split products each) -> TMEM [0, 128)
 #pragma unroll 1
     for (int h = 0; h < NH; ++h) {
@@ -587,10 +594,6 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_fwd_bf16x(const __grid_c
       }
     }
     __syncthreads();
-    // live rows only: every later reader of P G works row by row, and the
-    // cores read no row past the last neighbour.  (The adjoint core's dE/dQ,
-    // dE/dK stores stay whole-block: restricted to the live rows they made
-    // the width-256 core 16 % slower.)
     stg_to_global<false>(stg, a.PG + base * a.ldpg, a.ldpg, nn, a.ldpg < 128 ? a.ldpg : 128);
     fence_before_sync();
     __syncthreads();
@@ -765,16 +768,17 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_bwd_bf16x(const __grid_c
   constexpr int AW = NH * 128;  // attention width
   for (int atom = blockIdx.x; atom < a.n && sy.ok; atom += gridDim.x) {
     const int nn = a.nnei[atom];
-    const size_t base = (size_t)atom * NP;
+    const size_t base = a.row_off[atom], gbase = (size_t)atom * NP;
     const bool rv = row < nn;
     const float* qk0 = a.QK + base * ld;  // this atom's Q | K block
     // the next atom's Q and K rows, dPG and layer input into L2
     if (atom + (int)gridDim.x < a.n) {
-      const size_t nb = (size_t)(atom + gridDim.x) * NP;
-      if (tid < NP) prefetch_l2(a.QK + (nb + tid) * ld, (uint32_t)(2 * AW * sizeof(float)));
-      if (issuer) {
-        prefetch_l2(a.dPG + nb * a.ldpg, (uint32_t)(NP * a.ldpg * sizeof(float)));
-        prefetch_l2(a.G + nb * a.m1, (uint32_t)(NP * a.m1 * sizeof(float)));
+      const size_t nb = a.row_off[atom + gridDim.x];
+      const int rows = a.row_off[atom + gridDim.x + 1] - (int)nb;
+      if (tid < rows) prefetch_l2(a.QK + (nb + tid) * ld, (uint32_t)(2 * AW * sizeof(float)));
+      if (issuer && rows > 0) {
+        prefetch_l2(a.dPG + nb * a.ldpg, (uint32_t)(rows * a.ldpg * sizeof(float)));
+        prefetch_l2(a.G + nb * a.m1, (uint32_t)(rows * a.m1 * sizeof(float)));
       }
     }
     float v[32], q32[32];
@@ -791,7 +795,7 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_bwd_bf16x(const __grid_c
     load_blk(qk0, ld, nn, 128, q32);  // Q, first half
     store_blk_split(T[5], T[6], v);
     store_blk<false>(T[4], q32);
-    if (tid < 128) s_key[tid] = tid < nn ? reinterpret_cast<const float4*>(a.rw)[base + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < 128) s_key[tid] = tid < nn ? reinterpret_cast<const float4*>(a.rw)[gbase + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
     handoff();
     // dP = dPG G^T -> [128, 256); S = Q0_hi K0^T -> [0, 128)
     if (issuer) {
@@ -896,8 +900,8 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_bwd_bf16x(const __grid_c
       tmem_to_stg(tm + lane_off + c0, stg01, row, c0);
       tmem_to_stg(tm + lane_off + 128 + c0, stg23, row, c0);
       __syncthreads();
-      stg_to_global<false>(stg01, dqk, ld, 128, 128);
-      stg_to_global<false>(stg23, dqk + 128, ld, 128, 128);
+      stg_to_global<false>(stg01, dqk, ld, nn, 128);
+      stg_to_global<false>(stg23, dqk + 128, ld, nn, 128);
       __syncthreads();
       tmem_to_stg(tm + lane_off + 256 + c0, stg01, row, c0);
       tmem_to_stg(tm + lane_off + 384 + c0, stg23, row, c0);
@@ -913,11 +917,11 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_bwd_bf16x(const __grid_c
     __syncthreads();
     // dK (NH = 1: dQ | dK; NH = 2: dK0 | dK1) from the staging, and dgeo
     if constexpr (NH == 1) {
-      stg_to_global<false>(stg01, dqk, ld, 128, 128);
-      stg_to_global<false>(reinterpret_cast<float*>(T[2]), dqk + AW, ld, 128, 128);
+      stg_to_global<false>(stg01, dqk, ld, nn, 128);
+      stg_to_global<false>(reinterpret_cast<float*>(T[2]), dqk + AW, ld, nn, 128);
     } else {
-      stg_to_global<false>(stg01, dqk + AW, ld, 128, 128);
-      stg_to_global<false>(reinterpret_cast<float*>(T[2]), dqk + AW + 128, ld, 128, 128);
+      stg_to_global<false>(stg01, dqk + AW, ld, nn, 128);
+      stg_to_global<false>(reinterpret_cast<float*>(T[2]), dqk + AW + 128, ld, nn, 128);
     }
     if (tid < nn) {
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -928,7 +932,7 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_bwd_bf16x(const __grid_c
         s.x += r.x + c.x; s.y += r.y + c.y; s.z += r.z + c.z; s.w += r.w + c.w;
       }
       // one writer per row in a launch: a reduction without a return
-      atomicAdd(reinterpret_cast<float4*>(a.dgeo) + base + tid, s);
+      atomicAdd(reinterpret_cast<float4*>(a.dgeo) + gbase + tid, s);
     }
     fence_before_sync();
     __syncthreads();
@@ -1057,7 +1061,7 @@ void bf16x_free(dp_model* m) {
 }
 
 int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const float* bias, const float* R, int ldr,
-               float* C, int ldc, int M, int epi, cudaStream_t st) {
+               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev) {
   if (M <= 0) return DP_OK;
   CUtensorMap map;
   const cuuint64_t dims[2] = {(cuuint64_t)im.K, (cuuint64_t)M};
@@ -1080,11 +1084,11 @@ int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const flo
   a.nkb = im.nkb;
   a.bn_max = im.bn_max;
   a.epi = epi;
-  a.mtiles = (M + XBM - 1) / XBM;
+  a.m_dev = m_dev;
   a.err = m->d_err;
   // persistent: about one CTA per SM over the N blocks
   const int per_n = std::max(1, x_sm_count(m->device) / im.nnb);
-  dim3 grid((unsigned)std::min(a.mtiles, per_n), (unsigned)im.nnb);
+  dim3 grid((unsigned)std::min((M + XBM - 1) / XBM, per_n), (unsigned)im.nnb);
   k_gemm_bf16x<<<grid, XTHREADS, x_smem(im.bn_max), st>>>(map, a);
   note_launch();
   return DP_OK;
@@ -1103,6 +1107,7 @@ XCoreArgs core_args(dp_model* m, int n, int l) {
   a.dgeo = ws.dgeo;
   a.rw = ws.rw;
   a.nnei = ws.nnei;
+  a.row_off = ws.row_off;
   a.n = n;
   a.m1 = m->m1;
   a.ldpg = pg_ld(m->m1);

@@ -138,8 +138,8 @@ struct RowPos {
     const int atom = rg / NP;
     ti = a.atype[atom];
     tj = a.atype[a.nlist[rg]];
-    g0 = (size_t)atom * NP * a.m1 + (size_t)(rg % NP) * 4;
-    gs = NP * 4;
+    g0 = a.packed ? (size_t)p * a.m1 : (size_t)atom * NP * a.m1 + (size_t)(rg % NP) * 4;
+    gs = a.packed ? 4 : NP * 4;
   }
   __device__ size_t quad(int c) const { return g0 + (size_t)(c >> 2) * gs; }
 };

@@ -36,6 +36,11 @@ void launch_neighbors(const NbrArgs& a, cudaStream_t st);
 // arrays (ncells_total of them, at most cell_cap).  n is the pass's slots.
 void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell_base, int cb0, int ncells_total,
                              cudaStream_t st);
+// Live neighbour rows: row_off[i] (i <= n) = sum of nnei over atoms before i, and
+// rowmap[row_off[i] + s] = i * NP + s for s < nnei[i].  seg: scratch, one int per
+// ROW_SEG atoms.
+constexpr int ROW_SEG = 4096;
+void launch_row_list(const int* nnei, int n, int* row_off, int* rowmap, int* seg, cudaStream_t st);
 void launch_reverse(const int* nlist, int n, int* rev_cnt, int* rev_rows, int* err, cudaStream_t st);
 
 // --- environment matrix and its adjoint, forces, reductions (env.cu)
@@ -104,8 +109,9 @@ void launch_force_virial(const ForceArgs& a, cudaStream_t st);
 // --- FP32 SIMT network kernels (simt.cu)
 enum Epi { EPI_BIAS = 0, EPI_TANH = 1, EPI_RES_TANH = 2, EPI_ACCUM = 3, EPI_RES = 4 };
 // C[M][N] (ldc) = epi(A[M][K] (lda) * B[K][N] (ldb) + bias[N]); R is the residual (ldr).
+// m_dev non-null: the rows are *m_dev (device, <= M).
 void gemm_f32(const float* A, int lda, const float* B, int ldb, const float* bias, const float* R, int ldr,
-              float* C, int ldc, int M, int N, int K, int epi, cudaStream_t st);
+              float* C, int ldc, int M, int N, int K, int epi, cudaStream_t st, const int* m_dev = nullptr);
 
 struct EmbedArgs {
   const float* R;
@@ -117,29 +123,31 @@ struct EmbedArgs {
   const float* Gt;  // [ntypes][ntypes][m1]
   const float* b0t; // concat type-embedding mode: first-layer bias per (centre, neighbour)
                     // type [ntypes][ntypes][E0]; null: the b0 of the packed weights
-  float* G0;        // [rows][m1]
-  const float* dG0;  // backward only
+  float* G0;         // forward out: row p of the list at p * m1 (packed), or column-quad
+                     // interleaved in its atom's block
+  const float* dG0;  // backward in, laid out as G0
   float* dR;         // backward only: dR[:,0] +=
-  // row kernels: the list of live rows (atom * NP + slot) and its length (device)
-  const int* rowmap = nullptr;
+  const int* rowmap = nullptr;  // the list of live rows (atom * NP + slot) and its length (device)
   const int* nrows = nullptr;
+  int packed = 0;
 };
-// The net over a list of live rows, G0 and dG0 column-quad interleaved per atom
-// (embed.cu): forward, or adjoint.
+// The net over the list of live rows (embed.cu): forward, or adjoint.
 bool launch_embed_rows(const EmbedArgs& a, const int* widths, bool bwd, cudaStream_t st);
-bool launch_embed_fwd(const EmbedArgs& a, const int* widths, cudaStream_t st);
-bool launch_embed_bwd(const EmbedArgs& a, const int* widths, cudaStream_t st);
 
-void launch_ln_res_fwd(const float* Y, const float* Gin, const int* nlist, const float* gamma, const float* beta,
+// LayerNorm over packed rows: *nrows of them, at most rows.
+void launch_ln_res_fwd(const float* Y, const float* Gin, const int* nrows, const float* gamma, const float* beta,
                        float eps, float* Gout, float* stats, int rows, int m1, cudaStream_t st);
-void launch_ln_bwd(const float* dZ, const float* Y, const float* stats, const int* nlist, const float* gamma,
+void launch_ln_bwd(const float* dZ, const float* Y, const float* stats, const int* nrows, const float* gamma,
                    float* dY, int rows, int m1, cudaStream_t st);
 
+// Rows of QK, G, PG, dPG, dQK and dG are packed (atom i's at row_off[i]), those of
+// rw, w64 and dgeo at i * NP.
 struct AttnArgs {
   const float* QK;   // [rows][ldq]: Q | K (A columns each)
   const float* rw;   // [rows][4]
   const double* w64; // [rows] switch weights in FP64
   const int* nnei;
+  const int* row_off;
   int n, A, ldq;
   float shift;
   const float* G;    // [rows][m1] layer input
@@ -163,9 +171,10 @@ struct DescArgs {
   float* T;   // [n][4][m1]
   float* X;   // [n][fit_in]
   const float* dX;  // bwd
-  float* dG;        // bwd [rows][m1]
+  float* dG;        // bwd, laid out as G
   float* dR;        // bwd [rows][4] (written)
-  int cq;           // G and dG column-quad interleaved per atom (else row-major)
+  int cq;           // G and dG column-quad interleaved per atom (else packed rows, atom i's at row_off[i])
+  const int* row_off;
 };
 void launch_desc_fwd(const DescArgs& a, cudaStream_t st);
 void launch_desc_bwd(const DescArgs& a, cudaStream_t st);
@@ -201,23 +210,25 @@ struct JvpArgs {
   const int* nnei;      // [n]
   const int* atype;     // [n] (range-checked)
   int n, ntypes, m1, axis, fit_in, sel;
+  const int* row_off;   // [n + 1], rowmap: the packed rows of G, dG, Gd and dGd
+  const int* rowmap;
   const float* dstd;    // [ntypes][4]
   float rcs, rc;
   const float* R;       // [rows][4] environment rows
-  const float* G;       // [rows][m1] embedding output (row-major)
+  const float* G;       // [packed rows][m1] embedding output
   const float* T;       // [n][4][m1]
   const float* dX;      // [n][fit_in] dE/dX
-  const float* dG;      // [rows][m1] dE/dG
+  const float* dG;      // [packed rows][m1] dE/dG
   const float* w;       // packed embedding-net weights (W0 b0 W1 b1 W2 b2)
   const float* Gt;      // [ntypes][ntypes][m1]
   const float* b0t;     // concat mode: first-layer bias per (centre, neighbour) type, or null
   const double* v;      // [n][3] the direction
   float* Rd;            // [rows][4]   R'
-  float* Gd;            // [rows][m1]  G'
+  float* Gd;            // [packed rows][m1]  G'
   float* Td;            // [n][4][m1]  T'
   float* Xd;            // [n][fit_in] X'
   const float* dXd;     // [n][fit_in] (dE/dX)'
-  float* dGd;           // [rows][m1]  (dE/dG)'
+  float* dGd;           // [packed rows][m1]  (dE/dG)'
 };
 void launch_env_jvp(const JvpArgs& a, cudaStream_t st);
 // mode 0: G'; mode 1: grad += *scale * (dE/d(embedding weights))'

@@ -92,6 +92,9 @@ struct Workspace {
   int *cell_of, *cell_count, *cell_start, *cell_cursor, *cell_atoms;
   int cell_cap, cap_dim;
   int *nlist, *nnei, *ncand, *rev_cnt, *rev_rows;
+  // the live neighbour rows in order: first row of each atom [cap + 1], and each
+  // row's place atom * NP + slot (launch_row_list)
+  int *row_off, *rowmap, *row_seg;
   int* atype_c;  // device-checked copy of the atom types
   float4* coordf;  // FP32 coordinates (neighbour screen)
   // environment
@@ -99,7 +102,8 @@ struct Workspace {
   double* w64;
   // network
   // modular layer layout (FP32, bf16x): per layer Q | K, [P G, rowsum P], Y and
-  // the LayerNorm statistics; dE/d[P G, rowsum P] and dE/d[Q K] for the adjoint
+  // the LayerNorm statistics; dE/d[P G, rowsum P] and dE/d[Q K] for the adjoint;
+  // like G and dG there, row-major over the packed live rows
   std::vector<float*> G, QK, PG, Y, stats;
   float *dG, *dY, *dPG, *dQK;
   float *T, *X, *dX, *e;
@@ -198,10 +202,7 @@ using HostArrays = std::vector<std::pair<std::string, std::vector<double>>>;
 int tc_init_weights(dp_model* m, const HostArrays& arrays, std::string& msg);
 // tensor-core embedding net, tc_embed.cu
 int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg);
-void tc_embed_bf16(dp_model* m, int n, const int* atype, bool bwd, float* G0, const float* dG0, float* dR,
-                   float* H12, cudaStream_t st);
-void tc_live_rows(dp_model* m, int n, cudaStream_t st);
-void tc_embed_fused(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st);
+void tc_embed(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st);
 void tc_plan_buffers(dp_model* m, Arena& a, int cap);
 void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st);
 void tc_free_weights(dp_model* m);
@@ -215,7 +216,7 @@ int bf16x_init_weights(dp_model* m, std::string& msg);
 void bf16x_refresh(dp_model* m, cudaStream_t st);
 void bf16x_free(dp_model* m);
 int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const float* bias, const float* R, int ldr,
-               float* C, int ldc, int M, int epi, cudaStream_t st);
+               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev = nullptr);
 void attn_core_fwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 void attn_core_bwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 // the fused 16-bit layer kernels (tc.cu) serve DP_PREC_BF16 and DP_PREC_FP16X;

@@ -336,6 +336,68 @@ void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell
   note_launch();
 }
 
+// The list of live rows: a block of 256 threads takes ROWL_ATOMS atoms.  Its first
+// place is the sum of the counts before it: those of whole ROW_SEG segments from
+// seg (written by k_row_seg; a single segment needs none), the rest summed here.
+constexpr int ROWL_ATOMS = 32, ROWL_T = 256;
+
+__device__ __forceinline__ int block_sum(int v, int* s_red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int t = 0;
+#pragma unroll
+  for (int w = 0; w < ROWL_T / 32; ++w) t += s_red[w];
+  return t;
+}
+
+__global__ void __launch_bounds__(ROWL_T) k_row_seg(const int* __restrict__ nnei, int n, int* __restrict__ seg) {
+  __shared__ int s_red[ROWL_T / 32];
+  int v = 0;
+  for (int i = blockIdx.x * ROW_SEG + threadIdx.x; i < min(n, (int)(blockIdx.x + 1) * ROW_SEG); i += ROWL_T) v += nnei[i];
+  v = block_sum(v, s_red);
+  if (threadIdx.x == 0) seg[blockIdx.x] = v;
+}
+
+__global__ void __launch_bounds__(ROWL_T) k_row_list(const int* __restrict__ nnei, int n, const int* __restrict__ seg,
+                                                     int* __restrict__ row_off, int* __restrict__ rowmap) {
+  __shared__ int s_red[ROWL_T / 32], s_off[ROWL_ATOMS];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int first = blockIdx.x * ROWL_ATOMS, s0 = first / ROW_SEG;
+  int v = 0;
+  for (int k = t; k < s0; k += ROWL_T) v += seg[k];
+  for (int i = s0 * ROW_SEG + t; i < first; i += ROWL_T) v += nnei[i];
+  const int base = block_sum(v, s_red);
+  if (w == 0) {
+    const int nn = first + lane < n ? nnei[first + lane] : 0;
+    int x = nn;  // inclusive sum over the block's atoms
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+    s_off[lane] = base + x - nn;
+    if (first + lane < n) row_off[first + lane] = base + x - nn;
+    if (first + lane == n - 1) row_off[n] = base + x;
+  }
+  __syncthreads();
+  for (int j = w; j < ROWL_ATOMS && first + j < n; j += ROWL_T / 32) {
+    const int nj = nnei[first + j], oj = s_off[j];
+    for (int s = lane; s < nj; s += 32) rowmap[oj + s] = (first + j) * NP + s;
+  }
+}
+
+void launch_row_list(const int* nnei, int n, int* row_off, int* rowmap, int* seg, cudaStream_t st) {
+  if (n == 0) return;
+  if (n > ROW_SEG) {
+    k_row_seg<<<(n + ROW_SEG - 1) / ROW_SEG, ROWL_T, 0, st>>>(nnei, n, seg);
+    note_launch();
+  }
+  k_row_list<<<(n + ROWL_ATOMS - 1) / ROWL_ATOMS, ROWL_T, 0, st>>>(nnei, n, seg, row_off, rowmap);
+  note_launch();
+}
+
 void launch_reverse(const int* nlist, int n, int* rev_cnt, int* rev_rows, int* err, cudaStream_t st) {
   cudaMemsetAsync(rev_cnt, 0, sizeof(int) * (size_t)(n > 0 ? n : 1), st);
   if (n == 0) return;

@@ -22,7 +22,9 @@ template <int EPI, bool VEC>
 __global__ void __launch_bounds__(256, 2)
 k_sgemm128(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
            const float* __restrict__ bias, const float* __restrict__ R, int ldr, float* __restrict__ C, int ldc,
-           int M, int N, int K) {
+           int M, int N, int K, const int* __restrict__ m_dev) {
+  if (m_dev) M = *m_dev;
+  if ((long long)blockIdx.x * 128 >= M) return;
   __shared__ __align__(16) float As[2][GBK][GLD];  // k-major: As[k][row]
   __shared__ __align__(16) float Bs[2][GBK][GLD];  // Bs[k][column]
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -140,15 +142,16 @@ k_sgemm128(const float* __restrict__ A, int lda, const float* __restrict__ B, in
 
 template <int EPI>
 static void sgemm_launch(dim3 grid, bool vec, const float* A, int lda, const float* B, int ldb, const float* bias,
-                         const float* R, int ldr, float* C, int ldc, int M, int N, int K, cudaStream_t st) {
+                         const float* R, int ldr, float* C, int ldc, int M, int N, int K, const int* m_dev,
+                         cudaStream_t st) {
   if (vec)
-    k_sgemm128<EPI, true><<<grid, 256, 0, st>>>(A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K);
+    k_sgemm128<EPI, true><<<grid, 256, 0, st>>>(A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev);
   else
-    k_sgemm128<EPI, false><<<grid, 256, 0, st>>>(A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K);
+    k_sgemm128<EPI, false><<<grid, 256, 0, st>>>(A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev);
 }
 
 void gemm_f32(const float* A, int lda, const float* B, int ldb, const float* bias, const float* R, int ldr,
-              float* C, int ldc, int M, int N, int K, int epi, cudaStream_t st) {
+              float* C, int ldc, int M, int N, int K, int epi, cudaStream_t st, const int* m_dev) {
   if (M <= 0 || N <= 0) return;
   dim3 grid((unsigned)((M + 127) / 128), (unsigned)((N + 127) / 128));
   const bool res = epi == EPI_RES || epi == EPI_RES_TANH;
@@ -157,21 +160,20 @@ void gemm_f32(const float* A, int lda, const float* B, int ldb, const float* bia
   const bool vec = (addr & 15) == 0 && lda % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 && (!res || ldr % 4 == 0) &&
                    N % 4 == 0 && K % 4 == 0;
   switch (epi) {
-    case EPI_BIAS: sgemm_launch<EPI_BIAS>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, st); break;
-    case EPI_TANH: sgemm_launch<EPI_TANH>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, st); break;
-    case EPI_RES_TANH: sgemm_launch<EPI_RES_TANH>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, st); break;
-    case EPI_ACCUM: sgemm_launch<EPI_ACCUM>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, st); break;
-    default: sgemm_launch<EPI_RES>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, st); break;
+    case EPI_BIAS: sgemm_launch<EPI_BIAS>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev, st); break;
+    case EPI_TANH: sgemm_launch<EPI_TANH>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev, st); break;
+    case EPI_RES_TANH: sgemm_launch<EPI_RES_TANH>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev, st); break;
+    case EPI_ACCUM: sgemm_launch<EPI_ACCUM>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev, st); break;
+    default: sgemm_launch<EPI_RES>(grid, vec, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev, st); break;
   }
   note_launch();
 }
 
-// ------------------------------------------------------------ embedding net
-// G0_ij = net_s(R_ij,0) * (1 + Gt[t_i, t_j]); net_s = 1 -> E0 -> E1 -> E2 with
-// tanh and the residual rule (keep width: x + f; double: [x, x] + f).
-// A CTA takes 64 neighbour rows of one atom; activations of the block live in
-// shared memory and every layer is a small tiled product over the block, so
-// global rows are read and written whole (coalesced).
+// --------------------------------------- weight gradient of the embedding net
+// net_s = 1 -> E0 -> E1 -> E2 with tanh and the residual rule (keep width: x +
+// f; double: [x, x] + f).  A CTA takes 64 packed neighbour rows at a time;
+// their activations live in shared memory and every layer is a small tiled
+// product over the block.
 template <int E0, int E1, int E2>
 struct EmbedLayout {  // packed global weights: W0 b0 W1 b1 W2 b2
   static constexpr int W0 = 0, B0 = E0, W1 = 2 * E0, B1 = W1 + E0 * E1, W2 = B1 + E1, B2 = W2 + E1 * E2,
@@ -194,26 +196,27 @@ struct EmbedSmem {
   static constexpr int W0 = 0, B0 = E0, W1 = 2 * E0, B1 = W1 + E0 * E1, W2 = B1 + E1, B2 = W2 + E1 * P2,
                        X = B2 + E2, H1 = X + EROWS, H2 = H1 + EROWS * (E0 + 1), Z = H2 + EROWS * (E1 + 1),
                        DH2 = Z + EROWS * (E2 + 1), DZ2 = DH2 + EROWS * (E1 + 1), DH1 = DZ2 + EROWS * (E1 + 1),
-                       TJ = DH1 + EROWS * (E0 + 1), TOTAL = TJ + EROWS;  // TJ: the rows' neighbour types (int)
+                       TJ = DH1 + EROWS * (E0 + 1), TOTAL = TJ + EROWS;  // TJ: the rows' type pairs (int)
 };
 
 template <int E0, int E1, int E2>
-__device__ __forceinline__ void embed_load(float* sm, const EmbedArgs& a, size_t base, int cnt) {
+__device__ __forceinline__ void embed_load(float* sm, const EmbedArgs& a, int p0, int cnt) {
   using Lw = EmbedLayout<E0, E1, E2>;
   using S = EmbedSmem<E0, E1, E2>;
   for (int t = threadIdx.x; t < Lw::W2; t += ETHREADS) sm[t] = a.w[t];  // W0 b0 W1 b1 share offsets
   for (int t = threadIdx.x; t < E1 * E2; t += ETHREADS) sm[S::W2 + (t / E2) * S::P2 + t % E2] = a.w[Lw::W2 + t];
   for (int t = threadIdx.x; t < E2; t += ETHREADS) sm[S::B2 + t] = a.w[Lw::B2 + t];
   for (int r = threadIdx.x; r < EROWS; r += ETHREADS) {
-    sm[S::X + r] = r < cnt ? a.R[(base + r) * 4] : 0.f;
-    reinterpret_cast<int*>(sm + S::TJ)[r] = r < cnt ? a.atype[a.nlist[base + r]] : 0;
+    const int rg = r < cnt ? a.rowmap[p0 + r] : 0;
+    sm[S::X + r] = r < cnt ? a.R[(size_t)rg * 4] : 0.f;
+    reinterpret_cast<int*>(sm + S::TJ)[r] = r < cnt ? a.atype[rg / NP] * a.ntypes + a.atype[a.nlist[rg]] : 0;
   }
   __syncthreads();
 }
 
 // Layers 1 and 2, then Z = H2 W2 + b2 (4 rows per thread per weight load).
-// b0t: the centre type's rows of the concat mode's first-layer bias table
-// ([neighbour type][E0]), or null (strip mode: b0).
+// b0t: the concat mode's first-layer bias table ([type pair][E0]), or null
+// (strip mode: b0).
 template <int E0, int E1, int E2>
 __device__ __forceinline__ void embed_forward(float* sm, int cnt, const float* b0t) {
   using S = EmbedSmem<E0, E1, E2>;
@@ -261,131 +264,6 @@ __device__ __forceinline__ void embed_forward(float* sm, int cnt, const float* b
   __syncthreads();
 }
 
-template <int E0, int E1, int E2>
-__global__ void __launch_bounds__(ETHREADS) k_embed_fwd(EmbedArgs a) {
-  using S = EmbedSmem<E0, E1, E2>;
-  extern __shared__ float sm[];
-  const int atom = blockIdx.x >> 1, part = blockIdx.x & 1;
-  const int r0 = part * EROWS;
-  const int cnt = max(0, min(EROWS, a.nnei[atom] - r0));
-  const size_t base = (size_t)atom * NP + r0;
-  if (cnt > 0) {
-    embed_load<E0, E1, E2>(sm, a, base, cnt);
-    embed_forward<E0, E1, E2>(sm, cnt, a.b0t ? a.b0t + (size_t)a.atype[atom] * a.ntypes * E0 : nullptr);
-  }
-  const int ti = a.atype[atom];
-  for (int idx = threadIdx.x; idx < EROWS * E2; idx += ETHREADS) {
-    const int r = idx / E2, c = idx % E2;
-    float g = 0.f;
-    if (r < cnt) {
-      const int tj = a.atype[a.nlist[base + r]];
-      const float h3 = skip_in<E1, E2>(sm + S::H2 + r * (E1 + 1), c) + tanhf(sm[S::Z + r * (E2 + 1) + c]);
-      g = h3 * (1.f + a.Gt[((size_t)ti * a.ntypes + tj) * E2 + c]);
-    }
-    a.G0[(base + r) * a.m1 + c] = g;
-  }
-}
-
-// Adjoint: dR[:,0] += d net_s / dx . (dG0 * (1 + Gt)), recomputing the
-// forward activations of the block.
-template <int E0, int E1, int E2>
-__global__ void __launch_bounds__(ETHREADS) k_embed_bwd(EmbedArgs a) {
-  using S = EmbedSmem<E0, E1, E2>;
-  extern __shared__ float sm[];
-  const int atom = blockIdx.x >> 1, part = blockIdx.x & 1;
-  const int r0 = part * EROWS;
-  const int cnt = max(0, min(EROWS, a.nnei[atom] - r0));
-  if (cnt == 0) return;
-  const size_t base = (size_t)atom * NP + r0;
-  embed_load<E0, E1, E2>(sm, a, base, cnt);
-  embed_forward<E0, E1, E2>(sm, cnt, a.b0t ? a.b0t + (size_t)a.atype[atom] * a.ntypes * E0 : nullptr);
-  const int ti = a.atype[atom];
-  // Z <- dZ3 = g (1 - t3^2) with g = dG0 (1 + Gt); the skip part of dH2 is
-  // summed from g directly below
-  for (int idx = threadIdx.x; idx < EROWS * E2; idx += ETHREADS) {
-    const int r = idx / E2, c = idx % E2;
-    float dz = 0.f;
-    if (r < cnt) {
-      const int tj = a.atype[a.nlist[base + r]];
-      const float g = a.dG0[(base + r) * a.m1 + c] * (1.f + a.Gt[((size_t)ti * a.ntypes + tj) * E2 + c]);
-      const float t = tanhf(sm[S::Z + r * (E2 + 1) + c]);
-      dz = g * (1.f - t * t);
-    }
-    sm[S::Z + r * (E2 + 1) + c] = dz;
-  }
-  __syncthreads();
-  // dH2[r][b] = skip^T(g)[b] + sum_c W2[b][c] dZ3[r][c], four rows per
-  // thread so that each weight load serves four products (dZ3 is zero on
-  // rows past cnt)
-  for (int idx = threadIdx.x; idx < (EROWS / 4) * E1; idx += ETHREADS) {
-    const int r0 = (idx / E1) * 4, b = idx % E1;
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-    if (r0 < cnt) {
-      const float* dz = sm + S::Z + r0 * (E2 + 1);
-      const float* w2 = sm + S::W2 + b * S::P2;
-#pragma unroll 4
-      for (int c = 0; c < E2; ++c) {
-        const float w = w2[c];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) s[u] = fmaf(w, dz[u * (E2 + 1) + c], s[u]);
-      }
-      if (E2 == E1 || E2 == 2 * E1) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + u;
-          if (r >= cnt) break;
-          const int tj = a.atype[a.nlist[base + r]];
-          const float* gt = a.Gt + ((size_t)ti * a.ntypes + tj) * E2;
-          const float* dg = a.dG0 + (base + r) * a.m1;
-          for (int c = b; c < E2; c += E1) s[u] += dg[c] * (1.f + gt[c]);
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) sm[S::DH2 + (r0 + u) * (E1 + 1) + b] = r0 + u < cnt ? s[u] : 0.f;
-  }
-  __syncthreads();
-  // dZ2 = dH2 (1 - t2^2) with t2 = H2 - skip(H1)
-  for (int idx = threadIdx.x; idx < EROWS * E1; idx += ETHREADS) {
-    const int r = idx / E1, b = idx % E1;
-    const float t = sm[S::H2 + r * (E1 + 1) + b] - skip_in<E0, E1>(sm + S::H1 + r * (E0 + 1), b);
-    sm[S::DZ2 + r * (E1 + 1) + b] = sm[S::DH2 + r * (E1 + 1) + b] * (1.f - t * t);
-  }
-  __syncthreads();
-  // dH1[r][p] = skip^T(dH2)[p] + sum_b W1[p][b] dZ2[r][b]; term of dx: W0[p]
-  // dH1 (1 - H1^2); four rows per thread as above (dZ2 is zero past cnt)
-  for (int idx = threadIdx.x; idx < (EROWS / 4) * E0; idx += ETHREADS) {
-    const int r0 = (idx / E0) * 4, p = idx % E0;
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-    if (r0 < cnt) {
-      const float* dz2 = sm + S::DZ2 + r0 * (E1 + 1);
-      const float* w1 = sm + S::W1 + p * E1;
-#pragma unroll 5
-      for (int b = 0; b < E1; ++b) {
-        const float w = w1[b];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) s[u] = fmaf(w, dz2[u * (E1 + 1) + b], s[u]);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u;
-        if (E1 == E0 || E1 == 2 * E0)
-          for (int b = p; b < E1; b += E0) s[u] += sm[S::DH2 + r * (E1 + 1) + b];
-        const float h1 = sm[S::H1 + r * (E0 + 1) + p];
-        s[u] = s[u] * (1.f - h1 * h1) * sm[S::W0 + p];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) sm[S::DH1 + (r0 + u) * (E0 + 1) + p] = r0 + u < cnt ? s[u] : 0.f;
-  }
-  __syncthreads();
-  for (int r = threadIdx.x; r < cnt; r += ETHREADS) {
-    float dx = 0.f;
-    for (int p = 0; p < E0; ++p) dx += sm[S::DH1 + r * (E0 + 1) + p];
-    a.dR[(base + r) * 4] += dx;
-  }
-}
-
 // Weight gradients of the embedding net, scale * dE/d(W0 b0 W1 b1 W2 b2)
 // (packed layout), accumulated over every neighbour row.  Persistent CTAs
 // walk the 64-row blocks, keep per-CTA sums in shared memory and add them to
@@ -397,22 +275,19 @@ __global__ void __launch_bounds__(ETHREADS) k_embed_wgrad(EmbedArgs a, float* gr
   extern __shared__ float sm[];
   float* acc = sm + S::TOTAL;
   for (int t = threadIdx.x; t < Lw::TOTAL; t += ETHREADS) acc[t] = 0.f;
-  for (int blk = blockIdx.x; blk < 2 * a.n; blk += gridDim.x) {
-    const int atom = blk >> 1, part = blk & 1;
-    const int r0 = part * EROWS;
-    const int cnt = max(0, min(EROWS, a.nnei[atom] - r0));
-    if (cnt == 0) continue;  // uniform over the CTA
-    const size_t base = (size_t)atom * NP + r0;
+  const int* pair = reinterpret_cast<const int*>(sm + S::TJ);
+  const int nrows = *a.nrows;
+  for (int p0 = blockIdx.x * EROWS; p0 < nrows; p0 += gridDim.x * EROWS) {
+    const int cnt = min(EROWS, nrows - p0);
+    const size_t base = p0;
     __syncthreads();
-    embed_load<E0, E1, E2>(sm, a, base, cnt);
-    embed_forward<E0, E1, E2>(sm, cnt, a.b0t ? a.b0t + (size_t)a.atype[atom] * a.ntypes * E0 : nullptr);
-    const int ti = a.atype[atom];
+    embed_load<E0, E1, E2>(sm, a, p0, cnt);
+    embed_forward<E0, E1, E2>(sm, cnt, a.b0t);
     for (int idx = threadIdx.x; idx < EROWS * E2; idx += ETHREADS) {
       const int r = idx / E2, c = idx % E2;
       float dz = 0.f;
       if (r < cnt) {
-        const int tj = a.atype[a.nlist[base + r]];
-        const float g = a.dG0[(base + r) * a.m1 + c] * (1.f + a.Gt[((size_t)ti * a.ntypes + tj) * E2 + c]);
+        const float g = a.dG0[(base + r) * a.m1 + c] * (1.f + a.Gt[(size_t)pair[r] * E2 + c]);
         const float t = tanhf(sm[S::Z + r * (E2 + 1) + c]);
         dz = g * (1.f - t * t);
       }
@@ -427,8 +302,7 @@ __global__ void __launch_bounds__(ETHREADS) k_embed_wgrad(EmbedArgs a, float* gr
         const float* w2 = sm + S::W2 + b * S::P2;
         for (int c = 0; c < E2; ++c) sacc = fmaf(w2[c], dz[c], sacc);
         if (E2 == E1 || E2 == 2 * E1) {
-          const int tj = a.atype[a.nlist[base + r]];
-          const float* gt = a.Gt + ((size_t)ti * a.ntypes + tj) * E2;
+          const float* gt = a.Gt + (size_t)pair[r] * E2;
           const float* dg = a.dG0 + (base + r) * a.m1;
           for (int c = b; c < E2; c += E1) sacc += dg[c] * (1.f + gt[c]);
         }
@@ -502,39 +376,14 @@ bool launch_embed_wgrad(const EmbedArgs& a, const int* w, float* grad, const flo
   return false;
 }
 
-template <int E0, int E1, int E2>
-static void embed_launch(const EmbedArgs& a, bool bwd, cudaStream_t st) {
-  using S = EmbedSmem<E0, E1, E2>;
-  if (a.n == 0) return;
-  const unsigned grid = (unsigned)a.n * 2;
-  const size_t sm = sizeof(float) * S::TOTAL;
-  if (!bwd) {
-    cudaFuncSetAttribute(k_embed_fwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_embed_fwd<E0, E1, E2><<<grid, ETHREADS, sm, st>>>(a);
-  } else {
-    cudaFuncSetAttribute(k_embed_bwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_embed_bwd<E0, E1, E2><<<grid, ETHREADS, sm, st>>>(a);
-  }
-  note_launch();
-}
-
-static bool embed_dispatch(const EmbedArgs& a, const int* w, bool bwd, cudaStream_t st) {
-  if (w[0] == 25 && w[1] == 50 && w[2] == 100) { embed_launch<25, 50, 100>(a, bwd, st); return true; }
-  if (w[0] == 16 && w[1] == 32 && w[2] == 64) { embed_launch<16, 32, 64>(a, bwd, st); return true; }
-  if (w[0] == 32 && w[1] == 64 && w[2] == 128) { embed_launch<32, 64, 128>(a, bwd, st); return true; }
-  return false;
-}
-bool launch_embed_fwd(const EmbedArgs& a, const int* widths, cudaStream_t st) { return embed_dispatch(a, widths, false, st); }
-bool launch_embed_bwd(const EmbedArgs& a, const int* widths, cudaStream_t st) { return embed_dispatch(a, widths, true, st); }
-
 // ---------------------------------------------------------------- LayerNorm
-// G_out = G_in + LN(Y) on rows with a neighbour, G_out = G_in elsewhere.
-__global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restrict__ Gin, const int* __restrict__ nlist,
+// G_out = G_in + LN(Y), row by row.
+__global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restrict__ Gin, const int* __restrict__ nrows,
                              const float* __restrict__ gamma, const float* __restrict__ beta, float eps,
-                             float* __restrict__ Gout, float* __restrict__ stats, long long rows, int m1) {
+                             float* __restrict__ Gout, float* __restrict__ stats, int m1) {
   const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
+  if (row >= *nrows) return;
   const float* y = Y + row * m1;
   float v[4];
   float s = 0.f;
@@ -554,13 +403,12 @@ __global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restric
   }
   const float var = warp_sum(s2) / (float)m1;
   const float rstd = 1.0f / sqrtf(var + eps);
-  const bool valid = nlist[row] >= 0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int c = lane + 32 * q;
     if (c < m1) {
       const float gin = Gin[row * m1 + c];
-      Gout[row * m1 + c] = valid ? gin + (v[q] - mean) * rstd * gamma[c] + beta[c] : gin;
+      Gout[row * m1 + c] = gin + (v[q] - mean) * rstd * gamma[c] + beta[c];
     }
   }
   if (lane == 0) {
@@ -570,19 +418,18 @@ __global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restric
 }
 
 __global__ void k_ln_bwd(const float* __restrict__ dZ, const float* __restrict__ Y, const float* __restrict__ stats,
-                         const int* __restrict__ nlist, const float* __restrict__ gamma, float* __restrict__ dY,
-                         long long rows, int m1) {
+                         const int* __restrict__ nrows, const float* __restrict__ gamma, float* __restrict__ dY,
+                         int m1) {
   const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  const bool valid = nlist[row] >= 0;
+  if (row >= *nrows) return;
   const float mean = stats[2 * row], rstd = stats[2 * row + 1];
   float gz[4], yh[4];
   float s1 = 0.f, s2 = 0.f;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int c = lane + 32 * q;
-    if (c < m1 && valid) {
+    if (c < m1) {
       gz[q] = gamma[c] * dZ[row * m1 + c];
       yh[q] = (Y[row * m1 + c] - mean) * rstd;
     } else {
@@ -596,23 +443,22 @@ __global__ void k_ln_bwd(const float* __restrict__ dZ, const float* __restrict__
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int c = lane + 32 * q;
-    if (c < m1) dY[row * m1 + c] = valid ? rstd * (gz[q] - s1 - yh[q] * s2) : 0.f;
+    if (c < m1) dY[row * m1 + c] = rstd * (gz[q] - s1 - yh[q] * s2);
   }
 }
 
-void launch_ln_res_fwd(const float* Y, const float* Gin, const int* nlist, const float* gamma, const float* beta,
+void launch_ln_res_fwd(const float* Y, const float* Gin, const int* nrows, const float* gamma, const float* beta,
                        float eps, float* Gout, float* stats, int rows_i, int m1, cudaStream_t st) {
   long long rows = rows_i;
   if (rows == 0) return;
-  k_ln_res_fwd<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(Y, Gin, nlist, gamma, beta, eps, Gout, stats,
-                                                                      rows, m1);
+  k_ln_res_fwd<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(Y, Gin, nrows, gamma, beta, eps, Gout, stats, m1);
   note_launch();
 }
-void launch_ln_bwd(const float* dZ, const float* Y, const float* stats, const int* nlist, const float* gamma,
+void launch_ln_bwd(const float* dZ, const float* Y, const float* stats, const int* nrows, const float* gamma,
                    float* dY, int rows_i, int m1, cudaStream_t st) {
   long long rows = rows_i;
   if (rows == 0) return;
-  k_ln_bwd<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(dZ, Y, stats, nlist, gamma, dY, rows, m1);
+  k_ln_bwd<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(dZ, Y, stats, nrows, gamma, dY, m1);
   note_launch();
 }
 
@@ -772,11 +618,11 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
   const int ld = a.ldq;  // Q | K
   for (int atom = blockIdx.x; atom < a.n; atom += gridDim.x) {
     const int nn = a.nnei[atom];
-    const size_t base = (size_t)atom * NP;
+    const size_t base = a.row_off[atom], gbase = (size_t)atom * NP;
     __syncthreads();  // the previous atom is done with every shared array
     for (int r = tid; r < NP; r += FTF) {
-      rws[r] = r < nn ? reinterpret_cast<const float4*>(a.rw)[base + r] : make_float4(0.f, 0.f, 0.f, 0.f);
-      w2s[r] = split_pair(r < nn ? a.w64[base + r] : 0.0);
+      rws[r] = r < nn ? reinterpret_cast<const float4*>(a.rw)[gbase + r] : make_float4(0.f, 0.f, 0.f, 0.f);
+      w2s[r] = split_pair(r < nn ? a.w64[gbase + r] : 0.0);
     }
     float s[4][8];
 #pragma unroll
@@ -869,7 +715,8 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
       if (4 * ty < nn)
         for (int k = 0; k < nn4; k += 4) tile_fma4<4>(acc, X, Y, k, ty, tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) tile_store_row(a.PG + (base + 4 * ty + i) * a.ldpg, acc[i], c0, tx, a.ldpg);
+      for (int i = 0; i < 4; ++i)
+        if (4 * ty + i < nn) tile_store_row(a.PG + (base + 4 * ty + i) * a.ldpg, acc[i], c0, tx, a.ldpg);
     }
   }
 }
@@ -898,11 +745,11 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
   const int ld = a.ldq;  // Q | K, and dQ | dK
   for (int atom = blockIdx.x; atom < a.n; atom += gridDim.x) {
     const int nn = a.nnei[atom];
-    const size_t base = (size_t)atom * NP;
+    const size_t base = a.row_off[atom], gbase = (size_t)atom * NP;
     __syncthreads();  // the previous atom is done with every shared array
     for (int r = tid; r < NP; r += FTF) {
-      rws[r] = r < nn ? reinterpret_cast<const float4*>(a.rw)[base + r] : make_float4(0.f, 0.f, 0.f, 0.f);
-      w2s[r] = split_pair(r < nn ? a.w64[base + r] : 0.0);
+      rws[r] = r < nn ? reinterpret_cast<const float4*>(a.rw)[gbase + r] : make_float4(0.f, 0.f, 0.f, 0.f);
+      w2s[r] = split_pair(r < nn ? a.w64[gbase + r] : 0.0);
     }
     const bool live = 4 * ty < nn && 4 * tx < nn;
     float s[4][8], dp[4][8];
@@ -1038,7 +885,7 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
         acc.x += c.x; acc.y += c.y; acc.z += c.z; acc.w += c.w;
       }
       // one writer per row in a launch: a reduction without a return
-      atomicAdd(reinterpret_cast<float4*>(a.dgeo) + base + tid, acc);
+      atomicAdd(reinterpret_cast<float4*>(a.dgeo) + gbase + tid, acc);
     }
     const int nn4 = (nn + 3) & ~3;
     for (int c0 = 0; c0 < A; c0 += 128) {
@@ -1058,7 +905,8 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
       if (4 * ty < nn)
         for (int k = 0; k < nn4; k += 4) tile_fma4<4>(acc, B1, B0, k, ty, tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) tile_store_row(a.dQK + (base + 4 * ty + i) * ld, acc[i], c0, tx, A);
+      for (int i = 0; i < 4; ++i)
+        if (4 * ty + i < nn) tile_store_row(a.dQK + (base + 4 * ty + i) * ld, acc[i], c0, tx, A);
       // dK = dS^T Q: Q row-major in B0
       __syncthreads();
       for (int idx = tid; idx < NP * 32; idx += FTF) {
@@ -1074,7 +922,8 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
       if (4 * ty < nn)
         for (int j = 0; j < nn; ++j) tile_fma<4>(acc, B1, j * TLD + 4 * ty, B0, j * TLD + 4 * tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) tile_store_row(a.dQK + (base + 4 * ty + i) * ld + A, acc[i], c0, tx, A);
+      for (int i = 0; i < 4; ++i)
+        if (4 * ty + i < nn) tile_store_row(a.dQK + (base + 4 * ty + i) * ld + A, acc[i], c0, tx, A);
     }
     // dE/dG += P^T dPG: dPG row-major in B0 (columns below m1; m1 <= 128)
     __syncthreads();
@@ -1197,11 +1046,12 @@ __global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
       if (lane < 16) Ts[(lane >> 2) * a.m1 + 4 * q + (lane & 3)] = v * inv_sel;
     }
   } else {
+    const size_t gbase = a.row_off[atom];
     for (int c = threadIdx.x; c < a.m1; c += blockDim.x) {
       float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f;
       for (int s = 0; s < nn; ++s) {
         const float4 r = reinterpret_cast<const float4*>(a.R)[base + s];
-        const float gv = a.G[(base + s) * a.m1 + c];
+        const float gv = a.G[(gbase + s) * a.m1 + c];
         t0 = fmaf(r.x, gv, t0); t1 = fmaf(r.y, gv, t1); t2 = fmaf(r.z, gv, t2); t3 = fmaf(r.w, gv, t3);
       }
       Ts[c] = t0 * inv_sel; Ts[a.m1 + c] = t1 * inv_sel; Ts[2 * a.m1 + c] = t2 * inv_sel; Ts[3 * a.m1 + c] = t3 * inv_sel;
@@ -1284,26 +1134,25 @@ __global__ void k_desc_bwd(DescArgs a) {
     }
     return;
   }
-  // dG rows (all NP rows; zero on padding), a column quad per thread (m1 % 4 == 0)
+  // dG rows, a column quad per thread (m1 % 4 == 0)
   const int q4 = m1 / 4;
-  float4* dG4 = reinterpret_cast<float4*>(a.dG + base * m1);
-  for (int idx = threadIdx.x; idx < NP * q4; idx += blockDim.x) {
+  const size_t gbase = a.row_off[atom];
+  float4* dG4 = reinterpret_cast<float4*>(a.dG + gbase * m1);
+  for (int idx = threadIdx.x; idx < nn * q4; idx += blockDim.x) {
     const int s = idx / q4, q = idx % q4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (s < nn) {
-      const float4 r = reinterpret_cast<const float4*>(a.R)[base + s];
-      float* vp = &v.x;
+    const float4 r = reinterpret_cast<const float4*>(a.R)[base + s];
+    float4 v;
+    float* vp = &v.x;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int p = 4 * q + k;
-        vp[k] = r.x * dTs[p] + r.y * dTs[m1 + p] + r.z * dTs[2 * m1 + p] + r.w * dTs[3 * m1 + p];
-      }
+    for (int k = 0; k < 4; ++k) {
+      const int p = 4 * q + k;
+      vp[k] = r.x * dTs[p] + r.y * dTs[m1 + p] + r.z * dTs[2 * m1 + p] + r.w * dTs[3 * m1 + p];
     }
     dG4[idx] = v;
   }
   // dR rows: a warp per row, a column quad per lane
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const float4* G4 = reinterpret_cast<const float4*>(a.G + base * m1);
+  const float4* G4 = reinterpret_cast<const float4*>(a.G + gbase * m1);
   for (int s = warp; s < NP; s += nw) {
     float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
     if (s < nn) {

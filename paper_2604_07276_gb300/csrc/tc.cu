@@ -884,9 +884,6 @@ void tc_plan_buffers(dp_model* m, Arena& a, int cap) {
   ws.tc.p[2] = nullptr;
   // layers 1 and 2 of the tensor-core embedding net, for its adjoint
   ws.tc.p[5] = m->tcw.emb_W1_t ? a.take<float>(rows * (size_t)(m->emb[0] + m->emb[1])) : nullptr;
-  // the live neighbour rows the embedding net runs over, and their number
-  ws.tc.p[6] = a.take<int>(rows);
-  ws.tc.p[7] = a.take<int>(64);
 }
 
 
@@ -927,12 +924,11 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
   ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m->m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0]; ea.dG0 = ws.dG;
   ea.dR = ws.dR;
-  ea.rowmap = reinterpret_cast<const int*>(ws.tc.p[6]);
-  ea.nrows = reinterpret_cast<const int*>(ws.tc.p[7]);
+  ea.rowmap = ws.rowmap;
+  ea.nrows = ws.row_off + n;
   const bool emb_tc = m->tcw.emb_W1_t != nullptr;
-  tc_live_rows(m, n, st);
   if (emb_tc)
-    tc_embed_fused(m, n, atype, false, st);
+    tc_embed(m, n, atype, false, st);
   else
     launch_embed_rows(ea, m->emb, false, st);
   prof_mark(m, "embed_fwd", st);
@@ -955,7 +951,7 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
     prof_mark(m, "attn_bwd_tc", st);
   }
   if (emb_tc)
-    tc_embed_fused(m, n, atype, true, st);
+    tc_embed(m, n, atype, true, st);
   else
     launch_embed_rows(ea, m->emb, true, st);
   prof_mark(m, "embed_bwd", st);

@@ -37,7 +37,7 @@ int emb_sm_count(int dev) {
 // 32-64-128 net (both double their width per layer, E1 = 2 E0, E2 = 2 E1).
 constexpr int EMB_TA = 128 * 64 * 2;    // activation tile: 128 rows x 64 cols
 constexpr int EMB_TD = 128 * 128 * 2;   // dZ3 tile: 128 rows x 128 cols
-constexpr int EMB_MAXT = 8;             // atom types the staged type-pair rows allow
+constexpr int EMB_MAXT = 8;             // atom types (their type-pair table stays in L1)
 constexpr int EMB_THREADS = 256;
 static_assert(2 * EMB_TD == 4 * EMB_TA, "the dZ3 hi / lo tiles fill the activation tiles");
 
@@ -49,13 +49,10 @@ struct EmbShape {
   static constexpr int T1 = 64 * 64 * 2;               // W1 tile: 64 (E1 padded) rows x 64 cols
   static constexpr int T2 = E2P * 64 * 2;              // W2 tile: E2P rows x 64 cols
   static constexpr int WIMG = 2 * T1 + 2 * T2;         // W1 hi, W1 lo, W2 hi, W2 lo
-  static constexpr int GT = EMB_MAXT * E2 * 4;         // this atom's rows of the type-pair table
-  static constexpr int B0T = EMB_MAXT * E0 * 4;        // concat mode: this atom's rows of the first-layer bias table
-  static constexpr int F_B0 = WIMG + 4 * EMB_TA + GT;  // forward: bias rows after the type-pair rows
-  static constexpr int F_SMEM = F_B0 + B0T + 64;
-  // the adjoint reads layers 1 and 2 as stored (no bias rows); its dZ3 tiles
-  // reuse the four activation tiles
-  static constexpr int B_SMEM = WIMG + 4 * EMB_TA + GT + 512 + 64;
+  static constexpr int F_SMEM = WIMG + 4 * EMB_TA + 64;
+  // the adjoint's dZ3 tiles reuse the four activation tiles; 512 bytes for one
+  // partial dE/dx per row
+  static constexpr int B_SMEM = WIMG + 4 * EMB_TA + 512 + 64;
   static constexpr int SPLIT = (E1 / 2) & ~7;          // first layer-2 unit of half 1 (24 / 32)
   static constexpr int G2 = (E1 + 7) / 8;              // 8-column groups of layer 2
   static constexpr int G3 = (E2 + 7) / 8;              // 8-column groups of layer 3
@@ -75,21 +72,18 @@ struct EmbedTcArgs {
   const int* nnei;
   const int* atype;
   const float* Gt;        // [ntypes][ntypes][E2]
-  float* G0;              // fwd out, column-quad interleaved per atom (rm: row-major [rows][E2])
+  float* G0;              // fwd out, column-quad interleaved per atom (rm: packed rows [rows][E2])
   const float* dG0;       // bwd in, same layout as G0
   float* dR;              // bwd: dR[:,0] +=
   const float* b0t;       // concat type-embedding mode: first-layer bias per (centre,
                           // neighbour) type [ntypes][ntypes][E0]; null: b0 below
-  float* H12;             // [atom][E0 + E1 units][NP rows]: layers 1 and 2 of the net,
+  float* H12;             // [tile][E0 + E1 units][128 rows]: layers 1 and 2 of the net,
                           // written by the forward, read by the adjoint
   const uint4* wimg;      // W1/W2 hi/lo tiles (FP16 or BF16, as the kernel's operands)
   int n, ntypes;
-  int rm;                 // G0 and dG0 row-major (the modular layer layout) instead of interleaved
-  int live_only;          // G0's rows past the last neighbour are not written (their content is
-                          // undefined: the fused layer kernels never read them); else zeros.
-                          // The live-row kernels need 1 (a row past the list's end stores nothing)
-  const int* rowmap;      // live-row kernels: the live rows (atom * NP + slot) in tile order
-  const int* nrows;       // live-row kernels: their number (device)
+  int rm;                 // G0 and dG0 packed rows (the modular layer layout) instead of interleaved
+  const int* rowmap;      // the live rows (atom * NP + slot) in tile order
+  const int* nrows;       // their number (device)
   int* err;
   float W0[32], b0[32], b1[64], b2[128];  // the net's first layer and biases (first E0 / E1 / E2 used)
 };
@@ -213,19 +207,18 @@ __device__ __forceinline__ void embed_tc_front(const EmbedTcArgs& a, uint8_t* sm
 // Z3 = H2 W2; returns once Z3 is in TMEM columns [64, 64 + E2P).
 template <class S, bool F16, int H, class BeforeZ3>
 __device__ __forceinline__ void embed_bwd_front(const EmbedTcArgs& a, uint8_t* sm, uint32_t tm, Sync& sy, int row,
-                                                bool rv, int atom, int slot, float* h1, float* h2,
-                                                BeforeZ3 before_z3) {
+                                                bool rv, int tile, float* h1, float* h2, BeforeZ3 before_z3) {
   using O = EmbOwn<S, H>;
   uint8_t* sW2h = sm + 2 * S::T1;
   uint8_t* sW2l = sW2h + S::T2;
   uint8_t* sH2h = sm + S::WIMG + 2 * EMB_TA;
   uint8_t* sH2l = sH2h + EMB_TA;
   const bool issuer = threadIdx.x == 0;
-  const float* hs = a.H12 + (size_t)atom * (S::E0 + S::E1) * NP + slot;  // live rows only were stored
+  const float* hs = a.H12 + (size_t)tile * (S::E0 + S::E1) * 128 + row;  // live rows only were stored
 #pragma unroll
-  for (int p = 0; p < S::E0; ++p) h1[p] = rv ? hs[p * NP] : 0.f;
+  for (int p = 0; p < S::E0; ++p) h1[p] = rv ? hs[p * 128] : 0.f;
 #pragma unroll
-  for (int i = 0; i < O::nb; ++i) h2[i] = rv ? hs[(S::E0 + O::b0 + i) * NP] : 0.f;
+  for (int i = 0; i < O::nb; ++i) h2[i] = rv ? hs[(S::E0 + O::b0 + i) * 128] : 0.f;
 #pragma unroll
   for (int g = O::g_lo; g < O::g_hi; ++g) {
     float v[8];
@@ -247,27 +240,6 @@ __device__ __forceinline__ void embed_bwd_front(const EmbedTcArgs& a, uint8_t* s
   sy.wait();
 }
 
-// A row's inputs of the embedding net (s of the neighbour, its type), read
-// for the next atom while the current one is processed: the neighbour
-// count, s and the neighbour index at its start, the type at its end.
-struct EmbRowIn {
-  int nn = 0, nl = 0, tj = 0;
-  float x = 0.f;
-  __device__ void count(const EmbedTcArgs& a, int atom) { nn = atom < a.n ? a.nnei[atom] : 0; }
-  __device__ void rows(const EmbedTcArgs& a, int atom, int row) {
-    if (atom < a.n) {  // R and nlist are written for all NP rows: read unmasked, used masked
-      const size_t rg = (size_t)atom * NP + row;
-      x = a.R[rg * 4];
-      nl = a.nlist[rg];
-    }
-  }
-  __device__ void type(const EmbedTcArgs& a, int row) {
-    const bool rv = row < nn;
-    x = rv ? x : 0.f;
-    tj = rv ? a.atype[nl] : 0;
-  }
-};
-
 template <class S>
 __device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm, uint64_t*& bar, uint32_t*& s_tmem,
                                                int smem_bytes) {
@@ -286,37 +258,10 @@ __device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm
   handoff();
 }
 
-// Per atom: copy the centre type's rows of the type-pair table Gt[t_i][*]
-// (and, in concat mode and given s_b0, of the first-layer bias table) to
-// shared memory, read by neighbour type afterwards, and bring the next atom's
-// per-row inputs into L2.
-template <class S>
-__device__ __forceinline__ void embed_tc_atom_start(const EmbedTcArgs& a, float* s_gt, float* s_b0, int atom,
-                                                    bool bwd) {
-  const float4* src = reinterpret_cast<const float4*>(a.Gt + (size_t)a.atype[atom] * a.ntypes * S::E2);
-  float4* dst = reinterpret_cast<float4*>(s_gt);
-  for (int i = threadIdx.x; i < a.ntypes * S::E2 / 4; i += blockDim.x) dst[i] = src[i];
-  if (a.b0t && s_b0) {  // read by layer 1 right away: a barrier of its own
-    const float* b0 = a.b0t + (size_t)a.atype[atom] * a.ntypes * S::E0;
-    for (int i = threadIdx.x; i < a.ntypes * S::E0; i += blockDim.x) s_b0[i] = b0[i];
-    __syncthreads();
-  }
-  const int next = atom + gridDim.x;
-  if (threadIdx.x == 0 && next < a.n) {
-    const size_t base = (size_t)next * NP;
-    prefetch_l2(a.R + base * 4, NP * 4 * sizeof(float));
-    prefetch_l2(a.nlist + base, NP * sizeof(int));
-    if (bwd) {
-      prefetch_l2(a.dG0 + base * S::E2, NP * S::E2 * sizeof(float));
-      prefetch_l2(a.H12 + base * (S::E0 + S::E1), NP * (S::E0 + S::E1) * sizeof(float));
-    }
-  }
-}
-
 // Layer 3 forward of the owned outputs: G0[c] = (h2[c % E1] + tanh(z3 + b2)) (1 + Gt[t_i][t_j][c]).
 template <class S, int H>
 __device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, uint32_t taddr, const float* gt, const float* h2,
-                                              bool rv, float* out_blk, int row) {
+                                              bool rv, float* out_blk, int slot) {
   using O = EmbOwn<S, H>;
 #pragma unroll
   for (int k = 0; k < S::NK3; ++k) {
@@ -334,73 +279,9 @@ __device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, uint32_t tad
       float2 o;
       o.x = rv ? (h2[c % S::E1 - O::b0] + tanhf(z[i] + a.b2[c])) * (1.f + g2.x) : 0.f;
       o.y = rv ? (h2[(c + 1) % S::E1 - O::b0] + tanhf(z[i + 1] + a.b2[c + 1])) * (1.f + g2.y) : 0.f;
-      if (rv || !a.live_only)
-        __stcs(reinterpret_cast<float2*>(out_blk + (a.rm ? (size_t)row * S::E2 + c : cq_off(row, c))), o);
+      if (rv) __stcs(reinterpret_cast<float2*>(out_blk + (a.rm ? (size_t)slot * S::E2 + c : cq_off(slot, c))), o);
     }
   }
-}
-
-template <class S, bool F16>
-__global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd(const __grid_constant__ EmbedTcArgs a) {
-  extern __shared__ __align__(1024) uint8_t sm[];
-  if ((smem_u32(sm) & 1023u) != 0) {
-    if (threadIdx.x == 0) set_err(a.err, ERR_CAPACITY);
-    return;
-  }
-  uint64_t* bar;
-  uint32_t* s_tmem;
-  embed_tc_setup<S>(a, sm, bar, s_tmem, S::F_SMEM);
-  const uint32_t tm = *s_tmem;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
-  const int row = quad * 32 + lane;
-  const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-  float* s_gt = reinterpret_cast<float*>(sm + S::WIMG + 4 * EMB_TA);
-  float* s_b0 = reinterpret_cast<float*>(sm + S::F_B0);
-  Sync sy{bar, 0u, a.err};
-  float h1[S::E0], h2[S::E1 - S::SPLIT];
-  EmbRowIn in;
-  in.count(a, blockIdx.x);
-  in.rows(a, blockIdx.x, row);
-  in.type(a, row);
-  for (int atom = blockIdx.x; atom < a.n && sy.ok; atom += gridDim.x) {
-    const EmbRowIn cur = in;
-    const int nn = cur.nn, tj = cur.tj, next = atom + gridDim.x;
-    const bool rv = row < nn;
-    in.count(a, next);
-    embed_tc_atom_start<S>(a, s_gt, s_b0, atom, false);  // visible after the front's barriers
-    auto rows_next = [&] { in.rows(a, next, row); };
-    const float* b0row = a.b0t ? s_b0 + tj * S::E0 : nullptr;
-    if (half == 0)
-      embed_tc_front<S, F16, 0>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
-    else
-      embed_tc_front<S, F16, 1>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
-    if (rv) {  // layers 1 and 2 of a live row for the adjoint: this half's layer-1 units, its layer-2 units
-      float* hs = a.H12 + (size_t)atom * (S::E0 + S::E1) * NP + row;
-      if (half == 0) {
-#pragma unroll
-        for (int p = 0; p < 16; ++p) hs[p * NP] = h1[p];
-#pragma unroll
-        for (int i = 0; i < S::SPLIT; ++i) hs[(S::E0 + i) * NP] = h2[i];
-      } else {
-#pragma unroll
-        for (int p = 16; p < S::E0; ++p) hs[p * NP] = h1[p];
-#pragma unroll
-        for (int i = 0; i < S::E1 - S::SPLIT; ++i) hs[(S::E0 + S::SPLIT + i) * NP] = h2[i];
-      }
-    }
-    float* out = a.G0 + (size_t)atom * NP * S::E2;
-    if (half == 0)
-      embed_fwd_out<S, 0>(a, tm + lane_off, s_gt + tj * S::E2, h2, rv, out, row);
-    else
-      embed_fwd_out<S, 1>(a, tm + lane_off, s_gt + tj * S::E2, h2, rv, out, row);
-    in.type(a, row);
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-  }
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tm, 256);
 }
 
 // Adjoint of layer 3 for one half: dZ3 = g (1 - t3^2) with g = dG0 (1 + Gt)
@@ -538,13 +419,13 @@ __device__ __forceinline__ void embed_bwd_dz2(uint32_t taddr, const float* h1, c
   }
 }
 
-// rowg = atom * NP + slot: the row's place in the atom blocks (row is its
-// place in the tile); pre() runs with the row's first loads, before the wait
+// rowg = atom * NP + slot: the row's place in dR; slot: its place in its dE/dG0
+// block dg; pre() runs with the row's first loads, before the wait
 // for Z3.
 template <class S, bool F16, int H, class Pre>
 __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm, uint32_t tm, uint32_t lane_off,
-                                               Sync& sy, int row, bool rv, size_t rowg, const float* gt,
-                                               const float4* dg, float* xch, Pre pre) {
+                                               Sync& sy, int row, bool rv, int tile, size_t rowg, const float* gt,
+                                               const float4* dg, int slot, float* xch, Pre pre) {
   using O = EmbOwn<S, H>;
   const bool issuer = threadIdx.x == 0;
   uint8_t* sW1h = sm;
@@ -559,8 +440,7 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
   uint8_t* sDZ2l = sDZ2h + EMB_TA;
   float h1[S::E0], h2[O::nb];
   float4 d0[4];
-  const int atom = (int)(rowg / NP), slot = (int)(rowg - (size_t)atom * NP);
-  embed_bwd_front<S, F16, H>(a, sm, tm, sy, row, rv, atom, slot, h1, h2, [&] {
+  embed_bwd_front<S, F16, H>(a, sm, tm, sy, row, rv, tile, h1, h2, [&] {
     embed_bwd_load16<S, H>(dg, a.rm, 0, slot, rv, d0);
     embed_bwd_prefetch16<S, H>(dg, a.rm, 1, slot, rv);
     pre();
@@ -600,103 +480,15 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
   if (H == 0 && rv) atomicAdd(a.dR + rowg * 4, dx + xch[row]);
 }
 
-template <class S, bool F16>
-__global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd(const __grid_constant__ EmbedTcArgs a) {
-  extern __shared__ __align__(1024) uint8_t sm[];
-  if ((smem_u32(sm) & 1023u) != 0) {
-    if (threadIdx.x == 0) set_err(a.err, ERR_CAPACITY);
-    return;
-  }
-  uint64_t* bar;
-  uint32_t* s_tmem;
-  embed_tc_setup<S>(a, sm, bar, s_tmem, S::B_SMEM);
-  const uint32_t tm = *s_tmem;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
-  const int row = quad * 32 + lane;
-  const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-  float* s_gt = reinterpret_cast<float*>(sm + S::WIMG + 4 * EMB_TA);
-  float* xch = s_gt + EMB_MAXT * S::E2;  // [128] half 1's part of dE/dx
-  Sync sy{bar, 0u, a.err};
-  if (threadIdx.x == 0 && blockIdx.x < a.n)
-    prefetch_l2(a.dG0 + (size_t)blockIdx.x * NP * S::E2, NP * S::E2 * sizeof(float));
-  EmbRowIn in;
-  in.count(a, blockIdx.x);
-  in.rows(a, blockIdx.x, row);
-  in.type(a, row);
-  for (int atom = blockIdx.x; atom < a.n && sy.ok; atom += gridDim.x) {
-    const EmbRowIn cur = in;
-    const int nn = cur.nn, tj = cur.tj, next = atom + gridDim.x;
-    in.count(a, next);
-    in.rows(a, next, row);
-    if (nn == 0) {  // uniform over the CTA
-      in.type(a, row);
-      continue;
-    }
-    const bool rv = row < nn;
-    const size_t rowg = (size_t)atom * NP + row;
-    embed_tc_atom_start<S>(a, s_gt, nullptr, atom, true);  // visible after the front's barriers
-    const float4* dg = reinterpret_cast<const float4*>(a.dG0 + (size_t)atom * NP * S::E2);
-    if (half == 0)
-      embed_bwd_tail<S, F16, 0>(a, sm, tm, lane_off, sy, row, rv, rowg, s_gt + tj * S::E2, dg, xch, [] {});
-    else
-      embed_bwd_tail<S, F16, 1>(a, sm, tm, lane_off, sy, row, rv, rowg, s_gt + tj * S::E2, dg, xch, [] {});
-    in.type(a, row);
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-  }
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tm, 256);
-}
-
 // ------------------------------------------------- live-row tiles
 // The net treats every neighbour row on its own, so its tiles need not
-// follow the atoms: the live-row kernels below take 128 live rows at a time
-// from one list of all atoms' live rows (atom * NP + slot), so that no lane
-// of a tile holds a row past its atom's last neighbour (with 72-103
-// neighbours per atom, per-atom tiles leave lane quadrant 3, and with it
-// one of the SM's four schedulers, idle).  A row's results do not depend on
-// where in the list it is or which rows share its tile: every product row
-// and every element-wise step is the row's own.
-
-constexpr int LR_THREADS = 256;
-
-// The list: each block takes LR_THREADS atoms, reserves room for their live
-// rows with one atomic add and writes them, an atom's slots in order.  The
-// blocks' order in the list is that of their reservations.
-__global__ void __launch_bounds__(LR_THREADS) k_live_rows(const int* __restrict__ nnei, int n, int* __restrict__ count,
-                                                          int* __restrict__ rows) {
-  __shared__ int s_warp[LR_THREADS / 32];
-  __shared__ int s_base;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int first = blockIdx.x * LR_THREADS;
-  const int nn = first + t < n ? nnei[first + t] : 0;
-  int x = nn;  // inclusive sum over the warp's atoms
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, d);
-    if (lane >= d) x += y;
-  }
-  if (lane == 31) s_warp[w] = x;
-  __syncthreads();
-  if (t == 0) {
-    int tot = 0;
-    for (int k = 0; k < LR_THREADS / 32; ++k) {
-      const int c = s_warp[k];
-      s_warp[k] = tot;
-      tot += c;
-    }
-    s_base = tot > 0 ? atomicAdd(count, tot) : 0;
-  }
-  __syncthreads();
-  const int off = s_base + s_warp[w] + x - nn;  // this atom's first place in the list
-  for (int j = 0; j < 32; ++j) {                // the warp writes its atoms one at a time
-    const int nj = __shfl_sync(0xffffffffu, nn, j), oj = __shfl_sync(0xffffffffu, off, j);
-    const int aj = first + 32 * w + j;
-    for (int s = lane; s < nj; s += 32) rows[oj + s] = aj * NP + s;
-  }
-}
+// follow the atoms: they take 128 live rows at a time from the list of all
+// atoms' live rows (launch_row_list), so that no lane of a tile holds a row
+// past its atom's last neighbour (with 72-103 neighbours per atom, per-atom
+// tiles leave lane quadrant 3, and with it one of the SM's four schedulers,
+// idle).  A row's results do not depend on where in the list it is or which
+// rows share its tile: every product row and every element-wise step is the
+// row's own.
 
 // A row of a live-row tile: its place in the atom blocks (rg = atom * NP +
 // slot, -1 past the end of the list), s, and the centre and neighbour types.
@@ -730,7 +522,7 @@ struct LiveRowIn {
   }
 };
 
-template <class S>
+template <class S, bool F16>
 __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(const __grid_constant__ EmbedTcArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   if ((smem_u32(sm) & 1023u) != 0) {
@@ -759,28 +551,29 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
     auto rows_next = [&] { in.rows(a, true); };
     const float* b0row = a.b0t && rv ? a.b0t + ((size_t)cur.ti * a.ntypes + cur.tj) * S::E0 : nullptr;
     if (half == 0)
-      embed_tc_front<S, true, 0>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
+      embed_tc_front<S, F16, 0>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
     else
-      embed_tc_front<S, true, 1>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
-    if (rv) {  // layers 1 and 2 of the row for the adjoint, as the per-atom kernel stores them
-      float* hs = a.H12 + (size_t)cur.atom * (S::E0 + S::E1) * NP + cur.slot;
+      embed_tc_front<S, F16, 1>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
+    if (rv) {  // layers 1 and 2 of the row for the adjoint: this half's layer-1 units, its layer-2 units
+      float* hs = a.H12 + (size_t)tile * (S::E0 + S::E1) * 128 + row;
       if (half == 0) {
 #pragma unroll
-        for (int p = 0; p < 16; ++p) __stcs(hs + p * NP, h1[p]);
+        for (int p = 0; p < 16; ++p) __stcs(hs + p * 128, h1[p]);
 #pragma unroll
-        for (int i = 0; i < S::SPLIT; ++i) __stcs(hs + (S::E0 + i) * NP, h2[i]);
+        for (int i = 0; i < S::SPLIT; ++i) __stcs(hs + (S::E0 + i) * 128, h2[i]);
       } else {
 #pragma unroll
-        for (int p = 16; p < S::E0; ++p) __stcs(hs + p * NP, h1[p]);
+        for (int p = 16; p < S::E0; ++p) __stcs(hs + p * 128, h1[p]);
 #pragma unroll
-        for (int i = 0; i < S::E1 - S::SPLIT; ++i) __stcs(hs + (S::E0 + S::SPLIT + i) * NP, h2[i]);
+        for (int i = 0; i < S::E1 - S::SPLIT; ++i) __stcs(hs + (S::E0 + S::SPLIT + i) * 128, h2[i]);
       }
     }
-    float* out = a.G0 + (size_t)cur.atom * NP * S::E2;
+    float* out = a.G0 + (size_t)(a.rm ? tile : cur.atom) * NP * S::E2;
+    const int slot = a.rm ? row : cur.slot;
     if (half == 0)
-      embed_fwd_out<S, 0>(a, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, cur.slot);
+      embed_fwd_out<S, 0>(a, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
     else
-      embed_fwd_out<S, 1>(a, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, cur.slot);
+      embed_fwd_out<S, 1>(a, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
     in.type(a);
     fence_before_sync();
     __syncthreads();
@@ -791,7 +584,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
   if (warp == 0) tmem_dealloc(tm, 256);
 }
 
-template <class S>
+template <class S, bool F16>
 __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(const __grid_constant__ EmbedTcArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   if ((smem_u32(sm) & 1023u) != 0) {
@@ -805,7 +598,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
   const int row = quad * 32 + lane;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-  float* xch = reinterpret_cast<float*>(sm + S::WIMG + 4 * EMB_TA) + EMB_MAXT * S::E2;  // [128] half 1's dE/dx
+  float* xch = reinterpret_cast<float*>(sm + S::WIMG + 4 * EMB_TA);  // [128] half 1's dE/dx
   Sync sy{bar, 0u, a.err};
   const int nrows = *a.nrows;
   const int ntiles = (nrows + 127) / 128;
@@ -818,24 +611,28 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(
     const bool rv = cur.rg >= 0;
     in.map(a, nrows, tile + gridDim.x, row);
     // with the row's first loads: the next tile's neighbour indices, and its
-    // atoms' dE/dG0 and layer blocks brought into L2 (by the thread of an
-    // atom's first row in that tile)
+    // layers and dE/dG0 blocks (interleaved: its atoms', by the thread of an
+    // atom's first row in that tile) brought into L2
     auto pre = [&] {
       in.rows(a, false);
       if (half == 0 && in.rg >= 0) {
-        const int at = in.rg / NP;
-        if (row == 0 || in.rg == at * NP) {
-          prefetch_l2(a.dG0 + (size_t)at * NP * S::E2, NP * S::E2 * sizeof(float));
-          prefetch_l2(a.H12 + (size_t)at * (S::E0 + S::E1) * NP, NP * (S::E0 + S::E1) * sizeof(float));
+        const size_t nt = tile + gridDim.x;
+        if (row == 0) {
+          prefetch_l2(a.H12 + nt * (S::E0 + S::E1) * 128, 128 * (S::E0 + S::E1) * sizeof(float));
+          if (a.rm) prefetch_l2(a.dG0 + nt * 128 * S::E2, 128 * S::E2 * sizeof(float));
         }
+        const int at = in.rg / NP;
+        if (!a.rm && (row == 0 || in.rg == at * NP))
+          prefetch_l2(a.dG0 + (size_t)at * NP * S::E2, NP * S::E2 * sizeof(float));
       }
     };
     const size_t rowg = rv ? (size_t)cur.rg : 0;
-    const float4* dg = reinterpret_cast<const float4*>(a.dG0 + (size_t)cur.atom * NP * S::E2);
+    const float4* dg = reinterpret_cast<const float4*>(a.dG0 + (size_t)(a.rm ? tile : cur.atom) * NP * S::E2);
+    const int slot = a.rm ? row : cur.slot;
     if (half == 0)
-      embed_bwd_tail<S, true, 0>(a, sm, tm, lane_off, sy, row, rv, rowg, cur.gt(a, S::E2), dg, xch, pre);
+      embed_bwd_tail<S, F16, 0>(a, sm, tm, lane_off, sy, row, rv, tile, rowg, cur.gt(a, S::E2), dg, slot, xch, pre);
     else
-      embed_bwd_tail<S, true, 1>(a, sm, tm, lane_off, sy, row, rv, rowg, cur.gt(a, S::E2), dg, xch, pre);
+      embed_bwd_tail<S, F16, 1>(a, sm, tm, lane_off, sy, row, rv, tile, rowg, cur.gt(a, S::E2), dg, slot, xch, pre);
     in.type(a);
     fence_before_sync();
     __syncthreads();
@@ -881,10 +678,10 @@ std::vector<uint8_t> emb_image(const std::vector<double>& W1, const std::vector<
 
 template <class S>
 void emb_set_smem() {
-  cudaFuncSetAttribute(k_embed_tc_fwd<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
-  cudaFuncSetAttribute(k_embed_tc_bwd<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
-  cudaFuncSetAttribute(k_embed_tc_fwd_live<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
-  cudaFuncSetAttribute(k_embed_tc_bwd_live<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
 }
 
 template <class S>
@@ -937,33 +734,23 @@ int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg) {
 }
 
 namespace {
-// One launch of the tensor-core embedding net, forward or adjoint: live-row
-// tiles with FP16 operand splits (the fused 16-bit paths, given a row list),
-// or per-atom tiles with BF16 ones (bf16x).
-template <class S>
+// One launch of the tensor-core embedding net, forward or adjoint, with FP16
+// (the fused 16-bit paths) or BF16 (bf16x) operand splits.
+template <class S, bool F16>
 void tc_embed_launch_s(int grid, const EmbedTcArgs& et, bool bwd, cudaStream_t st) {
-  if (et.rowmap) {
-    if (!bwd) k_embed_tc_fwd_live<S><<<grid, EMB_THREADS, S::F_SMEM, st>>>(et);
-    if (bwd) k_embed_tc_bwd_live<S><<<grid, EMB_THREADS, S::B_SMEM, st>>>(et);
-  } else {
-    if (!bwd) k_embed_tc_fwd<S, false><<<grid, EMB_THREADS, S::F_SMEM, st>>>(et);
-    if (bwd) k_embed_tc_bwd<S, false><<<grid, EMB_THREADS, S::B_SMEM, st>>>(et);
-  }
+  if (!bwd) k_embed_tc_fwd_live<S, F16><<<grid, EMB_THREADS, S::F_SMEM, st>>>(et);
+  if (bwd) k_embed_tc_bwd_live<S, F16><<<grid, EMB_THREADS, S::B_SMEM, st>>>(et);
 }
 
-void tc_embed_launch(dp_model* m, const EmbedTcArgs& et, bool bwd, cudaStream_t st) {
-  const int per_sm = emb_is<EmbS100>(m) ? EmbS100::MIN_CTAS : EmbS128::MIN_CTAS;
-  // at most n tiles either way: n atoms, or n * NP live rows at most
-  const int grid = std::min(et.n, per_sm * emb_sm_count(m->device));
-  if (emb_is<EmbS100>(m))
-    tc_embed_launch_s<EmbS100>(grid, et, bwd, st);
-  else
-    tc_embed_launch_s<EmbS128>(grid, et, bwd, st);
-  note_launch();
-}
+}  // namespace
 
-EmbedTcArgs embed_tc_args(dp_model* m, int n, const int* atype) {
+// The embedding net on the tensor cores over the live-row list: forward (G0 ->
+// G[0]), or adjoint (dE/dG0 from dG, dR[:, 0] +=).  FP16 operand splits and the
+// interleaved layout in the fused paths, BF16 ones and packed rows in bf16x.
+void tc_embed(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st) {
+  if (n == 0) return;
   Workspace& ws = m->ws;
+  const bool f16 = fused_tc_precision(m->precision);
   EmbedTcArgs et{};
   et.R = ws.R; et.nlist = ws.nlist; et.nnei = ws.nnei; et.atype = atype; et.Gt = m->Gt;
   et.n = n; et.ntypes = m->nt; et.err = m->d_err; et.b0t = m->b0t;
@@ -971,50 +758,21 @@ EmbedTcArgs embed_tc_args(dp_model* m, int n, const int* atype) {
   memcpy(et.b0, m->tcw.emb_vec.b0, sizeof(et.b0));
   memcpy(et.b1, m->tcw.emb_vec.b1, sizeof(et.b1));
   memcpy(et.b2, m->tcw.emb_vec.b2, sizeof(et.b2));
-  return et;
-}
-}  // namespace
-
-// The embedding net of the bf16x mode on the tensor cores (BF16 hi + lo
-// splits of both operands), G0 and dE/dG0 row-major: forward, or adjoint
-// (dR[:, 0] +=).  H12 holds the layers the adjoint reads back.
-void tc_embed_bf16(dp_model* m, int n, const int* atype, bool bwd, float* G0, const float* dG0, float* dR,
-                   float* H12, cudaStream_t st) {
-  if (n == 0) return;
-  EmbedTcArgs et = embed_tc_args(m, n, atype);
-  et.G0 = G0; et.dG0 = dG0; et.dR = dR; et.H12 = H12; et.rm = 1;
-  et.wimg = reinterpret_cast<const uint4*>(m->tcw.emb_W2_t);
-  tc_embed_launch(m, et, bwd, st);
-}
-
-
-// The list of live neighbour rows the fused paths' embedding net runs over
-// (after the neighbour list, before the net's forward; its adjoint reads the
-// same list).
-void tc_live_rows(dp_model* m, int n, cudaStream_t st) {
-  if (n == 0) return;
-  Workspace& ws = m->ws;
-  int* count = reinterpret_cast<int*>(ws.tc.p[7]);
-  cudaMemsetAsync(count, 0, sizeof(int), st);
-  k_live_rows<<<(n + LR_THREADS - 1) / LR_THREADS, LR_THREADS, 0, st>>>(ws.nnei, n, count,
-                                                                          reinterpret_cast<int*>(ws.tc.p[6]));
-  note_launch();
-}
-
-// The embedding net of the fused 16-bit paths on the tensor cores (FP16 hi +
-// lo splits) over the live-row tiles of tc_live_rows, G0 and dE/dG0
-// column-quad interleaved per atom: forward (G0 -> G[0]), or adjoint (dE/dG0
-// from dG, dR[:, 0] +=).
-void tc_embed_fused(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st) {
-  if (n == 0) return;
-  Workspace& ws = m->ws;
-  EmbedTcArgs et = embed_tc_args(m, n, atype);
-  et.G0 = ws.G[0]; et.dG0 = ws.dG; et.dR = ws.dR; et.rm = 0; et.live_only = 1;
-  et.rowmap = reinterpret_cast<const int*>(ws.tc.p[6]);
-  et.nrows = reinterpret_cast<const int*>(ws.tc.p[7]);
+  et.G0 = ws.G[0]; et.dG0 = ws.dG; et.dR = ws.dR; et.rm = f16 ? 0 : 1;
+  et.rowmap = ws.rowmap;
+  et.nrows = ws.row_off + n;
   et.H12 = reinterpret_cast<float*>(ws.tc.p[5]);
-  et.wimg = reinterpret_cast<const uint4*>(m->tcw.emb_W1_t);
-  tc_embed_launch(m, et, bwd, st);
+  et.wimg = reinterpret_cast<const uint4*>(f16 ? m->tcw.emb_W1_t : m->tcw.emb_W2_t);
+  const int per_sm = emb_is<EmbS100>(m) ? EmbS100::MIN_CTAS : EmbS128::MIN_CTAS;
+  const int grid = std::min(n, per_sm * emb_sm_count(m->device));  // at most n * NP rows: n tiles
+  if (emb_is<EmbS100>(m)) {
+    if (f16) tc_embed_launch_s<EmbS100, true>(grid, et, bwd, st);
+    else tc_embed_launch_s<EmbS100, false>(grid, et, bwd, st);
+  } else {
+    if (f16) tc_embed_launch_s<EmbS128, true>(grid, et, bwd, st);
+    else tc_embed_launch_s<EmbS128, false>(grid, et, bwd, st);
+  }
+  note_launch();
 }
 
 }  // namespace dpa1

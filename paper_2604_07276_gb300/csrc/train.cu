@@ -162,7 +162,7 @@ __global__ void k_env_jvp(JvpArgs a) {
 
 // The embedding net G = net(s) (1 + Gt[t_i][t_j]), net: 1 -> E0 -> E1 -> E2,
 // tanh layers with the residual rule (same width: x + f; double: [x, x] + f),
-// input s = R_ij,0.  A CTA takes JROWS neighbour rows of one atom and
+// input s = R_ij,0.  A CTA takes JROWS packed neighbour rows and
 // evaluates the activations and their tangents (s' = R'_ij,0).  Mode 0 writes
 // G'.  Mode 1 also runs the adjoint from dE/dG and (dE/dG)' and adds
 // *scale times the tangents of the weight gradients to grad (per-CTA sums,
@@ -175,8 +175,8 @@ struct JvpEmbedSmem {
   static constexpr int P2 = E2 + 1, Q0 = E0 + 1, Q1 = E1 + 1;
   // packed weights as in the parameter vector, W2 rows padded to P2
   static constexpr int W0 = 0, B0 = E0, W1 = 2 * E0, B1 = W1 + E0 * E1, W2 = B1 + E1, B2 = W2 + E1 * P2;
-  static constexpr int X = B2 + E2, XD = X + JROWS;
-  static constexpr int H1 = XD + JROWS, H1D = H1 + JROWS * Q0;
+  static constexpr int X = B2 + E2, XD = X + JROWS, TP = XD + JROWS;  // TP: the rows' type pairs (int)
+  static constexpr int H1 = TP + JROWS, H1D = H1 + JROWS * Q0;
   static constexpr int H2 = H1D + JROWS * Q0, H2D = H2 + JROWS * Q1;
   static constexpr int Z3 = H2D + JROWS * Q1, Z3D = Z3 + JROWS * P2;
   static constexpr int FWD_TOTAL = Z3D + JROWS * P2;
@@ -204,22 +204,17 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, flo
   for (int t = tid; t < E2; t += JTHREADS) sm[S::B2 + t] = a.w[S::W2 + E1 * E2 + t];
   if (mode == 1)
     for (int t = tid; t < S::NW; t += JTHREADS) sm[S::ACC + t] = 0.f;
-  const int per_atom = NP / JROWS;
-  const int nblk = a.n * per_atom;
-  for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-    const int atom = blk / per_atom, r0 = (blk % per_atom) * JROWS;
-    const int cnt = max(0, min(JROWS, a.nnei[atom] - r0));
-    const size_t base = (size_t)atom * NP + r0;
-    if (cnt == 0) {  // uniform over the CTA
-      if (mode == 0)
-        for (int idx = tid; idx < JROWS * E2; idx += JTHREADS) a.Gd[(base + idx / E2) * a.m1 + idx % E2] = 0.f;
-      continue;
-    }
-    const int ti = a.atype[atom];
+  int* pair = reinterpret_cast<int*>(sm + S::TP);
+  const int nrows = a.row_off[a.n];
+  for (int p0 = blockIdx.x * JROWS; p0 < nrows; p0 += gridDim.x * JROWS) {
+    const int cnt = min(JROWS, nrows - p0);
+    const size_t base = p0;
     __syncthreads();  // the previous block is done with the activations
     for (int r = tid; r < JROWS; r += JTHREADS) {
-      sm[S::X + r] = r < cnt ? a.R[(base + r) * 4] : 0.f;
-      sm[S::XD + r] = r < cnt ? a.Rd[(base + r) * 4] : 0.f;
+      const int rg = r < cnt ? a.rowmap[p0 + r] : 0;
+      sm[S::X + r] = r < cnt ? a.R[(size_t)rg * 4] : 0.f;
+      sm[S::XD + r] = r < cnt ? a.Rd[(size_t)rg * 4] : 0.f;
+      pair[r] = r < cnt ? a.atype[rg / NP] * a.ntypes + a.atype[a.nlist[rg]] : 0;
     }
     __syncthreads();
     // layer 1: h1 = tanh(s W0 + b0), h1' = (1 - h1^2) s' W0
@@ -227,7 +222,7 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, flo
       const int r = idx / E0, p = idx % E0;
       float h = 0.f, hd = 0.f;
       if (r < cnt) {
-        const float b0 = a.b0t ? a.b0t[((size_t)ti * a.ntypes + a.atype[a.nlist[base + r]]) * E0 + p] : sm[S::B0 + p];
+        const float b0 = a.b0t ? a.b0t[(size_t)pair[r] * E0 + p] : sm[S::B0 + p];
         h = tanhf(fmaf(sm[S::X + r], sm[S::W0 + p], b0));
         hd = (1.f - h * h) * sm[S::XD + r] * sm[S::W0 + p];
       }
@@ -279,13 +274,9 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, flo
     if (mode == 0) {
       for (int idx = tid; idx < JROWS * E2; idx += JTHREADS) {
         const int r = idx / E2, c = idx % E2;
-        float gd = 0.f;
-        if (r < cnt) {
-          const int tj = a.atype[a.nlist[base + r]];
-          const float f = 1.f + a.Gt[((size_t)ti * a.ntypes + tj) * E2 + c];
-          gd = (jskip<E1, E2>(sm + S::H2D + r * S::Q1, c) + sm[S::Z3D + r * S::P2 + c]) * f;
-        }
-        a.Gd[(base + r) * a.m1 + c] = gd;
+        if (r >= cnt) continue;
+        const float f = 1.f + a.Gt[(size_t)pair[r] * E2 + c];
+        a.Gd[(base + r) * a.m1 + c] = (jskip<E1, E2>(sm + S::H2D + r * S::Q1, c) + sm[S::Z3D + r * S::P2 + c]) * f;
       }
       continue;
     }
@@ -295,8 +286,7 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, flo
       const int r = idx / E2, c = idx % E2;
       float dz = 0.f, dzd = 0.f;
       if (r < cnt) {
-        const int tj = a.atype[a.nlist[base + r]];
-        const float f = 1.f + a.Gt[((size_t)ti * a.ntypes + tj) * E2 + c];
+        const float f = 1.f + a.Gt[(size_t)pair[r] * E2 + c];
         const float g = a.dG[(base + r) * a.m1 + c] * f, gd = a.dGd[(base + r) * a.m1 + c] * f;
         const float t = sm[S::Z3 + r * S::P2 + c], td = sm[S::Z3D + r * S::P2 + c];
         dz = g * (1.f - t * t);
@@ -319,8 +309,7 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, flo
           dhd = fmaf(wv, dz3d[c], dhd);
         }
         if (E2 == E1 || E2 == 2 * E1) {
-          const int tj = a.atype[a.nlist[base + r]];
-          const float* gt = a.Gt + ((size_t)ti * a.ntypes + tj) * E2;
+          const float* gt = a.Gt + (size_t)pair[r] * E2;
           for (int c = b; c < E2; c += E1) {
             const float f = 1.f + gt[c];
             dh += a.dG[(base + r) * a.m1 + c] * f;
@@ -405,7 +394,7 @@ __global__ void k_desc_jvp_fwd(JvpArgs a) {
   float* Tds = Ts + 4 * m1;  // [4][m1]
   const int atom = blockIdx.x;
   const int nn = a.nnei[atom];
-  const size_t base = (size_t)atom * NP;
+  const size_t base = (size_t)atom * NP, gbase = a.row_off[atom];
   const float inv_sel = 1.0f / (float)a.sel;
   for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) {
     const int c = t / m1, p = t % m1;
@@ -413,8 +402,8 @@ __global__ void k_desc_jvp_fwd(JvpArgs a) {
     for (int s = 0; s < nn; ++s) {
       const float* r = a.R + (base + s) * 4;
       const float* rd = a.Rd + (base + s) * 4;
-      v = fmaf(rd[c], a.G[(base + s) * m1 + p], v);
-      v = fmaf(r[c], a.Gd[(base + s) * m1 + p], v);
+      v = fmaf(rd[c], a.G[(gbase + s) * m1 + p], v);
+      v = fmaf(r[c], a.Gd[(gbase + s) * m1 + p], v);
     }
     Tds[t] = v * inv_sel;
     Ts[t] = a.T[(size_t)atom * 4 * m1 + t];
@@ -444,7 +433,7 @@ __global__ void k_desc_jvp_bwd(JvpArgs a) {
   float* dDd = dD + m1 * ax;
   const int atom = blockIdx.x;
   const int nn = a.nnei[atom];
-  const size_t base = (size_t)atom * NP;
+  const size_t base = (size_t)atom * NP, gbase = a.row_off[atom];
   const float inv_sel = 1.0f / (float)a.sel;
   for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) {
     Ts[t] = a.T[(size_t)atom * 4 * m1 + t];
@@ -471,15 +460,13 @@ __global__ void k_desc_jvp_bwd(JvpArgs a) {
     dTds[t] = vd * inv_sel;
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < NP * m1; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < nn * m1; idx += blockDim.x) {
     const int s = idx / m1, p = idx % m1;
     float v = 0.f;
-    if (s < nn) {
-      const float* r = a.R + (base + s) * 4;
-      const float* rd = a.Rd + (base + s) * 4;
-      for (int c = 0; c < 4; ++c) v += rd[c] * dTs[c * m1 + p] + r[c] * dTds[c * m1 + p];
-    }
-    a.dGd[(base + s) * m1 + p] = v;
+    const float* r = a.R + (base + s) * 4;
+    const float* rd = a.Rd + (base + s) * 4;
+    for (int c = 0; c < 4; ++c) v += rd[c] * dTs[c * m1 + p] + r[c] * dTds[c * m1 + p];
+    a.dGd[(gbase + s) * m1 + p] = v;
   }
 }
 
