@@ -295,6 +295,7 @@ int alloc_workspace(dp_model* m, int cap) {
     ws.dHa = a.take<float>((size_t)cap * fmax);
     ws.dHb = a.take<float>((size_t)cap * fmax);
     ws.dZ = a.take<float>((size_t)cap * fmax);
+    ws.dZ2 = a.take<float>((size_t)cap * fmax);
     ws.partials = a.take<double>((size_t)((cap + 3) / 4 + 1) * 10);
     ws.coord = a.take<double>((size_t)cap * 3);
     ws.box = a.take<double>(9);
@@ -420,44 +421,56 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
                  res ? EPI_RES_TANH : EPI_TANH, st);
     else if (fit_tc)
       fit_gemm_tc(m, l, false, hin, fan, m->fitb[l], res ? hin : nullptr, fan, ws.H[l], out, n,
-                  res ? EPI_RES_TANH : EPI_TANH, st);
+                  res ? EPI_RES_TANH : EPI_TANH, nullptr, nullptr, nullptr, st);
     else
       gemm_f32(hin, fan, m->fitW[l], out, m->fitb[l], res ? hin : nullptr, fan, ws.H[l], out, n, out, fan,
                res ? EPI_RES_TANH : EPI_TANH, st);
     hin = ws.H[l];
     fan = out;
   }
-  // w_out and b_out are stored multiplied by out_scale
-  launch_energy_head(ws.H[m->nfit - 1], n, fan, m->w_out, m->d_b_out, 1.0f, m->ebias, atype, ws.e, st);
+  // w_out and b_out are stored multiplied by out_scale; a10, the fitting backward,
+  // is seeded with dE/dH_last = out_scale * w_out
+  const bool res_last = m->nfit > 1 && m->fit[m->nfit - 1] == m->fit[m->nfit - 2];
+  launch_energy_head(ws.H[m->nfit - 1], res_last ? ws.H[m->nfit - 2] : nullptr, n, m->call_nlocal, fan, m->w_out,
+                     m->d_b_out, m->ebias, atype, ws.e, ws.dHa, ws.dZ, st);
   const float* gs = m->grad_scale;  // non-null: add gs * dE/dtheta to the gradient
   if (gs) {
     launch_colsum(ws.H[m->nfit - 1], fan, m->grad + m->off_wout, fan, n, gs, (float)m->out_scale, st);
     launch_head_bias_grad(atype, n, m->grad + m->off_ebias, m->grad + m->off_bout, gs, (float)m->out_scale, st);
   }
-  // a10: fitting backward, seeded with dE/dH_last = out_scale * w_out
-  launch_fill_rows(ws.dHa, m->w_out, n, m->call_nlocal, fan, st);
-  float* dH = ws.dHa;
-  float* dHn = ws.dHb;
+  float *dH = ws.dHa, *dHn = ws.dHb, *dZ = ws.dZ, *dZn = ws.dZ2;
   for (int l = m->nfit - 1; l >= 0; --l) {
     const int out = m->fit[l];
     const int in = l > 0 ? m->fit[l - 1] : m->fit_in;
     const bool res = (l > 0 && out == in);
-    launch_tanh_bwd(dH, ws.H[l], res ? ws.H[l - 1] : nullptr, ws.dZ, (long long)n * out, st);
     if (gs) {
       const float* input = l > 0 ? ws.H[l - 1] : ws.X;
-      launch_wgrad(input, in, ws.dZ, out, m->grad + m->off_fitW[l], out, in, out, n, gs, st);
-      launch_colsum(ws.dZ, out, m->grad + m->off_fitb[l], out, n, gs, 1.0f, st);
+      launch_wgrad(input, in, dZ, out, m->grad + m->off_fitW[l], out, in, out, n, gs, st);
+      launch_colsum(dZ, out, m->grad + m->off_fitb[l], out, n, gs, 1.0f, st);
     }
     float* dst = l > 0 ? dHn : ws.dX;
-    if (fit_x)
-      gemm_bf16x(m, m->xw.fitT[l], ws.dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS,
-                 st);
-    else if (fit_tc)
-      fit_gemm_tc(m, l, true, ws.dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st);
-    else
-      gemm_f32(ws.dZ, out, m->fitWT[l], in, nullptr, res ? dH : nullptr, out, dst, in, n, in, out,
+    // the layer below: its dZ = dH (1 - t^2), t = H - its skip input, with the product
+    const float* Hc = l > 0 ? ws.H[l - 1] : nullptr;
+    const float* Hp = l > 1 && m->fit[l - 1] == m->fit[l - 2] ? ws.H[l - 2] : nullptr;
+    float* Z = l > 0 ? dZn : nullptr;
+    if (fit_x) {
+      // the persistent GEMM's four epilogue warps bind once a CTA walks many tiles:
+      // dZ is formed there for small boxes only (3,001 atoms: 171 -> 137 us for the
+      // fitting stage, with the narrower N blocks; 15,668: 308 -> 359 us)
+      const bool with = n <= 4096;
+      gemm_bf16x(m, m->xw.fitT[l], dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st,
+                 nullptr, Hc, Hp, with ? Z : nullptr);
+      if (!with && l > 0) launch_tanh_bwd(dst, Hc, Hp, Z, (long long)n * in, st);
+    } else if (fit_tc) {
+      fit_gemm_tc(m, l, true, dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, Hc, Hp, Z,
+                  st);
+    } else {
+      gemm_f32(dZ, out, m->fitWT[l], in, nullptr, res ? dH : nullptr, out, dst, in, n, in, out,
                res ? EPI_RES : EPI_BIAS, st);
+      if (l > 0) launch_tanh_bwd(dst, Hc, Hp, Z, (long long)n * in, st);
+    }
     std::swap(dH, dHn);
+    std::swap(dZ, dZn);
   }
   prof_mark(m, "fitting", st);
   // a11: descriptor backward -> dG (w.r.t. G_L) and dR

@@ -51,9 +51,10 @@ namespace {
 
 // ------------------------------------------------------------------- GEMM
 // C = epi(A B + bias (+ R)), A [M][K] FP32 row-major, B [K][N] from a
-// pre-split image.  Persistent: CTA (x, y) keeps N block y (<= 144 columns)
-// and walks the 128-row tiles x, x + gridDim.x, ...; the K loop runs in
-// stages of 64 through a two-stage ring that continues across tiles, and
+// pre-split image.  Persistent: CTA (x, y) keeps N block y (<= 144 columns;
+// 48 or 16 where the row tiles are too few to fill the SMs, as in the fitting
+// net of a small box) and walks the 128-row tiles x, x + gridDim.x, ...; the K
+// loop runs in stages of 64 through a ring that continues across tiles, and
 // the accumulator alternates between two TMEM buffers, so that the epilogue
 // of one tile overlaps the loads and products of the next.
 //   warp 0      : producer.  Two TMA boxes of A (128 rows x 32 K FP32,
@@ -66,7 +67,7 @@ namespace {
 //                 residual / accumulate -> global).  A warp takes its 32
 //                 rows 32 columns at a time through a shared staging block,
 //                 so that each global access covers 4 rows x 128 bytes.
-constexpr int XBM = 128, XBK = 64, XBN = 144, XSTAGES = 2, XTHREADS = 384;
+constexpr int XBM = 128, XBK = 64, XBN = 144, XSTAGES_MAX = 3, XTHREADS = 384;
 constexpr int XF32 = 2 * XBM * 32 * 4;  // FP32 staging of one stage: two TMA boxes (32 KB)
 constexpr int XAT = XBM * XBK * 2;      // one BF16 A tile (hi or lo): 16 KB
 constexpr int XSLD = 36;                // row stride (floats) of an epilogue warp's 32 x 32 staging block
@@ -79,7 +80,12 @@ struct XGemmArgs {
   float* C;             // [M][ldc]
   int ldr, ldc;
   int M, N, nkb, bn_max, epi;
+  int bn, stages;    // columns per CTA (see x_bn), depth of the ring
   const int* m_dev;  // non-null: the rows are *m_dev (device, <= M)
+  // fitting adjoint: Z = C (1 - t^2) with t = Hc - Hp (Hp null: Hc), all [M][ldc]; null: none
+  const float* Hc;
+  const float* Hp;
+  float* Z;
   int* err;
 };
 
@@ -104,20 +110,23 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo) {
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
+template <bool ZOUT>
 __global__ void __launch_bounds__(XTHREADS, 1)
 k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XGemmArgs a) {
   extern __shared__ uint8_t xsm_raw[];
   const uint32_t raw = smem_u32(xsm_raw);
   uint8_t* sm = xsm_raw + (((raw + 1023u) & ~1023u) - raw);  // 1024-byte aligned tiles
-  const int nb = blockIdx.y;
-  const int bn = min(XBN, ((a.N - nb * XBN) + 15) & ~15);  // MMA width of this N block
-  const int b_tile = a.bn_max * 128;
+  const int XSTAGES = a.stages;
+  const int nc0 = (int)blockIdx.y * a.bn;              // first column of this N block
+  const int bn = min(a.bn, ((a.N - nc0) + 15) & ~15);  // its MMA width
+  const int b_img = a.bn_max * 128;                    // bytes of one tile of the image
+  const int b_tile = a.bn * 128;
   const int stage_bytes = XF32 + 2 * XAT + 2 * b_tile;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + XSTAGES * stage_bytes);
   uint64_t* full = bars;                 // [XSTAGES] A boxes and B tiles arrived
-  uint64_t* conv = bars + XSTAGES;       // [XSTAGES] A split into hi / lo (128 arrivals)
-  uint64_t* empty = bars + 2 * XSTAGES;  // [XSTAGES] the stage's MMAs are done
-  uint64_t* tfull = bars + 3 * XSTAGES;  // [2] accumulator buffer complete
+  uint64_t* conv = bars + XSTAGES_MAX;       // [XSTAGES] A split into hi / lo (128 arrivals)
+  uint64_t* empty = bars + 2 * XSTAGES_MAX;  // [XSTAGES] the stage's MMAs are done
+  uint64_t* tfull = bars + 3 * XSTAGES_MAX;  // [2] accumulator buffer complete
   uint64_t* tempty = tfull + 2;          // [2] accumulator buffer read out (4 warp arrivals)
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tempty + 2);
   // [XBN + 32] this N block's bias (0 without one, and past the block: the
@@ -145,7 +154,7 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
   }
   if (warp == 2) tmem_alloc(s_tmem, 512);
   for (int c = threadIdx.x; c < XBN + 32; c += blockDim.x) {
-    const int n = nb * XBN + c;
+    const int n = nc0 + c;
     s_bias[c] = (a.bias && c < bn && n < a.N) ? a.bias[n] : 0.f;
   }
   fence_before_sync();
@@ -161,7 +170,7 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
   const int ntile = mtiles > (int)blockIdx.x ? (mtiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (warp == 0 && lane == 0) {
-    const uint8_t* img = a.bimg + (size_t)nb * a.nkb * 2 * b_tile;
+    const uint8_t* img = a.bimg + (size_t)(nc0 / XBN) * a.nkb * 2 * b_img + (nc0 % XBN) * 128;
     for (int it = 0; it < ntile && ok; ++it) {
       const int mb = blockIdx.x + it * gridDim.x;
       for (int kb = 0; kb < a.nkb && ok; ++kb) {
@@ -171,8 +180,8 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
         mbar_expect_tx(full + s, XF32 + 2 * bn * 128);
         x_tma_load_2d(sF(s), &tmA, kb * XBK, mb * XBM, full + s);
         x_tma_load_2d(sF(s) + XF32 / 2, &tmA, kb * XBK + 32, mb * XBM, full + s);
-        bulk_g2s(sBh(s), img + (size_t)(2 * kb) * b_tile, bn * 128, full + s);
-        bulk_g2s(sBl(s), img + (size_t)(2 * kb + 1) * b_tile, bn * 128, full + s);
+        bulk_g2s(sBh(s), img + (size_t)(2 * kb) * b_img, bn * 128, full + s);
+        bulk_g2s(sBl(s), img + (size_t)(2 * kb + 1) * b_img, bn * 128, full + s);
       }
     }
   } else if (warp == 1 && lane == 0) {
@@ -254,7 +263,7 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
         // 8 lanes per row, 4 rows per access: residual / accumulate, store
         const int q = 4 * (lane & 7);
         const int nl = c0 + q;  // column within the N block
-        const int n = nb * XBN + nl;
+        const int n = nc0 + nl;
         if (ok && nl < bn && n < a.N) {  // N % 4 == 0
           // four rows at a time: the residual / accumulator loads, then the stores
           const bool res = a.epi == EPI_RES_TANH || a.epi == EPI_RES, acc = a.epi == EPI_ACCUM;
@@ -275,7 +284,19 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const long long m = m0 + 4 * (k0 + k) + (lane >> 3);
-              if (m < M) *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o[k];
+              if (m < M) {
+                *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o[k];
+                if (ZOUT) {
+                  float4 t = *reinterpret_cast<const float4*>(a.Hc + m * a.ldc + n);
+                  if (a.Hp) {
+                    const float4 p = *reinterpret_cast<const float4*>(a.Hp + m * a.ldc + n);
+                    t.x -= p.x; t.y -= p.y; t.z -= p.z; t.w -= p.w;
+                  }
+                  *reinterpret_cast<float4*>(a.Z + m * a.ldc + n) =
+                      make_float4(o[k].x * (1.f - t.x * t.x), o[k].y * (1.f - t.y * t.y), o[k].z * (1.f - t.z * t.z),
+                                  o[k].w * (1.f - t.w * t.w));
+                }
+              }
             }
           }
         }
@@ -321,8 +342,20 @@ PFN_cuTensorMapEncodeTiled_v12000 g_x_encode = nullptr;
 
 // the stages, 1024 bytes of alignment slack, the barriers (128 bytes), the
 // bias (XBN + 32 floats) and the epilogue staging (4 blocks)
-int x_smem(int bn_max) {
-  return XSTAGES * (XF32 + 2 * XAT + 2 * bn_max * 128) + 1024 + 128 + (XBN + 32) * 4 + 4 * XSTG;
+int x_stages(int bn) { return bn <= 16 ? 3 : 2; }
+int x_smem(int bn) {
+  return x_stages(bn) * (XF32 + 2 * XAT + 2 * bn * 128) + 1024 + 128 + (XBN + 32) * 4 + 4 * XSTG;
+}
+static_assert(3 * (XF32 + 2 * XAT + 2 * 16 * 128) + 1024 + 128 + (XBN + 32) * 4 + 4 * XSTG <= 227 * 1024, "ring");
+static_assert(8 * (3 * XSTAGES_MAX + 4) + 4 <= 128, "barriers");
+
+// Columns per CTA for mt row tiles of an image's N columns: one block of the image
+// (bn_max), or 48 or 16 of its columns while that leaves SMs idle.
+int x_bn(int mt, const XImage& im, int sms) {
+  int bn = im.bn_max;
+  for (int next : {48, 16})
+    if (next < bn && (long long)mt * ((im.N + next - 1) / next) <= sms) bn = next;
+  return bn;
 }
 
 int x_sm_count(int dev) {
@@ -1032,7 +1065,8 @@ int bf16x_init_weights(dp_model* m, std::string& msg) {
     fan = m->fit[l];
   }
   bf16x_refresh(m, nullptr);
-  cudaFuncSetAttribute(k_gemm_bf16x, cudaFuncAttributeMaxDynamicSharedMemorySize, x_smem(XBN));
+  for (auto k : {k_gemm_bf16x<false>, k_gemm_bf16x<true>})
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(x_smem(XBN), x_smem(16)));
   cudaFuncSetAttribute(k_attn_core_fwd_bf16x<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, XF_SMEM);
   cudaFuncSetAttribute(k_attn_core_fwd_bf16x<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, XF_SMEM);
   cudaFuncSetAttribute(k_attn_core_bwd_bf16x<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
@@ -1061,7 +1095,8 @@ void bf16x_free(dp_model* m) {
 }
 
 int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const float* bias, const float* R, int ldr,
-               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev) {
+               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev, const float* Hc, const float* Hp,
+               float* Z) {
   if (M <= 0) return DP_OK;
   CUtensorMap map;
   const cuuint64_t dims[2] = {(cuuint64_t)im.K, (cuuint64_t)M};
@@ -1085,11 +1120,20 @@ int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const flo
   a.bn_max = im.bn_max;
   a.epi = epi;
   a.m_dev = m_dev;
+  a.Hc = Hc;
+  a.Hp = Hp;
+  a.Z = Z;
   a.err = m->d_err;
   // persistent: about one CTA per SM over the N blocks
-  const int per_n = std::max(1, x_sm_count(m->device) / im.nnb);
-  dim3 grid((unsigned)std::min((M + XBM - 1) / XBM, per_n), (unsigned)im.nnb);
-  k_gemm_bf16x<<<grid, XTHREADS, x_smem(im.bn_max), st>>>(map, a);
+  const int mt = (M + XBM - 1) / XBM, sms = x_sm_count(m->device);
+  a.bn = m_dev ? im.bn_max : x_bn(mt, im, sms);
+  a.stages = x_stages(a.bn);
+  const int nnb = (im.N + a.bn - 1) / a.bn;
+  dim3 grid((unsigned)std::min(mt, std::max(1, sms / nnb)), (unsigned)nnb);
+  if (Z)
+    k_gemm_bf16x<true><<<grid, XTHREADS, x_smem(a.bn), st>>>(map, a);
+  else
+    k_gemm_bf16x<false><<<grid, XTHREADS, x_smem(a.bn), st>>>(map, a);
   note_launch();
   return DP_OK;
 }

@@ -7,16 +7,24 @@
 // misses A_lo B_lo and the truncation of the low parts, ~2^-20 relative:
 // the products stay at FP32 accuracy.
 //
-// One CTA computes a 128-row x (<= 256)-column tile with the full K:
+// One CTA computes a 128-row x BN-column tile with the full K:
 //   warp 0      : producer.  A tiles (128 rows x 32 K, FP32) by TMA with the
 //                 128-byte swizzle, B_hi / B_lo tiles by 1D bulk copies of
-//                 pre-swizzled images; two pipeline stages.
-//   warps 4-7   : split each A tile in place (A_hi) and into its A_lo tile.
+//                 pre-swizzled images, through a ring of 2 - 6 stages.
+//   warps 4-11  : split each A tile in place (A_hi) and into its A_lo tile.
 //   warp 1      : issues the MMAs (one thread), accumulator in TMEM.
 //   warp 2      : allocates / frees TMEM.
-//   all 8 warps : the epilogue (TMEM -> bias, tanh, residual -> global); warp
-//                 w reads TMEM lane quadrant w % 4 and every other 16-column
+//   all warps   : the epilogue (TMEM -> bias, tanh, residual -> global; in the
+//                 backward pass also the next layer's dZ = dH (1 - t^2)); warp
+//                 w reads TMEM lane quadrant w % 4 and every third 16-column
 //                 chunk, starting at chunk w / 4.
+// BN: the widest tile (256 columns) reads A the fewest times, but a small box
+// has few 128-row tiles, and each CTA walks the whole K alone: BN shrinks until
+// the tiles fill the SMs once (192 atoms, K = 1608, N = 240: 2 CTAs -> 30), and
+// the ring deepens with the room that leaves.  A tile's sums do not depend on
+// BN.  With the dZ epilogue and the energy head's seed (7 launches, were 12) the
+// fitting stage of 192 atoms took 192 -> 107 us, of 582 208 -> 111, of 15,668
+// (one tile per SM row, BN = 240) 326 -> 310.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -39,9 +47,10 @@ namespace {
 constexpr int FBM = 128;            // rows per tile
 constexpr int FBK = 32;             // K per stage (one 128-byte swizzle row of FP32)
 constexpr int FNMAX = 256;          // output columns per tile
-constexpr int FSTAGES = 2;
+constexpr int FSTAGES_MAX = 6;
+constexpr int FSMEM = 220 * 1024;   // shared memory a CTA's ring may take
 constexpr int FA_TILE = FBM * FBK * 4;  // 16 KB
-constexpr int FTHREADS = 256;
+constexpr int FTHREADS = 384;
 
 struct FitGemmArgs {
   const uint8_t* bimg;  // B images: [n block][k block][hi, lo] tiles of bn_max rows x 128 bytes
@@ -51,7 +60,13 @@ struct FitGemmArgs {
   int ldr, ldc;
   int M, N, nkb;        // rows, output columns, K blocks of 32
   int bn_max;           // rows of one B image tile (multiple of 16, <= 256)
+  int bn;               // columns per CTA (multiple of 16; 256 is a multiple of it or it is N)
+  int stages;
   int epi;
+  // backward: Z = C (1 - t^2) with t = Hc - Hp (Hp null: Hc), all [M][ldc]; null: none
+  const float* Hc;
+  const float* Hp;
+  float* Z;
   int* err;
 };
 
@@ -98,14 +113,17 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
   extern __shared__ uint8_t fsm_raw[];
   const uint32_t raw = smem_u32(fsm_raw);
   uint8_t* sm = fsm_raw + (((raw + 1023u) & ~1023u) - raw);  // 1024-byte aligned tiles
-  const int bn = min(FNMAX, ((a.N - (int)blockIdx.y * FNMAX) + 15) & ~15);  // MMA width of this tile
-  const int b_tile = a.bn_max * 128;
+  const int FSTAGES = a.stages;
+  const int nc0 = (int)blockIdx.y * a.bn;                // first column of this tile
+  const int bn = min(a.bn, ((a.N - nc0) + 15) & ~15);    // its MMA width
+  const int b_img = a.bn_max * 128;                      // bytes of one tile of the image
+  const int b_tile = a.bn * 128;
   const int stage_bytes = 2 * FA_TILE + 2 * b_tile;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + FSTAGES * stage_bytes);
-  uint64_t* full = bars;              // [FSTAGES]
-  uint64_t* conv = bars + FSTAGES;    // [FSTAGES]
-  uint64_t* empty = bars + 2 * FSTAGES;
-  uint64_t* done = bars + 3 * FSTAGES;
+  uint64_t* full = bars;                   // [FSTAGES]
+  uint64_t* conv = bars + FSTAGES_MAX;     // [FSTAGES]
+  uint64_t* empty = bars + 2 * FSTAGES_MAX;
+  uint64_t* done = bars + 3 * FSTAGES_MAX;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(done + 1);
   auto sA = [&](int s) { return sm + s * stage_bytes; };
   auto sAl = [&](int s) { return sm + s * stage_bytes + FA_TILE; };
@@ -116,7 +134,7 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
   if (threadIdx.x == 0) {
     for (int s = 0; s < FSTAGES; ++s) {
       mbar_init(full + s, 1);
-      mbar_init(conv + s, 128);
+      mbar_init(conv + s, FTHREADS - 128);
       mbar_init(empty + s, 1);
     }
     mbar_init(done, 1);
@@ -127,20 +145,21 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
   __syncthreads();
   fence_after_sync();
   const uint32_t tm = *s_tmem;
-  const int mb = blockIdx.x, nb = blockIdx.y;
+  const int mb = blockIdx.x;
   Waiter wt{a.err};
 
   if (warp == 0 && lane == 0) {
     // producer
-    const uint8_t* img = a.bimg + (size_t)nb * a.nkb * 2 * b_tile;
+    // the tile's rows of the image (a block of 256 columns holds whole tiles)
+    const uint8_t* img = a.bimg + (size_t)(nc0 / FNMAX) * a.nkb * 2 * b_img + (nc0 % FNMAX) * 128;
     for (int kb = 0; kb < a.nkb && wt.ok; ++kb) {
       const int s = kb % FSTAGES, u = kb / FSTAGES;
       if (kb >= FSTAGES) wt.wait(empty + s, (u - 1) & 1);
       if (!wt.ok) break;
       mbar_expect_tx(full + s, FA_TILE + 2 * bn * 128);
       tma_load_2d(sA(s), &tmA, kb * FBK, mb * FBM, full + s);
-      bulk_g2s(sBh(s), img + (size_t)(2 * kb) * b_tile, bn * 128, full + s);
-      bulk_g2s(sBl(s), img + (size_t)(2 * kb + 1) * b_tile, bn * 128, full + s);
+      bulk_g2s(sBh(s), img + (size_t)(2 * kb) * b_img, bn * 128, full + s);
+      bulk_g2s(sBl(s), img + (size_t)(2 * kb + 1) * b_img, bn * 128, full + s);
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
@@ -165,7 +184,7 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
     }
     mma_commit(done);
   } else if (warp >= 4) {
-    // split A in place; thread t takes 16-byte pieces t, t + 128, ... of the
+    // split A in place; thread t takes 16-byte pieces t, t + 256, ... of the
     // tile, so that a warp touches 512 contiguous bytes (the swizzle only
     // permutes pieces within a row, and the split is element-wise)
     const int t = threadIdx.x - 128;
@@ -175,8 +194,8 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
       uint4* hi = reinterpret_cast<uint4*>(sA(s));
       uint4* lo = reinterpret_cast<uint4*>(sAl(s));
 #pragma unroll
-      for (int i = 0; i < FA_TILE / 16 / 128; ++i) {
-        const int q = i * 128 + t;
+      for (int i = 0; i < FA_TILE / 16 / (FTHREADS - 128); ++i) {
+        const int q = i * (FTHREADS - 128) + t;
         const uint4 x = hi[q];
         uint4 h, l;
         h.x = tf32_trunc(x.x); l.x = tf32_trunc(__float_as_uint(__uint_as_float(x.x) - __uint_as_float(h.x)));
@@ -199,10 +218,10 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
     const int r = (warp & 3) * 32 + lane;  // row in the tile = TMEM lane
     const long long m = (long long)mb * FBM + r;
     const uint32_t taddr = tm + ((uint32_t)((warp & 3) * 32) << 16);
-    for (int c0 = (warp >> 2) * 16; c0 < bn; c0 += 32) {
+    for (int c0 = (warp >> 2) * 16; c0 < bn; c0 += 48) {
       float v[16];
       tmem_ld16(taddr + c0, v);
-      const int n0 = nb * FNMAX + c0;
+      const int n0 = nc0 + c0;
       if (m >= a.M) continue;
 #pragma unroll
       for (int q = 0; q < 16; q += 4) {
@@ -223,6 +242,15 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
           o.x += rr.x; o.y += rr.y; o.z += rr.z; o.w += rr.w;
         }
         *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o;
+        if (a.Z) {
+          float4 t = *reinterpret_cast<const float4*>(a.Hc + m * a.ldc + n);
+          if (a.Hp) {
+            const float4 p = *reinterpret_cast<const float4*>(a.Hp + m * a.ldc + n);
+            t.x -= p.x; t.y -= p.y; t.z -= p.z; t.w -= p.w;
+          }
+          *reinterpret_cast<float4*>(a.Z + m * a.ldc + n) =
+              make_float4(o.x * (1.f - t.x * t.x), o.y * (1.f - t.y * t.y), o.z * (1.f - t.z * t.z), o.w * (1.f - t.w * t.w));
+        }
       }
     }
   }
@@ -272,7 +300,24 @@ ImageShape image_shape(int K, int N) {
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
-int fit_smem(int bn_max) { return FSTAGES * (2 * FA_TILE + 2 * bn_max * 128) + 1024 + 128; }
+int fit_stages(int bn) { return std::min(FSTAGES_MAX, FSMEM / (2 * FA_TILE + 2 * bn * 128)); }
+int fit_smem(int bn) { return fit_stages(bn) * (2 * FA_TILE + 2 * bn * 128) + 1024 + 256; }
+static_assert(FSMEM / (2 * FA_TILE + 2 * FNMAX * 128) >= 2, "two stages at the full width");
+static_assert(8 * (3 * FSTAGES_MAX + 1) + 4 <= 256, "barriers");
+
+// Columns per CTA for mt row tiles of an N-column product: the widest that fills
+// the SMs, down to 16.
+int fit_bn(int mt, int N, int sms) {
+  int bn = std::min(FNMAX, (N + 15) & ~15);
+  while (bn > 16) {
+    // narrower tiles are powers of two: none crosses two blocks of the image
+    int next = 16;
+    while (2 * next < bn) next *= 2;
+    if ((long long)mt * ((N + next - 1) / next) > sms) break;
+    bn = next;
+  }
+  return bn;
+}
 
 }  // namespace
 
@@ -313,11 +358,10 @@ int fit_tc_init(dp_model* m, std::string& msg) {
       }
       w.allocations.push_back(d);
       (dir == 0 ? w.fitW_t : w.fitWT_t).push_back(d);
-      const int smem = fit_smem(s.bn_max);
-      cudaFuncSetAttribute(k_fit_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(smem, fit_smem(FNMAX)));
     }
     fan = out;
   }
+  cudaFuncSetAttribute(k_fit_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM + 1024 + 256);
   fit_tc_refresh(m, nullptr);
   if (cudaDeviceSynchronize() != cudaSuccess) {
     msg = "building the fitting-net weight images failed";
@@ -346,7 +390,8 @@ void fit_tc_refresh(dp_model* m, cudaStream_t st) {
 }
 
 int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, const float* bias, const float* R,
-                int ldr, float* C, int ldc, int M, int epi, cudaStream_t st) {
+                int ldr, float* C, int ldc, int M, int epi, const float* Hc, const float* Hp, float* Z,
+                cudaStream_t st) {
   if (M <= 0) return DP_OK;
   const int fan = layer == 0 ? m->fit_in : m->fit[layer - 1];
   const int out = m->fit[layer];
@@ -371,10 +416,18 @@ int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, 
   a.N = s.N;
   a.nkb = s.nkb;
   a.bn_max = s.bn_max;
+  int sms = 1;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
+  const int mt = (M + FBM - 1) / FBM;
+  a.bn = fit_bn(mt, s.N, sms);
+  a.stages = fit_stages(a.bn);
   a.epi = epi;
+  a.Hc = Hc;
+  a.Hp = Hp;
+  a.Z = Z;
   a.err = m->d_err;
-  dim3 grid((unsigned)((M + FBM - 1) / FBM), (unsigned)s.nnb);
-  k_fit_gemm<<<grid, FTHREADS, fit_smem(s.bn_max), st>>>(map, a);
+  dim3 grid((unsigned)mt, (unsigned)((s.N + a.bn - 1) / a.bn));
+  k_fit_gemm<<<grid, FTHREADS, fit_smem(a.bn), st>>>(map, a);
   note_launch();
   return DP_OK;
 }

@@ -179,8 +179,12 @@ struct DescArgs {
 void launch_desc_fwd(const DescArgs& a, cudaStream_t st);
 void launch_desc_bwd(const DescArgs& a, cudaStream_t st);
 
-void launch_energy_head(const float* H, int n, int width, const float* w_out, const float* b_out, float out_scale,
-                        const float* ebias, const int* atype, float* e, cudaStream_t st);
+// e_i = w_out . H_i + b_out + ebias[t_i], and the seed of the adjoint: dH_i = w_out
+// (0 from atom nlocal on: ghosts seed no energy) and dZ_i = dH_i (1 - t^2) with t = H - Hprev
+// (Hprev null: t = H).
+void launch_energy_head(const float* H, const float* Hprev, int n, int nlocal, int width, const float* w_out,
+                        const float* b_out, const float* ebias, const int* atype, float* e, float* dH, float* dZ,
+                        cudaStream_t st);
 // dZ = dH * (1 - t^2) with t = Hcur - Hprev (Hprev may be null: t = Hcur)
 void launch_tanh_bwd(const float* dH, const float* Hcur, const float* Hprev, float* dZ, long long count,
                      cudaStream_t st);

@@ -108,7 +108,7 @@ struct Workspace {
   float *dG, *dY, *dPG, *dQK;
   float *T, *X, *dX, *e;
   std::vector<float*> H;
-  float *dHa, *dHb, *dZ;
+  float *dHa, *dHb, *dZ, *dZ2;
   double* partials;
   // host-API staging
   double *coord, *box, *force, *virial, *energy, *atom_energy;
@@ -216,7 +216,8 @@ int bf16x_init_weights(dp_model* m, std::string& msg);
 void bf16x_refresh(dp_model* m, cudaStream_t st);
 void bf16x_free(dp_model* m);
 int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const float* bias, const float* R, int ldr,
-               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev = nullptr);
+               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev = nullptr, const float* Hc = nullptr,
+               const float* Hp = nullptr, float* Z = nullptr);
 void attn_core_fwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 void attn_core_bwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 // the fused 16-bit layer kernels (tc.cu) serve DP_PREC_BF16 and DP_PREC_FP16X;
@@ -224,7 +225,8 @@ void attn_core_bwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 // stored Q | K and [P G, rowsum P], LayerNorm kernels)
 inline bool fused_tc_precision(int p) { return p == DP_PREC_BF16 || p == DP_PREC_FP16X; }
 int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, const float* bias, const float* R,
-                int ldr, float* C, int ldc, int M, int epi, cudaStream_t st);
+                int ldr, float* C, int ldc, int M, int epi, const float* Hc, const float* Hp, float* Z,
+                cudaStream_t st);
 // stages a7-a11 (descriptor, fitting forward / backward, descriptor backward)
 void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t st);
 }  // namespace dpa1

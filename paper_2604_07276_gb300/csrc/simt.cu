@@ -1185,23 +1185,33 @@ void launch_desc_bwd(const DescArgs& a, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------ fitting head
-__global__ void k_energy_head(const float* __restrict__ H, int n, int width, const float* __restrict__ w,
-                              const float* __restrict__ bptr, float out_scale, const float* __restrict__ ebias,
-                              const int* __restrict__ atype, float* __restrict__ e) {
+__global__ void k_energy_head(const float* __restrict__ H, const float* __restrict__ Hp, int n, int nlocal, int width,
+                              const float* __restrict__ w, const float* __restrict__ bptr,
+                              const float* __restrict__ ebias, const int* __restrict__ atype, float* __restrict__ e,
+                              float* __restrict__ dH, float* __restrict__ dZ) {
   const int atom = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (atom >= n) return;
   float s = 0.f;
-  for (int c = lane; c < width; c += 32) s = fmaf(H[(size_t)atom * width + c], w[c], s);
+  for (int c = lane; c < width; c += 32) {
+    const size_t i = (size_t)atom * width + c;
+    const float h = H[i], wc = w[c];
+    s = fmaf(h, wc, s);
+    const float t = Hp ? h - Hp[i] : h;
+    const float d = atom < nlocal ? wc : 0.f;
+    dH[i] = d;
+    dZ[i] = d * (1.f - t * t);
+  }
   s = warp_sum(s);
-  if (lane == 0) e[atom] = out_scale * (s + *bptr) + ebias[atype[atom]];
+  if (lane == 0) e[atom] = 1.0f * (s + *bptr) + ebias[atype[atom]];
 }
 
-void launch_energy_head(const float* H, int n, int width, const float* w_out, const float* b_out, float out_scale,
-                        const float* ebias, const int* atype, float* e, cudaStream_t st) {
+void launch_energy_head(const float* H, const float* Hprev, int n, int nlocal, int width, const float* w_out,
+                        const float* b_out, const float* ebias, const int* atype, float* e, float* dH, float* dZ,
+                        cudaStream_t st) {
   if (n == 0) return;
-  k_energy_head<<<(unsigned)(((long long)n * 32 + 255) / 256), 256, 0, st>>>(H, n, width, w_out, b_out, out_scale,
-                                                                          ebias, atype, e);
+  k_energy_head<<<(unsigned)(((long long)n * 32 + 255) / 256), 256, 0, st>>>(H, Hprev, n, nlocal, width, w_out, b_out,
+                                                                          ebias, atype, e, dH, dZ);
   note_launch();
 }
 
