@@ -357,6 +357,7 @@ NbrArgs nbr_args(dp_model* m, int n, const double* coord, const double* box, con
   a.cell_cursor = ws.cell_cursor; a.cell_atoms = ws.cell_atoms;
   a.nlist = ws.nlist + (size_t)rel * NP; a.nnei = ws.nnei + rel; a.ncand = ws.ncand + rel;
   a.atype_c = ws.atype_c + rel; a.coordf = ws.coordf + rel;
+  a.rev_cnt = ws.rev_cnt + rel;
   a.err = m->d_err;
   return a;
 }
@@ -517,7 +518,6 @@ void run_network_f32(dp_model* m, int n, const int* atype, cudaStream_t st) {
   }
   run_descriptor_fitting(m, n, atype, st);
   // a12: attention backward
-  cudaMemsetAsync(ws.dgeo, 0, sizeof(float) * (size_t)rows * 4, st);
   for (int l = L - 1; l >= 0; --l) {
     const AttnLayerW& w = m->attn[l];
     launch_ln_bwd(ws.dG, ws.Y[l], ws.stats[l], nrows, w.ln_g, ws.dY, rows, m1, st);
@@ -574,7 +574,6 @@ void run_network_bf16x(dp_model* m, int n, const int* atype, cudaStream_t st) {
     prof_mark(m, "wo_gemm_ln", st);
   }
   run_descriptor_fitting(m, n, atype, st);
-  cudaMemsetAsync(ws.dgeo, 0, sizeof(float) * (size_t)rows * 4, st);
   for (int l = L - 1; l >= 0; --l) {
     const AttnLayerW& w = m->attn[l];
     const XWeights::Layer& x = m->xw.layers[l];
@@ -615,7 +614,7 @@ int run_after_neighbors(dp_model* m, int n, const double* coord, const CellGrid*
   EnvArgs ea{};
   ea.coord = coord; ea.atype = atype; ea.grid = grid; ea.frame = frame; ea.nlist = ws.nlist; ea.n = nc;
   ea.davg = m->davg; ea.dstd = m->dstd; ea.rcs = (float)m->rcs; ea.rc = (float)m->rcut;
-  ea.R = ws.R; ea.rw = ws.rw; ea.rv = ws.rv;
+  ea.R = ws.R; ea.rw = ws.rw; ea.rv = ws.rv; ea.dgeo = ws.dgeo;
   // the FP32 path evaluates R in FP64 and keeps w in FP64 for its smooth logits
   ea.fp64 = m->precision == DP_PREC_FP32 ? 1 : 0;
   ea.w64 = ea.fp64 ? ws.w64 : nullptr;
@@ -1434,6 +1433,7 @@ int dp_nlist_noalloc(int natoms, const double* d_coord, const double* d_box, dou
   a.cell_cursor = s->cell_cursor; a.cell_atoms = s->cell_atoms;
   a.nlist = d_nlist; a.nnei = d_nnei; a.ncand = s->ncand; a.atype_c = s->types_c; a.coordf = s->coordf;
   a.err = d_status;
+  a.rev_cnt = nullptr;
   launch_neighbors(a, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, std::string("dp_nlist_noalloc: launch failed: ") + cudaGetErrorString(e));
@@ -1613,7 +1613,7 @@ int dp_md_run(dp_model* m, int natoms, double* d_coord, double* d_vel, const dou
     const void* key_dt = nullptr;
     memcpy(&key_dt, &dtv, sizeof(dtv) < sizeof(key_dt) ? sizeof(dtv) : sizeof(key_dt));
     std::vector<const void*> key = {d_coord, d_vel, d_mass, d_box, d_atype, d_force, d_energy, d_virial, d_thermo,
-                                    m->d_md_partial,
+                                    m->d_md_partial, m->ws.mem,
                                     reinterpret_cast<const void*>((intptr_t)natoms),
                                     reinterpret_cast<const void*>((intptr_t)nsteps),
                                     reinterpret_cast<const void*>((intptr_t)m->precision), key_dt};

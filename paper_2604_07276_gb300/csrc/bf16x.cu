@@ -113,6 +113,7 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo) {
 template <bool ZOUT>
 __global__ void __launch_bounds__(XTHREADS, 1)
 k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XGemmArgs a) {
+  pdl_wait();
   extern __shared__ uint8_t xsm_raw[];
   const uint32_t raw = smem_u32(xsm_raw);
   uint8_t* sm = xsm_raw + (((raw + 1023u) & ~1023u) - raw);  // 1024-byte aligned tiles
@@ -511,6 +512,7 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_fwd_bf16x(const __grid_c
   }
   if (warp == 0) tmem_alloc(s_tmem, 256);
   handoff();
+  pdl_wait();
   const uint32_t tm = *s_tmem;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
   const uint32_t tQh = smem_u32(sQh), tQl = smem_u32(sQl), tKh = smem_u32(sKh), tKl = smem_u32(sKl);
@@ -790,6 +792,7 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_bwd_bf16x(const __grid_c
   }
   if (warp == 0) tmem_alloc(s_tmem, 512);
   handoff();
+  pdl_wait();
   const uint32_t tm = *s_tmem;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
   uint32_t t[7];
@@ -1131,9 +1134,9 @@ int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const flo
   const int nnb = (im.N + a.bn - 1) / a.bn;
   dim3 grid((unsigned)std::min(mt, std::max(1, sms / nnb)), (unsigned)nnb);
   if (Z)
-    k_gemm_bf16x<true><<<grid, XTHREADS, x_smem(a.bn), st>>>(map, a);
+    launch_pdl(k_gemm_bf16x<true>, grid, XTHREADS, x_smem(a.bn), st, map, a);
   else
-    k_gemm_bf16x<false><<<grid, XTHREADS, x_smem(a.bn), st>>>(map, a);
+    launch_pdl(k_gemm_bf16x<false>, grid, XTHREADS, x_smem(a.bn), st, map, a);
   note_launch();
   return DP_OK;
 }
@@ -1168,9 +1171,9 @@ void attn_core_fwd_bf16x(dp_model* m, int n, int l, cudaStream_t st) {
   if (n == 0) return;
   const int grid = std::min(n, x_sm_count(m->device));
   if (m->A == 256)
-    k_attn_core_fwd_bf16x<2><<<grid, XC_NT, XF_SMEM, st>>>(core_args(m, n, l));
+    launch_pdl(k_attn_core_fwd_bf16x<2>, grid, XC_NT, XF_SMEM, st, core_args(m, n, l));
   else
-    k_attn_core_fwd_bf16x<1><<<grid, XC_NT, XF_SMEM, st>>>(core_args(m, n, l));
+    launch_pdl(k_attn_core_fwd_bf16x<1>, grid, XC_NT, XF_SMEM, st, core_args(m, n, l));
   note_launch();
 }
 
@@ -1178,9 +1181,9 @@ void attn_core_bwd_bf16x(dp_model* m, int n, int l, cudaStream_t st) {
   if (n == 0) return;
   const int grid = std::min(n, x_sm_count(m->device));
   if (m->A == 256)
-    k_attn_core_bwd_bf16x<2><<<grid, XC_NT, XB_SMEM, st>>>(core_args(m, n, l));
+    launch_pdl(k_attn_core_bwd_bf16x<2>, grid, XC_NT, XB_SMEM, st, core_args(m, n, l));
   else
-    k_attn_core_bwd_bf16x<1><<<grid, XC_NT, XB_SMEM, st>>>(core_args(m, n, l));
+    launch_pdl(k_attn_core_bwd_bf16x<1>, grid, XC_NT, XB_SMEM, st, core_args(m, n, l));
   note_launch();
 }
 

@@ -146,6 +146,7 @@ struct RowPos {
 
 template <int E0, int E1, int E2>
 __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::F_CTAS) k_embed_rows_fwd(EmbedArgs a) {
+  pdl_wait();
   using N = RowNet<E0, E1, E2>;
   extern __shared__ __align__(16) float sm[];
   row_weights<E0, E1, E2>(sm, a.w);
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::F_CTAS) k_embed_rows
 
 template <int E0, int E1, int E2>
 __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::B_CTAS) k_embed_rows_bwd(EmbedArgs a) {
+  pdl_wait();
   using N = RowNet<E0, E1, E2>;
   extern __shared__ __align__(16) float sm[];
   row_weights<E0, E1, E2>(sm, a.w);
@@ -298,10 +300,10 @@ void rows_launch(const EmbedArgs& a, bool bwd, cudaStream_t st) {
   const int grid = std::min(a.n, (bwd ? N::B_CTAS : N::F_CTAS) * std::max(1, sms));
   if (!bwd) {
     cudaFuncSetAttribute(k_embed_rows_fwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_embed_rows_fwd<E0, E1, E2><<<grid, ER_T, smem, st>>>(a);
+    launch_pdl(k_embed_rows_fwd<E0, E1, E2>, grid, ER_T, smem, st, a);
   } else {
     cudaFuncSetAttribute(k_embed_rows_bwd<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_embed_rows_bwd<E0, E1, E2><<<grid, ER_T, smem, st>>>(a);
+    launch_pdl(k_embed_rows_bwd<E0, E1, E2>, grid, ER_T, smem, st, a);
   }
   note_launch();
 }

@@ -15,6 +15,7 @@ namespace dpa1 {
 // relative, far below those paths' operand rounding.  Both store FP32.
 template <typename Real>
 __global__ void k_env(EnvArgs a) {
+  pdl_wait();
   long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long long)a.n * NP) return;
   const int i = (int)(row / NP);
@@ -57,15 +58,16 @@ __global__ void k_env(EnvArgs a) {
   reinterpret_cast<float4*>(a.R)[row] = R;
   reinterpret_cast<float4*>(a.rw)[row] = rw;
   reinterpret_cast<float4*>(a.rv)[row] = rv;
+  reinterpret_cast<float4*>(a.dgeo)[row] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 void launch_env(const EnvArgs& a, cudaStream_t st) {
   long long rows = (long long)a.n * NP;
   if (rows == 0) return;
   if (a.fp64)
-    k_env<double><<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(a);
+    launch_pdl(k_env<double>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
   else
-    k_env<float><<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(a);
+    launch_pdl(k_env<float>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
   note_launch();
 }
 
@@ -75,6 +77,7 @@ void launch_env(const EnvArgs& a, cudaStream_t st) {
 // Real = float uses the stored FP32 displacement.
 template <typename Real>
 __global__ void k_env_bwd(EnvBwdArgs a) {
+  pdl_wait();
   long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long long)a.n * NP) return;
   float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -128,9 +131,9 @@ void launch_env_bwd(const EnvBwdArgs& a, cudaStream_t st) {
   long long rows = (long long)a.n * NP;
   if (rows == 0) return;
   if (a.fp64)
-    k_env_bwd<double><<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(a);
+    launch_pdl(k_env_bwd<double>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
   else
-    k_env_bwd<float><<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(a);
+    launch_pdl(k_env_bwd<float>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
   note_launch();
 }
 
@@ -142,6 +145,7 @@ void launch_env_bwd(const EnvBwdArgs& a, cudaStream_t st) {
 // GPU is narrow), the per-block virial and energy in FP64.
 constexpr int FWARPS = FORCE_BLOCK_ATOMS;
 __global__ void __launch_bounds__(32 * FWARPS) k_force(ForceArgs a) {
+  pdl_wait();
   __shared__ int srev[FWARPS][REV_CAP];
   __shared__ double sred[FWARPS][10];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -215,6 +219,7 @@ __global__ void __launch_bounds__(32 * FWARPS) k_force(ForceArgs a) {
 // seg[b+1] - seg[0])), else one block over rows [0, nblocks).
 __global__ void k_finalize(const double* __restrict__ partials, int nblocks, const int* __restrict__ seg,
                            double* __restrict__ energy, double* __restrict__ virial) {
+  pdl_wait();
   __shared__ double red[10][32];
   const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;  // 10 warps, one per quantity
   int b0 = 0, cnt = nblocks;
@@ -243,16 +248,16 @@ __global__ void k_finalize(const double* __restrict__ partials, int nblocks, con
 void launch_force_virial(const ForceArgs& a, cudaStream_t st) {
   const int nb = a.n > 0 ? (a.n + FWARPS - 1) / FWARPS : 0;
   if (nb > 0) {
-    k_force<<<nb, 32 * FWARPS, 0, st>>>(a);
+    launch_pdl(k_force, nb, 32 * FWARPS, 0, st, a);
     note_launch();
   }
   if (a.seg) {
     if (a.nseg > 0) {
-      k_finalize<<<a.nseg, 320, 0, st>>>(a.partials, nb, a.seg, a.energy, a.virial);
+      launch_pdl(k_finalize, a.nseg, 320, 0, st, a.partials, nb, a.seg, a.energy, a.virial);
       note_launch();
     }
   } else {
-    k_finalize<<<1, 320, 0, st>>>(a.partials, nb, nullptr, a.energy, a.virial);
+    launch_pdl(k_finalize, 1, 320, 0, st, a.partials, nb, nullptr, a.energy, a.virial);
     note_launch();
   }
 }

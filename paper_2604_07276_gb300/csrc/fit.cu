@@ -145,6 +145,7 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
   __syncthreads();
   fence_after_sync();
   const uint32_t tm = *s_tmem;
+  pdl_wait();
   const int mb = blockIdx.x;
   Waiter wt{a.err};
 
@@ -427,7 +428,7 @@ int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, 
   a.Z = Z;
   a.err = m->d_err;
   dim3 grid((unsigned)mt, (unsigned)((s.N + a.bn - 1) / a.bn));
-  k_fit_gemm<<<grid, FTHREADS, fit_smem(a.bn), st>>>(map, a);
+  launch_pdl(k_fit_gemm, grid, FTHREADS, fit_smem(a.bn), st, map, a);
   note_launch();
   return DP_OK;
 }

@@ -24,6 +24,7 @@ struct NbrArgs {
   int* atype_c;    // out: types clamped to [0, ntypes)
   float4* coordf;  // scratch [n]: FP32 copy of the coordinates for the candidate screen
   int* err;
+  int* rev_cnt;    // out: zeroed for the reverse list (null: none)
   // packed batches, one frame per call: atoms [n, n_out) are padding (no
   // neighbours, type 0) and base is added to every neighbour index written
   // (0 and 0: plain call)
@@ -41,6 +42,7 @@ void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell
 // ROW_SEG atoms.
 constexpr int ROW_SEG = 4096;
 void launch_row_list(const int* nnei, int n, int* row_off, int* rowmap, int* seg, cudaStream_t st);
+// rev_cnt: zero on entry (the neighbour search clears it).
 void launch_reverse(const int* nlist, int n, int* rev_cnt, int* rev_rows, int* err, cudaStream_t st);
 
 // --- environment matrix and its adjoint, forces, reductions (env.cu)
@@ -57,6 +59,7 @@ struct EnvArgs {
   float* rw;  // [n*NP][4] (rhat_x, rhat_y, rhat_z, w)
   float* rv;  // [n*NP][4] (x, y, z, |r|)
   double* w64;  // [n*NP] switch weight in FP64
+  float* dgeo;  // [n*NP][4] zeroed: dE/d(rhat, w) of the adjoint
   int fp64;     // evaluate in FP64 (else FP32 from the FP64 displacement)
   const int* frame = nullptr;  // packed batches: frame of each atom, indexing grid[]
 };

@@ -13,6 +13,7 @@ constexpr double ACC = 9.648533212e-3;                       // (eV / A / amu) i
 // First half kick and drift: v += dt/2 F/m; x += dt v.
 __global__ void k_verlet_drift(int n, double dt, const double* __restrict__ mass, const double* __restrict__ f,
                                double* __restrict__ v, double* __restrict__ x) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * n) return;
   const double a = f[i] / mass[i / 3] * ACC;
@@ -30,6 +31,7 @@ int verlet_kick_blocks(int n) { return (3 * n + KICK_THREADS - 1) / KICK_THREADS
 __global__ void __launch_bounds__(KICK_THREADS) k_verlet_kick(int n, double dt, const double* __restrict__ mass,
                                                                 const double* __restrict__ f, double* __restrict__ v,
                                                                 double* __restrict__ partial) {
+  pdl_wait();
   __shared__ double red[KICK_THREADS / 32];
   const int i = blockIdx.x * KICK_THREADS + threadIdx.x;
   double ke = 0.0;
@@ -53,6 +55,7 @@ __global__ void __launch_bounds__(KICK_THREADS) k_verlet_kick(int n, double dt, 
 // FP64 in a fixed order (one block), and its record (E, kinetic, total).
 __global__ void k_verlet_thermo(int nb, const double* __restrict__ partial, const double* __restrict__ energy,
                                 int* __restrict__ counter, double* __restrict__ thermo, int nrec) {
+  pdl_wait();
   __shared__ double red[32];
   double ke = 0.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) ke += partial[b];
@@ -75,7 +78,7 @@ __global__ void k_verlet_thermo(int nb, const double* __restrict__ partial, cons
 
 void launch_verlet_drift(int n, double dt, const double* mass, const double* f, double* v, double* x, cudaStream_t st) {
   if (n == 0) return;
-  k_verlet_drift<<<(3 * n + 255) / 256, 256, 0, st>>>(n, dt, mass, f, v, x);
+  launch_pdl(k_verlet_drift, (3 * n + 255) / 256, 256, 0, st, n, dt, mass, f, v, x);
   note_launch();
 }
 
@@ -83,10 +86,10 @@ void launch_verlet_kick(int n, double dt, const double* mass, const double* f, d
                         const double* energy, int* counter, double* thermo, int nrec, cudaStream_t st) {
   const int nb = verlet_kick_blocks(n);
   if (nb > 0) {
-    k_verlet_kick<<<nb, KICK_THREADS, 0, st>>>(n, dt, mass, f, v, partial);
+    launch_pdl(k_verlet_kick, nb, KICK_THREADS, 0, st, n, dt, mass, f, v, partial);
     note_launch();
   }
-  k_verlet_thermo<<<1, 1024, 0, st>>>(nb, partial, energy, counter, thermo, nrec);
+  launch_pdl(k_verlet_thermo, 1, 1024, 0, st, nb, partial, energy, counter, thermo, nrec);
   note_launch();
 }
 

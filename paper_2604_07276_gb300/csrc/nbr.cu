@@ -1,17 +1,25 @@
 // Stages a1-a2: cell binning and the full neighbour list (Sec. II-C: DP
 // models need full lists; the O(N) cutoff search of Sec. II-A), plus the
 // reverse list used by the deterministic force gather.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace dpa1 {
 
-// One thread: validate the box and derive the cell grid.  Cell edges are
+// Clears the cell counters, and one thread validates the box and derives the cell grid.  Cell edges are
 // >= rcut, so every neighbour of an atom lies in the 27 cells around it; an
 // axis with fewer than 3 cells is treated as a single cell (no cell would
 // otherwise be visited twice).
 __global__ void k_cell_setup(const double* __restrict__ box, double rcut, int cap_dim,
-                             CellGrid* __restrict__ cg, int* __restrict__ err) {
+                             CellGrid* __restrict__ cg, int* __restrict__ err, int* __restrict__ cell_count,
+                             int* __restrict__ cell_cursor, int cell_cap) {
+  pdl_wait();
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cell_cap; c += gridDim.x * blockDim.x) {
+    cell_count[c] = 0;
+    cell_cursor[c] = 0;
+  }
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   CellGrid g;
   g.ok = 1;
@@ -49,6 +57,7 @@ __global__ void k_cell_count(const double* __restrict__ coord, const int* __rest
                              int* __restrict__ cell_count, int* __restrict__ atype_c, float4* __restrict__ coordf,
                              int* __restrict__ err, const int* __restrict__ frame, const int* __restrict__ cell_base,
                              int cb0) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int cbase = 0;
@@ -89,6 +98,7 @@ __global__ void k_cell_count(const double* __restrict__ coord, const int* __rest
 // Exclusive scan of the cell counts (one block).
 __global__ void k_cell_scan(const int* __restrict__ cell_count, int* __restrict__ cell_start,
                             const CellGrid* __restrict__ cgp, int ncells_given) {
+  pdl_wait();
   __shared__ int part[1024];
   __shared__ int carry;
   const int ncells = ncells_given >= 0 ? ncells_given : cgp->ncells;
@@ -115,6 +125,7 @@ __global__ void k_cell_scan(const int* __restrict__ cell_count, int* __restrict_
 
 __global__ void k_cell_fill(const int* __restrict__ cell_of, int n, const int* __restrict__ cell_start,
                             int* __restrict__ cell_cursor, int* __restrict__ cell_atoms) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int c = cell_of[i];
@@ -150,12 +161,14 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
             const int* __restrict__ cell_atoms, double rc2, int sel, int* __restrict__ nlist,
             int* __restrict__ nnei, int* __restrict__ ncand, int* __restrict__ atype_c,
             const float4* __restrict__ coordf, int* __restrict__ err, const int* __restrict__ frame,
-            const int* __restrict__ cell_base, int cb0) {
+            const int* __restrict__ cell_base, int cb0, int* __restrict__ rev_cnt) {
+  pdl_wait();
   __shared__ unsigned long long skey[NBR_WARPS][NBR_CAP];
   __shared__ int sidx[NBR_WARPS][NBR_CAP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * NBR_WARPS + warp;
   const int fi = frame && i < n ? frame[i] : 0;
+  if (rev_cnt && lane == 0 && i < n_out) rev_cnt[i] = 0;
   if (i >= n || fi < 0) {
     // padding atoms of a packed batch: no neighbours, a valid type
     if (i < n_out || (i < n && fi < 0)) {
@@ -283,6 +296,7 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
 // Reverse list: for every kept pair (i, slot) -> j, record row i*NP+slot under j.
 __global__ void k_rev_fill(const int* __restrict__ nlist, int n, int* __restrict__ rev_cnt,
                            int* __restrict__ rev_rows, int* __restrict__ err) {
+  pdl_wait();
   long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long long)n * NP) return;
   int j = nlist[row];
@@ -295,25 +309,24 @@ __global__ void k_rev_fill(const int* __restrict__ nlist, int n, int* __restrict
 }
 
 void launch_neighbors(const NbrArgs& a, cudaStream_t st) {
-  cudaMemsetAsync(a.cell_count, 0, sizeof(int) * (size_t)a.cell_cap, st);
-  cudaMemsetAsync(a.cell_cursor, 0, sizeof(int) * (size_t)a.cell_cap, st);
-  k_cell_setup<<<1, 1, 0, st>>>(a.box, a.rcut, a.cap_dim, a.grid, a.err);
+  launch_pdl(k_cell_setup, std::min(152, (a.cell_cap + 255) / 256), 256, 0, st, a.box, a.rcut, a.cap_dim, a.grid,
+             a.err, a.cell_count, a.cell_cursor, a.cell_cap);
   note_launch();
   const int n_out = a.n_out > a.n ? a.n_out : a.n;
   if (n_out == 0) return;
   const int tb = 256;
   if (a.n > 0) {
-    k_cell_count<<<(a.n + tb - 1) / tb, tb, 0, st>>>(a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of,
+    launch_pdl(k_cell_count, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of,
                                                     a.cell_count, a.atype_c, a.coordf, a.err, nullptr, nullptr, 0);
     note_launch();
-    k_cell_scan<<<1, 1024, 0, st>>>(a.cell_count, a.cell_start, a.grid, -1);
+    launch_pdl(k_cell_scan, 1, 1024, 0, st, a.cell_count, a.cell_start, a.grid, -1);
     note_launch();
-    k_cell_fill<<<(a.n + tb - 1) / tb, tb, 0, st>>>(a.cell_of, a.n, a.cell_start, a.cell_cursor, a.cell_atoms);
+    launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.cell_of, a.n, a.cell_start, a.cell_cursor, a.cell_atoms);
     note_launch();
   }
-  k_neighbors<<<(n_out + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st>>>(
+  launch_pdl(k_neighbors, (n_out + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st,
       a.coord, a.n, n_out, a.base, a.grid, a.cell_of, a.cell_start, a.cell_atoms, a.rcut * a.rcut, a.sel, a.nlist,
-      a.nnei, a.ncand, a.atype_c, a.coordf, a.err, nullptr, nullptr, 0);
+      a.nnei, a.ncand, a.atype_c, a.coordf, a.err, nullptr, nullptr, 0, a.rev_cnt);
   note_launch();
 }
 
@@ -323,16 +336,16 @@ void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell
   cudaMemsetAsync(a.cell_count, 0, sizeof(int) * (size_t)ncells_total, st);
   cudaMemsetAsync(a.cell_cursor, 0, sizeof(int) * (size_t)ncells_total, st);
   const int tb = 256;
-  k_cell_count<<<(a.n + tb - 1) / tb, tb, 0, st>>>(a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of, a.cell_count,
+  launch_pdl(k_cell_count, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of, a.cell_count,
                                                   a.atype_c, a.coordf, a.err, frame, cell_base, cb0);
   note_launch();
-  k_cell_scan<<<1, 1024, 0, st>>>(a.cell_count, a.cell_start, a.grid, ncells_total);
+  launch_pdl(k_cell_scan, 1, 1024, 0, st, a.cell_count, a.cell_start, a.grid, ncells_total);
   note_launch();
-  k_cell_fill<<<(a.n + tb - 1) / tb, tb, 0, st>>>(a.cell_of, a.n, a.cell_start, a.cell_cursor, a.cell_atoms);
+  launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.cell_of, a.n, a.cell_start, a.cell_cursor, a.cell_atoms);
   note_launch();
-  k_neighbors<<<(a.n + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st>>>(
+  launch_pdl(k_neighbors, (a.n + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st,
       a.coord, a.n, a.n, 0, a.grid, a.cell_of, a.cell_start, a.cell_atoms, a.rcut * a.rcut, a.sel, a.nlist, a.nnei,
-      a.ncand, a.atype_c, a.coordf, a.err, frame, cell_base, cb0);
+      a.ncand, a.atype_c, a.coordf, a.err, frame, cell_base, cb0, a.rev_cnt);
   note_launch();
 }
 
@@ -353,6 +366,7 @@ __device__ __forceinline__ int block_sum(int v, int* s_red) {
 }
 
 __global__ void __launch_bounds__(ROWL_T) k_row_seg(const int* __restrict__ nnei, int n, int* __restrict__ seg) {
+  pdl_wait();
   __shared__ int s_red[ROWL_T / 32];
   int v = 0;
   for (int i = blockIdx.x * ROW_SEG + threadIdx.x; i < min(n, (int)(blockIdx.x + 1) * ROW_SEG); i += ROWL_T) v += nnei[i];
@@ -362,6 +376,7 @@ __global__ void __launch_bounds__(ROWL_T) k_row_seg(const int* __restrict__ nnei
 
 __global__ void __launch_bounds__(ROWL_T) k_row_list(const int* __restrict__ nnei, int n, const int* __restrict__ seg,
                                                      int* __restrict__ row_off, int* __restrict__ rowmap) {
+  pdl_wait();
   __shared__ int s_red[ROWL_T / 32], s_off[ROWL_ATOMS];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int first = blockIdx.x * ROWL_ATOMS, s0 = first / ROW_SEG;
@@ -391,18 +406,17 @@ __global__ void __launch_bounds__(ROWL_T) k_row_list(const int* __restrict__ nne
 void launch_row_list(const int* nnei, int n, int* row_off, int* rowmap, int* seg, cudaStream_t st) {
   if (n == 0) return;
   if (n > ROW_SEG) {
-    k_row_seg<<<(n + ROW_SEG - 1) / ROW_SEG, ROWL_T, 0, st>>>(nnei, n, seg);
+    launch_pdl(k_row_seg, (n + ROW_SEG - 1) / ROW_SEG, ROWL_T, 0, st, nnei, n, seg);
     note_launch();
   }
-  k_row_list<<<(n + ROWL_ATOMS - 1) / ROWL_ATOMS, ROWL_T, 0, st>>>(nnei, n, seg, row_off, rowmap);
+  launch_pdl(k_row_list, (n + ROWL_ATOMS - 1) / ROWL_ATOMS, ROWL_T, 0, st, nnei, n, seg, row_off, rowmap);
   note_launch();
 }
 
 void launch_reverse(const int* nlist, int n, int* rev_cnt, int* rev_rows, int* err, cudaStream_t st) {
-  cudaMemsetAsync(rev_cnt, 0, sizeof(int) * (size_t)(n > 0 ? n : 1), st);
   if (n == 0) return;
   long long rows = (long long)n * NP;
-  k_rev_fill<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(nlist, n, rev_cnt, rev_rows, err);
+  launch_pdl(k_rev_fill, (unsigned)((rows + 255) / 256), 256, 0, st, nlist, n, rev_cnt, rev_rows, err);
   note_launch();
 }
 

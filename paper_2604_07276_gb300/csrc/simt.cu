@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(256, 2)
 k_sgemm128(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
            const float* __restrict__ bias, const float* __restrict__ R, int ldr, float* __restrict__ C, int ldc,
            int M, int N, int K, const int* __restrict__ m_dev) {
+  pdl_wait();
   if (m_dev) M = *m_dev;
   if ((long long)blockIdx.x * 128 >= M) return;
   __shared__ __align__(16) float As[2][GBK][GLD];  // k-major: As[k][row]
@@ -145,9 +146,9 @@ static void sgemm_launch(dim3 grid, bool vec, const float* A, int lda, const flo
                          const float* R, int ldr, float* C, int ldc, int M, int N, int K, const int* m_dev,
                          cudaStream_t st) {
   if (vec)
-    k_sgemm128<EPI, true><<<grid, 256, 0, st>>>(A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev);
+    launch_pdl(k_sgemm128<EPI, true>, grid, 256, 0, st, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev);
   else
-    k_sgemm128<EPI, false><<<grid, 256, 0, st>>>(A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev);
+    launch_pdl(k_sgemm128<EPI, false>, grid, 256, 0, st, A, lda, B, ldb, bias, R, ldr, C, ldc, M, N, K, m_dev);
 }
 
 void gemm_f32(const float* A, int lda, const float* B, int ldb, const float* bias, const float* R, int ldr,
@@ -270,6 +271,7 @@ __device__ __forceinline__ void embed_forward(float* sm, int cnt, const float* b
 // `grad` once at the end.
 template <int E0, int E1, int E2>
 __global__ void __launch_bounds__(ETHREADS) k_embed_wgrad(EmbedArgs a, float* grad, const float* scale) {
+  pdl_wait();
   using Lw = EmbedLayout<E0, E1, E2>;
   using S = EmbedSmem<E0, E1, E2>;
   extern __shared__ float sm[];
@@ -365,7 +367,7 @@ static void embed_wgrad_launch(const EmbedArgs& a, float* grad, const float* sca
   const size_t smem = sizeof(float) * (S::TOTAL + Lw::TOTAL);
   cudaFuncSetAttribute(k_embed_wgrad<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int grid = std::min(2 * a.n, 2 * sm_count());
-  k_embed_wgrad<E0, E1, E2><<<grid, ETHREADS, smem, st>>>(a, grad, scale);
+  launch_pdl(k_embed_wgrad<E0, E1, E2>, grid, ETHREADS, smem, st, a, grad, scale);
   note_launch();
 }
 
@@ -381,6 +383,7 @@ bool launch_embed_wgrad(const EmbedArgs& a, const int* w, float* grad, const flo
 __global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restrict__ Gin, const int* __restrict__ nrows,
                              const float* __restrict__ gamma, const float* __restrict__ beta, float eps,
                              float* __restrict__ Gout, float* __restrict__ stats, int m1) {
+  pdl_wait();
   const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= *nrows) return;
@@ -420,6 +423,7 @@ __global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restric
 __global__ void k_ln_bwd(const float* __restrict__ dZ, const float* __restrict__ Y, const float* __restrict__ stats,
                          const int* __restrict__ nrows, const float* __restrict__ gamma, float* __restrict__ dY,
                          int m1) {
+  pdl_wait();
   const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= *nrows) return;
@@ -451,14 +455,14 @@ void launch_ln_res_fwd(const float* Y, const float* Gin, const int* nrows, const
                        float eps, float* Gout, float* stats, int rows_i, int m1, cudaStream_t st) {
   long long rows = rows_i;
   if (rows == 0) return;
-  k_ln_res_fwd<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(Y, Gin, nrows, gamma, beta, eps, Gout, stats, m1);
+  launch_pdl(k_ln_res_fwd, (unsigned)((rows * 32 + 255) / 256), 256, 0, st, Y, Gin, nrows, gamma, beta, eps, Gout, stats, m1);
   note_launch();
 }
 void launch_ln_bwd(const float* dZ, const float* Y, const float* stats, const int* nrows, const float* gamma,
                    float* dY, int rows_i, int m1, cudaStream_t st) {
   long long rows = rows_i;
   if (rows == 0) return;
-  k_ln_bwd<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(dZ, Y, stats, nrows, gamma, dY, m1);
+  launch_pdl(k_ln_bwd, (unsigned)((rows * 32 + 255) / 256), 256, 0, st, dZ, Y, stats, nrows, gamma, dY, m1);
   note_launch();
 }
 
@@ -609,6 +613,7 @@ __device__ __forceinline__ void tile_store_row(float* dst, const float* accrow, 
 
 template <int A>
 __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale) {
+  pdl_wait();
   extern __shared__ float sm[];
   float* X = sm;                 // [128][TLD]: Q chunk (feature-major), then P (row-major)
   float* Y = X + 128 * TLD;      // [128][TLD]: K chunk (feature-major), then a part of [G 1] (key-major)
@@ -734,6 +739,7 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
 // column parts are summed over the 16 row groups in a fixed order.
 template <int A>
 __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale) {
+  pdl_wait();
   extern __shared__ float sm[];
   float* B0 = sm;               // [128][TLD] operand chunks
   float* B1 = B0 + 128 * TLD;   // [128][TLD] K / G chunk, then dS (row-major)
@@ -979,11 +985,11 @@ static void attn_f32_launch(const AttnArgs& a, bool bwd, cudaStream_t st) {
   if (!bwd) {
     const size_t smem = sizeof(float) * (2 * 128 * TLD + 4 * NP) + sizeof(float2) * NP;
     cudaFuncSetAttribute(k_attn_fwd_f32<A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_attn_fwd_f32<A><<<grid, FTF, smem, st>>>(a, scale);
+    launch_pdl(k_attn_fwd_f32<A>, grid, FTF, smem, st, a, scale);
   } else {
     const size_t smem = sizeof(float) * (3 * 128 * TLD + 8 * NP) + sizeof(float2) * NP;
     cudaFuncSetAttribute(k_attn_bwd_f32<A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_attn_bwd_f32<A><<<grid, FTF, smem, st>>>(a, scale);
+    launch_pdl(k_attn_bwd_f32<A>, grid, FTF, smem, st, a, scale);
   }
   note_launch();
 }
@@ -1007,6 +1013,7 @@ void launch_attn_bwd_f32(const AttnArgs& a, cudaStream_t st) {
 // A block of 128 threads per atom, 10 blocks per SM (48 registers): the kernel
 // waits on its loads, and more resident warps hide more of them.
 __global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
+  pdl_wait();
   extern __shared__ float sm[];
   float* Ts = sm;  // [4][m1]
   const int atom = blockIdx.x;
@@ -1074,6 +1081,7 @@ __global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
 // dT[c][p] = sum_b<axis dD[p][b] T[c][b] + (p < axis) sum_q dD[q][p] T[c][q];
 // dG_s = R_s dT / sel; dR_s = G_s dT^T / sel.
 __global__ void k_desc_bwd(DescArgs a) {
+  pdl_wait();
   extern __shared__ float sm[];
   const int m1 = a.m1, ax = a.axis;
   float* Ts = sm;              // [4][m1]
@@ -1174,13 +1182,13 @@ __global__ void k_desc_bwd(DescArgs a) {
 
 void launch_desc_fwd(const DescArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
-  k_desc_fwd<<<a.n, 128, sizeof(float) * 4 * a.m1, st>>>(a);
+  launch_pdl(k_desc_fwd, a.n, 128, sizeof(float) * 4 * a.m1, st, a);
   note_launch();
 }
 void launch_desc_bwd(const DescArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
   size_t sm = sizeof(float) * (8 * a.m1 + 2 * a.m1 * a.axis);
-  k_desc_bwd<<<a.n, 128, sm, st>>>(a);
+  launch_pdl(k_desc_bwd, a.n, 128, sm, st, a);
   note_launch();
 }
 
@@ -1189,6 +1197,7 @@ __global__ void k_energy_head(const float* __restrict__ H, const float* __restri
                               const float* __restrict__ w, const float* __restrict__ bptr,
                               const float* __restrict__ ebias, const int* __restrict__ atype, float* __restrict__ e,
                               float* __restrict__ dH, float* __restrict__ dZ) {
+  pdl_wait();
   const int atom = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (atom >= n) return;
@@ -1210,13 +1219,14 @@ void launch_energy_head(const float* H, const float* Hprev, int n, int nlocal, i
                         const float* b_out, const float* ebias, const int* atype, float* e, float* dH, float* dZ,
                         cudaStream_t st) {
   if (n == 0) return;
-  k_energy_head<<<(unsigned)(((long long)n * 32 + 255) / 256), 256, 0, st>>>(H, Hprev, n, nlocal, width, w_out, b_out,
+  launch_pdl(k_energy_head, (unsigned)(((long long)n * 32 + 255) / 256), 256, 0, st, H, Hprev, n, nlocal, width, w_out, b_out,
                                                                           ebias, atype, e, dH, dZ);
   note_launch();
 }
 
 __global__ void k_tanh_bwd(const float* __restrict__ dH, const float* __restrict__ Hc, const float* __restrict__ Hp,
                            float* __restrict__ dZ, long long count) {
+  pdl_wait();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float t = Hp ? Hc[i] - Hp[i] : Hc[i];
@@ -1226,12 +1236,13 @@ __global__ void k_tanh_bwd(const float* __restrict__ dH, const float* __restrict
 void launch_tanh_bwd(const float* dH, const float* Hcur, const float* Hprev, float* dZ, long long count,
                      cudaStream_t st) {
   if (count == 0) return;
-  k_tanh_bwd<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(dH, Hcur, Hprev, dZ, count);
+  launch_pdl(k_tanh_bwd, (unsigned)((count + 255) / 256), 256, 0, st, dH, Hcur, Hprev, dZ, count);
   note_launch();
 }
 
 __global__ void k_fill_rows(float* __restrict__ dst, const float* __restrict__ row, long long count, long long nlocal_el,
                             int width) {
+  pdl_wait();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   dst[i] = i < nlocal_el ? row[i % width] : 0.f;
@@ -1240,7 +1251,7 @@ __global__ void k_fill_rows(float* __restrict__ dst, const float* __restrict__ r
 void launch_fill_rows(float* dst, const float* row, int n, int nlocal, int width, cudaStream_t st) {
   long long count = (long long)n * width;
   if (count == 0) return;
-  k_fill_rows<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(dst, row, count, (long long)nlocal * width, width);
+  launch_pdl(k_fill_rows, (unsigned)((count + 255) / 256), 256, 0, st, dst, row, count, (long long)nlocal * width, width);
   note_launch();
 }
 

@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(NT, 1) k_layer_fwd_tc(const __grid_constant__ 
   }
   if (warp == 0) tmem_alloc(s_tmem, 512);
   handoff();
+  pdl_wait();
   const uint32_t tm = *s_tmem;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
   const uint32_t tA = smem_u32(sA), tB = smem_u32(sB), tC = smem_u32(sC), tD = smem_u32(sD);
@@ -421,6 +422,7 @@ __global__ void __launch_bounds__(NT, 1) k_layer_bwd_tc(const __grid_constant__ 
   }
   if (warp == 0) tmem_alloc(s_tmem, 512);
   handoff();
+  pdl_wait();
   const uint32_t tm = *s_tmem;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
   const uint32_t tA = smem_u32(sA), tB = smem_u32(sB), tC = smem_u32(sC), tD = smem_u32(sD);
@@ -934,19 +936,18 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
   prof_mark(m, "embed_fwd", st);
   for (int l = 0; l < L && n > 0; ++l) {
     if (f16)
-      k_layer_fwd_tc<true><<<grid, NT, F_SMEM, st>>>(largs(l));
+      launch_pdl(k_layer_fwd_tc<true>, grid, NT, F_SMEM, st, largs(l));
     else
-      k_layer_fwd_tc<false><<<grid, NT, F_SMEM, st>>>(largs(l));
+      launch_pdl(k_layer_fwd_tc<false>, grid, NT, F_SMEM, st, largs(l));
     note_launch();
     prof_mark(m, "attn_fwd_tc", st);
   }
   run_descriptor_fitting(m, n, atype, st);
-  cudaMemsetAsync(ws.dgeo, 0, sizeof(float) * rows * 4, st);
   for (int l = L - 1; l >= 0 && n > 0; --l) {
     if (f16)
-      k_layer_bwd_tc<true><<<grid, NT, B_SMEM, st>>>(largs(l));
+      launch_pdl(k_layer_bwd_tc<true>, grid, NT, B_SMEM, st, largs(l));
     else
-      k_layer_bwd_tc<false><<<grid, NT, B_SMEM, st>>>(largs(l));
+      launch_pdl(k_layer_bwd_tc<false>, grid, NT, B_SMEM, st, largs(l));
     note_launch();
     prof_mark(m, "attn_bwd_tc", st);
   }

@@ -532,6 +532,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
   uint64_t* bar;
   uint32_t* s_tmem;
   embed_tc_setup<S>(a, sm, bar, s_tmem, S::F_SMEM);
+  pdl_wait();
   const uint32_t tm = *s_tmem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
   const int row = quad * 32 + lane;
@@ -594,6 +595,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(
   uint64_t* bar;
   uint32_t* s_tmem;
   embed_tc_setup<S>(a, sm, bar, s_tmem, S::B_SMEM);
+  pdl_wait();
   const uint32_t tm = *s_tmem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
   const int row = quad * 32 + lane;
@@ -738,8 +740,8 @@ namespace {
 // (the fused 16-bit paths) or BF16 (bf16x) operand splits.
 template <class S, bool F16>
 void tc_embed_launch_s(int grid, const EmbedTcArgs& et, bool bwd, cudaStream_t st) {
-  if (!bwd) k_embed_tc_fwd_live<S, F16><<<grid, EMB_THREADS, S::F_SMEM, st>>>(et);
-  if (bwd) k_embed_tc_bwd_live<S, F16><<<grid, EMB_THREADS, S::B_SMEM, st>>>(et);
+  if (!bwd) launch_pdl(k_embed_tc_fwd_live<S, F16>, grid, EMB_THREADS, S::F_SMEM, st, et);
+  if (bwd) launch_pdl(k_embed_tc_bwd_live<S, F16>, grid, EMB_THREADS, S::B_SMEM, st, et);
 }
 
 }  // namespace

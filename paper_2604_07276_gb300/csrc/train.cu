@@ -23,6 +23,7 @@ namespace dpa1 {
 __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ A, int lda, const float* __restrict__ B,
                                                int ldb, float* __restrict__ C, int ldc, int I, int O, int N, int chunk,
                                                const float* __restrict__ scale) {
+  pdl_wait();
   __shared__ float As[16][64 + 4];
   __shared__ float Bs[16][64 + 4];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ A, int 
 // c[o] += scale * factor * sum_n B[n][o]
 __global__ void k_colsum(const float* __restrict__ B, int ldb, float* __restrict__ c, int O, int N, int chunk,
                          const float* __restrict__ scale, float factor) {
+  pdl_wait();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= O) return;
   const int n_begin = blockIdx.y * chunk, n_end = min(N, n_begin + chunk);
@@ -74,6 +76,7 @@ __global__ void k_colsum(const float* __restrict__ B, int ldb, float* __restrict
 // de_i/d ebias[t_i] = 1 and de_i/d b_out = out_scale for every atom.
 __global__ void k_head_bias_grad(const int* __restrict__ atype, int n, float* __restrict__ g_ebias,
                                  float* __restrict__ g_bout, const float* __restrict__ scale, float out_scale) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float s = *scale;
@@ -87,6 +90,7 @@ __global__ void k_train_prep(int n, const double* __restrict__ energy, double e_
                              const double* __restrict__ force, const double* __restrict__ force_ref, double pe,
                              double pf, double* __restrict__ v, double* __restrict__ loss,
                              float* __restrict__ scales) {
+  pdl_wait();
   __shared__ double red_s[32];
   double ss = 0.0;
   for (int k = threadIdx.x; k < 3 * n; k += blockDim.x) {
@@ -115,6 +119,7 @@ __global__ void k_train_prep(int n, const double* __restrict__ energy, double e_
 }
 
 __global__ void k_axpy(float* __restrict__ g, const float* __restrict__ src, int n, const float* __restrict__ scale) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) g[i] += *scale * src[i];
 }
@@ -125,6 +130,7 @@ __global__ void k_axpy(float* __restrict__ g, const float* __restrict__ src, int
 // (q r_a - avg_a)/std_a): s' = s_d d', (q r_a)' = q_d d' r_a + q r_a',
 // d' = r.r'/d.  (The image shift of r is constant.)
 __global__ void k_env_jvp(JvpArgs a) {
+  pdl_wait();
   const long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long long)a.n * NP) return;
   float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -195,6 +201,7 @@ __device__ __forceinline__ float jskip(const float* x, int o) {
 template <int E0, int E1, int E2>
 __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, float* __restrict__ grad,
                                                          const float* __restrict__ scale) {
+  pdl_wait();
   using S = JvpEmbedSmem<E0, E1, E2>;
   extern __shared__ float sm[];
   const int tid = threadIdx.x;
@@ -388,6 +395,7 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, flo
 // T' = (R'^T G + R^T G') / sel and D' = T'^T T_< + T^T T'_< (the type row of
 // X is constant).  One CTA per atom.
 __global__ void k_desc_jvp_fwd(JvpArgs a) {
+  pdl_wait();
   extern __shared__ float sm[];
   const int m1 = a.m1, ax = a.axis;
   float* Ts = sm;            // [4][m1]
@@ -423,6 +431,7 @@ __global__ void k_desc_jvp_fwd(JvpArgs a) {
 // dT = (dD T_< + [p < axis] dD^T T) / sel as in the descriptor adjoint, its
 // tangent by the product rule, and (dE/dG)' = R' dT + R dT'.
 __global__ void k_desc_jvp_bwd(JvpArgs a) {
+  pdl_wait();
   extern __shared__ float sm[];
   const int m1 = a.m1, ax = a.axis;
   float* Ts = sm;
@@ -472,6 +481,7 @@ __global__ void k_desc_jvp_bwd(JvpArgs a) {
 
 __global__ void k_tanh_jvp(const float* __restrict__ Zd, const float* __restrict__ H, const float* __restrict__ Hprev,
                            const float* __restrict__ Hprevd, float* __restrict__ Hd, long long count) {
+  pdl_wait();
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   const float t = Hprev ? H[k] - Hprev[k] : H[k];
@@ -482,6 +492,7 @@ __global__ void k_tanh_bwd_jvp(const float* __restrict__ dH, const float* __rest
                                const float* __restrict__ Hprev, const float* __restrict__ Hd,
                                const float* __restrict__ Hprevd, float* __restrict__ dZ, float* __restrict__ dZd,
                                long long count) {
+  pdl_wait();
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   const float t = Hprev ? H[k] - Hprev[k] : H[k];
@@ -534,7 +545,7 @@ void launch_wgrad(const float* A, int lda, const float* B, int ldb, float* C, in
   const int splits = std::min(64, std::max({1, N / 256, std::min(N / 32, 304 / tiles)}));
   const int chunk = (N + splits - 1) / splits;
   dim3 grid(blocks(I, 64), blocks(O, 64), splits);
-  k_wgrad<<<grid, 256, 0, st>>>(A, lda, B, ldb, C, ldc, I, O, N, chunk, scale);
+  launch_pdl(k_wgrad, grid, 256, 0, st, A, lda, B, ldb, C, ldc, I, O, N, chunk, scale);
   note_launch();
 }
 
@@ -543,33 +554,33 @@ void launch_colsum(const float* B, int ldb, float* c, int O, int N, const float*
   if (N <= 0 || O <= 0) return;
   const int splits = std::min(128, std::max(1, N / 32));
   const int chunk = (N + splits - 1) / splits;
-  k_colsum<<<dim3(blocks(O, 128), splits), 128, 0, st>>>(B, ldb, c, O, N, chunk, scale, factor);
+  launch_pdl(k_colsum, dim3(blocks(O, 128), splits), 128, 0, st, B, ldb, c, O, N, chunk, scale, factor);
   note_launch();
 }
 
 void launch_head_bias_grad(const int* atype, int n, float* g_ebias, float* g_bout, const float* scale, float out_scale,
                            cudaStream_t st) {
   if (n <= 0) return;
-  k_head_bias_grad<<<blocks(n, 256), 256, 0, st>>>(atype, n, g_ebias, g_bout, scale, out_scale);
+  launch_pdl(k_head_bias_grad, blocks(n, 256), 256, 0, st, atype, n, g_ebias, g_bout, scale, out_scale);
   note_launch();
 }
 
 void launch_train_prep(int n, const double* energy, double e_ref, const double* force, const double* force_ref,
                        double pe, double pf, double* v, double* loss, float* scales, cudaStream_t st) {
-  k_train_prep<<<1, 1024, 0, st>>>(n, energy, e_ref, force, force_ref, pe, pf, v, loss, scales);
+  launch_pdl(k_train_prep, 1, 1024, 0, st, n, energy, e_ref, force, force_ref, pe, pf, v, loss, scales);
   note_launch();
 }
 
 void launch_axpy(float* g, const float* src, int n, const float* scale, cudaStream_t st) {
   if (n <= 0) return;
-  k_axpy<<<blocks(n, 256), 256, 0, st>>>(g, src, n, scale);
+  launch_pdl(k_axpy, blocks(n, 256), 256, 0, st, g, src, n, scale);
   note_launch();
 }
 
 void launch_env_jvp(const JvpArgs& a, cudaStream_t st) {
   const long long rows = (long long)a.n * NP;
   if (rows == 0) return;
-  k_env_jvp<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(a);
+  launch_pdl(k_env_jvp, (unsigned)((rows + 255) / 256), 256, 0, st, a);
   note_launch();
 }
 
@@ -583,7 +594,7 @@ static void embed_jvp_launch(const JvpArgs& a, int mode, float* grad, const floa
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = mode == 1 ? std::min(nblk, 2 * std::max(1, sms)) : nblk;
-  k_embed_jvp<E0, E1, E2><<<grid, JTHREADS, smem, st>>>(a, mode, grad, scale);
+  launch_pdl(k_embed_jvp<E0, E1, E2>, grid, JTHREADS, smem, st, a, mode, grad, scale);
   note_launch();
 }
 
@@ -597,28 +608,28 @@ bool launch_embed_jvp(const JvpArgs& a, const int* w, int mode, float* grad, con
 
 void launch_desc_jvp_fwd(const JvpArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
-  k_desc_jvp_fwd<<<a.n, 128, sizeof(float) * 8 * a.m1, st>>>(a);
+  launch_pdl(k_desc_jvp_fwd, a.n, 128, sizeof(float) * 8 * a.m1, st, a);
   note_launch();
 }
 
 void launch_desc_jvp_bwd(const JvpArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
   const size_t smem = sizeof(float) * (16 * a.m1 + 2 * a.m1 * a.axis);
-  k_desc_jvp_bwd<<<a.n, 128, smem, st>>>(a);
+  launch_pdl(k_desc_jvp_bwd, a.n, 128, smem, st, a);
   note_launch();
 }
 
 void launch_tanh_jvp(const float* Zd, const float* H, const float* Hprev, const float* Hprevd, float* Hd,
                      long long count, cudaStream_t st) {
   if (count <= 0) return;
-  k_tanh_jvp<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(Zd, H, Hprev, Hprevd, Hd, count);
+  launch_pdl(k_tanh_jvp, (unsigned)((count + 255) / 256), 256, 0, st, Zd, H, Hprev, Hprevd, Hd, count);
   note_launch();
 }
 
 void launch_tanh_bwd_jvp(const float* dH, const float* dHd, const float* H, const float* Hprev, const float* Hd,
                          const float* Hprevd, float* dZ, float* dZd, long long count, cudaStream_t st) {
   if (count <= 0) return;
-  k_tanh_bwd_jvp<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(dH, dHd, H, Hprev, Hd, Hprevd, dZ, dZd, count);
+  launch_pdl(k_tanh_bwd_jvp, (unsigned)((count + 255) / 256), 256, 0, st, dH, dHd, H, Hprev, Hd, Hprevd, dZ, dZd, count);
   note_launch();
 }
 
