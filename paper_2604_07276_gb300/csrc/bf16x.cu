@@ -415,6 +415,12 @@ __device__ __forceinline__ void load_blk(const float* src, size_t ld, int nrows,
   }
 }
 
+// (a, b) = hi + lo: the packed BF16 roundings, and those of the residues.
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  hi = pack_bf16(a, b);
+  lo = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+}
+
 // The BF16 high parts (LO = false) or the BF16 roundings of the residues of a
 // block loaded by load_blk, into a 128 x 128 SW128 tile.
 template <bool LO>
@@ -422,17 +428,24 @@ __device__ __forceinline__ void store_blk(uint8_t* tile, const float* v) {
   const int c = 4 * (threadIdx.x & 31);
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
-    float x[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = LO ? v[4 * t + i] - round16<false>(v[4 * t + i]) : v[4 * t + i];
-    *reinterpret_cast<uint2*>(tile + sw128_offset(blk_row(t), c, 128)) =
-        make_uint2(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]));
+    uint2 h, l;
+    split2(v[4 * t], v[4 * t + 1], h.x, l.x);
+    split2(v[4 * t + 2], v[4 * t + 3], h.y, l.y);
+    *reinterpret_cast<uint2*>(tile + sw128_offset(blk_row(t), c, 128)) = LO ? l : h;
   }
 }
 
 __device__ __forceinline__ void store_blk_split(uint8_t* hi, uint8_t* lo, const float* v) {
-  store_blk<false>(hi, v);
-  store_blk<true>(lo, v);
+  const int c = 4 * (threadIdx.x & 31);
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    uint2 h, l;
+    split2(v[4 * t], v[4 * t + 1], h.x, l.x);
+    split2(v[4 * t + 2], v[4 * t + 3], h.y, l.y);
+    const uint32_t off = sw128_offset(blk_row(t), c, 128);
+    *reinterpret_cast<uint2*>(hi + off) = h;
+    *reinterpret_cast<uint2*>(lo + off) = l;
+  }
 }
 
 // FP32 staging of a 128 x 128 block in shared memory (64 KB): float4 q of
@@ -452,31 +465,22 @@ __device__ __forceinline__ void tmem_to_stg(uint32_t taddr, float* s, int row, i
 }
 
 // Rows [0, nrows), columns [0, ncols) of a staged block -> dst (row stride
-// ld), one row per warp access; ACC: dst += (a thread's loads are issued four
-// rows at a time before their stores).  ncols % 4 == 0, ncols <= 128.
+// ld), one row per warp access; ACC: dst +=, as reductions without a return
+// (one writer per element: the same FP32 add as a load, add and store, without
+// the round trip to memory).  ncols % 4 == 0, ncols <= 128.
 template <bool ACC>
 __device__ __forceinline__ void stg_to_global(float* s, float* dst, size_t ld, int nrows, int ncols) {
   const int q = threadIdx.x & 31;
   if (4 * q >= ncols) return;
 #pragma unroll
-  for (int t0 = 0; t0 < 8; t0 += 4) {
-    float4 x[4], y[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int r = blk_row(t0 + t);
-      if (r < nrows) {
-        x[t] = *stg4(s, r, q);
-        if (ACC) y[t] = *reinterpret_cast<const float4*>(dst + (size_t)r * ld + 4 * q);
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int r = blk_row(t0 + t);
-      if (r < nrows) {
-        if (ACC) { x[t].x += y[t].x; x[t].y += y[t].y; x[t].z += y[t].z; x[t].w += y[t].w; }
-        *reinterpret_cast<float4*>(dst + (size_t)r * ld + 4 * q) = x[t];
-      }
-    }
+  for (int t = 0; t < 8; ++t) {
+    const int r = blk_row(t);
+    if (r >= nrows) continue;
+    float4* p = reinterpret_cast<float4*>(dst + (size_t)r * ld + 4 * q);
+    if (ACC)
+      atomicAdd(p, *stg4(s, r, q));
+    else
+      *p = *stg4(s, r, q);
   }
 }
 
@@ -639,12 +643,15 @@ __global__ void __launch_bounds__(XC_NT, 1) k_attn_core_fwd_bf16x(const __grid_c
   if (warp == 0) tmem_dealloc(tm, 256);
 }
 
-// The softmax adjoint over this thread's 32 keys of its row, S and dP
-// re-read from TMEM in pieces of 8: A is recomputed with its row max and
-// normaliser; tsum = sum_k A_jk dA_jk with dA = dP w_j w_k c_jk; then per key
-// dLp = A (dA - tsum), dS = dLp w_j w_k scale -> TMEM over S, P -> the tile
+// The softmax adjoint over this thread's 32 keys of its row: the row max; then
+// e = exp(l' - max) and the gate cosine c of every key, kept in 128 free TMEM
+// columns each (tP + 128, tP + 256), with sum_k e_k and tsum = sum_k A_jk dA_jk
+// (dA = dP w_j w_k c_jk); then per key, in pieces of 8 from TMEM, A = e /
+// sum, dLp = A (dA - tsum), dS = dLp w_j w_k scale -> TMEM over S, P -> the tile
 // pt, dE/d(w_j w_k) = dP A c + dLp (l + shift), dE/dc = dP A w_j w_k.  dP
 // includes dpg1, the adjoint of the row sum of P (the same for every key).
+// Sixteen-key halves past the last neighbour, and lane quadrants whose rows are
+// all past it, only write the zeros that the products read.
 // The row part (this thread's row) and column parts (lanes 0-15: key c0 + h
 // + lane) of dE/drhat and dE/dw are returned.  pt's row lines also carry the
 // row exchanges, before P is stored.
@@ -653,47 +660,60 @@ __device__ __forceinline__ void softmax_adjoint(const XCoreArgs& a, uint8_t* pt,
                                                 float4& rpart, float4* cpart) {
   const int c0 = part * 32;
   const bool rv = row < nn;
+  rpart = cpart[0] = cpart[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto zeros = [&](int h) {
+    const float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int e8 = 0; e8 < 16; e8 += 8) {
+      sw128_store8(pt, row, c0 + h + e8, 128, make_uint4(0u, 0u, 0u, 0u));
+      tmem_st8_async(tS + h + e8, z);
+    }
+  };
+  if (quad * 32 >= nn) {  // the same for the quadrant's four warps
+    zeros(0);
+    zeros(16);
+    tmem_wait_st();
+    return;
+  }
   const RowXchg xr(pt, row, part, lane, quad);
   const float4 kj = s_key[row];
   const float wj = kj.w;
-  // the TMEM loads are warp-collective: their condition is uniform over the
+  // the TMEM accesses are warp-collective: their condition is uniform over the
   // warp (c0), the row mask (rv) is applied per lane
   const bool wlive = c0 < nn;
-  const bool live = wlive && rv;
+  float t[32];
   float mx = -INFINITY;
   if (wlive) {
+    tmem_ld32(tS, t);
 #pragma unroll
-    for (int e8 = 0; e8 < 32; e8 += 8) {
-      float t[8];
-      tmem_ld8(tS + e8, t);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int k = c0 + e8 + i;
-        if (k < nn && rv) mx = fmaxf(mx, (t[i] * a.scale + a.shift) * (wj * s_key[k].w));
-      }
+    for (int i = 0; i < 32; ++i) {
+      const int k = c0 + i;
+      if (k < nn && rv) mx = fmaxf(mx, (t[i] * a.scale + a.shift) * (wj * s_key[k].w));
     }
   }
   mx = xr.max(mx);
   const float mxs = mx == -INFINITY ? 0.f : mx;
   float sum = 0.f, esum = 0.f;  // sum_k e_k and sum_k e_k dA_k
   if (wlive) {
+    float u[32];
+    tmem_ld32(tP, u);
 #pragma unroll
-    for (int e8 = 0; e8 < 32; e8 += 8) {
-      float t[8], u[8];
-      tmem_ld8(tS + e8, t);
-      tmem_ld8(tP + e8, u);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int k = c0 + e8 + i;
-        if (k < nn && rv) {
-          const float4 kk = s_key[k];
-          const float ww = wj * kk.w;
-          const float e = exp_sfu((t[i] * a.scale + a.shift) * ww - mxs);
-          sum += e;
-          esum += e * (u[i] + dpg1) * ww * (kj.x * kk.x + kj.y * kk.y + kj.z * kk.z);
-        }
+    for (int i = 0; i < 32; ++i) {
+      const int k = c0 + i;
+      const float4 kk = s_key[k];
+      const float c = kj.x * kk.x + kj.y * kk.y + kj.z * kk.z;
+      float e = 0.f;
+      if (k < nn && rv) {
+        const float ww = wj * kk.w;
+        e = exp_sfu((t[i] * a.scale + a.shift) * ww - mxs);
+        sum += e;
+        esum += e * (u[i] + dpg1) * ww * c;
       }
+      t[i] = e;
+      u[i] = c;
     }
+    tmem_st32(tP + 128, t);
+    tmem_st32(tP + 256, u);
   }
   const float2 ss = xr.sum2(make_float2(sum, esum));
   const float inv = ss.x > 0.f ? 1.0f / ss.x : 0.f;
@@ -701,21 +721,23 @@ __device__ __forceinline__ void softmax_adjoint(const XCoreArgs& a, uint8_t* pt,
   float rw_ = 0.f, rx = 0.f, ry = 0.f, rz = 0.f;
 #pragma unroll 1
   for (int h = 0; h < 32; h += 16) {
+    if (c0 + h >= nn) {
+      zeros(h);
+      continue;
+    }
     float4 cph = make_float4(0.f, 0.f, 0.f, 0.f);
     float cw[16], dcv[16];
 #pragma unroll
     for (int e8 = 0; e8 < 16; e8 += 8) {
-      float t[8], u[8], pv[8];
-      tmem_ld8(tS + h + e8, t);
-      tmem_ld8(tP + h + e8, u);
+      float s8[8], u[8], ev[8], cv[8], pv[8];
+      tmem_ld8x4(tS + h + e8, tP + h + e8, tP + 128 + h + e8, tP + 256 + h + e8, s8, u, ev, cv);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const int k = c0 + h + e8 + i;
-        const float4 kk = s_key[k];
+        const float4 kk = s_key[c0 + h + e8 + i];
         const float ww = wj * kk.w;
-        const float c = kj.x * kk.x + kj.y * kk.y + kj.z * kk.z;
-        const float lg = t[i] * a.scale + a.shift;
-        const float A = (live && k < nn) ? exp_sfu(lg * ww - mxs) * inv : 0.f;
+        const float c = cv[i];
+        const float lg = s8[i] * a.scale + a.shift;
+        const float A = ev[i] * inv;
         const float dp = u[i] + dpg1;
         const float dA = dp * ww * c;
         const float dLp = A * (dA - tsum);
@@ -726,7 +748,7 @@ __device__ __forceinline__ void softmax_adjoint(const XCoreArgs& a, uint8_t* pt,
         cw[e8 + i] = H * wj;
         dcv[e8 + i] = dc;
         pv[i] = A * ww * c;
-        t[i] = dLp * ww * a.scale;  // dS
+        s8[i] = dLp * ww * a.scale;  // dS
       }
       uint4 w4;
       w4.x = pack_bf16(pv[0], pv[1]);
@@ -734,7 +756,7 @@ __device__ __forceinline__ void softmax_adjoint(const XCoreArgs& a, uint8_t* pt,
       w4.z = pack_bf16(pv[4], pv[5]);
       w4.w = pack_bf16(pv[6], pv[7]);
       sw128_store8(pt, row, c0 + h + e8, 128, w4);
-      tmem_st8_async(tS + h + e8, t);
+      tmem_st8_async(tS + h + e8, s8);
     }
     cph.w = warp_reduce_scatter16(cw);
     float tmp[16];
