@@ -537,7 +537,6 @@ void run_network_f32(dp_model* m, int n, const int* atype, cudaStream_t st) {
   }
   // a13: embedding backward -> dR[:,0]
   launch_embed_rows(ea, m->emb, true, st);
-  if (m->grad_scale) launch_embed_wgrad(ea, m->emb, m->grad, m->grad_scale, st);
   prof_mark(m, "embed_bwd", st);
 }
 
@@ -590,7 +589,6 @@ void run_network_bf16x(dp_model* m, int n, const int* atype, cudaStream_t st) {
     tc_embed(m, n, atype, true, st);
   } else {
     launch_embed_rows(ea, m->emb, true, st);
-    if (m->grad_scale) launch_embed_wgrad(ea, m->emb, m->grad, m->grad_scale, st);
   }
   prof_mark(m, "embed_bwd", st);
 }
@@ -684,7 +682,7 @@ void run_force_tangent(dp_model* m, int n, const double* coord, const double* v,
   const bool x16 = m->precision == DP_PREC_BF16X;
   // forward: R', G', T' and X'
   launch_env_jvp(a, st);
-  launch_embed_jvp(a, m->emb, 0, nullptr, scale, st);
+  launch_embed_jvp(a, m->emb, st);
   launch_desc_jvp_fwd(a, st);
   // fitting forward: H_l' = (1 - t_l^2) H_{l-1}' W_l (+ H_{l-1}')
   const float* hin = Xd;
@@ -738,9 +736,10 @@ void run_force_tangent(dp_model* m, int n, const double* coord, const double* v,
       gemm_f32(dZd, out, m->fitWT[l], in, nullptr, nullptr, 0, dXd, in, n, in, out, EPI_BIAS, st);
     }
   }
-  // descriptor adjoint's tangent -> (dE/dG)'; the embedding weights' tangent gradients
+  // descriptor adjoint's tangent -> (dE/dG)'; the embedding weights' gradients of
+  // both loss terms
   launch_desc_jvp_bwd(a, st);
-  launch_embed_jvp(a, m->emb, 1, m->grad, scale, st);
+  launch_embed_grad(a, m->emb, m->grad, m->d_scales, st);
 }
 
 int read_status(dp_model* m) {

@@ -195,7 +195,6 @@ void launch_tanh_bwd(const float* dH, const float* Hcur, const float* Hprev, flo
 void launch_fill_rows(float* dst, const float* row, int n, int nlocal, int width, cudaStream_t st);
 
 // --- training of the student (train.cu, simt.cu)
-bool launch_embed_wgrad(const EmbedArgs& a, const int* widths, float* grad, const float* scale, cudaStream_t st);
 void launch_wgrad(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int I, int O, int N,
                   const float* scale, cudaStream_t st);
 void launch_colsum(const float* B, int ldb, float* c, int O, int N, const float* scale, float factor, cudaStream_t st);
@@ -238,9 +237,10 @@ struct JvpArgs {
   float* dGd;           // [packed rows][m1]  (dE/dG)'
 };
 void launch_env_jvp(const JvpArgs& a, cudaStream_t st);
-// mode 0: G'; mode 1: grad += *scale * (dE/d(embedding weights))'
-bool launch_embed_jvp(const JvpArgs& a, const int* widths, int mode, float* grad, const float* scale,
-                      cudaStream_t st);
+// G'.
+bool launch_embed_jvp(const JvpArgs& a, const int* widths, cudaStream_t st);
+// grad += scales[1] dE/d(embedding weights) + scales[2] (dE/d(embedding weights))'.
+bool launch_embed_grad(const JvpArgs& a, const int* widths, float* grad, const float* scales, cudaStream_t st);
 void launch_desc_jvp_fwd(const JvpArgs& a, cudaStream_t st);
 void launch_desc_jvp_bwd(const JvpArgs& a, cudaStream_t st);
 // H' = (1 - t^2) Z' + Hprev' with t = H - Hprev (Hprev, Hprev' null: t = H, no skip)

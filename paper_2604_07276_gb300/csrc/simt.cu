@@ -170,214 +170,6 @@ void gemm_f32(const float* A, int lda, const float* B, int ldb, const float* bia
   note_launch();
 }
 
-// --------------------------------------- weight gradient of the embedding net
-// net_s = 1 -> E0 -> E1 -> E2 with tanh and the residual rule (keep width: x +
-// f; double: [x, x] + f).  A CTA takes 64 packed neighbour rows at a time;
-// their activations live in shared memory and every layer is a small tiled
-// product over the block.
-template <int E0, int E1, int E2>
-struct EmbedLayout {  // packed global weights: W0 b0 W1 b1 W2 b2
-  static constexpr int W0 = 0, B0 = E0, W1 = 2 * E0, B1 = W1 + E0 * E1, W2 = B1 + E1, B2 = W2 + E1 * E2,
-                       TOTAL = B2 + E2;
-};
-
-constexpr int EROWS = 64;  // neighbour rows per CTA
-constexpr int ETHREADS = 256;
-
-template <int IN, int OUT>
-__device__ __forceinline__ float skip_in(const float* x, int o) {
-  return OUT == IN ? x[o] : (OUT == 2 * IN ? x[o % IN] : 0.f);
-}
-
-// Shared layout (floats); W2 is kept with row stride E2 + 1 (bank-conflict
-// free for both of its access patterns), activations with row stride n + 1.
-template <int E0, int E1, int E2>
-struct EmbedSmem {
-  static constexpr int P2 = E2 + 1;
-  static constexpr int W0 = 0, B0 = E0, W1 = 2 * E0, B1 = W1 + E0 * E1, W2 = B1 + E1, B2 = W2 + E1 * P2,
-                       X = B2 + E2, H1 = X + EROWS, H2 = H1 + EROWS * (E0 + 1), Z = H2 + EROWS * (E1 + 1),
-                       DH2 = Z + EROWS * (E2 + 1), DZ2 = DH2 + EROWS * (E1 + 1), DH1 = DZ2 + EROWS * (E1 + 1),
-                       TJ = DH1 + EROWS * (E0 + 1), TOTAL = TJ + EROWS;  // TJ: the rows' type pairs (int)
-};
-
-template <int E0, int E1, int E2>
-__device__ __forceinline__ void embed_load(float* sm, const EmbedArgs& a, int p0, int cnt) {
-  using Lw = EmbedLayout<E0, E1, E2>;
-  using S = EmbedSmem<E0, E1, E2>;
-  for (int t = threadIdx.x; t < Lw::W2; t += ETHREADS) sm[t] = a.w[t];  // W0 b0 W1 b1 share offsets
-  for (int t = threadIdx.x; t < E1 * E2; t += ETHREADS) sm[S::W2 + (t / E2) * S::P2 + t % E2] = a.w[Lw::W2 + t];
-  for (int t = threadIdx.x; t < E2; t += ETHREADS) sm[S::B2 + t] = a.w[Lw::B2 + t];
-  for (int r = threadIdx.x; r < EROWS; r += ETHREADS) {
-    const int rg = r < cnt ? a.rowmap[p0 + r] : 0;
-    sm[S::X + r] = r < cnt ? a.R[(size_t)rg * 4] : 0.f;
-    reinterpret_cast<int*>(sm + S::TJ)[r] = r < cnt ? a.atype[rg / NP] * a.ntypes + a.atype[a.nlist[rg]] : 0;
-  }
-  __syncthreads();
-}
-
-// Layers 1 and 2, then Z = H2 W2 + b2 (4 rows per thread per weight load).
-// b0t: the concat mode's first-layer bias table ([type pair][E0]), or null
-// (strip mode: b0).
-template <int E0, int E1, int E2>
-__device__ __forceinline__ void embed_forward(float* sm, int cnt, const float* b0t) {
-  using S = EmbedSmem<E0, E1, E2>;
-  const int* tj = reinterpret_cast<const int*>(sm + S::TJ);
-  for (int idx = threadIdx.x; idx < EROWS * E0; idx += ETHREADS) {
-    const int r = idx / E0, p = idx % E0;
-    const float b = b0t ? b0t[tj[r] * E0 + p] : sm[S::B0 + p];
-    sm[S::H1 + r * (E0 + 1) + p] = r < cnt ? tanhf(fmaf(sm[S::X + r], sm[S::W0 + p], b)) : 0.f;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < (EROWS / 4) * E1; idx += ETHREADS) {  // four rows per thread
-    const int r0 = (idx / E1) * 4, b = idx % E1;
-    const float* h1 = sm + S::H1 + r0 * (E0 + 1);
-    float z[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) z[u] = sm[S::B1 + b];
-#pragma unroll 5
-    for (int p = 0; p < E0; ++p) {
-      const float w = sm[S::W1 + p * E1 + b];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) z[u] = fmaf(h1[u * (E0 + 1) + p], w, z[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = r0 + u;
-      sm[S::H2 + r * (E1 + 1) + b] = r < cnt ? skip_in<E0, E1>(h1 + u * (E0 + 1), b) + tanhf(z[u]) : 0.f;
-    }
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < (EROWS / 4) * E2; idx += ETHREADS) {
-    const int r0 = (idx / E2) * 4, c = idx % E2;
-    float z0 = sm[S::B2 + c], z1 = z0, z2 = z0, z3 = z0;
-    const float* h = sm + S::H2 + r0 * (E1 + 1);
-#pragma unroll 5
-    for (int b = 0; b < E1; ++b) {
-      const float wv = sm[S::W2 + b * S::P2 + c];
-      z0 = fmaf(h[b], wv, z0);
-      z1 = fmaf(h[(E1 + 1) + b], wv, z1);
-      z2 = fmaf(h[2 * (E1 + 1) + b], wv, z2);
-      z3 = fmaf(h[3 * (E1 + 1) + b], wv, z3);
-    }
-    float* zr = sm + S::Z + r0 * (E2 + 1) + c;
-    zr[0] = z0; zr[E2 + 1] = z1; zr[2 * (E2 + 1)] = z2; zr[3 * (E2 + 1)] = z3;
-  }
-  __syncthreads();
-}
-
-// Weight gradients of the embedding net, scale * dE/d(W0 b0 W1 b1 W2 b2)
-// (packed layout), accumulated over every neighbour row.  Persistent CTAs
-// walk the 64-row blocks, keep per-CTA sums in shared memory and add them to
-// `grad` once at the end.
-template <int E0, int E1, int E2>
-__global__ void __launch_bounds__(ETHREADS) k_embed_wgrad(EmbedArgs a, float* grad, const float* scale) {
-  pdl_wait();
-  using Lw = EmbedLayout<E0, E1, E2>;
-  using S = EmbedSmem<E0, E1, E2>;
-  extern __shared__ float sm[];
-  float* acc = sm + S::TOTAL;
-  for (int t = threadIdx.x; t < Lw::TOTAL; t += ETHREADS) acc[t] = 0.f;
-  const int* pair = reinterpret_cast<const int*>(sm + S::TJ);
-  const int nrows = *a.nrows;
-  for (int p0 = blockIdx.x * EROWS; p0 < nrows; p0 += gridDim.x * EROWS) {
-    const int cnt = min(EROWS, nrows - p0);
-    const size_t base = p0;
-    __syncthreads();
-    embed_load<E0, E1, E2>(sm, a, p0, cnt);
-    embed_forward<E0, E1, E2>(sm, cnt, a.b0t);
-    for (int idx = threadIdx.x; idx < EROWS * E2; idx += ETHREADS) {
-      const int r = idx / E2, c = idx % E2;
-      float dz = 0.f;
-      if (r < cnt) {
-        const float g = a.dG0[(base + r) * a.m1 + c] * (1.f + a.Gt[(size_t)pair[r] * E2 + c]);
-        const float t = tanhf(sm[S::Z + r * (E2 + 1) + c]);
-        dz = g * (1.f - t * t);
-      }
-      sm[S::Z + r * (E2 + 1) + c] = dz;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < EROWS * E1; idx += ETHREADS) {
-      const int r = idx / E1, b = idx % E1;
-      float sacc = 0.f;
-      if (r < cnt) {
-        const float* dz = sm + S::Z + r * (E2 + 1);
-        const float* w2 = sm + S::W2 + b * S::P2;
-        for (int c = 0; c < E2; ++c) sacc = fmaf(w2[c], dz[c], sacc);
-        if (E2 == E1 || E2 == 2 * E1) {
-          const float* gt = a.Gt + (size_t)pair[r] * E2;
-          const float* dg = a.dG0 + (base + r) * a.m1;
-          for (int c = b; c < E2; c += E1) sacc += dg[c] * (1.f + gt[c]);
-        }
-      }
-      sm[S::DH2 + r * (E1 + 1) + b] = sacc;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < EROWS * E1; idx += ETHREADS) {
-      const int r = idx / E1, b = idx % E1;
-      const float t = sm[S::H2 + r * (E1 + 1) + b] - skip_in<E0, E1>(sm + S::H1 + r * (E0 + 1), b);
-      sm[S::DZ2 + r * (E1 + 1) + b] = r < cnt ? sm[S::DH2 + r * (E1 + 1) + b] * (1.f - t * t) : 0.f;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < EROWS * E0; idx += ETHREADS) {
-      const int r = idx / E0, q = idx % E0;
-      float sacc = 0.f;
-      if (r < cnt) {
-        const float* dz2 = sm + S::DZ2 + r * (E1 + 1);
-        const float* w1 = sm + S::W1 + q * E1;
-        for (int b = 0; b < E1; ++b) sacc = fmaf(w1[b], dz2[b], sacc);
-        if (E1 == E0 || E1 == 2 * E0)
-          for (int b = q; b < E1; b += E0) sacc += sm[S::DH2 + r * (E1 + 1) + b];
-        const float h1 = sm[S::H1 + r * (E0 + 1) + q];
-        sacc *= (1.f - h1 * h1);  // dz1
-      }
-      sm[S::DH1 + r * (E0 + 1) + q] = sacc;
-    }
-    __syncthreads();
-    // accumulate this block's weight gradients (rows >= cnt are zero everywhere)
-    for (int t = threadIdx.x; t < Lw::TOTAL; t += ETHREADS) {
-      float g = 0.f;
-      if (t < Lw::B0) {
-        for (int r = 0; r < EROWS; ++r) g = fmaf(sm[S::X + r], sm[S::DH1 + r * (E0 + 1) + t], g);
-      } else if (t < Lw::W1) {
-        for (int r = 0; r < EROWS; ++r) g += sm[S::DH1 + r * (E0 + 1) + (t - Lw::B0)];
-      } else if (t < Lw::B1) {
-        const int q = (t - Lw::W1) / E1, b = (t - Lw::W1) % E1;
-        for (int r = 0; r < EROWS; ++r) g = fmaf(sm[S::H1 + r * (E0 + 1) + q], sm[S::DZ2 + r * (E1 + 1) + b], g);
-      } else if (t < Lw::W2) {
-        for (int r = 0; r < EROWS; ++r) g += sm[S::DZ2 + r * (E1 + 1) + (t - Lw::B1)];
-      } else if (t < Lw::B2) {
-        const int b = (t - Lw::W2) / E2, c = (t - Lw::W2) % E2;
-        for (int r = 0; r < EROWS; ++r) g = fmaf(sm[S::H2 + r * (E1 + 1) + b], sm[S::Z + r * (E2 + 1) + c], g);
-      } else {
-        for (int r = 0; r < EROWS; ++r) g += sm[S::Z + r * (E2 + 1) + (t - Lw::B2)];
-      }
-      acc[t] += g;
-    }
-  }
-  __syncthreads();
-  const float sc = *scale;
-  for (int t = threadIdx.x; t < Lw::TOTAL; t += ETHREADS) atomicAdd(&grad[t], sc * acc[t]);
-}
-
-template <int E0, int E1, int E2>
-static void embed_wgrad_launch(const EmbedArgs& a, float* grad, const float* scale, cudaStream_t st) {
-  using Lw = EmbedLayout<E0, E1, E2>;
-  using S = EmbedSmem<E0, E1, E2>;
-  if (a.n == 0) return;
-  const size_t smem = sizeof(float) * (S::TOTAL + Lw::TOTAL);
-  cudaFuncSetAttribute(k_embed_wgrad<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const int grid = std::min(2 * a.n, 2 * sm_count());
-  launch_pdl(k_embed_wgrad<E0, E1, E2>, grid, ETHREADS, smem, st, a, grad, scale);
-  note_launch();
-}
-
-bool launch_embed_wgrad(const EmbedArgs& a, const int* w, float* grad, const float* scale, cudaStream_t st) {
-  if (w[0] == 25 && w[1] == 50 && w[2] == 100) { embed_wgrad_launch<25, 50, 100>(a, grad, scale, st); return true; }
-  if (w[0] == 16 && w[1] == 32 && w[2] == 64) { embed_wgrad_launch<16, 32, 64>(a, grad, scale, st); return true; }
-  if (w[0] == 32 && w[1] == 64 && w[2] == 128) { embed_wgrad_launch<32, 64, 128>(a, grad, scale, st); return true; }
-  return false;
-}
-
 // ---------------------------------------------------------------- LayerNorm
 // G_out = G_in + LN(Y), row by row.
 __global__ void k_ln_res_fwd(const float* __restrict__ Y, const float* __restrict__ Gin, const int* __restrict__ nrows,

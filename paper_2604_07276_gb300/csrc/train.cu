@@ -168,227 +168,365 @@ __global__ void k_env_jvp(JvpArgs a) {
 
 // The embedding net G = net(s) (1 + Gt[t_i][t_j]), net: 1 -> E0 -> E1 -> E2,
 // tanh layers with the residual rule (same width: x + f; double: [x, x] + f),
-// input s = R_ij,0.  A CTA takes JROWS packed neighbour rows and
+// input s = R_ij,0, over the packed live rows.  A CTA takes JROWS rows and
 // evaluates the activations and their tangents (s' = R'_ij,0).  Mode 0 writes
-// G'.  Mode 1 also runs the adjoint from dE/dG and (dE/dG)' and adds
-// *scale times the tangents of the weight gradients to grad (per-CTA sums,
-// one atomic add per weight at the end).
-constexpr int JROWS = 32;
+// G'.  Mode 1 also runs the adjoint from dE/dG and (dE/dG)' and adds the weight
+// gradients of both loss terms to grad: with s1, s2 the scales of the energy and
+// force terms, the tangents are seeded with s2 s' and s2 (dE/dG)' + s1 dE/dG,
+// which (everything being linear in them) makes sum_r in' (x) dz + in (x) dz' the
+// sum of s2 times the tangent of the energy's weight gradient and s1 times that
+// gradient itself: no pass of its own for the latter.
+//
+// Activations lie in shared memory as [unit][row]; a thread owns 4 rows x 1 - 4
+// units of a layer, its value and tangent sums sharing the weight loads (3
+// 16-byte loads for 32 FMAs in the widest layer), and fixed elements of the weight
+// gradients, 2 x 4 of W2, whose sums stay in registers until the last block.  (A
+// thread per element with 4-byte loads, and a separate pass for the energy term,
+// took 409 us per 582-atom frame; this takes 168.)
+constexpr int JROWS = 64;
 constexpr int JTHREADS = 256;
+constexpr int JLD = JROWS + 4;   // row stride of a unit's rows (16-byte aligned)
+constexpr int JQ = JROWS / 4;    // row quads
 
 template <int E0, int E1, int E2>
 struct JvpEmbedSmem {
-  static constexpr int P2 = E2 + 1, Q0 = E0 + 1, Q1 = E1 + 1;
-  // packed weights as in the parameter vector, W2 rows padded to P2
-  static constexpr int W0 = 0, B0 = E0, W1 = 2 * E0, B1 = W1 + E0 * E1, W2 = B1 + E1, B2 = W2 + E1 * P2;
-  static constexpr int X = B2 + E2, XD = X + JROWS, TP = XD + JROWS;  // TP: the rows' type pairs (int)
-  static constexpr int H1 = TP + JROWS, H1D = H1 + JROWS * Q0;
-  static constexpr int H2 = H1D + JROWS * Q0, H2D = H2 + JROWS * Q1;
-  static constexpr int Z3 = H2D + JROWS * Q1, Z3D = Z3 + JROWS * P2;
-  static constexpr int FWD_TOTAL = Z3D + JROWS * P2;
-  // mode 1 only
-  static constexpr int DH2 = FWD_TOTAL, DH2D = DH2 + JROWS * Q1, DZ2 = DH2D + JROWS * Q1, DZ2D = DZ2 + JROWS * Q1;
-  static constexpr int DZ1 = DZ2D + JROWS * Q1, DZ1D = DZ1 + JROWS * Q0;
-  static constexpr int NW = B2 + E2 - E1 * (P2 - E2);  // packed weight count
-  static constexpr int ACC = DZ1D + JROWS * Q0, TOTAL = ACC + NW;
+  static constexpr int pad4(int x) { return (x + 3) / 4 * 4; }
+  static constexpr int L1 = pad4(E1), L2 = pad4(E2), L0 = pad4(E0);
+  // packed weights in the parameter vector
+  static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2, NW = gB2 + E2;
+  // shared memory (floats)
+  static constexpr int W1 = 0, W2 = W1 + E0 * L1, W0 = W2 + E1 * L2, B0 = W0 + L0, B1 = B0 + L0, B2 = B1 + L1,
+                       X = B2 + L2, XD = X + JROWS, TP = XD + JROWS;  // TP: the rows' type pairs (int)
+  static constexpr int H1 = TP + JROWS, H1D = H1 + E0 * JLD, H2 = H1D + E0 * JLD, H2D = H2 + E1 * JLD;
+  static constexpr int FWD_TOTAL = H2D + E1 * JLD;
+  // mode 1: the transposes W2^T [E2][L1], W1^T [E1][L0], dz3 and dz3'; once those
+  // are used up, dH2, dH2', dz2, dz2' lie over them; dz1, dz1'
+  static constexpr int W2T = FWD_TOTAL, W1T = W2T + E2 * L1, Z3 = W1T + E1 * L0, Z3D = Z3 + E2 * JLD;
+  static constexpr int DH2 = Z3, DH2D = DH2 + E1 * JLD, DZ2 = DH2D + E1 * JLD, DZ2D = DZ2 + E1 * JLD;
+  static constexpr int DZ1 = Z3 + (2 * E2 > 4 * E1 ? 2 * E2 : 4 * E1) * JLD, DZ1D = DZ1 + E0 * JLD;
+  static constexpr int TOTAL = DZ1D + E0 * JLD;
+  static_assert(TOTAL * 4 <= 227 * 1024, "shared memory");
 };
 
 template <int IN, int OUT>
-__device__ __forceinline__ float jskip(const float* x, int o) {
-  return OUT == IN ? x[o] : (OUT == 2 * IN ? x[o % IN] : 0.f);
+__device__ __forceinline__ int jskip(int o) {  // the skip input of output o, or -1
+  return OUT == IN ? o : (OUT == 2 * IN ? (o < IN ? o : o - IN) : -1);
 }
 
-template <int E0, int E1, int E2>
-__global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, int mode, float* __restrict__ grad,
-                                                         const float* __restrict__ scale) {
+__device__ __forceinline__ float4 jld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void jst4(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// z[u][o] += sum_k in[k][r + u] W[k][c + o], u < 4, o < OC, and likewise zd from ind.
+template <int K, int OC, int LDW>
+__device__ __forceinline__ void jtile(const float* in, const float* ind, const float* W, int r, int c, float (&z)[4][OC],
+                                      float (&zd)[4][OC]) {
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    const float4 h4 = jld4(in + k * JLD + r), d4 = jld4(ind + k * JLD + r);
+    const float h[4] = {h4.x, h4.y, h4.z, h4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w};
+    float w[OC];
+    if constexpr (OC == 4) {
+      const float4 w4 = jld4(W + k * LDW + c);
+      w[0] = w4.x; w[1] = w4.y; w[2] = w4.z; w[3] = w4.w;
+    } else {
+#pragma unroll
+      for (int o = 0; o < OC; ++o) w[o] = W[k * LDW + c + o];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int o = 0; o < OC; ++o) {
+        z[u][o] = fmaf(h[u], w[o], z[u][o]);
+        zd[u][o] = fmaf(d[u], w[o], zd[u][o]);
+      }
+  }
+}
+
+// acc[i][j] += sum over the block's rows of a'[i] b[j] + a[i] b'[j] (units a0 + i,
+// b0 + j of the [unit][row] arrays).
+template <int I, int J>
+__device__ __forceinline__ void jouter(const float* A, const float* AD, const float* B, const float* BD, int a0, int b0,
+                                       float (&acc)[I][J]) {
+#pragma unroll 2
+  for (int r = 0; r < JROWS; r += 4) {
+    float a[I][4], ad[I][4];
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+      const float4 x = jld4(A + (a0 + i) * JLD + r), y = jld4(AD + (a0 + i) * JLD + r);
+      a[i][0] = x.x; a[i][1] = x.y; a[i][2] = x.z; a[i][3] = x.w;
+      ad[i][0] = y.x; ad[i][1] = y.y; ad[i][2] = y.z; ad[i][3] = y.w;
+    }
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const float4 x = jld4(B + (b0 + j) * JLD + r), y = jld4(BD + (b0 + j) * JLD + r);
+      const float b[4] = {x.x, x.y, x.z, x.w}, bd[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int i = 0; i < I; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[i][j] = fmaf(ad[i][u], b[u], fmaf(a[i][u], bd[u], acc[i][j]));
+    }
+  }
+}
+
+template <int E0, int E1, int E2, int MODE>
+__global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __restrict__ grad,
+                                                         const float* __restrict__ scales) {
   pdl_wait();
   using S = JvpEmbedSmem<E0, E1, E2>;
-  extern __shared__ float sm[];
+  static_assert(E1 % 2 == 0 && E2 % 4 == 0, "register tiles");
+  extern __shared__ __align__(16) float sm[];
   const int tid = threadIdx.x;
-  // weights (packed W0 b0 W1 b1 | W2 | b2)
-  for (int t = tid; t < S::W2; t += JTHREADS) sm[t] = a.w[t];
-  for (int t = tid; t < E1 * E2; t += JTHREADS) sm[S::W2 + (t / E2) * S::P2 + t % E2] = a.w[S::W2 + t];
-  for (int t = tid; t < E2; t += JTHREADS) sm[S::B2 + t] = a.w[S::W2 + E1 * E2 + t];
-  if (mode == 1)
-    for (int t = tid; t < S::NW; t += JTHREADS) sm[S::ACC + t] = 0.f;
-  int* pair = reinterpret_cast<int*>(sm + S::TP);
+  for (int t = tid; t < E0 * E1; t += JTHREADS) sm[S::W1 + (t / E1) * S::L1 + t % E1] = a.w[S::gW1 + t];
+  for (int t = tid; t < E1 * E2; t += JTHREADS) sm[S::W2 + (t / E2) * S::L2 + t % E2] = a.w[S::gW2 + t];
+  for (int t = tid; t < E0; t += JTHREADS) {
+    sm[S::W0 + t] = a.w[t];
+    sm[S::B0 + t] = a.w[S::gB0 + t];
+  }
+  for (int t = tid; t < E1; t += JTHREADS) sm[S::B1 + t] = a.w[S::gB1 + t];
+  for (int t = tid; t < E2; t += JTHREADS) sm[S::B2 + t] = a.w[S::gB2 + t];
+  float s1 = 0.f, s2 = 1.f;
+  if (MODE == 1) {
+    s1 = scales[1];
+    s2 = scales[2];
+    for (int t = tid; t < E1 * E2; t += JTHREADS) sm[S::W2T + (t % E2) * S::L1 + t / E2] = a.w[S::gW2 + t];
+    for (int t = tid; t < E0 * E1; t += JTHREADS) sm[S::W1T + (t % E1) * S::L0 + t / E1] = a.w[S::gW1 + t];
+  }
+  // this thread's elements of the weight gradients: N2 tasks of 2 x 4 of W2, N1 of
+  // 1 x 2 of W1 and NB of the others (W0, b0, b1, b2)
+  constexpr int T2 = (E1 / 2) * (E2 / 4), T1 = E0 * (E1 / 2), TB = 2 * E0 + E1 + E2;
+  constexpr int N2 = (T2 + JTHREADS - 1) / JTHREADS, N1 = (T1 + JTHREADS - 1) / JTHREADS,
+                NB = (TB + JTHREADS - 1) / JTHREADS;
+  float g2[N2][2][4] = {}, g1[N1][1][2] = {}, gb[NB] = {};
+  const int* pair = reinterpret_cast<const int*>(sm + S::TP);
   const int nrows = a.row_off[a.n];
   for (int p0 = blockIdx.x * JROWS; p0 < nrows; p0 += gridDim.x * JROWS) {
     const int cnt = min(JROWS, nrows - p0);
-    const size_t base = p0;
     __syncthreads();  // the previous block is done with the activations
     for (int r = tid; r < JROWS; r += JTHREADS) {
       const int rg = r < cnt ? a.rowmap[p0 + r] : 0;
       sm[S::X + r] = r < cnt ? a.R[(size_t)rg * 4] : 0.f;
-      sm[S::XD + r] = r < cnt ? a.Rd[(size_t)rg * 4] : 0.f;
-      pair[r] = r < cnt ? a.atype[rg / NP] * a.ntypes + a.atype[a.nlist[rg]] : 0;
+      sm[S::XD + r] = r < cnt ? (MODE == 1 ? s2 : 1.f) * a.Rd[(size_t)rg * 4] : 0.f;
+      reinterpret_cast<int*>(sm + S::TP)[r] = r < cnt ? a.atype[rg / NP] * a.ntypes + a.atype[a.nlist[rg]] : 0;
     }
     __syncthreads();
     // layer 1: h1 = tanh(s W0 + b0), h1' = (1 - h1^2) s' W0
     for (int idx = tid; idx < JROWS * E0; idx += JTHREADS) {
-      const int r = idx / E0, p = idx % E0;
-      float h = 0.f, hd = 0.f;
-      if (r < cnt) {
-        const float b0 = a.b0t ? a.b0t[(size_t)pair[r] * E0 + p] : sm[S::B0 + p];
-        h = tanhf(fmaf(sm[S::X + r], sm[S::W0 + p], b0));
-        hd = (1.f - h * h) * sm[S::XD + r] * sm[S::W0 + p];
-      }
-      sm[S::H1 + r * S::Q0 + p] = h;
-      sm[S::H1D + r * S::Q0 + p] = hd;
+      const int r = idx % JROWS, p = idx / JROWS;
+      const float b0 = a.b0t ? a.b0t[(size_t)pair[r] * E0 + p] : sm[S::B0 + p];
+      const float h = tanhf(fmaf(sm[S::X + r], sm[S::W0 + p], b0));
+      sm[S::H1 + p * JLD + r] = h;
+      sm[S::H1D + p * JLD + r] = (1.f - h * h) * sm[S::XD + r] * sm[S::W0 + p];
     }
     __syncthreads();
     // layer 2: H2 = skip(h1) + tanh(h1 W1 + b1), and its tangent
-    for (int idx = tid; idx < JROWS * E1; idx += JTHREADS) {
-      const int r = idx / E1, b = idx % E1;
-      float h = 0.f, hd = 0.f;
-      if (r < cnt) {
-        const float* h1 = sm + S::H1 + r * S::Q0;
-        const float* h1d = sm + S::H1D + r * S::Q0;
-        float z = sm[S::B1 + b], zd = 0.f;
-        for (int p = 0; p < E0; ++p) {
-          const float wv = sm[S::W1 + p * E1 + b];
-          z = fmaf(h1[p], wv, z);
-          zd = fmaf(h1d[p], wv, zd);
+    for (int task = tid; task < JQ * (E1 / 2); task += JTHREADS) {
+      const int r = (task % JQ) * 4, c = (task / JQ) * 2;
+      float z[4][2], zd[4][2] = {};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int o = 0; o < 2; ++o) z[u][o] = sm[S::B1 + c + o];
+      jtile<E0, 2, S::L1>(sm + S::H1, sm + S::H1D, sm + S::W1, r, c, z, zd);
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const int sk = jskip<E0, E1>(c + o);
+        float h[4], hd[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float t = tanhf(z[u][o]);
+          h[u] = (sk >= 0 ? sm[S::H1 + sk * JLD + r + u] : 0.f) + t;
+          hd[u] = (sk >= 0 ? sm[S::H1D + sk * JLD + r + u] : 0.f) + (1.f - t * t) * zd[u][o];
         }
-        const float t = tanhf(z);
-        h = jskip<E0, E1>(h1, b) + t;
-        hd = jskip<E0, E1>(h1d, b) + (1.f - t * t) * zd;
+        jst4(sm + S::H2 + (c + o) * JLD + r, h);
+        jst4(sm + S::H2D + (c + o) * JLD + r, hd);
       }
-      sm[S::H2 + r * S::Q1 + b] = h;
-      sm[S::H2D + r * S::Q1 + b] = hd;
     }
     __syncthreads();
-    // layer 3 pre-activation: t3 = tanh(H2 W2 + b2) and t3'
-    for (int idx = tid; idx < JROWS * E2; idx += JTHREADS) {
-      const int r = idx / E2, c = idx % E2;
-      float t = 0.f, td = 0.f;
-      if (r < cnt) {
-        const float* h2 = sm + S::H2 + r * S::Q1;
-        const float* h2d = sm + S::H2D + r * S::Q1;
-        float z = sm[S::B2 + c], zd = 0.f;
-        for (int b = 0; b < E1; ++b) {
-          const float wv = sm[S::W2 + b * S::P2 + c];
-          z = fmaf(h2[b], wv, z);
-          zd = fmaf(h2d[b], wv, zd);
-        }
-        t = tanhf(z);
-        td = (1.f - t * t) * zd;
-      }
-      sm[S::Z3 + r * S::P2 + c] = t;
-      sm[S::Z3D + r * S::P2 + c] = td;
-    }
-    __syncthreads();
-    if (mode == 0) {
-      for (int idx = tid; idx < JROWS * E2; idx += JTHREADS) {
-        const int r = idx / E2, c = idx % E2;
-        if (r >= cnt) continue;
-        const float f = 1.f + a.Gt[(size_t)pair[r] * E2 + c];
-        a.Gd[(base + r) * a.m1 + c] = (jskip<E1, E2>(sm + S::H2D + r * S::Q1, c) + sm[S::Z3D + r * S::P2 + c]) * f;
-      }
-      continue;
-    }
-    // adjoint of layer 3 with g = dE/dG (1 + Gt): dz3 = g (1 - t3^2),
-    // dz3' = g' (1 - t3^2) - 2 g t3 t3' (in place of t3, t3')
-    for (int idx = tid; idx < JROWS * E2; idx += JTHREADS) {
-      const int r = idx / E2, c = idx % E2;
-      float dz = 0.f, dzd = 0.f;
-      if (r < cnt) {
-        const float f = 1.f + a.Gt[(size_t)pair[r] * E2 + c];
-        const float g = a.dG[(base + r) * a.m1 + c] * f, gd = a.dGd[(base + r) * a.m1 + c] * f;
-        const float t = sm[S::Z3 + r * S::P2 + c], td = sm[S::Z3D + r * S::P2 + c];
-        dz = g * (1.f - t * t);
-        dzd = gd * (1.f - t * t) - 2.f * g * t * td;
-      }
-      sm[S::Z3 + r * S::P2 + c] = dz;
-      sm[S::Z3D + r * S::P2 + c] = dzd;
-    }
-    __syncthreads();
-    // dH2 = W2 dz3 + skip^T(g), dz2 = dH2 (1 - t2^2) with t2 = H2 - skip(h1)
-    for (int idx = tid; idx < JROWS * E1; idx += JTHREADS) {
-      const int r = idx / E1, b = idx % E1;
-      float dh = 0.f, dhd = 0.f, dz = 0.f, dzd = 0.f;
-      if (r < cnt) {
-        const float* dz3 = sm + S::Z3 + r * S::P2;
-        const float* dz3d = sm + S::Z3D + r * S::P2;
-        for (int c = 0; c < E2; ++c) {
-          const float wv = sm[S::W2 + b * S::P2 + c];
-          dh = fmaf(wv, dz3[c], dh);
-          dhd = fmaf(wv, dz3d[c], dhd);
-        }
-        if (E2 == E1 || E2 == 2 * E1) {
-          const float* gt = a.Gt + (size_t)pair[r] * E2;
-          for (int c = b; c < E2; c += E1) {
-            const float f = 1.f + gt[c];
-            dh += a.dG[(base + r) * a.m1 + c] * f;
-            dhd += a.dGd[(base + r) * a.m1 + c] * f;
+    // layer 3: t3 = tanh(H2 W2 + b2), t3'; mode 0: G' out; mode 1: its adjoint with
+    // g = dE/dG (1 + Gt): dz3 = g (1 - t3^2), dz3' = g' (1 - t3^2) - 2 g t3 t3'
+    for (int task = tid; task < JQ * (E2 / 4); task += JTHREADS) {
+      const int r = (task % JQ) * 4, c = (task / JQ) * 4;
+      float z[4][4], zd[4][4] = {};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) z[u][o] = sm[S::B2 + c + o];
+      jtile<E1, 4, S::L2>(sm + S::H2, sm + S::H2D, sm + S::W2, r, c, z, zd);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool live = r + u < cnt;
+        const size_t at = (size_t)(p0 + r + u) * a.m1 + c;
+        const float4 f4 = jld4(a.Gt + (size_t)pair[r + u] * E2 + c);
+        const float f[4] = {1.f + f4.x, 1.f + f4.y, 1.f + f4.z, 1.f + f4.w};
+        if (MODE == 0) {
+          float gd[4];
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            const int sk = jskip<E1, E2>(c + o);
+            const float t = tanhf(z[u][o]);
+            gd[o] = ((sk >= 0 ? sm[S::H2D + sk * JLD + r + u] : 0.f) + (1.f - t * t) * zd[u][o]) * f[o];
+          }
+          if (live) jst4(a.Gd + at, gd);
+        } else {
+          float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f), qd4 = q4;
+          if (live) {
+            q4 = jld4(a.dG + at);
+            qd4 = jld4(a.dGd + at);
+          }
+          const float q[4] = {q4.x, q4.y, q4.z, q4.w}, qd[4] = {qd4.x, qd4.y, qd4.z, qd4.w};
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            const float g = q[o] * f[o], gd = fmaf(s2, qd[o], s1 * q[o]) * f[o];
+            const float t = tanhf(z[u][o]), td = (1.f - t * t) * zd[u][o];
+            z[u][o] = g * (1.f - t * t);
+            zd[u][o] = gd * (1.f - t * t) - 2.f * g * t * td;
           }
         }
-        const float t = sm[S::H2 + r * S::Q1 + b] - jskip<E0, E1>(sm + S::H1 + r * S::Q0, b);
-        const float td = sm[S::H2D + r * S::Q1 + b] - jskip<E0, E1>(sm + S::H1D + r * S::Q0, b);
-        dz = dh * (1.f - t * t);
-        dzd = dhd * (1.f - t * t) - 2.f * dh * t * td;
       }
-      sm[S::DH2 + r * S::Q1 + b] = dh;
-      sm[S::DH2D + r * S::Q1 + b] = dhd;
-      sm[S::DZ2 + r * S::Q1 + b] = dz;
-      sm[S::DZ2D + r * S::Q1 + b] = dzd;
+      if (MODE == 1) {
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const float v[4] = {z[0][o], z[1][o], z[2][o], z[3][o]}, vd[4] = {zd[0][o], zd[1][o], zd[2][o], zd[3][o]};
+          jst4(sm + S::Z3 + (c + o) * JLD + r, v);
+          jst4(sm + S::Z3D + (c + o) * JLD + r, vd);
+        }
+      }
+    }
+    if (MODE == 0) continue;
+    __syncthreads();
+    // dH2 = W2 dz3 + skip^T(g) and its tangent, kept in registers until W2's
+    // gradient has read dz3
+    constexpr int TH = JQ * (E1 / 2), NH = (TH + JTHREADS - 1) / JTHREADS;
+    float dh[NH][4][2], dhd[NH][4][2];
+#pragma unroll
+    for (int k = 0; k < NH; ++k) {
+      const int task = tid + k * JTHREADS;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) dh[k][u][0] = dh[k][u][1] = dhd[k][u][0] = dhd[k][u][1] = 0.f;
+      if (task >= TH) continue;
+      const int r = (task % JQ) * 4, b = (task / JQ) * 2;
+      jtile<E2, 2, S::L1>(sm + S::Z3, sm + S::Z3D, sm + S::W2T, r, b, dh[k], dhd[k]);
+      if (E2 == E1 || E2 == 2 * E1) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (r + u >= cnt) break;
+          const float* gt = a.Gt + (size_t)pair[r + u] * E2;
+          const size_t at = (size_t)(p0 + r + u) * a.m1;
+          for (int c = b; c < E2; c += E1)
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+              const float f = 1.f + gt[c + o], q = a.dG[at + c + o], qd = a.dGd[at + c + o];
+              dh[k][u][o] += q * f;
+              dhd[k][u][o] += fmaf(s2, qd, s1 * q) * f;
+            }
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < N2; ++k) {
+      const int task = tid + k * JTHREADS;
+      if (task < T2) jouter<2, 4>(sm + S::H2, sm + S::H2D, sm + S::Z3, sm + S::Z3D, 2 * (task / (E2 / 4)), 4 * (task % (E2 / 4)), g2[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {  // b2: sum of dz3'
+      const int t = tid + k * JTHREADS - (2 * E0 + E1);
+      if (t >= 0 && t < E2)
+        for (int r = 0; r < JROWS; ++r) gb[k] += sm[S::Z3D + t * JLD + r];
+    }
+    __syncthreads();
+    // dz2 = dH2 (1 - t2^2) with t2 = H2 - skip(h1), over dz3's place
+#pragma unroll
+    for (int k = 0; k < NH; ++k) {
+      const int task = tid + k * JTHREADS;
+      if (task >= TH) continue;
+      const int r = (task % JQ) * 4, b = (task / JQ) * 2;
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const int sk = jskip<E0, E1>(b + o);
+        float d[4], dd[4], e[4], ed[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float t = sm[S::H2 + (b + o) * JLD + r + u] - (sk >= 0 ? sm[S::H1 + sk * JLD + r + u] : 0.f);
+          const float td = sm[S::H2D + (b + o) * JLD + r + u] - (sk >= 0 ? sm[S::H1D + sk * JLD + r + u] : 0.f);
+          d[u] = dh[k][u][o];
+          dd[u] = dhd[k][u][o];
+          e[u] = d[u] * (1.f - t * t);
+          ed[u] = dd[u] * (1.f - t * t) - 2.f * d[u] * t * td;
+        }
+        jst4(sm + S::DH2 + (b + o) * JLD + r, d);
+        jst4(sm + S::DH2D + (b + o) * JLD + r, dd);
+        jst4(sm + S::DZ2 + (b + o) * JLD + r, e);
+        jst4(sm + S::DZ2D + (b + o) * JLD + r, ed);
+      }
     }
     __syncthreads();
     // dh1 = W1 dz2 + skip^T(dH2), dz1 = dh1 (1 - h1^2)
-    for (int idx = tid; idx < JROWS * E0; idx += JTHREADS) {
-      const int r = idx / E0, p = idx % E0;
-      float dz = 0.f, dzd = 0.f;
-      if (r < cnt) {
-        float dh = 0.f, dhd = 0.f;
-        for (int b = 0; b < E1; ++b) {
-          const float wv = sm[S::W1 + p * E1 + b];
-          dh = fmaf(wv, sm[S::DZ2 + r * S::Q1 + b], dh);
-          dhd = fmaf(wv, sm[S::DZ2D + r * S::Q1 + b], dhd);
-        }
+    for (int task = tid; task < JQ * E0; task += JTHREADS) {
+      const int r = (task % JQ) * 4, p = task / JQ;
+      float d1[4][1] = {}, d1d[4][1] = {};
+      jtile<E1, 1, S::L0>(sm + S::DZ2, sm + S::DZ2D, sm + S::W1T, r, p, d1, d1d);
+      float e[4], ed[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float d = d1[u][0], dd = d1d[u][0];
         if (E1 == E0 || E1 == 2 * E0)
           for (int b = p; b < E1; b += E0) {
-            dh += sm[S::DH2 + r * S::Q1 + b];
-            dhd += sm[S::DH2D + r * S::Q1 + b];
+            d += sm[S::DH2 + b * JLD + r + u];
+            dd += sm[S::DH2D + b * JLD + r + u];
           }
-        const float h = sm[S::H1 + r * S::Q0 + p], hd = sm[S::H1D + r * S::Q0 + p];
-        dz = dh * (1.f - h * h);
-        dzd = dhd * (1.f - h * h) - 2.f * dh * h * hd;
+        const float h = sm[S::H1 + p * JLD + r + u], hd = sm[S::H1D + p * JLD + r + u];
+        e[u] = d * (1.f - h * h);
+        ed[u] = dd * (1.f - h * h) - 2.f * d * h * hd;
       }
-      sm[S::DZ1 + r * S::Q0 + p] = dz;
-      sm[S::DZ1D + r * S::Q0 + p] = dzd;
+      jst4(sm + S::DZ1 + p * JLD + r, e);
+      jst4(sm + S::DZ1D + p * JLD + r, ed);
+    }
+    // W1's gradient (dz2) does not wait for dz1
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+      const int task = tid + k * JTHREADS;
+      if (task < T1) jouter<1, 2>(sm + S::H1, sm + S::H1D, sm + S::DZ2, sm + S::DZ2D, task / (E1 / 2), 2 * (task % (E1 / 2)), g1[k]);
     }
     __syncthreads();
-    // tangents of the weight gradients: (sum_r in (x) dz)' = sum_r in' (x) dz + in (x) dz'
-    for (int t = tid; t < S::NW; t += JTHREADS) {
-      float g = 0.f;
-      if (t < S::B0) {
-        for (int r = 0; r < cnt; ++r)
-          g += sm[S::XD + r] * sm[S::DZ1 + r * S::Q0 + t] + sm[S::X + r] * sm[S::DZ1D + r * S::Q0 + t];
-      } else if (t < S::W1) {
-        for (int r = 0; r < cnt; ++r) g += sm[S::DZ1D + r * S::Q0 + (t - S::B0)];
-      } else if (t < S::B1) {
-        const int p = (t - S::W1) / E1, b = (t - S::W1) % E1;
-        for (int r = 0; r < cnt; ++r)
-          g += sm[S::H1D + r * S::Q0 + p] * sm[S::DZ2 + r * S::Q1 + b] +
-               sm[S::H1 + r * S::Q0 + p] * sm[S::DZ2D + r * S::Q1 + b];
-      } else if (t < S::W2) {
-        for (int r = 0; r < cnt; ++r) g += sm[S::DZ2D + r * S::Q1 + (t - S::B1)];
-      } else if (t < S::W2 + E1 * E2) {
-        const int b = (t - S::W2) / E2, c = (t - S::W2) % E2;
-        for (int r = 0; r < cnt; ++r)
-          g += sm[S::H2D + r * S::Q1 + b] * sm[S::Z3 + r * S::P2 + c] +
-               sm[S::H2 + r * S::Q1 + b] * sm[S::Z3D + r * S::P2 + c];
-      } else {
-        const int c = t - S::W2 - E1 * E2;
-        for (int r = 0; r < cnt; ++r) g += sm[S::Z3D + r * S::P2 + c];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {  // W0, b0, b1
+      const int t = tid + k * JTHREADS;
+      if (t < E0) {
+        for (int r = 0; r < JROWS; ++r)
+          gb[k] += sm[S::XD + r] * sm[S::DZ1 + t * JLD + r] + sm[S::X + r] * sm[S::DZ1D + t * JLD + r];
+      } else if (t < 2 * E0) {
+        for (int r = 0; r < JROWS; ++r) gb[k] += sm[S::DZ1D + (t - E0) * JLD + r];
+      } else if (t < 2 * E0 + E1) {
+        for (int r = 0; r < JROWS; ++r) gb[k] += sm[S::DZ2D + (t - 2 * E0) * JLD + r];
       }
-      sm[S::ACC + t] += g;
     }
   }
-  if (mode == 1) {
-    __syncthreads();
-    const float sc = *scale;
-    for (int t = tid; t < S::NW; t += JTHREADS) atomicAdd(&grad[t], sc * sm[S::ACC + t]);
+  if (MODE == 0) return;
+#pragma unroll
+  for (int k = 0; k < N2; ++k) {
+    const int task = tid + k * JTHREADS;
+    if (task < T2)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          atomicAdd(grad + S::gW2 + (2 * (task / (E2 / 4)) + i) * E2 + 4 * (task % (E2 / 4)) + j, g2[k][i][j]);
+  }
+#pragma unroll
+  for (int k = 0; k < N1; ++k) {
+    const int task = tid + k * JTHREADS;
+    if (task < T1)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) atomicAdd(grad + S::gW1 + (task / (E1 / 2)) * E1 + 2 * (task % (E1 / 2)) + j, g1[k][0][j]);
+  }
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    const int t = tid + k * JTHREADS;
+    if (t < 2 * E0) atomicAdd(grad + t, gb[k]);
+    else if (t < 2 * E0 + E1) atomicAdd(grad + S::gB1 + t - 2 * E0, gb[k]);
+    else if (t < TB) atomicAdd(grad + S::gB2 + t - 2 * E0 - E1, gb[k]);
   }
 }
 
@@ -584,26 +722,36 @@ void launch_env_jvp(const JvpArgs& a, cudaStream_t st) {
   note_launch();
 }
 
-template <int E0, int E1, int E2>
-static void embed_jvp_launch(const JvpArgs& a, int mode, float* grad, const float* scale, cudaStream_t st) {
+template <int E0, int E1, int E2, int MODE>
+static void embed_jvp_launch(const JvpArgs& a, float* grad, const float* scales, cudaStream_t st) {
   using S = JvpEmbedSmem<E0, E1, E2>;
-  const size_t smem = sizeof(float) * (mode == 1 ? S::TOTAL : S::FWD_TOTAL);
-  cudaFuncSetAttribute(k_embed_jvp<E0, E1, E2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * S::TOTAL));
-  const int nblk = a.n * (NP / JROWS);
-  int sms = 0, dev = 0;
+  const size_t smem = sizeof(float) * (MODE == 1 ? S::TOTAL : S::FWD_TOTAL);
+  cudaFuncSetAttribute(k_embed_jvp<E0, E1, E2, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int sms = 0, dev = 0, per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = mode == 1 ? std::min(nblk, 2 * std::max(1, sms)) : nblk;
-  launch_pdl(k_embed_jvp<E0, E1, E2>, grid, JTHREADS, smem, st, a, mode, grad, scale);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_embed_jvp<E0, E1, E2, MODE>, JTHREADS, smem);
+  // at most n * NP rows
+  const int grid = std::min(a.n * (NP / JROWS), std::max(1, per_sm) * std::max(1, sms));
+  launch_pdl(k_embed_jvp<E0, E1, E2, MODE>, grid, JTHREADS, smem, st, a, grad, scales);
   note_launch();
 }
 
-bool launch_embed_jvp(const JvpArgs& a, const int* w, int mode, float* grad, const float* scale, cudaStream_t st) {
+template <int MODE>
+static bool embed_jvp_dispatch(const JvpArgs& a, const int* w, float* grad, const float* scales, cudaStream_t st) {
   if (a.n == 0) return true;
-  if (w[0] == 16 && w[1] == 32 && w[2] == 64) { embed_jvp_launch<16, 32, 64>(a, mode, grad, scale, st); return true; }
-  if (w[0] == 25 && w[1] == 50 && w[2] == 100) { embed_jvp_launch<25, 50, 100>(a, mode, grad, scale, st); return true; }
-  if (w[0] == 32 && w[1] == 64 && w[2] == 128) { embed_jvp_launch<32, 64, 128>(a, mode, grad, scale, st); return true; }
+  if (w[0] == 16 && w[1] == 32 && w[2] == 64) { embed_jvp_launch<16, 32, 64, MODE>(a, grad, scales, st); return true; }
+  if (w[0] == 25 && w[1] == 50 && w[2] == 100) { embed_jvp_launch<25, 50, 100, MODE>(a, grad, scales, st); return true; }
+  if (w[0] == 32 && w[1] == 64 && w[2] == 128) { embed_jvp_launch<32, 64, 128, MODE>(a, grad, scales, st); return true; }
   return false;
+}
+
+bool launch_embed_jvp(const JvpArgs& a, const int* w, cudaStream_t st) {
+  return embed_jvp_dispatch<0>(a, w, nullptr, nullptr, st);
+}
+
+bool launch_embed_grad(const JvpArgs& a, const int* w, float* grad, const float* scales, cudaStream_t st) {
+  return embed_jvp_dispatch<1>(a, w, grad, scales, st);
 }
 
 void launch_desc_jvp_fwd(const JvpArgs& a, cudaStream_t st) {
