@@ -803,8 +803,10 @@ void launch_attn_bwd_f32(const AttnArgs& a, cudaStream_t st) {
 // ------------------------------------------------------------- descriptor
 // T = R^T G / sel (4 x m1); D = T^T T[:, :axis]; X = [D (row-major), Z[t_i]].
 // A block of 128 threads per atom, 10 blocks per SM (48 registers): the kernel
-// waits on its loads, and more resident warps hide more of them.
-__global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
+// waits on its loads, and more resident warps hide more of them.  CQ: G and dG
+// interleaved per atom (the fused paths), else packed rows.
+template <bool CQ>
+__global__ void __launch_bounds__(128, CQ ? 10 : 6) k_desc_fwd(DescArgs a) {
   pdl_wait();
   extern __shared__ float sm[];
   float* Ts = sm;  // [4][m1]
@@ -812,7 +814,7 @@ __global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
   const int nn = a.nnei[atom];
   const size_t base = (size_t)atom * NP;
   const float inv_sel = 1.0f / (float)a.sel;
-  if (a.cq) {
+  if (CQ) {
     // a warp per column quad, its lanes over the rows
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const float4* G4 = reinterpret_cast<const float4*>(a.G + base * a.m1);
@@ -848,6 +850,7 @@ __global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
     const size_t gbase = a.row_off[atom];
     for (int c = threadIdx.x; c < a.m1; c += blockDim.x) {
       float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f;
+#pragma unroll 8  // eight rows' loads in flight ahead of the FMA chains
       for (int s = 0; s < nn; ++s) {
         const float4 r = reinterpret_cast<const float4*>(a.R)[base + s];
         const float gv = a.G[(gbase + s) * a.m1 + c];
@@ -872,7 +875,8 @@ __global__ void __launch_bounds__(128, 10) k_desc_fwd(DescArgs a) {
 
 // dT[c][p] = sum_b<axis dD[p][b] T[c][b] + (p < axis) sum_q dD[q][p] T[c][q];
 // dG_s = R_s dT / sel; dR_s = G_s dT^T / sel.
-__global__ void k_desc_bwd(DescArgs a) {
+template <bool CQ>
+__global__ void __launch_bounds__(128, 10) k_desc_bwd(DescArgs a) {
   pdl_wait();
   extern __shared__ float sm[];
   const int m1 = a.m1, ax = a.axis;
@@ -895,12 +899,14 @@ __global__ void k_desc_bwd(DescArgs a) {
     const int c = t / m1, p = t % m1;
     float v = 0.f;
     for (int b = 0; b < ax; ++b) v = fmaf(dDt[b * m1 + p], Ts[c * m1 + b], v);
-    if (p < ax)
+    if (p < ax) {
+#pragma unroll 8
       for (int q = 0; q < m1; ++q) v = fmaf(dD[q * ax + p], Ts[c * m1 + q], v);
+    }
     dTs[t] = v * inv_sel;
   }
   __syncthreads();
-  if (a.cq) {
+  if constexpr (CQ) {
     // A thread per row: its dG row in column quads (consecutive threads ->
     // consecutive rows; live rows only: the fused layer kernels and the
     // embedding adjoint read no others) and its dR row, with the columns of
@@ -934,53 +940,73 @@ __global__ void k_desc_bwd(DescArgs a) {
     }
     return;
   }
-  // dG rows, a column quad per thread (m1 % 4 == 0)
+  // Packed rows: a warp per row, a column quad per lane (m1 / 4 <= 32), whose four
+  // rows of dT stay in registers: dG = R dT, dR = G dT^T.  Two rows at a time, so
+  // that their loads and reductions overlap (four spill at 10 blocks per SM).
+  // 15,668 atoms in bf16x: 651 us with a thread per dG element and a second pass
+  // over G for dR, 332 now.
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int q4 = m1 / 4;
   const size_t gbase = a.row_off[atom];
-  float4* dG4 = reinterpret_cast<float4*>(a.dG + gbase * m1);
-  for (int idx = threadIdx.x; idx < nn * q4; idx += blockDim.x) {
-    const int s = idx / q4, q = idx % q4;
-    const float4 r = reinterpret_cast<const float4*>(a.R)[base + s];
-    float4 v;
-    float* vp = &v.x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int p = 4 * q + k;
-      vp[k] = r.x * dTs[p] + r.y * dTs[m1 + p] + r.z * dTs[2 * m1 + p] + r.w * dTs[3 * m1 + p];
-    }
-    dG4[idx] = v;
-  }
-  // dR rows: a warp per row, a column quad per lane
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const float4* G4 = reinterpret_cast<const float4*>(a.G + gbase * m1);
-  for (int s = warp; s < NP; s += nw) {
-    float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
-    if (s < nn) {
-      for (int q = lane; q < q4; q += 32) {
-        const float4 g = G4[(size_t)s * q4 + q];
-        const float gg[4] = {g.x, g.y, g.z, g.w};
+  float4* dG4 = reinterpret_cast<float4*>(a.dG + gbase * m1);
+  const float4* R4 = reinterpret_cast<const float4*>(a.R) + base;
+  float4* dR4 = reinterpret_cast<float4*>(a.dR) + base;
+  const bool on = lane < q4;
+  float t[4][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int p = 4 * q + k;
-          d0 = fmaf(gg[k], dTs[p], d0); d1 = fmaf(gg[k], dTs[m1 + p], d1);
-          d2 = fmaf(gg[k], dTs[2 * m1 + p], d2); d3 = fmaf(gg[k], dTs[3 * m1 + p], d3);
-        }
-      }
-    }
-    d0 = warp_sum(d0); d1 = warp_sum(d1); d2 = warp_sum(d2); d3 = warp_sum(d3);
-    if (lane == 0) reinterpret_cast<float4*>(a.dR)[base + s] = make_float4(d0, d1, d2, d3);
+  for (int c = 0; c < 4; ++c) {
+    const float4 x = on ? reinterpret_cast<const float4*>(dTs + c * m1)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    t[c][0] = x.x; t[c][1] = x.y; t[c][2] = x.z; t[c][3] = x.w;
   }
+  constexpr int RB = 2;
+  for (int s0 = warp; s0 < nn; s0 += nw * RB) {
+    float4 g[RB], r[RB];
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const int s = s0 + i * nw;
+      g[i] = on && s < nn ? G4[(size_t)s * q4 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+      r[i] = s < nn ? R4[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float d[RB][4];
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const int s = s0 + i * nw;
+      const float gg[4] = {g[i].x, g[i].y, g[i].z, g[i].w};
+      float4 v;
+      float* vp = &v.x;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) d[i][c] = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        vp[k] = r[i].x * t[0][k] + r[i].y * t[1][k] + r[i].z * t[2][k] + r[i].w * t[3][k];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d[i][c] = fmaf(gg[k], t[c][k], d[i][c]);
+      }
+      if (on && s < nn) dG4[(size_t)s * q4 + lane] = v;
+    }
+#pragma unroll
+    for (int i = 0; i < RB; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) d[i][c] = warp_sum(d[i][c]);
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const int s = s0 + i * nw;
+      if (lane == 0 && s < nn) dR4[s] = make_float4(d[i][0], d[i][1], d[i][2], d[i][3]);
+    }
+  }
+  for (int s = nn + threadIdx.x; s < NP; s += blockDim.x) dR4[s] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 void launch_desc_fwd(const DescArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
-  launch_pdl(k_desc_fwd, a.n, 128, sizeof(float) * 4 * a.m1, st, a);
+  launch_pdl(a.cq ? k_desc_fwd<true> : k_desc_fwd<false>, a.n, 128, sizeof(float) * 4 * a.m1, st, a);
   note_launch();
 }
 void launch_desc_bwd(const DescArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
   size_t sm = sizeof(float) * (8 * a.m1 + 2 * a.m1 * a.axis);
-  launch_pdl(k_desc_bwd, a.n, 128, sm, st, a);
+  launch_pdl(a.cq ? k_desc_bwd<true> : k_desc_bwd<false>, a.n, 128, sm, st, a);
   note_launch();
 }
 

@@ -545,6 +545,7 @@ __global__ void k_desc_jvp_fwd(JvpArgs a) {
   for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) {
     const int c = t / m1, p = t % m1;
     float v = 0.f;
+#pragma unroll 8
     for (int s = 0; s < nn; ++s) {
       const float* r = a.R + (base + s) * 4;
       const float* rd = a.Rd + (base + s) * 4;
