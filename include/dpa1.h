@@ -143,6 +143,15 @@ DP_API int dp_compute_batch(dp_model* m, int nframes, const int* atom_offsets, c
  * dp_compute_device and before capturing it in a CUDA graph). */
 DP_API int dp_reserve(dp_model* m, int max_atoms);
 
+/* Gradient of the energy with respect to the cell h (rows = cell vectors) at
+ * fixed Cartesian coordinates, from a call's coordinates, forces and virial (all
+ * DEVICE, on the current device): dE/dh = h^-T (sum_k x_k (x) F_k - W).  d_out
+ * [nout]: dE/dh in the first 9 entries, then a flag (1 if h is singular, the
+ * gradient then unspecified), the rest is scratch; nout >= 10 + 9 * min(152,
+ * max(1, ceil(natoms / 1024))), else DP_ERR_ARG.  Never synchronises. */
+DP_API int dp_box_gradient(int natoms, const double* d_coord, const double* d_box, const double* d_force,
+                           const double* d_virial, double* d_out, int nout, void* cuda_stream);
+
 /* Switch the arithmetic of the network products (enum dp_precision). */
 DP_API int dp_set_precision(dp_model* m, int precision);
 

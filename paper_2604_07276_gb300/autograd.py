@@ -19,12 +19,21 @@ from __future__ import annotations
 
 import torch
 
-from .binding import DPA1
+from .binding import DPA1, box_gradient as _box_gradient_device
 
 
 def box_gradient(coord: torch.Tensor, box: torch.Tensor, force: torch.Tensor, virial: torch.Tensor) -> torch.Tensor:
     """dE/dh [9] (row-major, h = box.view(3, 3)) from the coordinates the
-    call was given, its forces and its virial (all float64)."""
+    call was given, its forces and its virial (all float64).
+
+    CUDA tensors that need no derivative of the result go through the library
+    (two launches instead of about ten); anything else through PyTorch."""
+    ts = (coord, box, force, virial)
+    if all(t.is_cuda and t.dtype == torch.float64 and t.is_contiguous() and t.device == coord.device for t in ts) and \
+            not (torch.is_grad_enabled() and any(t.requires_grad for t in ts)) and \
+            coord.dim() == 2 and coord.shape[1] == 3 and force.shape == coord.shape and box.numel() == 9 and \
+            virial.numel() == 9:
+        return _box_gradient_device(coord, box, force, virial)
     h = box.reshape(3, 3).to(torch.float64)
     xf = coord.to(torch.float64).transpose(0, 1) @ force.to(torch.float64)
     return torch.linalg.solve(h.transpose(0, 1), xf - virial.reshape(3, 3).to(torch.float64)).reshape(9)

@@ -22,7 +22,7 @@ STATUS = {0: "DP_OK", -1: "DP_ERR_ARG", -2: "DP_ERR_IO", -3: "DP_ERR_BOX", -4: "
 PRECISION = {"fp32": 0, "bf16": 1, "fp16x": 2, "bf16x": 3}
 
 EXPORTS = ("dp_init", "dp_compute", "dp_compute_device", "dp_compute_local", "dp_compute_device_local", "dp_compute_batch", "dp_reserve", "dp_set_precision",
-           "dp_get_status", "dp_nlist_device", "dp_stats", "dp_inspect_weights", "dp_debug_copy", "dp_debug_poison",
+           "dp_get_status", "dp_box_gradient", "dp_nlist_device", "dp_stats", "dp_inspect_weights", "dp_debug_copy", "dp_debug_poison",
            "dp_set_profiling", "dp_stage_times", "dp_kernel_launches", "dp_nlist_noalloc", "dp_md_run", "dp_param_count", "dp_get_params",
            "dp_set_params", "dp_get_grad", "dp_zero_grad", "dp_train_frame", "dp_adam_step", "dp_last_error",
            "dp_free")
@@ -57,6 +57,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.dp_reserve.argtypes = [P, ctypes.c_int]
     lib.dp_set_precision.argtypes = [P, ctypes.c_int]
     lib.dp_get_status.argtypes = [P]
+    lib.dp_box_gradient.argtypes = [ctypes.c_int, P, P, P, P, P, ctypes.c_int, P]
     lib.dp_nlist_device.argtypes = [P, ctypes.c_int, P, P, P, P, P]
     lib.dp_stats.argtypes = [P, I, ctypes.POINTER(ctypes.c_longlong)]
     lib.dp_inspect_weights.argtypes = [ctypes.c_char_p, I, D]
@@ -119,6 +120,22 @@ def nlist_noalloc(coord, box, rcut: float, sel: int, nlist, nnei, status, stream
     st = stream if stream is not None else torch.cuda.current_stream(coord.device).cuda_stream
     _check(load_library().dp_nlist_noalloc(int(coord.shape[0]), coord.data_ptr(), box.data_ptr(), float(rcut),
                                            int(sel), nlist.data_ptr(), nnei.data_ptr(), status.data_ptr(), st))
+
+
+def box_gradient(coord, box, force, virial):
+    """``dp_box_gradient`` on contiguous float64 CUDA tensors of one device:
+    dE/dh [9]; raises ``torch.linalg.LinAlgError`` for a singular cell."""
+    import torch
+
+    n = int(coord.shape[0])
+    nout = 10 + 9 * min(152, max(1, -(-n // 1024)))
+    out = torch.empty(nout, dtype=torch.float64, device=coord.device)
+    with torch.cuda.device(coord.device):
+        _check(load_library().dp_box_gradient(n, coord.data_ptr(), box.data_ptr(), force.data_ptr(), virial.data_ptr(),
+                                              out.data_ptr(), nout, torch.cuda.current_stream().cuda_stream))
+    if out[9].item() != 0.0:
+        raise torch.linalg.LinAlgError("box_gradient: the cell is singular")
+    return out[:9]
 
 
 def kernel_launches() -> int:

@@ -1239,6 +1239,17 @@ int dp_compute_batch(dp_model* m, int nframes, const int* off, const double* coo
   return read_status(m);
 }
 
+int dp_box_gradient(int natoms, const double* d_coord, const double* d_box, const double* d_force,
+                    const double* d_virial, double* d_out, int nout, void* stream) {
+  if (natoms < 0 || !d_box || !d_virial || !d_out || (natoms > 0 && (!d_coord || !d_force)))
+    return fail(DP_ERR_ARG, "dp_box_gradient: bad arguments");
+  if (nout < 10 + 9 * box_grad_blocks(natoms)) return fail(DP_ERR_ARG, "dp_box_gradient: out is too small");
+  launch_box_grad(natoms, d_coord, d_box, d_force, d_virial, d_out, reinterpret_cast<cudaStream_t>(stream));
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(DP_ERR_CUDA, std::string("dp_box_gradient: launch failed: ") + cudaGetErrorString(e));
+  return DP_OK;
+}
+
 int dp_get_status(dp_model* m) {
   if (check_model(m)) return DP_ERR_ARG;
   CUDA_TRY(cudaSetDevice(m->device));

@@ -262,4 +262,82 @@ void launch_force_virial(const ForceArgs& a, cudaStream_t st) {
   }
 }
 
+// The gradient of E with respect to the cell h (rows = cell vectors) at fixed
+// Cartesian coordinates, dE/dh = h^-T (sum_k x_k (x) F_k - W): per-block sums of the
+// nine products, then one warp adds them in order and solves the 3 x 3 system by
+// elimination with partial pivoting.  out: dE/dh [9], a flag (1: h singular), then
+// the block sums.
+constexpr int BG_T = 256;
+__global__ void __launch_bounds__(BG_T) k_box_grad_sum(int n, const double* __restrict__ x, const double* __restrict__ f,
+                                                       double* __restrict__ part) {
+  pdl_wait();
+  __shared__ double red[9][BG_T / 32];
+  double s[9] = {};
+  for (int k = blockIdx.x * BG_T + threadIdx.x; k < n; k += gridDim.x * BG_T) {
+    const double a[3] = {x[3 * k], x[3 * k + 1], x[3 * k + 2]}, b[3] = {f[3 * k], f[3 * k + 1], f[3 * k + 2]};
+#pragma unroll
+    for (int i = 0; i < 9; ++i) s[i] = fma(a[i / 3], b[i % 3], s[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    s[i] = warp_sum_d(s[i]);
+    if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = s[i];
+  }
+  __syncthreads();
+  if (threadIdx.x < 9) {
+    double t = 0.0;
+    for (int w = 0; w < BG_T / 32; ++w) t += red[threadIdx.x][w];
+    part[9 * blockIdx.x + threadIdx.x] = t;
+  }
+}
+
+__global__ void k_box_grad_solve(int nblocks, const double* __restrict__ part, const double* __restrict__ box,
+                                 const double* __restrict__ virial, double* __restrict__ out) {
+  pdl_wait();
+  __shared__ double M[9];
+  if (threadIdx.x < 9) {
+    double t = 0.0;
+    for (int b = 0; b < nblocks; ++b) t += part[9 * b + threadIdx.x];
+    M[threadIdx.x] = t - virial[threadIdx.x];
+  }
+  __syncwarp();
+  if (threadIdx.x != 0) return;
+  double A[3][6];  // [h^T | M]
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) {
+      A[i][j] = box[3 * j + i];
+      A[i][3 + j] = M[3 * i + j];
+    }
+  double flag = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    int p = c;
+    for (int r = c + 1; r < 3; ++r)
+      if (fabs(A[r][c]) > fabs(A[p][c])) p = r;
+    if (A[p][c] == 0.0) flag = 1.0;
+    for (int j = 0; j < 6; ++j) {
+      const double t = A[c][j];
+      A[c][j] = A[p][j];
+      A[p][j] = t;
+    }
+    for (int r = 0; r < 3; ++r) {
+      if (r == c) continue;
+      const double m = A[r][c] / A[c][c];
+      for (int j = c; j < 6; ++j) A[r][j] -= m * A[c][j];
+    }
+  }
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) out[3 * i + j] = A[i][3 + j] / A[i][i];
+  out[9] = flag;
+}
+
+int box_grad_blocks(int n) { return n < 1 ? 1 : (n + 4 * BG_T - 1) / (4 * BG_T) < 152 ? (n + 4 * BG_T - 1) / (4 * BG_T) : 152; }
+
+void launch_box_grad(int n, const double* x, const double* box, const double* f, const double* virial, double* out,
+                     cudaStream_t st) {
+  const int nb = box_grad_blocks(n);
+  launch_pdl(k_box_grad_sum, nb, BG_T, 0, st, n, x, f, out + 10);
+  launch_pdl(k_box_grad_solve, 1, 32, 0, st, nb, out + 10, box, virial, out);
+  note_launch(2);
+}
+
 }  // namespace dpa1

@@ -108,6 +108,10 @@ struct ForceArgs {
   int nseg = 0;
 };
 void launch_force_virial(const ForceArgs& a, cudaStream_t st);
+// dE/dh from coordinates, forces and virial; out [10 + 9 box_grad_blocks(n)].
+int box_grad_blocks(int n);
+void launch_box_grad(int n, const double* x, const double* box, const double* f, const double* virial, double* out,
+                     cudaStream_t st);
 
 // --- FP32 SIMT network kernels (simt.cu)
 enum Epi { EPI_BIAS = 0, EPI_TANH = 1, EPI_RES_TANH = 2, EPI_ACCUM = 3, EPI_RES = 4 };
