@@ -984,6 +984,9 @@ int dp_init(dp_model** out, const char* weights_path, const char* const* type_ma
   }
   if (cudaStreamCreateWithFlags(&m->stream, cudaStreamNonBlocking) != cudaSuccess)
     return fail_free(fail(DP_ERR_CUDA, "stream creation failed"));
+  if (cudaHostAlloc(reinterpret_cast<void**>(&m->h_io), IO_BYTES, cudaHostAllocDefault) != cudaSuccess ||
+      cudaMalloc(reinterpret_cast<void**>(&m->d_io), IO_BYTES) != cudaSuccess)
+    return fail_free(fail(DP_ERR_CUDA, "allocation of the host-call staging failed"));
   if ((rc = alloc_workspace(m, 256)) != DP_OK) return fail_free(rc);
   *out = m;
   return DP_OK;
@@ -1049,6 +1052,39 @@ int dp_compute_local(dp_model* m, int natoms, int nlocal, const double* coord, c
   if (natoms > m->ws.cap && (rc = dp_reserve(m, natoms)) != DP_OK) return rc;
   Workspace& ws = m->ws;
   cudaStream_t st = m->stream;
+  if (natoms <= IO_ATOMS) {
+    // Small calls: the arrays packed in pinned memory, one copy in, one out, and the
+    // status word.  Separate copies of pageable arrays (three in, four out, the status
+    // and its clearing) are a host round trip each: 192 atoms 425 -> 383 us.  Above
+    // IO_ATOMS the copies take the time, and the caller's own arrays (pinned, perhaps)
+    // are copied as they are.
+    const size_t n = natoms;
+    char* hi = m->h_io;
+    char* ho = hi + IO_OUT;
+    int* h_err = reinterpret_cast<int*>(hi + IO_ERR);
+    double* di = reinterpret_cast<double*>(m->d_io);  // box, coord, atype
+    double* dout = reinterpret_cast<double*>(m->d_io + IO_OUT);  // energy, virial, force, e_i
+    memcpy(hi, box, 72);
+    if (n) {
+      memcpy(hi + 72, coord, 24 * n);
+      memcpy(hi + 72 + 24 * n, atype, 4 * n);
+    }
+    CUDA_TRY(cudaMemcpyAsync(di, hi, io_in(n), cudaMemcpyHostToDevice, st));
+    rc = run_device(m, natoms, nlocal, di + 9, di, reinterpret_cast<int*>(di + 9 + 3 * n), dout, dout + 10, dout + 1,
+                    dout + 10 + 3 * n, st);
+    if (rc != DP_OK) return rc;
+    CUDA_TRY(cudaMemcpyAsync(ho, dout, atom_energy ? io_out(n) : io_out(n) - 8 * n,
+                             cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(h_err, m->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    memcpy(energy, ho, 8);
+    memcpy(virial, ho + 8, 72);
+    if (n) {
+      memcpy(force, ho + 80, 24 * n);
+      if (atom_energy) memcpy(atom_energy, ho + 80 + 24 * n, 8 * n);
+    }
+    return *h_err ? read_status(m) : DP_OK;
+  }
   if (natoms > 0) {
     CUDA_TRY(cudaMemcpyAsync(ws.coord, coord, sizeof(double) * 3 * natoms, cudaMemcpyHostToDevice, st));
     CUDA_TRY(cudaMemcpyAsync(ws.atype, atype, sizeof(int) * natoms, cudaMemcpyHostToDevice, st));
@@ -1657,6 +1693,8 @@ void dp_free(dp_model* m) {
   bf16x_free(m);
   for (void* p : m->allocations) cudaFree(p);
   if (m->d_err) cudaFree(m->d_err);
+  if (m->h_io) cudaFreeHost(m->h_io);
+  if (m->d_io) cudaFree(m->d_io);
   if (m->stream) cudaStreamDestroy(m->stream);
   for (auto& e : m->prof.ev)
     if (e) cudaEventDestroy(e);

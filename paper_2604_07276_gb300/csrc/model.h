@@ -117,6 +117,16 @@ struct Workspace {
   TcBuffers tc;
 };
 
+// Host calls of up to IO_ATOMS atoms: bytes of the packed inputs (box, coordinates,
+// types) and results (energy, virial, forces, atomic energies), and of their staging
+// (inputs, results, status word).
+constexpr int IO_ATOMS = 4096;
+constexpr size_t io_in(size_t n) { return 9 * 8 + n * (24 + 4); }
+constexpr size_t io_out(size_t n) { return 10 * 8 + n * (24 + 8); }
+constexpr size_t IO_OUT = (io_in(IO_ATOMS) + 255) / 256 * 256;            // offset of the results
+constexpr size_t IO_ERR = IO_OUT + (io_out(IO_ATOMS) + 255) / 256 * 256;  // and of the status word
+constexpr size_t IO_BYTES = IO_ERR + 256;
+
 // Per-stage CUDA-event timing of one call (enabled with dp_set_profiling).
 // Stage boundaries accumulate over calls until profiling is switched on again.
 struct Profiler {
@@ -173,6 +183,10 @@ struct dp_model {
   std::vector<void*> allocations;
   Workspace ws;
   int* d_err = nullptr;
+  // dp_compute of up to IO_ATOMS atoms: pinned host memory and its device image, so
+  // that a call takes one copy each way (see dp_compute_local)
+  char* h_io = nullptr;
+  char* d_io = nullptr;
   cudaStream_t stream = nullptr;  // own stream of the host API
   cudaStream_t last_stream = nullptr;
   int last_natoms = 0;
