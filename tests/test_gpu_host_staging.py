@@ -25,6 +25,7 @@ def test_host_call_equals_device_call(default_model, n):
     f64 = torch.float64
     E, F, W, e = (torch.zeros(s, dtype=f64, device="cuda") for s in (1, (n, 3), 9, n))
     m.compute_device(dev(coord, f64), dev(p.box9(box), f64), dev(atype, torch.int32), E, F, W, e)
+    torch.cuda.synchronize()  # the host call runs on the model's own stream
     for want in (True, False):
         hE, hF, hW, he = m.compute(coord, box, atype, atom_energy=want)
         assert hE == E.item() and np.array_equal(hF, F.cpu().numpy())
