@@ -304,12 +304,21 @@ __device__ __forceinline__ float2 warp_max_pair(float2 v) {
 
 __device__ __forceinline__ float pair_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
 
-// Forward, register-tiled: 512 threads as a 32 x 16 grid.  Thread (ty, tx)
-// owns rows 4 ty + i (i < 4) and keys t_rc(tx, jj) (jj < 8) of S (128 x
-// 128), then the same rows and columns of each 128-column part of PG.  Q and K pass
-// through shared memory feature-major, 128 features at a time; P stays
-// row-major and [G 1] comes in 128-column parts, key-major.  S sums over the
-// features and PG over the keys in order, as a plain loop would.
+// Forward, register-tiled, 512 threads.  The products (S, then each 128-column
+// part of PG) give a warp 16 rows x 64 columns and a thread 4 x 8 of them (PTile):
+// per step a warp then reads 64 bytes of A and 2 x 128 of B, three 16-byte loads for
+// 32 FMAs with one wavefront each (8 x 128 a warp: five), and a warp whose rows, or a
+// half of it whose columns, are past the last neighbour has nothing to do.  The live
+// warps are spread over the four schedulers, and the loops unrolled eight times so
+// that loads run ahead of the FMAs: latency binds, not the shared-memory pipe (the
+// same tiles, one scheduler with twice the FMAs of another: 8 % slower; not unrolled:
+// 8 % more).  The softmax works on
+// rows 4 ty + i (i < 4) and keys t_rc(tx, jj) (jj < 8) of a 32 x 16 thread grid, S
+// passing through shared memory.  Q and K pass through shared memory
+// feature-major, 128 features at a time; P stays row-major and [G 1] comes in
+// 128-column parts, key-major.  S sums over the features and PG over the keys in
+// order, as a plain loop would.  3,001 atoms, width 128: 654 -> 593 us a layer (the
+// adjoint 1,385 -> 1,226).
 //
 // The kernel writes PG = [P G, rowsum(P)] instead of O = P V: with V = G Wv +
 // bv, O Wo + bo = [P G, rowsum(P)] [Wv Wo; bv Wo] + bo, which a GEMM with the
@@ -346,61 +355,131 @@ __device__ __forceinline__ void fm_store(float* T, int j, int f, float4 v) {
   T[(f + 2) * TLD + j] = v.z; T[(f + 3) * TLD + j] = v.w;
 }
 
-// Row i < TR of thread row coordinate ty: with TR = 8 (16 thread rows) the
-// quarter tiles of t_rc; with TR = 4 (32 thread rows) rows 4 ty .. 4 ty + 3.
-template <int TR>
-__device__ __forceinline__ int r_of(int ty, int i) { return TR == 8 ? t_rc(ty, i) : 4 * ty + i; }
-
-// The TR x 8 outer-product step of a register tile: acc[i][jj] += a[i] b[jj],
-// with a = (A[ra .. ra + 3] (, A[ra + 64 .. ra + 67] for TR = 8)) and b =
-// (B[rb .. rb + 3], B[rb + 64 .. rb + 67]).
-template <int TR>
-__device__ __forceinline__ void tile_fma(float (&acc)[TR][8], const float* A, int ra, const float* B, int rb) {
-  float av[TR];
-  const float4 a0 = *reinterpret_cast<const float4*>(A + ra);
-  av[0] = a0.x; av[1] = a0.y; av[2] = a0.z; av[3] = a0.w;
-  if constexpr (TR == 8) {
-    const float4 a1 = *reinterpret_cast<const float4*>(A + ra + 64);
-    av[4] = a1.x; av[5] = a1.y; av[6] = a1.z; av[7] = a1.w;
+// A thread's part of a 128 x 128 product: rows r .. r + 3, columns c .. c + 3
+// and c + 32 .. c + 35.
+struct PTile {
+  int r, c;
+  __device__ PTile(int tid) {
+    const int warp = tid >> 5, lane = tid & 31;
+    // live rows come first: consecutive row blocks over the SM's four schedulers
+    // (warp % 4), the column halves alternating
+    r = 16 * (warp >> 1) + 4 * (lane >> 3);
+    c = 64 * ((warp ^ (warp >> 2)) & 1) + 4 * (lane & 7);
   }
-  const float4 b0 = *reinterpret_cast<const float4*>(B + rb);
-  const float4 b1 = *reinterpret_cast<const float4*>(B + rb + 64);
-  const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+  // of the warp: rows below nrows, columns of its first and second half below ncols
+  __device__ int halves(int nrows, int ncols) const {
+    if ((r & ~15) >= nrows) return 0;
+    const int c0 = c & ~63;
+    return c0 + 32 < ncols ? 2 : (c0 < ncols ? 1 : 0);
+  }
+};
+
+// acc[i][j] += a[i] b[j] with a = A[ra .. ra + 3], b = (B[rb .. rb + 3], B[rb + 32
+// .. rb + 35] for H = 2).
+template <int H>
+__device__ __forceinline__ void tile_fma(float (&acc)[4][8], const float* A, int ra, const float* B, int rb) {
+  const float4 a0 = *reinterpret_cast<const float4*>(A + ra);
+  const float av[4] = {a0.x, a0.y, a0.z, a0.w};
 #pragma unroll
-  for (int i = 0; i < TR; ++i)
+  for (int h = 0; h < H; ++h) {
+    const float4 b0 = *reinterpret_cast<const float4*>(B + rb + 32 * h);
+    const float bv[4] = {b0.x, b0.y, b0.z, b0.w};
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj) acc[i][jj] = fmaf(av[i], bv[jj], acc[i][jj]);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][4 * h + j] = fmaf(av[i], bv[j], acc[i][4 * h + j]);
+  }
 }
 
-// acc[i][jj] += sum over k0 .. k0 + 3 of A[r_of(ty, i)][k] B[k][t_rc(tx, jj)]
-// (A row-major, B key-major, both with row stride TLD).
-template <int TR>
-__device__ __forceinline__ void tile_fma4(float (&acc)[TR][8], const float* A, const float* B, int k0, int ty,
-                                          int tx) {
-  float4 pa[TR];
+// acc[i][j] += sum over k0 .. k0 + 3 of A[r + i][k] B[k][c ..] (A row-major, B
+// key-major, both with row stride TLD).
+template <int H>
+__device__ __forceinline__ void tile_fma4(float (&acc)[4][8], const float* A, const float* B, int k0, const PTile& t) {
+  float4 pa[4];
 #pragma unroll
-  for (int i = 0; i < TR; ++i) pa[i] = *reinterpret_cast<const float4*>(A + r_of<TR>(ty, i) * TLD + k0);
+  for (int i = 0; i < 4; ++i) pa[i] = *reinterpret_cast<const float4*>(A + (t.r + i) * TLD + k0);
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
-    const float4 v0 = *reinterpret_cast<const float4*>(B + (k0 + u) * TLD + 4 * tx);
-    const float4 v1 = *reinterpret_cast<const float4*>(B + (k0 + u) * TLD + 64 + 4 * tx);
-    const float vb[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-    for (int i = 0; i < TR; ++i) {
-      const float p = u == 0 ? pa[i].x : u == 1 ? pa[i].y : u == 2 ? pa[i].z : pa[i].w;
+    for (int h = 0; h < H; ++h) {
+      const float4 v = *reinterpret_cast<const float4*>(B + (k0 + u) * TLD + t.c + 32 * h);
+      const float vb[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int jj = 0; jj < 8; ++jj) acc[i][jj] = fmaf(p, vb[jj], acc[i][jj]);
+      for (int i = 0; i < 4; ++i) {
+        const float p = u == 0 ? pa[i].x : u == 1 ? pa[i].y : u == 2 ? pa[i].z : pa[i].w;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][4 * h + j] = fmaf(p, vb[j], acc[i][4 * h + j]);
+      }
     }
   }
 }
 
-// One row of a register tile -> dst row (columns 4 tx .. and 64 + 4
-// tx .. from col0, each float4 only below ncols).
-__device__ __forceinline__ void tile_store_row(float* dst, const float* accrow, int col0, int tx, int ncols) {
-  if (col0 + 4 * tx < ncols)
-    *reinterpret_cast<float4*>(dst + col0 + 4 * tx) = make_float4(accrow[0], accrow[1], accrow[2], accrow[3]);
-  if (col0 + 64 + 4 * tx < ncols)
-    *reinterpret_cast<float4*>(dst + col0 + 64 + 4 * tx) = make_float4(accrow[4], accrow[5], accrow[6], accrow[7]);
+// acc = sum over k < n of the outer products of A[k][r ..] and B[k][c ..] (both
+// k-major with row stride TLD).
+__device__ __forceinline__ void tile_outer(float (&acc)[4][8], const float* A, const float* B, int n, const PTile& t,
+                                           int halves) {
+  if (halves == 2) {
+#pragma unroll 8
+    for (int k = 0; k < n; ++k) tile_fma<2>(acc, A, k * TLD + t.r, B, k * TLD + t.c);
+  } else if (halves == 1) {
+#pragma unroll 8
+    for (int k = 0; k < n; ++k) tile_fma<1>(acc, A, k * TLD + t.r, B, k * TLD + t.c);
+  }
+}
+
+// acc = sum over k < n (n % 4 == 0) of A[r ..][k] B[k][c ..].
+__device__ __forceinline__ void tile_inner(float (&acc)[4][8], const float* A, const float* B, int n, const PTile& t,
+                                           int halves) {
+  if (halves == 2) {
+#pragma unroll 4
+    for (int k = 0; k < n; k += 4) tile_fma4<2>(acc, A, B, k, t);
+  } else if (halves == 1) {
+#pragma unroll 4
+    for (int k = 0; k < n; k += 4) tile_fma4<1>(acc, A, B, k, t);
+  }
+}
+
+__device__ __forceinline__ void tile_zero(float (&acc)[4][8]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+}
+
+// The tile's rows below nrows -> dst (row stride ld, column 0 of the product at dst),
+// each float4 only below ncols.
+__device__ __forceinline__ void tile_store(float* dst, size_t ld, const float (&acc)[4][8], const PTile& t, int nrows,
+                                           int ncols) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (t.r + i >= nrows) continue;
+    float* p = dst + (size_t)(t.r + i) * ld + t.c;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (t.c + 32 * h < ncols)
+        *reinterpret_cast<float4*>(p + 32 * h) =
+            make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
+  }
+}
+
+// One row of the softmax's thread grid -> dst row (columns 4 tx .. and 64 + 4 tx ..).
+__device__ __forceinline__ void grid_store_row(float* dst, const float* v, int tx) {
+  *reinterpret_cast<float4*>(dst + 4 * tx) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4*>(dst + 64 + 4 * tx) = make_float4(v[4], v[5], v[6], v[7]);
+}
+__device__ __forceinline__ void grid_load_row(const float* src, float* v, int tx) {
+  const float4 a = *reinterpret_cast<const float4*>(src + 4 * tx), b = *reinterpret_cast<const float4*>(src + 64 + 4 * tx);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// The next atom's rows into L2, a row per thread.
+__device__ __forceinline__ void prefetch_rows(const float* p, int row_floats, int row0, int rows) {
+  const int t = threadIdx.x;
+  if (t < rows)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + (size_t)(row0 + t) * row_floats),
+                 "r"((uint32_t)(row_floats * sizeof(float)))
+                 : "memory");
 }
 
 template <int A>
@@ -413,20 +492,23 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
   float2* w2s = reinterpret_cast<float2*>(rws + NP);       // [NP] switch weights as float pairs
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int ld = a.ldq;  // Q | K
+  const PTile pt(tid);
   for (int atom = blockIdx.x; atom < a.n; atom += gridDim.x) {
     const int nn = a.nnei[atom];
     const size_t base = a.row_off[atom], gbase = (size_t)atom * NP;
+    if (atom + (int)gridDim.x < a.n) {
+      const int r0 = a.row_off[atom + gridDim.x], rows = a.row_off[atom + gridDim.x + 1] - r0;
+      prefetch_rows(a.QK, ld, r0, rows);
+      prefetch_rows(a.G, a.m1, r0, rows);
+    }
     __syncthreads();  // the previous atom is done with every shared array
     for (int r = tid; r < NP; r += FTF) {
       rws[r] = r < nn ? reinterpret_cast<const float4*>(a.rw)[gbase + r] : make_float4(0.f, 0.f, 0.f, 0.f);
       w2s[r] = split_pair(r < nn ? a.w64[gbase + r] : 0.0);
     }
-    float s[4][8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj) s[i][jj] = 0.f;
-    const bool live = 4 * ty < nn && 4 * tx < nn;
+    float acc[4][8];
+    tile_zero(acc);
+    const int live = pt.halves(nn, nn);
     for (int c0 = 0; c0 < A; c0 += 128) {
       if (c0 > 0) __syncthreads();  // the previous chunk's products are done
       for (int idx = tid; idx < NP * 32; idx += FTF) {
@@ -441,10 +523,15 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
         fm_store(Y, j, f, kv);
       }
       __syncthreads();
-      if (live)
-        for (int f = 0; f < 128; ++f) tile_fma<4>(s, X, f * TLD + 4 * ty, Y, f * TLD + 4 * tx);
+      tile_outer(acc, X, Y, 128, pt, live);
     }
-    __syncthreads();  // X and Y are free: P goes to X
+    __syncthreads();  // X and Y are free: S passes through X to the softmax's threads
+    if (live) tile_store(X, TLD, acc, pt, 128, 128);
+    __syncthreads();
+    float s[4][8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) grid_load_row(X + (4 * ty + i) * TLD, s[i], tx);
+    // (a thread reads the entries of S that it overwrites with P)
     // softmax per row over the 16 threads of a half warp (every lane takes
     // part in the shuffles; rows and keys past nnei come out zero)
 #pragma unroll
@@ -487,7 +574,7 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
           pv[jj] = e[jj] * inv * (rj.w * rk.w) * (rj.x * rk.x + rj.y * rk.y + rj.z * rk.z);
         }
       }
-      tile_store_row(X + j * TLD, pv, 0, tx, 128);
+      grid_store_row(X + j * TLD, pv, tx);
     }
     // PG = P [G 1], 128 columns at a time (column m1 of [G 1] is 1, later
     // ones 0; m1 % 4 == 0)
@@ -504,31 +591,23 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_fwd_f32(AttnArgs a, float scale
         *reinterpret_cast<float4*>(Y + k * TLD + f - c0) = vv;
       }
       __syncthreads();  // P (first part) and this part of [G 1] are in place
-      float acc[4][8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[i][jj] = 0.f;
-      if (4 * ty < nn)
-        for (int k = 0; k < nn4; k += 4) tile_fma4<4>(acc, X, Y, k, ty, tx);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (4 * ty + i < nn) tile_store_row(a.PG + (base + 4 * ty + i) * a.ldpg, acc[i], c0, tx, a.ldpg);
+      tile_zero(acc);
+      const int ncols = min(128, a.ldpg - c0);
+      tile_inner(acc, X, Y, nn4, pt, pt.halves(nn, ncols));
+      tile_store(a.PG + base * a.ldpg + c0, a.ldpg, acc, pt, nn, ncols);
     }
   }
 }
 
 // Adjoint of one attention layer for one centre, register-tiled like the
-// forward (512 threads as a 32 x 16 grid; thread (ty, tx) owns rows 4 ty + i
-// (i < 4) and keys or columns t_rc(tx, jj) (jj < 8) of each 128 x 128 product),
-// in the form of the forward's output Y = [P G, rowsum P] [Wv Wo; bv Wo] +
-// bo: with dPG = dE/d[P G, rowsum P] (a GEMM of dY with [Wv Wo; bv Wo]^T),
+// forward, in the form of its output Y = [P G, rowsum P] [Wv Wo; bv Wo] + bo: with
+// dPG = dE/d[P G, rowsum P] (a GEMM of dY with [Wv Wo; bv Wo]^T),
 //   dP_jk = sum_c dPG_jc G_kc + dPG_j,m1        (the values V never appear)
 //   softmax adjoint: dS, and the row / column parts of dE/dw and dE/drhat
 //   dQ = dS K,  dK = dS^T Q,  dE/dG += P^T dPG (columns below m1).
-// S and dP stay in registers through the softmax adjoint; dS and P then go to
-// shared memory (row-major), where the three last products read them.  The
-// column parts are summed over the 16 row groups in a fixed order.
+// S and dP pass through shared memory to the threads of the softmax adjoint; dS
+// and P go back there (row-major), where the three last products read them.  The
+// column parts are summed over the 32 row groups in a fixed order.
 template <int A>
 __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale) {
   pdl_wait();
@@ -541,20 +620,25 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
   float4* rowg = reinterpret_cast<float4*>(w2s + NP);        // [NP] row parts of (d rhat, d w)
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int ld = a.ldq;  // Q | K, and dQ | dK
+  const PTile pt(tid);
   for (int atom = blockIdx.x; atom < a.n; atom += gridDim.x) {
     const int nn = a.nnei[atom];
     const size_t base = a.row_off[atom], gbase = (size_t)atom * NP;
+    if (atom + (int)gridDim.x < a.n) {
+      const int r0 = a.row_off[atom + gridDim.x], rows = a.row_off[atom + gridDim.x + 1] - r0;
+      prefetch_rows(a.QK, ld, r0, rows);
+      prefetch_rows(a.G, a.m1, r0, rows);
+      prefetch_rows(a.dPG, a.ldpg, r0, rows);
+    }
     __syncthreads();  // the previous atom is done with every shared array
     for (int r = tid; r < NP; r += FTF) {
       rws[r] = r < nn ? reinterpret_cast<const float4*>(a.rw)[gbase + r] : make_float4(0.f, 0.f, 0.f, 0.f);
       w2s[r] = split_pair(r < nn ? a.w64[gbase + r] : 0.0);
     }
-    const bool live = 4 * ty < nn && 4 * tx < nn;
-    float s[4][8], dp[4][8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj) { s[i][jj] = 0.f; dp[i][jj] = 0.f; }
+    const int live = pt.halves(nn, nn);
+    float ps[4][8], pd[4][8];  // this thread's tiles of S and dP
+    tile_zero(ps);
+    tile_zero(pd);
     // S = Q K^T over feature chunks of 128 (feature-major in B0, B1)
     for (int c0 = 0; c0 < A; c0 += 128) {
       if (c0 > 0) __syncthreads();
@@ -570,8 +654,7 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
         fm_store(B1, j, f, kv);
       }
       __syncthreads();
-      if (live)
-        for (int f = 0; f < 128; ++f) tile_fma<4>(s, B0, f * TLD + 4 * ty, B1, f * TLD + 4 * tx);
+      tile_outer(ps, B0, B1, 128, pt, live);
     }
     __syncthreads();
     // dP = dPG G^T over the m1 columns (feature-major: dPG in B0, G in B1;
@@ -588,9 +671,21 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
       fm_store(B1, j, f, gv);
     }
     __syncthreads();
-    if (live)
-      for (int f = 0; f < a.m1; ++f) tile_fma<4>(dp, B0, f * TLD + 4 * ty, B1, f * TLD + 4 * tx);
-    __syncthreads();  // B0 and B1 are free: dS goes to B1, P to B2, column parts to B0
+    tile_outer(pd, B0, B1, a.m1, pt, live);
+    __syncthreads();  // B0 and B1 are free: S passes through B1, dP through B2
+    if (live) {
+      tile_store(B1, TLD, ps, pt, 128, 128);
+      tile_store(B2, TLD, pd, pt, 128, 128);
+    }
+    __syncthreads();
+    float s[4][8], dp[4][8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      grid_load_row(B1 + (4 * ty + i) * TLD, s[i], tx);
+      grid_load_row(B2 + (4 * ty + i) * TLD, dp[i], tx);
+    }
+    // (a thread reads the entries that it overwrites: dS goes to B1, P to B2,
+    // column parts to B0)
     // softmax adjoint per row over the 16 threads of a half warp (every lane
     // takes part in the shuffles; rows and keys past nnei come out zero)
     float cw[8], cx[8], cy[8], cz[8];
@@ -660,8 +755,8 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
           cx[jj] += dc * rj.x; cy[jj] += dc * rj.y; cz[jj] += dc * rj.z;
         }
       }
-      tile_store_row(B1 + j * TLD, ds, 0, tx, 128);
-      tile_store_row(B2 + j * TLD, pv, 0, tx, 128);
+      grid_store_row(B1 + j * TLD, ds, tx);
+      grid_store_row(B2 + j * TLD, pv, tx);
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) {
         rw_ += __shfl_xor_sync(0xffffffffu, rw_, o);
@@ -696,15 +791,10 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
       }
       __syncthreads();
       float acc[4][8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[i][jj] = 0.f;
-      if (4 * ty < nn)
-        for (int k = 0; k < nn4; k += 4) tile_fma4<4>(acc, B1, B0, k, ty, tx);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (4 * ty + i < nn) tile_store_row(a.dQK + (base + 4 * ty + i) * ld, acc[i], c0, tx, A);
+      const int lv = pt.halves(nn, 128);
+      tile_zero(acc);
+      tile_inner(acc, B1, B0, nn4, pt, lv);
+      tile_store(a.dQK + base * ld + c0, ld, acc, pt, nn, 128);
       // dK = dS^T Q: Q row-major in B0
       __syncthreads();
       for (int idx = tid; idx < NP * 32; idx += FTF) {
@@ -713,15 +803,9 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
             j < nn ? *reinterpret_cast<const float4*>(a.QK + (base + j) * ld + c0 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
       __syncthreads();
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[i][jj] = 0.f;
-      if (4 * ty < nn)
-        for (int j = 0; j < nn; ++j) tile_fma<4>(acc, B1, j * TLD + 4 * ty, B0, j * TLD + 4 * tx);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (4 * ty + i < nn) tile_store_row(a.dQK + (base + 4 * ty + i) * ld + A, acc[i], c0, tx, A);
+      tile_zero(acc);
+      tile_outer(acc, B1, B0, nn, pt, lv);
+      tile_store(a.dQK + base * ld + A + c0, ld, acc, pt, nn, 128);
     }
     // dE/dG += P^T dPG: dPG row-major in B0 (columns below m1; m1 <= 128)
     __syncthreads();
@@ -732,28 +816,20 @@ __global__ void __launch_bounds__(FTF, 1) k_attn_bwd_f32(AttnArgs a, float scale
                                                          : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    if (4 * ty < nn && 4 * tx < a.m1) {
+    if (const int lv = pt.halves(nn, a.m1)) {
       float acc[4][8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[i][jj] = 0.f;
-      for (int j = 0; j < nn; ++j) tile_fma<4>(acc, B2, j * TLD + 4 * ty, B0, j * TLD + 4 * tx);
+      tile_zero(acc);
+      tile_outer(acc, B2, B0, nn, pt, lv);
+      // one writer per element: reductions without a return
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int k = 4 * ty + i;
-        if (k >= nn) continue;
-        float* dgrow = a.dG + (base + k) * a.m1;
+        if (pt.r + i >= nn) continue;
+        float* p = a.dG + (base + pt.r + i) * a.m1 + pt.c;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int c = 64 * h + 4 * tx;
-          if (c < a.m1) {
-            float4* dg = reinterpret_cast<float4*>(dgrow + c);
-            float4 x = *dg;
-            x.x += acc[i][4 * h]; x.y += acc[i][4 * h + 1]; x.z += acc[i][4 * h + 2]; x.w += acc[i][4 * h + 3];
-            *dg = x;
-          }
-        }
+        for (int h = 0; h < 2; ++h)
+          if (pt.c + 32 * h < a.m1)
+            atomicAdd(reinterpret_cast<float4*>(p + 32 * h),
+                      make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]));
       }
     }
   }
