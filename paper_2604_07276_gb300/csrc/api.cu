@@ -249,9 +249,8 @@ int alloc_workspace(dp_model* m, int cap) {
     ws.cell_of = a.take<int>(cap);
     ws.cell_count = a.take<int>(ws.cell_cap);
     ws.cell_start = a.take<int>(ws.cell_cap + 1);
-    ws.cell_cursor = a.take<int>(ws.cell_cap);
-    ws.cell_atoms = a.take<int>(cap);
-    ws.coordf = a.take<float4>(cap);
+    ws.cell_rank = a.take<int>(cap);
+    ws.cell_pos = a.take<float4>(cap);
     ws.nlist = a.take<int>(rows);
     ws.nnei = a.take<int>(cap);
     ws.ncand = a.take<int>(cap);
@@ -345,7 +344,7 @@ int translate_err(int bits) {
 
 // Stages a1-a2 on the stream.
 // Neighbour-stage arguments for n atoms at coord, with the list, counts,
-// clamped types and FP32 coordinates written from workspace slot rel on.
+// clamped types and reverse list written from workspace slot rel on.
 NbrArgs nbr_args(dp_model* m, int n, const double* coord, const double* box, const int* atype, CellGrid* grid,
                  int rel) {
   Workspace& ws = m->ws;
@@ -354,10 +353,10 @@ NbrArgs nbr_args(dp_model* m, int n, const double* coord, const double* box, con
   a.n = n; a.ntypes = m->nt; a.sel = m->sel; a.rcut = m->rcut;
   a.cap_dim = ws.cap_dim; a.cell_cap = ws.cell_cap; a.grid = grid;
   a.cell_of = ws.cell_of; a.cell_count = ws.cell_count; a.cell_start = ws.cell_start;
-  a.cell_cursor = ws.cell_cursor; a.cell_atoms = ws.cell_atoms;
+  a.cell_rank = ws.cell_rank; a.cell_pos = ws.cell_pos;
   a.nlist = ws.nlist + (size_t)rel * NP; a.nnei = ws.nnei + rel; a.ncand = ws.ncand + rel;
-  a.atype_c = ws.atype_c + rel; a.coordf = ws.coordf + rel;
-  a.rev_cnt = ws.rev_cnt + rel;
+  a.atype_c = ws.atype_c + rel;
+  a.rev_cnt = ws.rev_cnt + rel; a.rev_rows = ws.rev_rows + (size_t)rel * REV_CAP;
   a.err = m->d_err;
   return a;
 }
@@ -636,7 +635,6 @@ int run_after_neighbors(dp_model* m, int n, const double* coord, const CellGrid*
   launch_env_bwd(eb, st);
   prof_mark(m, "env_bwd", st);
   // a15: forces, virial, energy
-  launch_reverse(ws.nlist, n, ws.rev_cnt, ws.rev_rows, m->d_err, st);
   ForceArgs fa{};
   fa.g = ws.g; fa.rv = ws.rv; fa.nnei = ws.nnei; fa.rev_cnt = ws.rev_cnt; fa.rev_rows = ws.rev_rows; fa.e = ws.e;
   fa.n = n; fa.nlocal = m->call_nlocal; fa.force = force; fa.atom_energy = atom_energy; fa.partials = ws.partials;
@@ -1176,6 +1174,7 @@ int dp_compute_batch(dp_model* m, int nframes, const int* off, const double* coo
       if (nc < 3) nc = 1;
       if (nc > m->ws.cap_dim) nc = m->ws.cap_dim;
       g.nc[d] = nc;
+      g.scale[d] = (double)nc / L;
     }
     g.ncells = g.nc[0] * g.nc[1] * g.nc[2];
     grids[f] = g;
@@ -1432,13 +1431,12 @@ struct NoAllocScratch {
   CellGrid grid;
   int cell_count[NA_MAX_CELLS];
   int cell_start[NA_MAX_CELLS + 1];
-  int cell_cursor[NA_MAX_CELLS];
   int cell_of[NA_MAX_ATOMS];
-  int cell_atoms[NA_MAX_ATOMS];
+  int cell_rank[NA_MAX_ATOMS];
   int ncand[NA_MAX_ATOMS];
   int types[NA_MAX_ATOMS];    // all zero: the list does not depend on types
   int types_c[NA_MAX_ATOMS];
-  float4 coordf[NA_MAX_ATOMS];  // FP32 coordinates for the candidate screen
+  float4 cell_pos[NA_MAX_ATOMS];
 };
 __device__ __align__(256) NoAllocScratch g_nbr_scratch;
 constexpr int NA_MAX_DEVICES = 64;
@@ -1476,10 +1474,10 @@ int dp_nlist_noalloc(int natoms, const double* d_coord, const double* d_box, dou
   a.n = natoms; a.ntypes = 1; a.sel = sel; a.rcut = rcut;
   a.cap_dim = NA_CAP_DIM; a.cell_cap = NA_MAX_CELLS; a.grid = &s->grid;
   a.cell_of = s->cell_of; a.cell_count = s->cell_count; a.cell_start = s->cell_start;
-  a.cell_cursor = s->cell_cursor; a.cell_atoms = s->cell_atoms;
-  a.nlist = d_nlist; a.nnei = d_nnei; a.ncand = s->ncand; a.atype_c = s->types_c; a.coordf = s->coordf;
+  a.cell_rank = s->cell_rank; a.cell_pos = s->cell_pos;
+  a.nlist = d_nlist; a.nnei = d_nnei; a.ncand = s->ncand; a.atype_c = s->types_c;
   a.err = d_status;
-  a.rev_cnt = nullptr;
+  a.rev_cnt = nullptr; a.rev_rows = nullptr;
   launch_neighbors(a, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, std::string("dp_nlist_noalloc: launch failed: ") + cudaGetErrorString(e));

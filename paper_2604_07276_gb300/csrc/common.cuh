@@ -65,6 +65,7 @@ enum ErrBits : int {
 // Cell grid derived on the device from the (device) box.
 struct CellGrid {
   double L[3];
+  double scale[3];  // nc / L
   int nc[3];
   int ncells;
   int ok;
@@ -116,6 +117,45 @@ __device__ __forceinline__ float warp_reduce_scatter16(float* v) {
 // bit for bit.
 __device__ __forceinline__ double mic(double d, double L) {
   return __dsub_rn(d, __dmul_rn(L, rint(__ddiv_rn(d, L))));
+}
+
+// mic() without its division when no image shift is possible: for |d| < L/2 the
+// rounded d / L lies in [-0.5, 0.5], rint gives 0 and mic returns d up to the sign of
+// a zero.  The test compares the high words (strictly less there: less in value; NaN
+// is not), since an FP64 instruction of this GPU takes as long as 32 of FP32.
+__device__ __forceinline__ double mic_near(double d, double L) {
+  return (__double2hiint(d) & 0x7fffffff) < __double2hiint(L) - 0x100000 ? d : mic(d, L);
+}
+
+// Sorts 32 R unsigned values over a warp in ascending order: a bitonic network in
+// registers, lane l ending up with places R l to R l + R - 1.  Strides below R need
+// no exchange, the others one shuffle per value; in shared memory each of the
+// network's stages waited for its loads and stores (128 values: 28 stages).
+template <int R>
+__device__ __forceinline__ void warp_sort(unsigned (&k)[R]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int kk = 2; kk <= 32 * R; kk <<= 1)
+#pragma unroll
+    for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+      if (jj >= R) {
+        const bool up = kk == 32 * R || (lane & (kk / R)) == 0, low = (lane & (jj / R)) == 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const unsigned o = __shfl_xor_sync(0xffffffffu, k[r], jj / R);
+          k[r] = up == low ? min(k[r], o) : max(k[r], o);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if ((r & jj) == 0) {
+            const bool up = kk < R ? (r & kk) == 0 : kk == 32 * R || (lane & (kk / R)) == 0;
+            const unsigned a = k[r], b = k[r | jj], lo = min(a, b), hi = max(a, b);
+            k[r] = up ? lo : hi;
+            k[r | jj] = up ? hi : lo;
+          }
+      }
+    }
 }
 
 // (dx*dx + dy*dy) + dz*dz without contraction.

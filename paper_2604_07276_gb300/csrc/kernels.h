@@ -19,12 +19,14 @@ struct NbrArgs {
   double rcut;
   int cap_dim, cell_cap;
   CellGrid* grid;
-  int *cell_of, *cell_count, *cell_start, *cell_cursor, *cell_atoms;
+  int *cell_of, *cell_count, *cell_start, *cell_rank;
+  float4* cell_pos;  // scratch [n]: the atoms cell by cell, FP32 coordinates and the index (bits)
   int *nlist, *nnei, *ncand;
   int* atype_c;    // out: types clamped to [0, ntypes)
-  float4* coordf;  // scratch [n]: FP32 copy of the coordinates for the candidate screen
   int* err;
-  int* rev_cnt;    // out: zeroed for the reverse list (null: none)
+  // out, the reverse list (null: none): how many rows list an atom, and which
+  // (REV_CAP places an atom, in no order)
+  int *rev_cnt, *rev_rows;
   // packed batches, one frame per call: atoms [n, n_out) are padding (no
   // neighbours, type 0) and base is added to every neighbour index written
   // (0 and 0: plain call)
@@ -42,8 +44,6 @@ void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell
 // ROW_SEG atoms.
 constexpr int ROW_SEG = 4096;
 void launch_row_list(const int* nnei, int n, int* row_off, int* rowmap, int* seg, cudaStream_t st);
-// rev_cnt: zero on entry (the neighbour search clears it).
-void launch_reverse(const int* nlist, int n, int* rev_cnt, int* rev_rows, int* err, cudaStream_t st);
 
 // --- environment matrix and its adjoint, forces, reductions (env.cu)
 struct EnvArgs {

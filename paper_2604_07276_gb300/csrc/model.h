@@ -89,14 +89,14 @@ struct Workspace {
   size_t bytes = 0;
   // neighbour search
   CellGrid* grid;
-  int *cell_of, *cell_count, *cell_start, *cell_cursor, *cell_atoms;
+  int *cell_of, *cell_count, *cell_start, *cell_rank;
+  float4* cell_pos;  // the atoms cell by cell: FP32 coordinates, index
   int cell_cap, cap_dim;
   int *nlist, *nnei, *ncand, *rev_cnt, *rev_rows;
   // the live neighbour rows in order: first row of each atom [cap + 1], and each
   // row's place atom * NP + slot (launch_row_list)
   int *row_off, *rowmap, *row_seg;
   int* atype_c;  // device-checked copy of the atom types
-  float4* coordf;  // FP32 coordinates (neighbour screen)
   // environment
   float *R, *rw, *rv, *dR, *dgeo, *g;
   double* w64;

@@ -14,12 +14,9 @@ namespace dpa1 {
 // otherwise be visited twice).
 __global__ void k_cell_setup(const double* __restrict__ box, double rcut, int cap_dim,
                              CellGrid* __restrict__ cg, int* __restrict__ err, int* __restrict__ cell_count,
-                             int* __restrict__ cell_cursor, int cell_cap) {
+                             int cell_cap) {
   pdl_wait();
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cell_cap; c += gridDim.x * blockDim.x) {
-    cell_count[c] = 0;
-    cell_cursor[c] = 0;
-  }
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cell_cap; c += gridDim.x * blockDim.x) cell_count[c] = 0;
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   CellGrid g;
   g.ok = 1;
@@ -33,6 +30,7 @@ __global__ void k_cell_setup(const double* __restrict__ box, double rcut, int ca
     if (nc < 3) nc = 1;
     if (nc > cap_dim) nc = cap_dim;
     g.nc[a] = nc;
+    g.scale[a] = (double)nc / L;
   }
   g.ncells = g.nc[0] * g.nc[1] * g.nc[2];
   if (!g.ok) {
@@ -40,26 +38,30 @@ __global__ void k_cell_setup(const double* __restrict__ box, double rcut, int ca
     g.nc[0] = g.nc[1] = g.nc[2] = 1;
     g.ncells = 1;
     g.L[0] = g.L[1] = g.L[2] = 1.0;
+    g.scale[0] = g.scale[1] = g.scale[2] = 1.0;
   }
   *cg = g;
 }
 
-__device__ __forceinline__ int cell_coord(double x, double L, int nc) {
-  double w = x - L * floor(x / L);
-  int c = (int)(w * (double)nc / L);
+// A coordinate inside the box needs no division (its floor is 0).
+__device__ __forceinline__ int cell_coord(double x, double L, double scale, int nc) {
+  double w = x >= 0.0 && x < L ? x : x - L * floor(x / L);
+  int c = (int)(w * scale);
   return c < 0 ? 0 : (c >= nc ? nc - 1 : c);
 }
 
 // frame non-null (packed batches): slot i belongs to frame frame[i] (-1:
-// padding, no cell) with grid cgp[f] and cells from cell_base[f] - cb0 on.
+// padding, no cell) with grid cgp[f] and cells from cell_base[f] - cb0 on.  An atom's
+// rank in its cell is what the count was before it.
 __global__ void k_cell_count(const double* __restrict__ coord, const int* __restrict__ atype, int n,
                              int ntypes, const CellGrid* __restrict__ cgp, int* __restrict__ cell_of,
-                             int* __restrict__ cell_count, int* __restrict__ atype_c, float4* __restrict__ coordf,
-                             int* __restrict__ err, const int* __restrict__ frame, const int* __restrict__ cell_base,
-                             int cb0) {
+                             int* __restrict__ cell_count, int* __restrict__ cell_rank, int* __restrict__ atype_c,
+                             int* __restrict__ rev_cnt, int* __restrict__ err, const int* __restrict__ frame,
+                             const int* __restrict__ cell_base, int cb0) {
   pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  if (rev_cnt) rev_cnt[i] = 0;
   int cbase = 0;
   const CellGrid* gp = cgp;
   if (frame) {
@@ -74,14 +76,13 @@ __global__ void k_cell_count(const double* __restrict__ coord, const int* __rest
   }
   const CellGrid g = *gp;
   double x = coord[3 * i], y = coord[3 * i + 1], z = coord[3 * i + 2];
-  coordf[i] = make_float4((float)x, (float)y, (float)z, 0.f);
   int c = 0;
   if (!isfinite(x) || !isfinite(y) || !isfinite(z)) {
     set_err(err, ERR_NAN);
   } else {
-    int cx = cell_coord(x, g.L[0], g.nc[0]);
-    int cy = cell_coord(y, g.L[1], g.nc[1]);
-    int cz = cell_coord(z, g.L[2], g.nc[2]);
+    int cx = cell_coord(x, g.L[0], g.scale[0], g.nc[0]);
+    int cy = cell_coord(y, g.L[1], g.scale[1], g.nc[1]);
+    int cz = cell_coord(z, g.L[2], g.scale[2], g.nc[2]);
     c = (cz * g.nc[1] + cy) * g.nc[0] + cx;
   }
   c += cbase;
@@ -92,7 +93,7 @@ __global__ void k_cell_count(const double* __restrict__ coord, const int* __rest
   }
   atype_c[i] = t;
   cell_of[i] = c;
-  atomicAdd(&cell_count[c], 1);
+  cell_rank[i] = atomicAdd(&cell_count[c], 1);
 }
 
 // Exclusive scan of the cell counts (one block).
@@ -123,15 +124,17 @@ __global__ void k_cell_scan(const int* __restrict__ cell_count, int* __restrict_
   if (threadIdx.x == 0) cell_start[ncells] = carry;
 }
 
-__global__ void k_cell_fill(const int* __restrict__ cell_of, int n, const int* __restrict__ cell_start,
-                            int* __restrict__ cell_cursor, int* __restrict__ cell_atoms) {
+// The atoms cell by cell: FP32 coordinates for the candidate screen, the index in w.
+__global__ void k_cell_fill(const double* __restrict__ coord, const int* __restrict__ cell_of,
+                            const int* __restrict__ cell_rank, int n, const int* __restrict__ cell_start,
+                            float4* __restrict__ cell_pos) {
   pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int c = cell_of[i];
   if (c < 0) return;  // padding of a packed batch
-  int pos = cell_start[c] + atomicAdd(&cell_cursor[c], 1);
-  cell_atoms[pos] = i;
+  cell_pos[cell_start[c] + cell_rank[i]] =
+      make_float4((float)coord[3 * i], (float)coord[3 * i + 1], (float)coord[3 * i + 2], __int_as_float(i));
 }
 
 // Sort keys: the bit pattern of d^2 >= 0 (+0 or positive, never NaN) read as an
@@ -140,35 +143,83 @@ __device__ __forceinline__ bool key_gt(unsigned long long da, int ja, unsigned l
   return da > db || (da == db && ja > jb);
 }
 
-// mic() without its division when no image shift is possible: for |d| < L/2
-// the rounded d / L lies in [-0.5, 0.5], rint gives 0 and mic returns d up to
-// the sign of a zero, which the squared distance does not see.
-__device__ __forceinline__ double mic_near(double d, double L) {
-  return fabs(d) < 0.5 * L ? d : mic(d, L);
+constexpr int NBR_WARPS = 4;
+constexpr int NBR_SEGS = 18;  // 9 rows of 3 cells along x, each cut in two by the box edge at most
+
+// One warp's buffers.
+struct NbrShared {
+  unsigned long long key[NBR_CAP];  // bits of d^2
+  int idx[NBR_CAP];                 // candidate
+  unsigned char order[NBR_CAP];     // candidates' places, sorted
+  int2 seg[NBR_SEGS];               // running end of a segment's candidates, its offset in cell_pos
+};
+
+// The order of the cnt <= 32 R candidates by (d^2, j).  The registers sort 24 bits of
+// d^2 - the value's exponent and 20 fraction bits below rc^2, everything under
+// rc^2 / 65,536 alike - with the place in the low byte; pairs of neighbours that these
+// bits leave undecided are put right by exchanges on the full key.
+template <int R>
+__device__ __forceinline__ void sort_candidates(NbrShared& sh, int cnt, int hi_rc2, int lane) {
+  unsigned k[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int e = 32 * r + lane;
+    k[r] = 0xffffffffu;
+    if (e < cnt) {
+      const int hi = (int)(sh.key[e] >> 32) - (hi_rc2 - 0xffffff);
+      k[r] = (unsigned)max(hi, 0) << 8 | (unsigned)e;
+    }
+  }
+  warp_sort<R>(k);
+  const unsigned next = __shfl_down_sync(0xffffffffu, k[0], 1);
+  bool tie = false;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int p = R * lane + r;  // the place after it: p + 1
+    sh.order[p] = (unsigned char)(k[r] & 0xff);
+    tie |= p + 1 < cnt && k[r] >> 8 == (r + 1 < R ? k[(r + 1) % R] : next) >> 8;
+  }
+  __syncwarp();
+  if (!__any_sync(0xffffffffu, tie)) return;
+  // odd-even transposition sorts cnt values in cnt rounds at most
+  for (int round = 0; round < cnt; round += 2) {
+    bool moved = false;
+    for (int odd = 0; odd < 2; ++odd) {
+      for (int p = 2 * lane + odd; p + 1 < cnt; p += 64) {
+        const int x = sh.order[p], y = sh.order[p + 1];
+        if (key_gt(sh.key[x], sh.idx[x], sh.key[y], sh.idx[y])) {
+          sh.order[p] = (unsigned char)y;
+          sh.order[p + 1] = (unsigned char)x;
+          moved = true;
+        }
+      }
+      __syncwarp();
+    }
+    if (!__any_sync(0xffffffffu, moved)) break;
+  }
 }
 
 // One warp per centre atom: gather every candidate j != i with d^2 < rc^2 from
 // the 27 surrounding cells (screened in FP32, decided in FP64 and
-// bit-reproducible), then bitonic-sort the candidates by (d^2, j) and keep the
-// first sel.  FP64 is slow on this part, so it is kept to the ~11 % of
-// candidates that pass the screen.
-constexpr int NBR_WARPS = 4;
-// 10 blocks per SM (48 registers, no spills): the search is latency-bound and
-// gains from the extra resident warps
-__global__ void __launch_bounds__(32 * NBR_WARPS, 10)
+// bit-reproducible), then sort the candidates by (d^2, j) and keep the first sel; a
+// kept pair also enters j's reverse list, as row i * NP + slot.  FP64 is slow on this
+// part, so it is kept to the ~11 % of candidates that pass the screen.  A chain of
+// dependent loads and of sort stages binds, so loads go out in groups of four, a row
+// of cells is one stretch, and the sort stays in registers.  15,668 atoms: the
+// search's kernels took 181 us, and 26 for the reverse list's own -> 87 together; 192
+// atoms: 42 + 6 -> 32.  63 registers: held to 48 for two more blocks an SM, 183.
+__global__ void __launch_bounds__(32 * NBR_WARPS, 8)
 k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const CellGrid* __restrict__ cgp,
             const int* __restrict__ cell_of, const int* __restrict__ cell_start,
-            const int* __restrict__ cell_atoms, double rc2, int sel, int* __restrict__ nlist,
-            int* __restrict__ nnei, int* __restrict__ ncand, int* __restrict__ atype_c,
-            const float4* __restrict__ coordf, int* __restrict__ err, const int* __restrict__ frame,
-            const int* __restrict__ cell_base, int cb0, int* __restrict__ rev_cnt) {
+            const float4* __restrict__ cell_pos, double rc2, int sel, int* __restrict__ nlist,
+            int* __restrict__ nnei, int* __restrict__ ncand, int* __restrict__ atype_c, int* __restrict__ err,
+            const int* __restrict__ frame, const int* __restrict__ cell_base, int cb0, int* __restrict__ rev_cnt,
+            int* __restrict__ rev_rows) {
   pdl_wait();
-  __shared__ unsigned long long skey[NBR_WARPS][NBR_CAP];
-  __shared__ int sidx[NBR_WARPS][NBR_CAP];
+  __shared__ NbrShared s_sh[NBR_WARPS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * NBR_WARPS + warp;
   const int fi = frame && i < n ? frame[i] : 0;
-  if (rev_cnt && lane == 0 && i < n_out) rev_cnt[i] = 0;
   if (i >= n || fi < 0) {
     // padding atoms of a packed batch: no neighbours, a valid type
     if (i < n_out || (i < n && fi < 0)) {
@@ -177,62 +228,96 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
         nnei[i] = 0;
         ncand[i] = 0;
         atype_c[i] = 0;
+        if (rev_cnt) rev_cnt[i] = 0;
       }
     }
     return;
   }
-  const CellGrid g = cgp[frame ? fi : 0];
-  const int cbase = frame ? cell_base[fi] - cb0 : 0;  // the frame's first cell
-  unsigned long long* key = skey[warp];
-  int* idx = sidx[warp];
+  NbrShared& sh = s_sh[warp];
+  const CellGrid* g = cgp + (frame ? fi : 0);
   const double xi = coord[3 * i], yi = coord[3 * i + 1], zi = coord[3 * i + 2];
-  const float4 pi = coordf[i];
-  const int ci = cell_of[i] - cbase;
-  const int cx = ci % g.nc[0], cy = (ci / g.nc[0]) % g.nc[1], cz = ci / (g.nc[0] * g.nc[1]);
-  const int ox = g.nc[0] >= 3 ? 1 : 0, oy = g.nc[1] >= 3 ? 1 : 0, oz = g.nc[2] >= 3 ? 1 : 0;
-  const float Lf[3] = {(float)g.L[0], (float)g.L[1], (float)g.L[2]};
-  const float iLf[3] = {1.0f / Lf[0], 1.0f / Lf[1], 1.0f / Lf[2]};
-  const float rc2_screen = (float)rc2 * 1.0001f + 1e-4f;
-  // pass 1: FP32 screen of every candidate in the 27 cells; survivors are
-  // compacted into idx[] so that the FP64 decision below runs on full warps
-  // (this part's FP64 rate is low, and a divergent FP64 branch costs the whole
-  // warp)
-  // a neighbouring cell's index along an axis, wrapped without a division
-  // (offsets are -1, 0 or +1)
-  auto wrap = [](int x, int nc) { return x < 0 ? x + nc : (x >= nc ? x - nc : x); };
-  int ns = 0;
-  for (int dz = -oz; dz <= oz; ++dz)
-    for (int dy = -oy; dy <= oy; ++dy)
-      for (int dx = -ox; dx <= ox; ++dx) {
-        const int nx = wrap(cx + dx, g.nc[0]);
-        const int ny = wrap(cy + dy, g.nc[1]);
-        const int nz = wrap(cz + dz, g.nc[2]);
-        int c = cbase + (nz * g.nc[1] + ny) * g.nc[0] + nx;
-        int b = cell_start[c], e = cell_start[c + 1];
-        for (int base = b; base < e; base += 32) {
-          int t = base + lane;
-          bool pass = false;
-          int j = -1;
-          if (t < e) {
-            j = cell_atoms[t];
-            // a component of the FP32 difference is off by at most ~1e-5 A
-            // and the squared distance near rc^2 by ~1.3e-4 A^2, far inside
-            // the margin, so a pair rejected here is never a neighbour (where
-            // FP32 and FP64 pick different images, both distances exceed
-            // L/2 > rcut)
-            const float4 pj = coordf[j];
-            float fx = pj.x - pi.x, fy = pj.y - pi.y, fz = pj.z - pi.z;
-            fx -= Lf[0] * rintf(fx * iLf[0]);
-            fy -= Lf[1] * rintf(fy * iLf[1]);
-            fz -= Lf[2] * rintf(fz * iLf[2]);
-            pass = j != i && fx * fx + fy * fy + fz * fz < rc2_screen;
-          }
-          const unsigned bal = __ballot_sync(0xffffffffu, pass);
-          const int pos = ns + __popc(bal & ((1u << lane) - 1u));
-          if (pass && pos < NBR_CAP) idx[pos] = j;
-          ns += __popc(bal);
-        }
+  const float fxi = (float)xi, fyi = (float)yi, fzi = (float)zi;
+  const float Lx = (float)g->L[0], Ly = (float)g->L[1], Lz = (float)g->L[2];
+  const float iLx = 1.0f / Lx, iLy = 1.0f / Ly, iLz = 1.0f / Lz;
+  // The cells of a row along x follow each other in cell_pos: a lane finds one
+  // contiguous stretch of candidates (part 1: what wraps around the box edge).
+  int ns = 0, total;
+  {
+    const int cbase = frame ? cell_base[fi] - cb0 : 0;  // the frame's first cell
+    const int nx = g->nc[0], ny = g->nc[1], nz = g->nc[2];
+    const int ci = cell_of[i] - cbase;
+    const int cx = ci % nx, cy = (ci / nx) % ny, cz = ci / (nx * ny);
+    const int row = lane >> 1, dy = row % 3 - 1, dz = row / 3 - 1;
+    int b = 0, cnt = 0;
+    // an axis of fewer than 3 cells has one, visited once
+    if (lane < NBR_SEGS && (ny >= 3 || dy == 0) && (nz >= 3 || dz == 0)) {
+      auto wrap = [](int x, int nc) { return x < 0 ? x + nc : (x >= nc ? x - nc : x); };
+      int lo = cx, hi = cx;
+      if (nx >= 3) { lo = cx - 1; hi = cx + 1; }
+      if (lane & 1) {
+        if (lo < 0) lo = hi = nx - 1;
+        else if (hi >= nx) lo = hi = 0;
+        else lo = 0, hi = -1;
+      } else {
+        lo = max(lo, 0);
+        hi = min(hi, nx - 1);
       }
+      if (lo <= hi) {
+        const int c = cbase + (wrap(cz + dz, nz) * ny + wrap(cy + dy, ny)) * nx;
+        b = cell_start[c + lo];
+        cnt = cell_start[c + hi + 1] - b;
+      }
+    }
+    int end = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, end, d);
+      if (lane >= d) end += y;
+    }
+    if (lane < NBR_SEGS) sh.seg[lane] = make_int2(end, b - (end - cnt));
+    total = __shfl_sync(0xffffffffu, end, 31);
+    __syncwarp();
+  }
+  // pass 1: FP32 screen of the candidates, all lanes busy and NBR_U loads under way;
+  // survivors are compacted into idx[] so that the FP64 decision below runs on full
+  // warps (this part's FP64 rate is low, and a divergent FP64 branch costs the whole
+  // warp).  A component of the FP32 difference is off by at most ~1e-5 A and the
+  // squared distance near rc^2 by ~1.3e-4 A^2, far inside the margin, so a pair
+  // rejected here is never a neighbour (where FP32 and FP64 pick different images,
+  // both distances exceed L/2 > rcut).
+  constexpr int NBR_U = 4;
+  const float rc2_screen = (float)rc2 * 1.0001f + 1e-4f;
+  constexpr float RINT = 12582912.f;  // 1.5 * 2^23: x + RINT - RINT rounds x to an integer
+  int cur = 0;
+  int2 seg = sh.seg[0];
+  for (int b = 0; b < total; b += 32 * NBR_U) {
+    float4 p[NBR_U];
+#pragma unroll
+    for (int u = 0; u < NBR_U; ++u) {
+      const int t = b + 32 * u + lane;
+      p[u].w = __int_as_float(i);  // no candidate
+      if (t < total) {
+        while (t >= seg.x) seg = sh.seg[++cur];
+        p[u] = cell_pos[t + seg.y];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NBR_U; ++u) {
+      const int j = __float_as_int(p[u].w);
+      bool pass = false;
+      if (j != i) {
+        float fx = p[u].x - fxi, fy = p[u].y - fyi, fz = p[u].z - fzi;
+        fx -= Lx * (__fmaf_rn(fx, iLx, RINT) - RINT);
+        fy -= Ly * (__fmaf_rn(fy, iLy, RINT) - RINT);
+        fz -= Lz * (__fmaf_rn(fz, iLz, RINT) - RINT);
+        pass = fx * fx + fy * fy + fz * fz < rc2_screen;
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, pass);
+      const int pos = ns + __popc(bal & ((1u << lane) - 1u));
+      if (pass && pos < NBR_CAP) sh.idx[pos] = j;
+      ns += __popc(bal);
+    }
+  }
   if (ns > NBR_CAP) {
     if (lane == 0) set_err(err, ERR_CAPACITY);
     ns = NBR_CAP;
@@ -241,92 +326,74 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
   // pass 2: the exact FP64 decision on the survivors, compacted in place
   // (a write never reaches an entry that is still to be read)
   int cnt = 0;
-  for (int base = 0; base < ns; base += 32) {
-    const int t = base + lane;
+  const unsigned long long rc2_bits = (unsigned long long)__double_as_longlong(rc2);
+  for (int b = 0; b < ns; b += 32) {
+    const int t = b + lane;
     bool hit = false;
-    double d2 = 0.0;
+    unsigned long long d2 = 0;
     int j = -1;
     if (t < ns) {
-      j = idx[t];
-      const double ddx = mic_near(__dsub_rn(coord[3 * j], xi), g.L[0]);
-      const double ddy = mic_near(__dsub_rn(coord[3 * j + 1], yi), g.L[1]);
-      const double ddz = mic_near(__dsub_rn(coord[3 * j + 2], zi), g.L[2]);
-      d2 = sqdist(ddx, ddy, ddz);
-      hit = d2 < rc2;
+      j = sh.idx[t];
+      const double ddx = mic_near(__dsub_rn(coord[3 * j], xi), g->L[0]);
+      const double ddy = mic_near(__dsub_rn(coord[3 * j + 1], yi), g->L[1]);
+      const double ddz = mic_near(__dsub_rn(coord[3 * j + 2], zi), g->L[2]);
+      d2 = (unsigned long long)__double_as_longlong(sqdist(ddx, ddy, ddz));
+      hit = d2 < rc2_bits;
     }
     const unsigned bal = __ballot_sync(0xffffffffu, hit);
     const int pos = cnt + __popc(bal & ((1u << lane) - 1u));
     if (hit) {
-      key[pos] = (unsigned long long)__double_as_longlong(d2);
-      idx[pos] = j;
+      sh.key[pos] = d2;
+      sh.idx[pos] = j;
     }
     cnt += __popc(bal);
     __syncwarp();
   }
   if (lane == 0) ncand[i] = cnt;
-  int P = 1;
-  while (P < cnt) P <<= 1;
-  for (int t = cnt + lane; t < P; t += 32) {
-    key[t] = 0x7ff0000000000000ULL;  // +inf
-    idx[t] = 0x7fffffff;
-  }
-  __syncwarp();
-  // the bitonic network, a lane per compare-exchange pair (t, t + jj): pair
-  // q has t = q with a zero bit inserted at jj
-  for (int k = 2; k <= P; k <<= 1)
-    for (int jj = k >> 1; jj > 0; jj >>= 1) {
-      for (int q = lane; q < (P >> 1); q += 32) {
-        const int t = ((q & ~(jj - 1)) << 1) | (q & (jj - 1)), o = t | jj;
-        const bool asc = (t & k) == 0;
-        const unsigned long long ka = key[t], kb = key[o];
-        const int ia = idx[t], ib = idx[o];
-        const bool sw = asc ? key_gt(ka, ia, kb, ib) : key_gt(kb, ib, ka, ia);
-        if (sw) {
-          key[t] = kb; key[o] = ka;
-          idx[t] = ib; idx[o] = ia;
-        }
-      }
-      __syncwarp();
-    }
-  const int keep = cnt < sel ? cnt : sel;
-  for (int s = lane; s < NP; s += 32) nlist[(size_t)i * NP + s] = s < keep ? idx[s] + base : -1;
-  if (lane == 0) nnei[i] = keep;
-}
-
-// Reverse list: for every kept pair (i, slot) -> j, record row i*NP+slot under j.
-__global__ void k_rev_fill(const int* __restrict__ nlist, int n, int* __restrict__ rev_cnt,
-                           int* __restrict__ rev_rows, int* __restrict__ err) {
-  pdl_wait();
-  long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= (long long)n * NP) return;
-  int j = nlist[row];
-  if (j < 0) return;
-  int pos = atomicAdd(&rev_cnt[j], 1);
-  if (pos < REV_CAP)
-    rev_rows[(size_t)j * REV_CAP + pos] = (int)row;
+  const int hi_rc2 = __double2hiint(rc2);
+  if (cnt <= 32)
+    sort_candidates<1>(sh, cnt, hi_rc2, lane);
+  else if (cnt <= 64)
+    sort_candidates<2>(sh, cnt, hi_rc2, lane);
+  else if (cnt <= 128)
+    sort_candidates<4>(sh, cnt, hi_rc2, lane);
   else
-    set_err(err, ERR_CAPACITY);
+    sort_candidates<8>(sh, cnt, hi_rc2, lane);
+  const int keep = cnt < sel ? cnt : sel;
+  for (int s = lane; s < NP; s += 32) {
+    const int j = s < keep ? sh.idx[sh.order[s]] : -1;
+    nlist[(size_t)i * NP + s] = j >= 0 ? j + base : -1;
+    if (rev_rows && j >= 0) {
+      const int pos = atomicAdd(&rev_cnt[j], 1);
+      if (pos < REV_CAP)
+        rev_rows[(size_t)j * REV_CAP + pos] = (i + base) * NP + s;
+      else
+        set_err(err, ERR_CAPACITY);
+    }
+  }
+  if (lane == 0) nnei[i] = keep;
 }
 
 void launch_neighbors(const NbrArgs& a, cudaStream_t st) {
   launch_pdl(k_cell_setup, std::min(152, (a.cell_cap + 255) / 256), 256, 0, st, a.box, a.rcut, a.cap_dim, a.grid,
-             a.err, a.cell_count, a.cell_cursor, a.cell_cap);
+             a.err, a.cell_count, a.cell_cap);
   note_launch();
   const int n_out = a.n_out > a.n ? a.n_out : a.n;
   if (n_out == 0) return;
   const int tb = 256;
   if (a.n > 0) {
     launch_pdl(k_cell_count, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of,
-                                                    a.cell_count, a.atype_c, a.coordf, a.err, nullptr, nullptr, 0);
+               a.cell_count, a.cell_rank, a.atype_c, a.rev_cnt, a.err, nullptr, nullptr, 0);
     note_launch();
     launch_pdl(k_cell_scan, 1, 1024, 0, st, a.cell_count, a.cell_start, a.grid, -1);
     note_launch();
-    launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.cell_of, a.n, a.cell_start, a.cell_cursor, a.cell_atoms);
+    launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.cell_of, a.cell_rank, a.n, a.cell_start,
+               a.cell_pos);
     note_launch();
   }
   launch_pdl(k_neighbors, (n_out + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st,
-      a.coord, a.n, n_out, a.base, a.grid, a.cell_of, a.cell_start, a.cell_atoms, a.rcut * a.rcut, a.sel, a.nlist,
-      a.nnei, a.ncand, a.atype_c, a.coordf, a.err, nullptr, nullptr, 0, a.rev_cnt);
+             a.coord, a.n, n_out, a.base, a.grid, a.cell_of, a.cell_start, a.cell_pos, a.rcut * a.rcut, a.sel, a.nlist,
+             a.nnei, a.ncand, a.atype_c, a.err, nullptr, nullptr, 0, a.rev_cnt, a.rev_rows);
   note_launch();
 }
 
@@ -334,18 +401,18 @@ void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell
                              cudaStream_t st) {
   if (a.n == 0) return;
   cudaMemsetAsync(a.cell_count, 0, sizeof(int) * (size_t)ncells_total, st);
-  cudaMemsetAsync(a.cell_cursor, 0, sizeof(int) * (size_t)ncells_total, st);
   const int tb = 256;
-  launch_pdl(k_cell_count, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of, a.cell_count,
-                                                  a.atype_c, a.coordf, a.err, frame, cell_base, cb0);
+  launch_pdl(k_cell_count, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.atype, a.n, a.ntypes, a.grid, a.cell_of,
+             a.cell_count, a.cell_rank, a.atype_c, a.rev_cnt, a.err, frame, cell_base, cb0);
   note_launch();
   launch_pdl(k_cell_scan, 1, 1024, 0, st, a.cell_count, a.cell_start, a.grid, ncells_total);
   note_launch();
-  launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.cell_of, a.n, a.cell_start, a.cell_cursor, a.cell_atoms);
+  launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.cell_of, a.cell_rank, a.n, a.cell_start,
+             a.cell_pos);
   note_launch();
   launch_pdl(k_neighbors, (a.n + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st,
-      a.coord, a.n, a.n, 0, a.grid, a.cell_of, a.cell_start, a.cell_atoms, a.rcut * a.rcut, a.sel, a.nlist, a.nnei,
-      a.ncand, a.atype_c, a.coordf, a.err, frame, cell_base, cb0, a.rev_cnt);
+             a.coord, a.n, a.n, 0, a.grid, a.cell_of, a.cell_start, a.cell_pos, a.rcut * a.rcut, a.sel, a.nlist, a.nnei,
+             a.ncand, a.atype_c, a.err, frame, cell_base, cb0, a.rev_cnt, a.rev_rows);
   note_launch();
 }
 
@@ -410,13 +477,6 @@ void launch_row_list(const int* nnei, int n, int* row_off, int* rowmap, int* seg
     note_launch();
   }
   launch_pdl(k_row_list, (n + ROWL_ATOMS - 1) / ROWL_ATOMS, ROWL_T, 0, st, nnei, n, seg, row_off, rowmap);
-  note_launch();
-}
-
-void launch_reverse(const int* nlist, int n, int* rev_cnt, int* rev_rows, int* err, cudaStream_t st) {
-  if (n == 0) return;
-  long long rows = (long long)n * NP;
-  launch_pdl(k_rev_fill, (unsigned)((rows + 255) / 256), 256, 0, st, nlist, n, rev_cnt, rev_rows, err);
   note_launch();
 }
 
