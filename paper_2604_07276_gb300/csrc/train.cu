@@ -180,9 +180,11 @@ __global__ void k_env_jvp(JvpArgs a) {
 // Activations lie in shared memory as [unit][row]; a thread owns 4 rows x 1 - 4
 // units of a layer, its value and tangent sums sharing the weight loads (3
 // 16-byte loads for 32 FMAs in the widest layer), and fixed elements of the weight
-// gradients, 2 x 4 of W2, whose sums stay in registers until the last block.  (A
-// thread per element with 4-byte loads, and a separate pass for the energy term,
-// took 409 us per 582-atom frame; this takes 168.)
+// gradients, 2 x 4 of W2, whose sums stay in registers until the last block, as do its
+// rows' parts of the bias gradients.  Shared-memory wavefronts and scattered loads bind:
+// per 582-atom frame 136 us with neighbouring units in one thread (8-way bank conflicts
+// in W2's gradient), dE/dG read once more for the skip's adjoint and the bias sums taken
+// from shared memory by a few warps; 84 us now.
 constexpr int JROWS = 64;
 constexpr int JTHREADS = 256;
 constexpr int JLD = JROWS + 4;   // row stride of a unit's rows (16-byte aligned)
@@ -200,11 +202,10 @@ struct JvpEmbedSmem {
   static constexpr int H1 = TP + JROWS, H1D = H1 + E0 * JLD, H2 = H1D + E0 * JLD, H2D = H2 + E1 * JLD;
   static constexpr int FWD_TOTAL = H2D + E1 * JLD;
   // mode 1: the transposes W2^T [E2][L1], W1^T [E1][L0], dz3 and dz3'; once those
-  // are used up, dH2, dH2', dz2, dz2' lie over them; dz1, dz1'
+  // are used up, dH2, dH2', dz2, dz2' lie over them
   static constexpr int W2T = FWD_TOTAL, W1T = W2T + E2 * L1, Z3 = W1T + E1 * L0, Z3D = Z3 + E2 * JLD;
   static constexpr int DH2 = Z3, DH2D = DH2 + E1 * JLD, DZ2 = DH2D + E1 * JLD, DZ2D = DZ2 + E1 * JLD;
-  static constexpr int DZ1 = Z3 + (2 * E2 > 4 * E1 ? 2 * E2 : 4 * E1) * JLD, DZ1D = DZ1 + E0 * JLD;
-  static constexpr int TOTAL = DZ1D + E0 * JLD;
+  static constexpr int TOTAL = Z3 + (2 * E2 > 4 * E1 ? 2 * E2 : 4 * E1) * JLD;
   static_assert(TOTAL * 4 <= 227 * 1024, "shared memory");
 };
 
@@ -218,8 +219,9 @@ __device__ __forceinline__ void jst4(float* p, const float* v) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// z[u][o] += sum_k in[k][r + u] W[k][c + o], u < 4, o < OC, and likewise zd from ind.
-template <int K, int OC, int LDW>
+// z[u][o] += sum_k in[k][r + u] W[k][unit o], u < 4, o < OC, and likewise zd from ind.
+// The units are c + o, or with HALF c, c + 1, c + HALF, c + HALF + 1.
+template <int K, int OC, int LDW, int HALF = 0>
 __device__ __forceinline__ void jtile(const float* in, const float* ind, const float* W, int r, int c, float (&z)[4][OC],
                                       float (&zd)[4][OC]) {
 #pragma unroll 4
@@ -227,7 +229,11 @@ __device__ __forceinline__ void jtile(const float* in, const float* ind, const f
     const float4 h4 = jld4(in + k * JLD + r), d4 = jld4(ind + k * JLD + r);
     const float h[4] = {h4.x, h4.y, h4.z, h4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w};
     float w[OC];
-    if constexpr (OC == 4) {
+    if constexpr (HALF > 0) {
+      const float2 x = *reinterpret_cast<const float2*>(W + k * LDW + c);
+      const float2 y = *reinterpret_cast<const float2*>(W + k * LDW + c + HALF);
+      w[0] = x.x; w[1] = x.y; w[2] = y.x; w[3] = y.y;
+    } else if constexpr (OC == 4) {
       const float4 w4 = jld4(W + k * LDW + c);
       w[0] = w4.x; w[1] = w4.y; w[2] = w4.z; w[3] = w4.w;
     } else {
@@ -245,8 +251,9 @@ __device__ __forceinline__ void jtile(const float* in, const float* ind, const f
 }
 
 // acc[i][j] += sum over the block's rows of a'[i] b[j] + a[i] b'[j] (units a0 + i,
-// b0 + j of the [unit][row] arrays).
-template <int I, int J>
+// b0 + j BS of the [unit][row] arrays; neighbouring threads take neighbouring b0, whose
+// rows are JLD apart: 16-byte loads without bank conflicts).
+template <int I, int J, int BS>
 __device__ __forceinline__ void jouter(const float* A, const float* AD, const float* B, const float* BD, int a0, int b0,
                                        float (&acc)[I][J]) {
 #pragma unroll 2
@@ -260,7 +267,7 @@ __device__ __forceinline__ void jouter(const float* A, const float* AD, const fl
     }
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-      const float4 x = jld4(B + (b0 + j) * JLD + r), y = jld4(BD + (b0 + j) * JLD + r);
+      const float4 x = jld4(B + (b0 + j * BS) * JLD + r), y = jld4(BD + (b0 + j * BS) * JLD + r);
       const float b[4] = {x.x, x.y, x.z, x.w}, bd[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
       for (int i = 0; i < I; ++i)
@@ -275,7 +282,7 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
                                                          const float* __restrict__ scales) {
   pdl_wait();
   using S = JvpEmbedSmem<E0, E1, E2>;
-  static_assert(E1 % 2 == 0 && E2 % 4 == 0, "register tiles");
+  static_assert(E1 % 2 == 0 && E1 == 2 * E0 && E2 == 2 * E1, "register tiles");
   extern __shared__ __align__(16) float sm[];
   const int tid = threadIdx.x;
   for (int t = tid; t < E0 * E1; t += JTHREADS) sm[S::W1 + (t / E1) * S::L1 + t % E1] = a.w[S::gW1 + t];
@@ -294,11 +301,12 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
     for (int t = tid; t < E0 * E1; t += JTHREADS) sm[S::W1T + (t % E1) * S::L0 + t / E1] = a.w[S::gW1 + t];
   }
   // this thread's elements of the weight gradients: N2 tasks of 2 x 4 of W2, N1 of
-  // 1 x 2 of W1 and NB of the others (W0, b0, b1, b2)
-  constexpr int T2 = (E1 / 2) * (E2 / 4), T1 = E0 * (E1 / 2), TB = 2 * E0 + E1 + E2;
+  // 1 x 2 of W1; and its rows' part of the others (NH tasks of 4 rows x 2 units of
+  // layers 2 and 3: b2, b1; N0 of 4 rows x 1 unit of layer 1: W0, b0)
+  constexpr int T2 = (E1 / 2) * (E2 / 4), T1 = E0 * (E1 / 2), TH = JQ * (E1 / 2), T0 = JQ * E0;
   constexpr int N2 = (T2 + JTHREADS - 1) / JTHREADS, N1 = (T1 + JTHREADS - 1) / JTHREADS,
-                NB = (TB + JTHREADS - 1) / JTHREADS;
-  float g2[N2][2][4] = {}, g1[N1][1][2] = {}, gb[NB] = {};
+                NH = (TH + JTHREADS - 1) / JTHREADS, N0 = (T0 + JTHREADS - 1) / JTHREADS;
+  float g2[N2][2][4] = {}, g1[N1][1][2] = {}, gb2[NH][4] = {}, gb1[NH][2] = {}, g0[N0][2] = {};
   const int* pair = reinterpret_cast<const int*>(sm + S::TP);
   const int nrows = a.row_off[a.n];
   for (int p0 = blockIdx.x * JROWS; p0 < nrows; p0 += gridDim.x * JROWS) {
@@ -345,22 +353,28 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
     }
     __syncthreads();
     // layer 3: t3 = tanh(H2 W2 + b2), t3'; mode 0: G' out; mode 1: its adjoint with
-    // g = dE/dG (1 + Gt): dz3 = g (1 - t3^2), dz3' = g' (1 - t3^2) - 2 g t3 t3'
-    for (int task = tid; task < JQ * (E2 / 4); task += JTHREADS) {
-      const int r = (task % JQ) * 4, c = (task / JQ) * 4;
+    // g = dE/dG (1 + Gt): dz3 = g (1 - t3^2), dz3' = g' (1 - t3^2) - 2 g t3 t3'.  There a
+    // thread's units are c, c + 1 and those E1 further, so that it holds skip^T(g) for
+    // its 4 rows x 2 units of dH2, the start of the sums dh
+    float dh[NH][4][2], dhd[NH][4][2];
+#pragma unroll
+    for (int k = 0; k < NH; ++k) {
+      const int task = tid + k * JTHREADS;
+      if (task >= TH) continue;
+      const int r = (task % JQ) * 4, c = (task / JQ) * (MODE == 0 ? 4 : 2);
       float z[4][4], zd[4][4] = {};
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int o = 0; o < 4; ++o) z[u][o] = sm[S::B2 + c + o];
-      jtile<E1, 4, S::L2>(sm + S::H2, sm + S::H2D, sm + S::W2, r, c, z, zd);
+        for (int o = 0; o < 4; ++o) z[u][o] = sm[S::B2 + c + (MODE == 0 || o < 2 ? o : E1 + o - 2)];
+      jtile<E1, 4, S::L2, MODE == 0 ? 0 : E1>(sm + S::H2, sm + S::H2D, sm + S::W2, r, c, z, zd);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const bool live = r + u < cnt;
         const size_t at = (size_t)(p0 + r + u) * a.m1 + c;
-        const float4 f4 = jld4(a.Gt + (size_t)pair[r + u] * E2 + c);
-        const float f[4] = {1.f + f4.x, 1.f + f4.y, 1.f + f4.z, 1.f + f4.w};
         if (MODE == 0) {
+          const float4 f4 = jld4(a.Gt + (size_t)pair[r + u] * E2 + c);
+          const float f[4] = {1.f + f4.x, 1.f + f4.y, 1.f + f4.z, 1.f + f4.w};
           float gd[4];
 #pragma unroll
           for (int o = 0; o < 4; ++o) {
@@ -370,18 +384,28 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
           }
           if (live) jst4(a.Gd + at, gd);
         } else {
-          float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f), qd4 = q4;
-          if (live) {
-            q4 = jld4(a.dG + at);
-            qd4 = jld4(a.dGd + at);
+          float q[4] = {}, qd[4] = {}, f[4];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float2 x = *reinterpret_cast<const float2*>(a.Gt + (size_t)pair[r + u] * E2 + c + h * E1);
+            f[2 * h] = 1.f + x.x; f[2 * h + 1] = 1.f + x.y;
+            if (live) {
+              const float2 y = *reinterpret_cast<const float2*>(a.dG + at + h * E1);
+              const float2 yd = *reinterpret_cast<const float2*>(a.dGd + at + h * E1);
+              q[2 * h] = y.x; q[2 * h + 1] = y.y;
+              qd[2 * h] = yd.x; qd[2 * h + 1] = yd.y;
+            }
           }
-          const float q[4] = {q4.x, q4.y, q4.z, q4.w}, qd[4] = {qd4.x, qd4.y, qd4.z, qd4.w};
+          dh[k][u][0] = dh[k][u][1] = dhd[k][u][0] = dhd[k][u][1] = 0.f;
 #pragma unroll
           for (int o = 0; o < 4; ++o) {
             const float g = q[o] * f[o], gd = fmaf(s2, qd[o], s1 * q[o]) * f[o];
             const float t = tanhf(z[u][o]), td = (1.f - t * t) * zd[u][o];
             z[u][o] = g * (1.f - t * t);
             zd[u][o] = gd * (1.f - t * t) - 2.f * g * t * td;
+            gb2[k][o] += zd[u][o];
+            dh[k][u][o & 1] += g;
+            dhd[k][u][o & 1] += gd;
           }
         }
       }
@@ -389,51 +413,27 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
 #pragma unroll
         for (int o = 0; o < 4; ++o) {
           const float v[4] = {z[0][o], z[1][o], z[2][o], z[3][o]}, vd[4] = {zd[0][o], zd[1][o], zd[2][o], zd[3][o]};
-          jst4(sm + S::Z3 + (c + o) * JLD + r, v);
-          jst4(sm + S::Z3D + (c + o) * JLD + r, vd);
+          const int cu = c + (o & 1) + (o >> 1) * E1;
+          jst4(sm + S::Z3 + cu * JLD + r, v);
+          jst4(sm + S::Z3D + cu * JLD + r, vd);
         }
       }
     }
     if (MODE == 0) continue;
     __syncthreads();
-    // dH2 = W2 dz3 + skip^T(g) and its tangent, kept in registers until W2's
+    // dH2 = skip^T(g) + W2 dz3 and its tangent, kept in registers until W2's
     // gradient has read dz3
-    constexpr int TH = JQ * (E1 / 2), NH = (TH + JTHREADS - 1) / JTHREADS;
-    float dh[NH][4][2], dhd[NH][4][2];
 #pragma unroll
     for (int k = 0; k < NH; ++k) {
       const int task = tid + k * JTHREADS;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) dh[k][u][0] = dh[k][u][1] = dhd[k][u][0] = dhd[k][u][1] = 0.f;
       if (task >= TH) continue;
       const int r = (task % JQ) * 4, b = (task / JQ) * 2;
       jtile<E2, 2, S::L1>(sm + S::Z3, sm + S::Z3D, sm + S::W2T, r, b, dh[k], dhd[k]);
-      if (E2 == E1 || E2 == 2 * E1) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (r + u >= cnt) break;
-          const float* gt = a.Gt + (size_t)pair[r + u] * E2;
-          const size_t at = (size_t)(p0 + r + u) * a.m1;
-          for (int c = b; c < E2; c += E1)
-#pragma unroll
-            for (int o = 0; o < 2; ++o) {
-              const float f = 1.f + gt[c + o], q = a.dG[at + c + o], qd = a.dGd[at + c + o];
-              dh[k][u][o] += q * f;
-              dhd[k][u][o] += fmaf(s2, qd, s1 * q) * f;
-            }
-        }
-      }
     }
 #pragma unroll
     for (int k = 0; k < N2; ++k) {
       const int task = tid + k * JTHREADS;
-      if (task < T2) jouter<2, 4>(sm + S::H2, sm + S::H2D, sm + S::Z3, sm + S::Z3D, 2 * (task / (E2 / 4)), 4 * (task % (E2 / 4)), g2[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {  // b2: sum of dz3'
-      const int t = tid + k * JTHREADS - (2 * E0 + E1);
-      if (t >= 0 && t < E2)
-        for (int r = 0; r < JROWS; ++r) gb[k] += sm[S::Z3D + t * JLD + r];
+      if (task < T2) jouter<2, 4, E2 / 4>(sm + S::H2, sm + S::H2D, sm + S::Z3, sm + S::Z3D, 2 * (task / (E2 / 4)), task % (E2 / 4), g2[k]);
     }
     __syncthreads();
     // dz2 = dH2 (1 - t2^2) with t2 = H2 - skip(h1), over dz3's place
@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
           dd[u] = dhd[k][u][o];
           e[u] = d[u] * (1.f - t * t);
           ed[u] = dd[u] * (1.f - t * t) - 2.f * d[u] * t * td;
+          gb1[k][o] += ed[u];
         }
         jst4(sm + S::DH2 + (b + o) * JLD + r, d);
         jst4(sm + S::DH2D + (b + o) * JLD + r, dd);
@@ -463,7 +464,10 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
     }
     __syncthreads();
     // dh1 = W1 dz2 + skip^T(dH2), dz1 = dh1 (1 - h1^2)
-    for (int task = tid; task < JQ * E0; task += JTHREADS) {
+#pragma unroll
+    for (int k = 0; k < N0; ++k) {
+      const int task = tid + k * JTHREADS;
+      if (task >= T0) continue;
       const int r = (task % JQ) * 4, p = task / JQ;
       float d1[4][1] = {}, d1d[4][1] = {};
       jtile<E1, 1, S::L0>(sm + S::DZ2, sm + S::DZ2D, sm + S::W1T, r, p, d1, d1d);
@@ -471,36 +475,23 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         float d = d1[u][0], dd = d1d[u][0];
-        if (E1 == E0 || E1 == 2 * E0)
-          for (int b = p; b < E1; b += E0) {
-            d += sm[S::DH2 + b * JLD + r + u];
-            dd += sm[S::DH2D + b * JLD + r + u];
-          }
+#pragma unroll
+        for (int b = p; b < E1; b += E0) {
+          d += sm[S::DH2 + b * JLD + r + u];
+          dd += sm[S::DH2D + b * JLD + r + u];
+        }
         const float h = sm[S::H1 + p * JLD + r + u], hd = sm[S::H1D + p * JLD + r + u];
         e[u] = d * (1.f - h * h);
         ed[u] = dd * (1.f - h * h) - 2.f * d * h * hd;
+        g0[k][0] += sm[S::XD + r + u] * e[u] + sm[S::X + r + u] * ed[u];
+        g0[k][1] += ed[u];
       }
-      jst4(sm + S::DZ1 + p * JLD + r, e);
-      jst4(sm + S::DZ1D + p * JLD + r, ed);
     }
     // W1's gradient (dz2) does not wait for dz1
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
       const int task = tid + k * JTHREADS;
-      if (task < T1) jouter<1, 2>(sm + S::H1, sm + S::H1D, sm + S::DZ2, sm + S::DZ2D, task / (E1 / 2), 2 * (task % (E1 / 2)), g1[k]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {  // W0, b0, b1
-      const int t = tid + k * JTHREADS;
-      if (t < E0) {
-        for (int r = 0; r < JROWS; ++r)
-          gb[k] += sm[S::XD + r] * sm[S::DZ1 + t * JLD + r] + sm[S::X + r] * sm[S::DZ1D + t * JLD + r];
-      } else if (t < 2 * E0) {
-        for (int r = 0; r < JROWS; ++r) gb[k] += sm[S::DZ1D + (t - E0) * JLD + r];
-      } else if (t < 2 * E0 + E1) {
-        for (int r = 0; r < JROWS; ++r) gb[k] += sm[S::DZ2D + (t - 2 * E0) * JLD + r];
-      }
+      if (task < T1) jouter<1, 2, E1 / 2>(sm + S::H1, sm + S::H1D, sm + S::DZ2, sm + S::DZ2D, task / (E1 / 2), task % (E1 / 2), g1[k]);
     }
   }
   if (MODE == 0) return;
@@ -512,21 +503,35 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
       for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          atomicAdd(grad + S::gW2 + (2 * (task / (E2 / 4)) + i) * E2 + 4 * (task % (E2 / 4)) + j, g2[k][i][j]);
+          atomicAdd(grad + S::gW2 + (2 * (task / (E2 / 4)) + i) * E2 + task % (E2 / 4) + j * (E2 / 4), g2[k][i][j]);
   }
 #pragma unroll
   for (int k = 0; k < N1; ++k) {
     const int task = tid + k * JTHREADS;
     if (task < T1)
 #pragma unroll
-      for (int j = 0; j < 2; ++j) atomicAdd(grad + S::gW1 + (task / (E1 / 2)) * E1 + 2 * (task % (E1 / 2)) + j, g1[k][0][j]);
+      for (int j = 0; j < 2; ++j) atomicAdd(grad + S::gW1 + (task / (E1 / 2)) * E1 + task % (E1 / 2) + j * (E1 / 2), g1[k][0][j]);
+  }
+  // the JQ threads of a unit are neighbouring lanes
+  static_assert(JQ == 16 && JTHREADS % 32 == 0, "half warps");
+  auto unit_sum = [&](float v, bool live, int at) {
+#pragma unroll
+    for (int o = JQ / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (live && tid % JQ == 0) atomicAdd(grad + at, v);
+  };
+#pragma unroll
+  for (int k = 0; k < NH; ++k) {
+    const int task = tid + k * JTHREADS, c = (task / JQ) * 2;
+#pragma unroll
+    for (int o = 0; o < 4; ++o) unit_sum(gb2[k][o], task < TH, S::gB2 + c + (o & 1) + (o >> 1) * E1);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) unit_sum(gb1[k][o], task < TH, S::gB1 + c + o);
   }
 #pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    const int t = tid + k * JTHREADS;
-    if (t < 2 * E0) atomicAdd(grad + t, gb[k]);
-    else if (t < 2 * E0 + E1) atomicAdd(grad + S::gB1 + t - 2 * E0, gb[k]);
-    else if (t < TB) atomicAdd(grad + S::gB2 + t - 2 * E0 - E1, gb[k]);
+  for (int k = 0; k < N0; ++k) {
+    const int task = tid + k * JTHREADS;
+    unit_sum(g0[k][0], task < T0, task / JQ);
+    unit_sum(g0[k][1], task < T0, E0 + task / JQ);
   }
 }
 
