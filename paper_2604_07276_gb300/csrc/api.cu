@@ -431,22 +431,18 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
   // w_out and b_out are stored multiplied by out_scale; a10, the fitting backward,
   // is seeded with dE/dH_last = out_scale * w_out
   const bool res_last = m->nfit > 1 && m->fit[m->nfit - 1] == m->fit[m->nfit - 2];
+  const FitKeep* keep = m->fit_keep;
+  float *dH = keep ? keep->dH[m->nfit - 1] : ws.dHa, *dHn = ws.dHb;
+  float *dZ = keep ? keep->dZ[m->nfit - 1] : ws.dZ, *dZn = ws.dZ2;
   launch_energy_head(ws.H[m->nfit - 1], res_last ? ws.H[m->nfit - 2] : nullptr, n, m->call_nlocal, fan, m->w_out,
-                     m->d_b_out, m->ebias, atype, ws.e, ws.dHa, ws.dZ, st);
-  const float* gs = m->grad_scale;  // non-null: add gs * dE/dtheta to the gradient
-  if (gs) {
-    launch_colsum(ws.H[m->nfit - 1], fan, m->grad + m->off_wout, fan, n, gs, (float)m->out_scale, st);
-    launch_head_bias_grad(atype, n, m->grad + m->off_ebias, m->grad + m->off_bout, gs, (float)m->out_scale, st);
-  }
-  float *dH = ws.dHa, *dHn = ws.dHb, *dZ = ws.dZ, *dZn = ws.dZ2;
+                     m->d_b_out, m->ebias, atype, ws.e, dH, dZ, st);
   for (int l = m->nfit - 1; l >= 0; --l) {
     const int out = m->fit[l];
     const int in = l > 0 ? m->fit[l - 1] : m->fit_in;
     const bool res = (l > 0 && out == in);
-    if (gs) {
-      const float* input = l > 0 ? ws.H[l - 1] : ws.X;
-      launch_wgrad(input, in, dZ, out, m->grad + m->off_fitW[l], out, in, out, n, gs, st);
-      launch_colsum(dZ, out, m->grad + m->off_fitb[l], out, n, gs, 1.0f, st);
+    if (keep && l > 0) {
+      dHn = keep->dH[l - 1];
+      dZn = keep->dZ[l - 1];
     }
     float* dst = l > 0 ? dHn : ws.dX;
     // the layer below: its dZ = dH (1 - t^2), t = H - its skip input, with the product
@@ -549,7 +545,7 @@ void run_network_bf16x(dp_model* m, int n, const int* atype, cudaStream_t st) {
   const int* nrows = ws.row_off + n;  // the live rows (device)
   // the 25-50-100 embedding net on the tensor cores (BF16 two-term splits),
   // other nets, and any net while its weight gradient is wanted, in FP32
-  const bool emb_tc = m->tcw.emb_W2_t != nullptr && !m->grad_scale;
+  const bool emb_tc = m->tcw.emb_W2_t != nullptr && !m->fit_keep;
   EmbedArgs ea{};
   ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0];
@@ -660,12 +656,13 @@ int run_device(dp_model* m, int n, int nlocal, const double* coord, const double
   return run_after_neighbors(m, n, coord, ws.grid, nullptr, nullptr, 0, energy, force, virial, atom_energy, st);
 }
 
-// The tangent, along the atom displacement field v, of the energy-weight
-// gradient of the evaluation that just ran (FP32 path, no attention layer,
-// its intermediates still in the workspace), added to grad times *scale.
+// The weight gradients of both loss terms of the evaluation that just ran (no
+// attention layer, its intermediates still in the workspace, the fitting adjoint in
+// keep): grad += s1 dE/dtheta + s2 (dE/dtheta)', ' being the tangent along the atom
+// displacement field v and s1, s2 = d_scales[1], [2].
 void run_force_tangent(dp_model* m, int n, const double* coord, const double* v, float* Rd, float* Gd, float* dGd,
-                       float* Td, float* Xd, float* dXd, const std::vector<float*>& Hd, float* const* dH,
-                       float* const* dHd, float* dZ, float* dZd, float* Zd, const float* scale, cudaStream_t st) {
+                       float* Td, float* Xd, float* dXd, const std::vector<float*>& Hd, const FitKeep& keep,
+                       float* const* dHd, float* dZd, float* Zd, cudaStream_t st) {
   Workspace& ws = m->ws;
   JvpArgs a{};
   a.row_off = ws.row_off; a.rowmap = ws.rowmap;
@@ -696,11 +693,11 @@ void run_force_tangent(dp_model* m, int n, const double* coord, const double* v,
     hin = Hd[l];
     fan = out;
   }
-  // energy head: (dE/dw_out)' = out_scale sum_i H_last,i'
-  launch_colsum(Hd[m->nfit - 1], fan, m->grad + m->off_wout, fan, n, scale, (float)m->out_scale, st);
-  // fitting adjoint and its tangent (dE/dH_last = out_scale w_out is constant)
-  launch_fill_rows(dH[0], m->w_out, n, n, fan, st);
-  cudaMemsetAsync(dHd[0], 0, sizeof(float) * (size_t)n * fan, st);
+  const float* scales = m->d_scales;
+  launch_head_grad(ws.H[m->nfit - 1], Hd[m->nfit - 1], a.atype, m->grad + m->off_wout, m->grad + m->off_bout,
+                   m->grad + m->off_ebias, fan, n, scales, (float)m->out_scale, st);
+  // tangent of the fitting adjoint (dE/dH_last = out_scale w_out is constant)
+  const float* dHdc = nullptr;
   int cur = 0;
   for (int l = m->nfit - 1; l >= 0; --l) {
     const int out = m->fit[l];
@@ -708,31 +705,20 @@ void run_force_tangent(dp_model* m, int n, const double* coord, const double* v,
     const bool res = (l > 0 && out == in);
     const float* Hprev = res ? ws.H[l - 1] : nullptr;
     const float* Hprevd = res ? Hd[l - 1] : nullptr;
-    launch_tanh_bwd_jvp(dH[cur], dHd[cur], ws.H[l], Hprev, Hd[l], Hprevd, dZ, dZd, (long long)n * out, st);
+    launch_tanh_bwd_jvp(keep.dH[l], dHdc, ws.H[l], Hprev, Hd[l], Hprevd, dZd, (long long)n * out, st);
     const float* input = l > 0 ? ws.H[l - 1] : ws.X;
     const float* inputd = l > 0 ? Hd[l - 1] : Xd;
-    launch_wgrad(inputd, in, dZ, out, m->grad + m->off_fitW[l], out, in, out, n, scale, st);
-    launch_wgrad(input, in, dZd, out, m->grad + m->off_fitW[l], out, in, out, n, scale, st);
-    launch_colsum(dZd, out, m->grad + m->off_fitb[l], out, n, scale, 1.0f, st);
-    if (l > 0) {
-      if (x16) {
-        gemm_bf16x(m, m->xw.fitT[l], dZ, out, nullptr, res ? dH[cur] : nullptr, out, dH[1 - cur], in, n,
-                   res ? EPI_RES : EPI_BIAS, st);
-        gemm_bf16x(m, m->xw.fitT[l], dZd, out, nullptr, res ? dHd[cur] : nullptr, out, dHd[1 - cur], in, n,
-                   res ? EPI_RES : EPI_BIAS, st);
-      } else {
-        gemm_f32(dZ, out, m->fitWT[l], in, nullptr, res ? dH[cur] : nullptr, out, dH[1 - cur], in, n, in, out,
-                 res ? EPI_RES : EPI_BIAS, st);
-        gemm_f32(dZd, out, m->fitWT[l], in, nullptr, res ? dHd[cur] : nullptr, out, dHd[1 - cur], in, n, in, out,
-                 res ? EPI_RES : EPI_BIAS, st);
-      }
-      cur = 1 - cur;
-    } else if (x16) {
-      gemm_bf16x(m, m->xw.fitT[l], dZd, out, nullptr, nullptr, 0, dXd, in, n, EPI_BIAS, st);
-    } else {
-      // dE/dX itself is still in the workspace from the evaluation
-      gemm_f32(dZd, out, m->fitWT[l], in, nullptr, nullptr, 0, dXd, in, n, in, out, EPI_BIAS, st);
-    }
+    launch_fit_grad(input, inputd, keep.dZ[l], dZd, m->grad + m->off_fitW[l], m->grad + m->off_fitb[l], in, out, n,
+                    scales, st);
+    // dE/dX itself is still in the workspace from the evaluation
+    float* dst = l > 0 ? dHd[cur] : dXd;
+    const float* skip = res ? dHdc : nullptr;
+    if (x16)
+      gemm_bf16x(m, m->xw.fitT[l], dZd, out, nullptr, skip, out, dst, in, n, skip ? EPI_RES : EPI_BIAS, st);
+    else
+      gemm_f32(dZd, out, m->fitWT[l], in, nullptr, skip, out, dst, in, n, in, out, skip ? EPI_RES : EPI_BIAS, st);
+    dHdc = dst;
+    cur = 1 - cur;
   }
   // descriptor adjoint's tangent -> (dE/dG)'; the embedding weights' gradients of
   // both loss terms
@@ -1536,15 +1522,15 @@ int dp_train_frame(dp_model* m, int natoms, const double* d_coord, const double*
   for (int l = 0; l < nfit; ++l) fmax = std::max(fmax, m->fit[l]);
   struct TrainBufs {
     double *energy, *virial, *force, *v;
-    float *gE, *Rd, *Gd, *dGd, *Td, *Xd, *dXd, *dH[2], *dHd[2], *dZ, *dZd, *Zd;
+    float *Rd, *Gd, *dGd, *Td, *Xd, *dXd, *dHd[2], *dZd, *Zd;
     std::vector<float*> Hd;
+    FitKeep keep;
   } b;
   auto plan = [&](Arena& a) {
     b.energy = a.take<double>(1);
     b.virial = a.take<double>(9);
     b.force = a.take<double>((size_t)cap * 3);
     b.v = a.take<double>((size_t)cap * 3);
-    b.gE = a.take<float>((size_t)m->ntheta);
     b.Rd = a.take<float>(rows * 4);
     b.Gd = a.take<float>(rows * m1);
     b.dGd = a.take<float>(rows * m1);
@@ -1553,11 +1539,13 @@ int dp_train_frame(dp_model* m, int natoms, const double* d_coord, const double*
     b.dXd = a.take<float>((size_t)cap * m->fit_in);
     b.Hd.assign(nfit, nullptr);
     for (int l = 0; l < nfit; ++l) b.Hd[l] = a.take<float>((size_t)cap * m->fit[l]);
-    for (int k = 0; k < 2; ++k) {
-      b.dH[k] = a.take<float>((size_t)cap * fmax);
-      b.dHd[k] = a.take<float>((size_t)cap * fmax);
+    b.keep.dH.assign(nfit, nullptr);
+    b.keep.dZ.assign(nfit, nullptr);
+    for (int l = 0; l < nfit; ++l) {
+      b.keep.dH[l] = a.take<float>((size_t)cap * m->fit[l]);
+      b.keep.dZ[l] = a.take<float>((size_t)cap * m->fit[l]);
     }
-    b.dZ = a.take<float>((size_t)cap * fmax);
+    for (int k = 0; k < 2; ++k) b.dHd[k] = a.take<float>((size_t)cap * fmax);
     b.dZd = a.take<float>((size_t)cap * fmax);
     b.Zd = a.take<float>((size_t)cap * fmax);
   };
@@ -1577,21 +1565,17 @@ int dp_train_frame(dp_model* m, int natoms, const double* d_coord, const double*
   real.base = reinterpret_cast<char*>(m->t_buf);
   real.cap = probe.off;
   plan(real);
-  // 1. the energy evaluation, with dE/dtheta (unscaled) into gE
-  CUDA_TRY(cudaMemsetAsync(b.gE, 0, sizeof(float) * (size_t)m->ntheta, st));
-  float* grad_keep = m->grad;
-  m->grad = b.gE;
-  m->grad_scale = m->d_scales;  // 1
+  // 1. the evaluation, its fitting adjoint kept
+  m->fit_keep = &b.keep;
   int rc = run_device(m, natoms, natoms, d_coord, d_box, d_atype, b.energy, b.force, b.virial, nullptr, st);
-  m->grad = grad_keep;
-  m->grad_scale = nullptr;
+  m->fit_keep = nullptr;
   if (rc != DP_OK) return rc;
-  // 2. loss, scales and v = F - F_ref; the energy term of the gradient
+  // 2. loss, scales and v = F - F_ref
   launch_train_prep(natoms, b.energy, e_ref, b.force, d_force_ref, pe, pf, b.v, d_loss, m->d_scales, st);
-  launch_axpy(m->grad, b.gE, m->ntheta, m->d_scales + 1, st);
-  // 3. the force term: the tangent of dE/dtheta along v, scaled by -2 pf / 3N
-  run_force_tangent(m, natoms, d_coord, b.v, b.Rd, b.Gd, b.dGd, b.Td, b.Xd, b.dXd, b.Hd, b.dH, b.dHd, b.dZ, b.dZd,
-                    b.Zd, m->d_scales + 2, st);
+  // 3. the gradient: the energy term, and the tangent of dE/dtheta along v times
+  // -2 pf / 3N
+  run_force_tangent(m, natoms, d_coord, b.v, b.Rd, b.Gd, b.dGd, b.Td, b.Xd, b.dXd, b.Hd, b.keep, b.dHd, b.dZd, b.Zd,
+                    st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DP_ERR_CUDA, std::string("dp_train_frame: launch failed: ") + cudaGetErrorString(e));
   return DP_OK;

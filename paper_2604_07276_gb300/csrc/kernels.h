@@ -195,21 +195,18 @@ void launch_energy_head(const float* H, const float* Hprev, int n, int nlocal, i
 // dZ = dH * (1 - t^2) with t = Hcur - Hprev (Hprev may be null: t = Hcur)
 void launch_tanh_bwd(const float* dH, const float* Hcur, const float* Hprev, float* dZ, long long count,
                      cudaStream_t st);
-// dst[i][:] = row for i < nlocal, 0 for nlocal <= i < n (ghost atoms seed no energy)
-void launch_fill_rows(float* dst, const float* row, int n, int nlocal, int width, cudaStream_t st);
 
 // --- training of the student (train.cu, simt.cu)
-void launch_wgrad(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int I, int O, int N,
-                  const float* scale, cudaStream_t st);
-void launch_colsum(const float* B, int ldb, float* c, int O, int N, const float* scale, float factor, cudaStream_t st);
-void launch_head_bias_grad(const int* atype, int n, float* g_ebias, float* g_bout, const float* scale, float out_scale,
-                           cudaStream_t st);
+// A fitting layer's weight and bias gradients: C[I][O] += A'^T (s2 dZ) + A^T (s2 dZ' + s1
+// dZ), c[O] += column sums of s2 dZ' + s1 dZ, with s1, s2 = scales[1], scales[2].
+void launch_fit_grad(const float* A, const float* Ad, const float* dZ, const float* dZd, float* C, float* c, int I,
+                     int O, int N, const float* scales, cudaStream_t st);
+void launch_head_grad(const float* H, const float* Hd, const int* atype, float* g_wout, float* g_bout, float* g_ebias,
+                      int O, int N, const float* scales, float out_scale, cudaStream_t st);
 // loss of one frame, the gradient scales (1, energy term, force term) and
 // the direction v = F - F_ref of the force term
 void launch_train_prep(int n, const double* energy, double e_ref, const double* force, const double* force_ref,
                        double pe, double pf, double* v, double* loss, float* scales, cudaStream_t st);
-// g[i] += *scale * src[i]
-void launch_axpy(float* g, const float* src, int n, const float* scale, cudaStream_t st);
 
 // Tangents (forward mode) of an energy evaluation of the FP32 path without
 // attention layers, along the atom displacement field v, and of its adjoint.
@@ -250,9 +247,9 @@ void launch_desc_jvp_bwd(const JvpArgs& a, cudaStream_t st);
 // H' = (1 - t^2) Z' + Hprev' with t = H - Hprev (Hprev, Hprev' null: t = H, no skip)
 void launch_tanh_jvp(const float* Zd, const float* H, const float* Hprev, const float* Hprevd, float* Hd,
                      long long count, cudaStream_t st);
-// dZ = dH (1 - t^2), dZ' = dH' (1 - t^2) - 2 dH t t' with t = H - Hprev, t' = H' - Hprev'
+// dZ' = dH' (1 - t^2) - 2 dH t t' with t = H - Hprev, t' = H' - Hprev' (dH' null: zero)
 void launch_tanh_bwd_jvp(const float* dH, const float* dHd, const float* H, const float* Hprev, const float* Hd,
-                         const float* Hprevd, float* dZ, float* dZd, long long count, cudaStream_t st);
+                         const float* Hprevd, float* dZd, long long count, cudaStream_t st);
 void launch_adam(float* theta, float* g, float* m1, float* m2, int n, float lr, float b1, float b2, float eps,
                  float bc1, float bc2, cudaStream_t st);
 void launch_transpose(const float* W, int R, int C, float* WT, cudaStream_t st);

@@ -83,6 +83,11 @@ struct TcBuffers {
   void* p[32] = {};
 };
 
+// Adjoint of the fitting net, a buffer per layer (training).
+struct FitKeep {
+  std::vector<float*> dH, dZ;
+};
+
 struct Workspace {
   int cap = 0;  // atoms
   void* mem = nullptr;
@@ -166,10 +171,12 @@ struct dp_model {
   float* adam_m = nullptr;
   float* adam_v = nullptr;
   int adam_t = 0;
-  const float* grad_scale = nullptr;  // non-null: the next evaluation adds scale * dE/dtheta to grad
+  // non-null: the next evaluation leaves every fitting layer's dE/dH and dE/dZ there,
+  // layer by layer, and runs the embedding net in FP32
+  const dpa1::FitKeep* fit_keep = nullptr;
   float* d_scales = nullptr;          // [4]: 1, energy-loss scale, force-loss scale, 0
   void* t_buf = nullptr;              // training scratch: energy, virial, forces, the direction
-                                      // v = F - F_ref, dE/dtheta, and the tangents of the evaluation
+                                      // v = F - F_ref, the fitting adjoint and the tangents of the evaluation
   int t_cap = 0;                      // atoms t_buf is laid out for
   // device weights
   float *emb_packed, *Gt, *tebd, *davg, *dstd, *ebias, *w_out;

@@ -18,70 +18,91 @@
 
 namespace dpa1 {
 
-// C[i][o] += scale * sum_n A[n][i] * B[n][o]; the n range is split over
-// grid.z slices that add their parts atomically.
-__global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ A, int lda, const float* __restrict__ B,
-                                               int ldb, float* __restrict__ C, int ldc, int I, int O, int N, int chunk,
-                                               const float* __restrict__ scale) {
+// Gradient of a fitting layer, both loss terms at once: with s1, s2 the energy and
+// force terms' scales, M = s2 dZ' + s1 dZ and D = s2 dZ,
+//   C[i][o] += sum_n A'[n][i] D[n][o] + A[n][i] M[n][o],  c[o] += sum_n M[n][o]
+// (A the layer's input, ' the tangents).  The n range is split over grid.z slices that
+// add their parts atomically.  A frame of some hundred atoms is a chain of launches and
+// load latencies, hence one launch a layer, and 32 rows of all four operands fetched at
+// once.  A launch for each of the three products and two sums of a layer took 34 us a
+// layer of a 582-atom frame (and one more to add the energy term up), this 11.
+constexpr int WG_ROWS = 32;
+__global__ void __launch_bounds__(256) k_fit_grad(const float* __restrict__ A, const float* __restrict__ Ad,
+                                                  const float* __restrict__ dZ, const float* __restrict__ dZd,
+                                                  float* __restrict__ C, float* __restrict__ c, int I, int O, int N,
+                                                  int chunk, const float* __restrict__ scales) {
   pdl_wait();
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
+  __shared__ float As[WG_ROWS][64 + 4], Ads[WG_ROWS][64 + 4], Ms[WG_ROWS][64 + 4], Ds[WG_ROWS][64 + 4];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int i0 = blockIdx.x * 64, o0 = blockIdx.y * 64;
   const int n_begin = blockIdx.z * chunk;
   const int n_end = min(N, n_begin + chunk);
-  float acc[4][4] = {};
-  for (int n0 = n_begin; n0 < n_end; n0 += 16) {
-    for (int t = threadIdx.x; t < 16 * 64; t += 256) {
-      const int k = t / 64, c = t % 64;
-      const int n = n0 + k;
-      As[k][c] = (n < n_end && i0 + c < I) ? A[(size_t)n * lda + i0 + c] : 0.f;
-      Bs[k][c] = (n < n_end && o0 + c < O) ? B[(size_t)n * ldb + o0 + c] : 0.f;
+  const float s1 = scales[1], s2 = scales[2];
+  float acc[4][4] = {}, bias = 0.f;
+  for (int n0 = n_begin; n0 < n_end; n0 += WG_ROWS) {
+#pragma unroll
+    for (int q = 0; q < WG_ROWS * 64 / 256; ++q) {
+      const int t = threadIdx.x + 256 * q, k = t / 64, j = t % 64, n = n0 + k;
+      const bool ai = n < n_end && i0 + j < I, bo = n < n_end && o0 + j < O;
+      const size_t ia = (size_t)n * I + i0 + j, ib = (size_t)n * O + o0 + j;
+      As[k][j] = ai ? A[ia] : 0.f;
+      Ads[k][j] = ai ? Ad[ia] : 0.f;
+      const float z = bo ? dZ[ib] : 0.f, zd = bo ? dZd[ib] : 0.f;
+      Ms[k][j] = fmaf(s2, zd, s1 * z);
+      Ds[k][j] = s2 * z;
     }
     __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < WG_ROWS; ++k) {
+      float a[4], ad[4], m[4], d[4];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      float a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) { a[q] = As[k][ty * 4 + q]; b[q] = Bs[k][tx * 4 + q]; }
+      for (int q = 0; q < 4; ++q) {
+        a[q] = As[k][ty * 4 + q]; ad[q] = Ads[k][ty * 4 + q];
+        m[q] = Ms[k][tx * 4 + q]; d[q] = Ds[k][tx * 4 + q];
+      }
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
+        for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(a[p], m[q], fmaf(ad[p], d[q], acc[p][q]));
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 64) {
+#pragma unroll 8
+      for (int k = 0; k < WG_ROWS; ++k) bias += Ms[k][threadIdx.x];
     }
     __syncthreads();
   }
-  const float s = *scale;
 #pragma unroll
   for (int p = 0; p < 4; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int i = i0 + ty * 4 + p, o = o0 + tx * 4 + q;
-      if (i < I && o < O) atomicAdd(&C[(size_t)i * ldc + o], s * acc[p][q]);
+      if (i < I && o < O) atomicAdd(&C[(size_t)i * O + o], acc[p][q]);
     }
+  if (blockIdx.x == 0 && threadIdx.x < 64 && o0 + (int)threadIdx.x < O) atomicAdd(&c[o0 + threadIdx.x], bias);
 }
 
-// c[o] += scale * factor * sum_n B[n][o]
-__global__ void k_colsum(const float* __restrict__ B, int ldb, float* __restrict__ c, int O, int N, int chunk,
-                         const float* __restrict__ scale, float factor) {
+// Gradient of the energy head, e_i = out_scale (H_i . w_out + b_out) + ebias[t_i]:
+// w_out[o] += out_scale sum_n s1 H[n][o] + s2 H'[n][o]; b_out and ebias, constant in
+// the forces, s1 out_scale and s1 an atom.
+__global__ void k_head_grad(const float* __restrict__ H, const float* __restrict__ Hd, const int* __restrict__ atype,
+                            float* __restrict__ g_wout, float* __restrict__ g_bout, float* __restrict__ g_ebias, int O,
+                            int N, int chunk, const float* __restrict__ scales, float out_scale) {
   pdl_wait();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= O) return;
   const int n_begin = blockIdx.y * chunk, n_end = min(N, n_begin + chunk);
-  float s = 0.f;
-  for (int n = n_begin; n < n_end; ++n) s += B[(size_t)n * ldb + o];
-  atomicAdd(&c[o], *scale * factor * s);
-}
-
-// de_i/d ebias[t_i] = 1 and de_i/d b_out = out_scale for every atom.
-__global__ void k_head_bias_grad(const int* __restrict__ atype, int n, float* __restrict__ g_ebias,
-                                 float* __restrict__ g_bout, const float* __restrict__ scale, float out_scale) {
-  pdl_wait();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float s = *scale;
-  atomicAdd(&g_ebias[atype[i]], s);
-  atomicAdd(g_bout, s * out_scale);
+  const float s1 = scales[1], s2 = scales[2];
+  if (blockIdx.x == 0) {
+    for (int n = n_begin + threadIdx.x; n < n_end; n += blockDim.x) atomicAdd(&g_ebias[atype[n]], s1);
+    if (threadIdx.x == 0 && n_end > n_begin) atomicAdd(g_bout, s1 * out_scale * (float)(n_end - n_begin));
+  }
+  if (o >= O) return;
+  float s = 0.f, sd = 0.f;
+#pragma unroll 8
+  for (int n = n_begin; n < n_end; ++n) {
+    s += H[(size_t)n * O + o];
+    sd += Hd[(size_t)n * O + o];
+  }
+  atomicAdd(&g_wout[o], out_scale * fmaf(s2, sd, s1 * s));
 }
 
 // One block: loss of the frame, the gradient scales and the direction
@@ -116,12 +137,6 @@ __global__ void k_train_prep(int n, const double* __restrict__ energy, double e_
     scales[2] = (float)(-2.0 * pf / (3.0 * nn));
     scales[3] = 0.f;
   }
-}
-
-__global__ void k_axpy(float* __restrict__ g, const float* __restrict__ src, int n, const float* __restrict__ scale) {
-  pdl_wait();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) g[i] += *scale * src[i];
 }
 
 // ------------------------------------------------------------------ tangents
@@ -634,16 +649,14 @@ __global__ void k_tanh_jvp(const float* __restrict__ Zd, const float* __restrict
 
 __global__ void k_tanh_bwd_jvp(const float* __restrict__ dH, const float* __restrict__ dHd, const float* __restrict__ H,
                                const float* __restrict__ Hprev, const float* __restrict__ Hd,
-                               const float* __restrict__ Hprevd, float* __restrict__ dZ, float* __restrict__ dZd,
-                               long long count) {
+                               const float* __restrict__ Hprevd, float* __restrict__ dZd, long long count) {
   pdl_wait();
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   const float t = Hprev ? H[k] - Hprev[k] : H[k];
   const float td = Hprevd ? Hd[k] - Hprevd[k] : Hd[k];
   const float d = dH[k];
-  dZ[k] = d * (1.f - t * t);
-  dZd[k] = dHd[k] * (1.f - t * t) - 2.f * d * t * td;
+  dZd[k] = (dHd ? dHd[k] * (1.f - t * t) : 0.f) - 2.f * d * t * td;
 }
 
 __global__ void k_adam(float* __restrict__ theta, float* __restrict__ g, float* __restrict__ m1, float* __restrict__ m2,
@@ -679,45 +692,34 @@ __global__ void k_add_rows(const float* __restrict__ rows, const float* __restri
 
 static int blocks(long long n, int t) { return (int)((n + t - 1) / t); }
 
-void launch_wgrad(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int I, int O, int N,
-                  const float* scale, cudaStream_t st) {
+void launch_fit_grad(const float* A, const float* Ad, const float* dZ, const float* dZd, float* C, float* c, int I,
+                     int O, int N, const float* scales, cudaStream_t st) {
   if (N <= 0 || I <= 0 || O <= 0) return;
   // slices of the rows: 256 rows or more each in large frames; in small ones down
-  // to 32, until the grid holds two blocks per SM (582 atoms: 2 slices -> 17, the
-  // kernel 53 -> 11 us)
+  // to 32, until the grid holds two blocks per SM (582 atoms: 2 slices -> 17, 53 -> 11 us
+  // for one product)
   const int tiles = blocks(I, 64) * blocks(O, 64);
   const int splits = std::min(64, std::max({1, N / 256, std::min(N / 32, 304 / tiles)}));
-  const int chunk = (N + splits - 1) / splits;
-  dim3 grid(blocks(I, 64), blocks(O, 64), splits);
-  launch_pdl(k_wgrad, grid, 256, 0, st, A, lda, B, ldb, C, ldc, I, O, N, chunk, scale);
+  // whole groups of WG_ROWS
+  const int chunk = blocks(blocks(N, splits), WG_ROWS) * WG_ROWS;
+  launch_pdl(k_fit_grad, dim3(blocks(I, 64), blocks(O, 64), blocks(N, chunk)), 256, 0, st, A, Ad, dZ, dZd, C, c, I, O,
+             N, chunk, scales);
   note_launch();
 }
 
-void launch_colsum(const float* B, int ldb, float* c, int O, int N, const float* scale, float factor,
-                   cudaStream_t st) {
+void launch_head_grad(const float* H, const float* Hd, const int* atype, float* g_wout, float* g_bout, float* g_ebias,
+                      int O, int N, const float* scales, float out_scale, cudaStream_t st) {
   if (N <= 0 || O <= 0) return;
   const int splits = std::min(128, std::max(1, N / 32));
   const int chunk = (N + splits - 1) / splits;
-  launch_pdl(k_colsum, dim3(blocks(O, 128), splits), 128, 0, st, B, ldb, c, O, N, chunk, scale, factor);
-  note_launch();
-}
-
-void launch_head_bias_grad(const int* atype, int n, float* g_ebias, float* g_bout, const float* scale, float out_scale,
-                           cudaStream_t st) {
-  if (n <= 0) return;
-  launch_pdl(k_head_bias_grad, blocks(n, 256), 256, 0, st, atype, n, g_ebias, g_bout, scale, out_scale);
+  launch_pdl(k_head_grad, dim3(blocks(O, 128), splits), 128, 0, st, H, Hd, atype, g_wout, g_bout, g_ebias, O, N, chunk,
+             scales, out_scale);
   note_launch();
 }
 
 void launch_train_prep(int n, const double* energy, double e_ref, const double* force, const double* force_ref,
                        double pe, double pf, double* v, double* loss, float* scales, cudaStream_t st) {
   launch_pdl(k_train_prep, 1, 1024, 0, st, n, energy, e_ref, force, force_ref, pe, pf, v, loss, scales);
-  note_launch();
-}
-
-void launch_axpy(float* g, const float* src, int n, const float* scale, cudaStream_t st) {
-  if (n <= 0) return;
-  launch_pdl(k_axpy, blocks(n, 256), 256, 0, st, g, src, n, scale);
   note_launch();
 }
 
@@ -781,9 +783,9 @@ void launch_tanh_jvp(const float* Zd, const float* H, const float* Hprev, const 
 }
 
 void launch_tanh_bwd_jvp(const float* dH, const float* dHd, const float* H, const float* Hprev, const float* Hd,
-                         const float* Hprevd, float* dZ, float* dZd, long long count, cudaStream_t st) {
+                         const float* Hprevd, float* dZd, long long count, cudaStream_t st) {
   if (count <= 0) return;
-  launch_pdl(k_tanh_bwd_jvp, (unsigned)((count + 255) / 256), 256, 0, st, dH, dHd, H, Hprev, Hd, Hprevd, dZ, dZd, count);
+  launch_pdl(k_tanh_bwd_jvp, (unsigned)((count + 255) / 256), 256, 0, st, dH, dHd, H, Hprev, Hd, Hprevd, dZd, count);
   note_launch();
 }
 
