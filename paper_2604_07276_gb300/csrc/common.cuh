@@ -127,6 +127,19 @@ __device__ __forceinline__ double mic_near(double d, double L) {
   return (__double2hiint(d) & 0x7fffffff) < __double2hiint(L) - 0x100000 ? d : mic(d, L);
 }
 
+// For the FP64 environment kernels, whose blocks of 2 NP threads hold the rows of two
+// atoms: rec[4 a + c] = 1 / dstd[t_a][c], rec[8] = 1 / (rc - rcs).  An FP64 division is
+// some twenty instructions at a 64th of the FP32 rate, and with one a row for each of
+// these the divisions bound the kernels: rows of the FP32 path, 3,001 atoms, 64 -> 45 us
+// and 86 -> 63 (adjoint), tangents of 582 atoms 21 -> 15.
+__device__ __forceinline__ void env_reciprocals(double* rec, const float* dstd, const int* atype, int n, double rcs,
+                                                double rc) {
+  const int t = threadIdx.x, i = 2 * blockIdx.x + (t >> 2);
+  if (t < 8 && i < n) rec[t] = 1.0 / (double)dstd[4 * atype[i] + (t & 3)];
+  if (t == 8) rec[8] = 1.0 / (rc - rcs);
+  __syncthreads();
+}
+
 // Sorts 32 R unsigned values over a warp in ascending order: a bitonic network in
 // registers, lane l ending up with places R l to R l + R - 1.  Strides below R need
 // no exchange, the others one shuffle per value; in shared memory each of the

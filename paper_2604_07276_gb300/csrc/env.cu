@@ -16,6 +16,8 @@ namespace dpa1 {
 template <typename Real>
 __global__ void k_env(EnvArgs a) {
   pdl_wait();
+  __shared__ double rec[sizeof(Real) == 8 ? 9 : 1];
+  if constexpr (sizeof(Real) == 8) env_reciprocals(rec, a.dstd, a.atype, a.n, a.rcs, a.rc);
   long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long long)a.n * NP) return;
   const int i = (int)(row / NP);
@@ -36,7 +38,9 @@ __global__ void k_env(EnvArgs a) {
     if (d < rcs) {
       sw = 1;
     } else if (d < rc) {
-      const Real u = (d - rcs) / (rc - rcs);
+      Real u;
+      if constexpr (sizeof(Real) == 8) u = (d - rcs) * rec[8];
+      else u = (d - rcs) / (rc - rcs);
       sw = u * u * u * ((Real)-6 * u * u + (Real)15 * u - (Real)10) + (Real)1;
     } else {
       sw = 0;
@@ -47,8 +51,13 @@ __global__ void k_env(EnvArgs a) {
     const int t = a.atype[i];
     const float* av = a.davg + 4 * t;
     const float* sv = a.dstd + 4 * t;
-    R = make_float4((float)((s - (Real)av[0]) / (Real)sv[0]), (float)((s * hx - (Real)av[1]) / (Real)sv[1]),
-                    (float)((s * hy - (Real)av[2]) / (Real)sv[2]), (float)((s * hz - (Real)av[3]) / (Real)sv[3]));
+    if constexpr (sizeof(Real) == 8) {
+      const double* iv = rec + 4 * (i & 1);
+      R = make_float4((float)((s - av[0]) * iv[0]), (float)((s * hx - av[1]) * iv[1]), (float)((s * hy - av[2]) * iv[2]),
+                      (float)((s * hz - av[3]) * iv[3]));
+    } else {
+      R = make_float4((s - av[0]) / sv[0], (s * hx - av[1]) / sv[1], (s * hy - av[2]) / sv[2], (s * hz - av[3]) / sv[3]);
+    }
     rw = make_float4((float)hx, (float)hy, (float)hz, (float)sw);
     rv = make_float4((float)dx, (float)dy, (float)dz, (float)d);
     w64 = sw;
@@ -64,9 +73,9 @@ void launch_env(const EnvArgs& a, cudaStream_t st) {
   long long rows = (long long)a.n * NP;
   if (rows == 0) return;
   if (a.fp64)
-    launch_pdl(k_env<double>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
+    launch_pdl(k_env<double>, (unsigned)((rows + 2 * NP - 1) / (2 * NP)), 2 * NP, 0, st, a);
   else
-    launch_pdl(k_env<float>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
+    launch_pdl(k_env<float>, (unsigned)((rows + 2 * NP - 1) / (2 * NP)), 2 * NP, 0, st, a);
   note_launch();
 }
 
@@ -77,6 +86,8 @@ void launch_env(const EnvArgs& a, cudaStream_t st) {
 template <typename Real>
 __global__ void k_env_bwd(EnvBwdArgs a) {
   pdl_wait();
+  __shared__ double rec[sizeof(Real) == 8 ? 9 : 1];
+  if constexpr (sizeof(Real) == 8) env_reciprocals(rec, a.dstd, a.atype, a.n, a.rcs, a.rc);
   long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= (long long)a.n * NP) return;
   float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -105,9 +116,13 @@ __global__ void k_env_bwd(EnvBwdArgs a) {
       sw = 1; dsw = 0;
     } else if (d < rc) {
       const Real wdt = rc - rcs;
-      const Real u = (d - rcs) / wdt;
+      Real u;
+      if constexpr (sizeof(Real) == 8) u = (d - rcs) * rec[8];
+      else u = (d - rcs) / wdt;
       sw = u * u * u * (Real(-6) * u * u + Real(15) * u - Real(10)) + Real(1);
-      dsw = Real(-30) * u * u * (u - Real(1)) * (u - Real(1)) / wdt;
+      dsw = Real(-30) * u * u * (u - Real(1)) * (u - Real(1));
+      if constexpr (sizeof(Real) == 8) dsw *= rec[8];
+      else dsw /= wdt;
     } else {
       sw = 0; dsw = 0;
     }
@@ -115,7 +130,13 @@ __global__ void k_env_bwd(EnvBwdArgs a) {
     const Real q = sw * inv * inv;                // s / d
     const Real dq = dsw * inv * inv - Real(2) * sw * inv * inv * inv;
     const float* sv = a.dstd + 4 * t;
-    const Real r0 = (Real)dR.x / sv[0], r1 = (Real)dR.y / sv[1], r2 = (Real)dR.z / sv[2], r3 = (Real)dR.w / sv[3];
+    Real r0, r1, r2, r3;
+    if constexpr (sizeof(Real) == 8) {
+      const double* iv = rec + 4 * (i & 1);
+      r0 = dR.x * iv[0]; r1 = dR.y * iv[1]; r2 = dR.z * iv[2]; r3 = dR.w * iv[3];
+    } else {
+      r0 = dR.x / sv[0]; r1 = dR.y / sv[1]; r2 = dR.z / sv[2]; r3 = dR.w / sv[3];
+    }
     const Real vdotr = r1 * rx + r2 * ry + r3 * rz;
     const Real radial = r0 * ds + dq * vdotr + (Real)dg.w * dsw;  // coefficient of rhat
     const Real hdot = (Real)dg.x * hx + (Real)dg.y * hy + (Real)dg.z * hz;
@@ -130,9 +151,9 @@ void launch_env_bwd(const EnvBwdArgs& a, cudaStream_t st) {
   long long rows = (long long)a.n * NP;
   if (rows == 0) return;
   if (a.fp64)
-    launch_pdl(k_env_bwd<double>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
+    launch_pdl(k_env_bwd<double>, (unsigned)((rows + 2 * NP - 1) / (2 * NP)), 2 * NP, 0, st, a);
   else
-    launch_pdl(k_env_bwd<float>, (unsigned)((rows + 255) / 256), 256, 0, st, a);
+    launch_pdl(k_env_bwd<float>, (unsigned)((rows + 2 * NP - 1) / (2 * NP)), 2 * NP, 0, st, a);
   note_launch();
 }
 

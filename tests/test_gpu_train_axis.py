@@ -1,0 +1,43 @@
+"""The training gradient over descriptor axis widths (the tangent kernels spread the
+axis columns' sums over the block: one column, an odd number, as many as the embedding
+is wide), against the oracle's double backward (FP32 sums: 1e-5 relative, as for the
+student)."""
+
+import dataclasses
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import OracleModel
+from oracle.student import loss_and_grad
+
+from gpu_helpers import weight_file
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("embed,axis", [((16, 32, 64), 1), ((16, 32, 64), 64), ((25, 50, 100), 7), ((32, 64, 128), 40)])
+def test_axis(embed, axis):
+    import torch
+
+    import paper_2604_07276_gb300 as p
+
+    cfg = dataclasses.replace(synth.STUDENT_CONFIG, embed=embed, axis=axis, fitting=(32, 32))
+    w = synth.make_weights(cfg, seed=10, bias_scale=0.1, stats=True)
+    coord, atype, box = synth.lattice_system(70, seed=7, density=0.03)
+    n = len(atype)
+    f_ref = np.random.default_rng(3).normal(size=(n, 3))
+    L, _, _, g = loss_and_grad(OracleModel.from_numpy(cfg, w), coord, box, atype, 0.5, f_ref)
+    m = p.DPA1(weight_file(cfg, w, f"trainaxis_{embed[0]}_{axis}"), precision="fp32")
+    m.reserve(n)
+    m.debug_poison()
+    dev = lambda a, t: torch.tensor(np.asarray(a), dtype=t, device="cuda")
+    loss = torch.zeros(3, dtype=torch.float64, device="cuda")
+    m.zero_grad()
+    m.train_frame(dev(coord, torch.float64), dev(p.box9(box), torch.float64), dev(atype, torch.int32), 0.5,
+                  dev(f_ref, torch.float64), loss)
+    got = m.get_grad()
+    assert np.linalg.norm(got - g) <= 1e-5 * np.linalg.norm(g)
+    assert abs(float(loss[0]) - L) <= 1e-5 * abs(L)
+    m.close()
