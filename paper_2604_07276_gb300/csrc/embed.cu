@@ -7,10 +7,11 @@
 // in its registers (and, where an index runs, in its own shared-memory column),
 // the weights are read from shared memory as 16-byte broadcasts.  The products
 // run on pairs of outputs (fma.rn.f32x2: two FP32 FMAs, each rounded as fmaf):
-// the bound is the issue of FMAs, weight loads and tanhf (E0 + E1 + E2 per row
-// and direction), so 6 instructions for 8 FMAs instead of 10 count.  Two rows
-// per thread, which halve the weight loads, measured no gain.  Every product
-// sums in the order of a plain loop over its inputs.
+// the bound is shared memory's data path (two wavefronts for 16 bytes to every lane,
+// 80 - 87 % busy), then the issue of FMAs and tanhf (E0 + E1 + E2 per row and
+// direction).  Two rows per thread, which halve the weight loads, leave 12 warps on an
+// SM: 272 us against 283 forward, the adjoint spills.  Every product sums in the order
+// of a plain loop over its inputs.
 #include <algorithm>
 
 #include "common.cuh"
@@ -47,7 +48,7 @@ struct RowNet {
   static constexpr int Q1 = (E1 + 3) / 4 * 4, Q0 = (E0 + 3) / 4 * 4;
   static constexpr int W2T = FWD, W1T = W2T + P2 * Q1, BWD = W1T + E1 * Q0;
   // CTAs per SM that registers and shared memory (228 KB) allow
-  static constexpr int F_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 3 : 2), B_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 2 : 1);
+  static constexpr int F_CTAS = E1 <= 32 ? 4 : (E1 <= 50 ? 3 : 2), B_CTAS = E1 <= 32 ? 3 : (E1 <= 50 ? 2 : 1);
   static_assert(F_CTAS * (FWD * 4 + 1024) <= 228 * 1024 && B_CTAS * (BWD * 4 + 1024) <= 228 * 1024, "shared memory");
 };
 
@@ -76,36 +77,38 @@ __device__ __forceinline__ void row_weights(float* sm, const float* __restrict__
   __syncthreads();
 }
 
-// z[u] = bias[c + u] + sum_k in[k] W[k][c + u], u < 8 (W with row stride LD;
-// in[k] as the pair (in[k], in[k]))
+// z[u] = bias[c + u] + sum_k in[k] W[k][c + u], u < 8 (W with row stride LD).  The
+// pair (in[k], in[k]) is made here: held as pairs the inputs take twice the registers,
+// and the adjoint spilled (16-32-64, 1.36 M rows: 578 -> 508 us).
 template <int K, int LD>
-__device__ __forceinline__ void row_block(const f2* in, const float* W, const float* bias, int c, float* z) {
+__device__ __forceinline__ void row_block(const float* in, const float* W, const float* bias, int c, float* z) {
   const ulonglong2 b0 = f2_ld4(bias + c), b1 = f2_ld4(bias + c + 4);
   f2 acc[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const ulonglong2 w0 = f2_ld4(W + k * LD + c), w1 = f2_ld4(W + k * LD + c + 4);
-    f2_fma(acc[0], in[k], w0.x);
-    f2_fma(acc[1], in[k], w0.y);
-    f2_fma(acc[2], in[k], w1.x);
-    f2_fma(acc[3], in[k], w1.y);
+    const f2 h = f2_pack(in[k], in[k]);
+    f2_fma(acc[0], h, w0.x);
+    f2_fma(acc[1], h, w0.y);
+    f2_fma(acc[2], h, w1.x);
+    f2_fma(acc[3], h, w1.y);
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) f2_unpack(acc[q], z[2 * q], z[2 * q + 1]);
 }
 
 // Layers 1 and 2 of this thread's row: its shared columns H1 and H2 and the
-// layer-2 units in h2 (each as a pair of itself).
+// layer-2 units in h2.
 template <int E0, int E1, int E2>
-__device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, f2* h2) {
+__device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, float* h2) {
   using N = RowNet<E0, E1, E2>;
   float* c1 = sm + N::H1 + threadIdx.x;
   float* c2 = sm + N::H2 + threadIdx.x;
-  f2 h1[E0];
+  float h1[E0];
 #pragma unroll
   for (int p = 0; p < E0; ++p) {
     const float h = tanhf(fmaf(x, sm[N::W0 + p], b0t ? b0t[p] : sm[N::B0 + p]));
-    h1[p] = f2_pack(h, h);
+    h1[p] = h;
     c1[p * ER_T] = h;
   }
 #pragma unroll 1
@@ -120,10 +123,7 @@ __device__ __forceinline__ void row_front(float* sm, float x, const float* b0t, 
       }
   }
 #pragma unroll
-  for (int b = 0; b < E1; ++b) {
-    const float h = c2[b * ER_T];
-    h2[b] = f2_pack(h, h);
-  }
+  for (int b = 0; b < E1; ++b) h2[b] = c2[b * ER_T];
 }
 
 // Where a list row's data lie: row rg = atom * NP + slot of the per-row
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::F_CTAS) k_embed_rows
   for (int p0 = blockIdx.x * ER_T; p0 < nrows; p0 += gridDim.x * ER_T) {
     const RowPos r(a, p0 + threadIdx.x, nrows);
     const size_t pair = (size_t)r.ti * a.ntypes + r.tj;
-    f2 h2[E1];
+    float h2[E1];
     row_front<E0, E1, E2>(sm, r.rg >= 0 ? a.R[(size_t)r.rg * 4] : 0.f, a.b0t ? a.b0t + pair * E0 : nullptr, h2);
     const float4* gt4 = reinterpret_cast<const float4*>(a.Gt + pair * E2);
     const float* c2 = sm + N::H2 + threadIdx.x;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(ER_T, RowNet<E0, E1, E2>::B_CTAS) k_embed_rows
     const RowPos r(a, p0 + threadIdx.x, nrows);
     const bool live = r.rg >= 0;
     const size_t pair = (size_t)r.ti * a.ntypes + r.tj;
-    f2 h2[E1];
+    float h2[E1];
     row_front<E0, E1, E2>(sm, live ? a.R[(size_t)r.rg * 4] : 0.f, a.b0t ? a.b0t + pair * E0 : nullptr, h2);
     const float4* gt4 = reinterpret_cast<const float4*>(a.Gt + pair * E2);
     // dH2[b] = sum_c W2[b][c] dZ3[c], dZ3 = g (1 - t3^2), g = dG0 (1 + Gt)
