@@ -76,3 +76,20 @@ def test_cells(box, outside):
     if outside:
         coord = coord + rng.integers(-2, 3, (n, 3)) * box
     _check(coord, box)
+
+
+@pytest.mark.parametrize("n", [1, 2, 1023, 1025, 2047, 2048, 2049])
+def test_atom_counts(n):
+    """Around the largest box whose cells one block sorts."""
+    rng = np.random.default_rng(n)
+    box = np.array([14.0, 19.0, 13.5]) * max(1.0, n / 280.0) ** (1 / 3)
+    _check(rng.random((n, 3)) * box, box)
+
+
+@pytest.mark.parametrize("edge", [96.5, 97.5, 195.0])
+def test_many_cells(edge):
+    """Few atoms in 4,096 cells and more."""
+    rng = np.random.default_rng(int(edge))
+    coord = rng.random((300, 3)) * edge
+    coord[150:] = coord[:150] + rng.normal(size=(150, 3)) * 2.5
+    _check(coord, np.array([edge, edge, edge]))
