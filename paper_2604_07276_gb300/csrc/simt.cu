@@ -938,12 +938,20 @@ __global__ void __launch_bounds__(128, CQ ? 10 : 6) k_desc_fwd(DescArgs a) {
   __syncthreads();
   for (int t = threadIdx.x; t < 4 * a.m1; t += blockDim.x) a.T[(size_t)atom * 4 * a.m1 + t] = Ts[t];
   float* x = a.X + (size_t)atom * a.fit_in;
+  // D, element p * axis + b: (p, b) advance without a division
+  const int dp = blockDim.x / a.axis, db = blockDim.x % a.axis;
+  int p = threadIdx.x / a.axis, b = threadIdx.x % a.axis;
   for (int idx = threadIdx.x; idx < a.m1 * a.axis; idx += blockDim.x) {
-    const int p = idx / a.axis, b = idx % a.axis;
     float d = 0.f;
 #pragma unroll
     for (int c = 0; c < 4; ++c) d = fmaf(Ts[c * a.m1 + p], Ts[c * a.m1 + b], d);
     x[idx] = d;
+    p += dp;
+    b += db;
+    if (b >= a.axis) {
+      b -= a.axis;
+      ++p;
+    }
   }
   const int ti = a.atype[atom];
   for (int t = threadIdx.x; t < a.tebd_dim; t += blockDim.x) x[a.m1 * a.axis + t] = a.tebd[ti * a.tebd_dim + t];
@@ -965,21 +973,42 @@ __global__ void __launch_bounds__(128, 10) k_desc_bwd(DescArgs a) {
   const size_t base = (size_t)atom * NP;
   const float inv_sel = 1.0f / (float)a.sel;
   for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) Ts[t] = a.T[(size_t)atom * 4 * m1 + t];
-  for (int t = threadIdx.x; t < m1 * ax; t += blockDim.x) {
-    const float v = a.dX[(size_t)atom * a.fit_in + t];
-    dD[t] = v;
-    dDt[(t % ax) * m1 + t / ax] = v;
+  {
+    const float* dX = a.dX + (size_t)atom * a.fit_in;
+    const int dp = blockDim.x / ax, db = blockDim.x % ax;
+    int p = threadIdx.x / ax, b = threadIdx.x % ax;
+#pragma unroll 4
+    for (int t = threadIdx.x; t < m1 * ax; t += blockDim.x) {
+      const float v = dX[t];
+      dD[t] = v;
+      dDt[b * m1 + p] = v;
+      p += dp;
+      b += db;
+      if (b >= ax) {
+        b -= ax;
+        ++p;
+      }
+    }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) {
-    const int c = t / m1, p = t % m1;
-    float v = 0.f;
-    for (int b = 0; b < ax; ++b) v = fmaf(dDt[b * m1 + p], Ts[c * m1 + b], v);
-    if (p < ax) {
-#pragma unroll 8
-      for (int q = 0; q < m1; ++q) v = fmaf(dD[q * ax + p], Ts[c * m1 + q], v);
+  for (int p = threadIdx.x; p < m1; p += blockDim.x) {
+    float v[4] = {};
+    for (int b = 0; b < ax; ++b) {
+      const float d = dDt[b * m1 + p];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = fmaf(d, Ts[c * m1 + b], v[c]);
     }
-    dTs[t] = v * inv_sel;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) dTs[c * m1 + p] = p < ax ? v[c] : v[c] * inv_sel;
+  }
+  __syncthreads();
+  // the axis columns' other term: all four rows of T at once, in as few warps
+  for (int t = threadIdx.x; t < 4 * ax; t += blockDim.x) {
+    const int c = t / ax, p = t % ax;
+    float v = dTs[c * m1 + p];
+#pragma unroll 8
+    for (int q = 0; q < m1; ++q) v = fmaf(dD[q * ax + p], Ts[c * m1 + q], v);
+    dTs[c * m1 + p] = v * inv_sel;
   }
   __syncthreads();
   if constexpr (CQ) {
@@ -1020,7 +1049,7 @@ __global__ void __launch_bounds__(128, 10) k_desc_bwd(DescArgs a) {
   // rows of dT stay in registers: dG = R dT, dR = G dT^T.  Two rows at a time, so
   // that their loads and reductions overlap (four spill at 10 blocks per SM).
   // 15,668 atoms in bf16x: 651 us with a thread per dG element and a second pass
-  // over G for dR, 332 now.
+  // over G for dR, 332 so, 311 without the integer divisions of the first part.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int q4 = m1 / 4;
   const size_t gbase = a.row_off[atom];

@@ -9,10 +9,10 @@ import numpy as np
 import pytest
 
 import synth
-from oracle import OracleModel
+from oracle import OracleModel, energy_force_virial
 from oracle.student import loss_and_grad
 
-from gpu_helpers import weight_file
+from gpu_helpers import BF16_ATOM_ENERGY, BF16_FORCE_RMSE, force_rmse, weight_file
 
 pytestmark = pytest.mark.gpu
 
@@ -41,3 +41,22 @@ def test_axis(embed, axis):
     assert np.linalg.norm(got - g) <= 1e-5 * np.linalg.norm(g)
     assert abs(float(loss[0]) - L) <= 1e-5 * abs(L)
     m.close()
+
+
+@pytest.mark.parametrize("axis", [1, 7, 48, 64])
+def test_axis_interleaved(axis):
+    """The descriptor and its adjoint on the column-quad layout (fp16x), forces and
+    atomic energies against the FP64 oracle."""
+    import paper_2604_07276_gb300 as p
+
+    cfg = dataclasses.replace(synth.STUDENT_CONFIG, axis=axis, fitting=(32, 32))
+    w = synth.make_weights(cfg, seed=11, bias_scale=0.1, stats=True)
+    coord, atype, box = synth.lattice_system(70, seed=8, density=0.03)
+    _, re, rF, _ = energy_force_virial(OracleModel.from_numpy(cfg, w), coord, box, atype)
+    m = p.DPA1(weight_file(cfg, w, f"axis_{axis}"), precision="fp16x")
+    m.reserve(len(atype))
+    m.debug_poison()
+    _, F, _, e = m.compute(coord, box, atype, atom_energy=True)
+    m.close()
+    assert force_rmse(F, rF) <= BF16_FORCE_RMSE
+    assert np.abs(e - re).max() <= BF16_ATOM_ENERGY
