@@ -394,8 +394,9 @@ __global__ void k_batch_unpack(const double* __restrict__ forceP, const int* __r
 
 namespace dpa1 {
 // Stages a7-a11 shared by both precisions: descriptor, fitting forward and
-// backward, descriptor backward (dE/dG of the last layer and dE/dR).
-void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t st) {
+// backward, descriptor backward (dE/dG of the last layer and dE/dR; with fold only its
+// dT, into dG's place: the embedding's adjoint does the rest).
+void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t st, bool fold) {
   Workspace& ws = m->ws;
   const int L = m->nattn, m1 = m->m1;
   // a7: descriptor
@@ -470,7 +471,10 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
   }
   prof_mark(m, "fitting", st);
   // a11: descriptor backward -> dG (w.r.t. G_L) and dR
-  launch_desc_bwd(da, st);
+  if (fold)
+    launch_desc_dt(da, st);
+  else
+    launch_desc_bwd(da, st);
   prof_mark(m, "desc_bwd", st);
 }
 

@@ -133,7 +133,10 @@ struct EmbedArgs {
   float* G0;         // forward out: row p of the list at p * m1 (packed), or column-quad
                      // interleaved in its atom's block
   const float* dG0;  // backward in, laid out as G0
-  float* dR;         // backward only: dR[:,0] +=
+  float* dR;         // backward only: dR[:,0] += (with dT: dR written)
+  // backward, instead of dG0: the descriptor's dT [n][4][m1] (launch_desc_dt), no layer
+  // between the net and the descriptor
+  const float* dT = nullptr;
   const int* rowmap = nullptr;  // the list of live rows (atom * NP + slot) and its length (device)
   const int* nrows = nullptr;
   int packed = 0;
@@ -185,6 +188,8 @@ struct DescArgs {
 };
 void launch_desc_fwd(const DescArgs& a, cudaStream_t st);
 void launch_desc_bwd(const DescArgs& a, cudaStream_t st);
+// The first part of the adjoint alone, dT [n][4][m1], into dG's place.
+void launch_desc_dt(const DescArgs& a, cudaStream_t st);
 
 // e_i = w_out . H_i + b_out + ebias[t_i], and the seed of the adjoint: dH_i = w_out
 // (0 from atom nlocal on: ghosts seed no energy) and dZ_i = dH_i (1 - t^2) with t = H - Hprev

@@ -249,5 +249,5 @@ int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, 
                 int ldr, float* C, int ldc, int M, int epi, const float* Hc, const float* Hp, float* Z,
                 cudaStream_t st);
 // stages a7-a11 (descriptor, fitting forward / backward, descriptor backward)
-void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t st);
+void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t st, bool fold = false);
 }  // namespace dpa1

@@ -959,18 +959,13 @@ __global__ void __launch_bounds__(128, CQ ? 10 : 6) k_desc_fwd(DescArgs a) {
 
 // dT[c][p] = sum_b<axis dD[p][b] T[c][b] + (p < axis) sum_q dD[q][p] T[c][q];
 // dG_s = R_s dT / sel; dR_s = G_s dT^T / sel.
-template <bool CQ>
-__global__ void __launch_bounds__(128, 10) k_desc_bwd(DescArgs a) {
-  pdl_wait();
-  extern __shared__ float sm[];
+// The adjoint's first part, a block per atom: dT [4][m1] in shared memory.
+__device__ __forceinline__ float* desc_dt(const DescArgs& a, float* sm, int atom) {
   const int m1 = a.m1, ax = a.axis;
   float* Ts = sm;              // [4][m1]
   float* dTs = Ts + 4 * m1;    // [4][m1]
   float* dD = dTs + 4 * m1;    // [m1][axis]
   float* dDt = dD + m1 * ax;   // [axis][m1]: dD transposed, so that threads with consecutive p read consecutive words
-  const int atom = blockIdx.x;
-  const int nn = a.nnei[atom];
-  const size_t base = (size_t)atom * NP;
   const float inv_sel = 1.0f / (float)a.sel;
   for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) Ts[t] = a.T[(size_t)atom * 4 * m1 + t];
   {
@@ -1011,6 +1006,26 @@ __global__ void __launch_bounds__(128, 10) k_desc_bwd(DescArgs a) {
     dTs[c * m1 + p] = v * inv_sel;
   }
   __syncthreads();
+  return dTs;
+}
+
+__global__ void __launch_bounds__(128, 10) k_desc_dt(DescArgs a) {
+  pdl_wait();
+  extern __shared__ float sm[];
+  const int atom = blockIdx.x, m1 = a.m1;
+  const float* dTs = desc_dt(a, sm, atom);
+  for (int t = threadIdx.x; t < 4 * m1; t += blockDim.x) a.dG[(size_t)atom * 4 * m1 + t] = dTs[t];
+}
+
+template <bool CQ>
+__global__ void __launch_bounds__(128, 10) k_desc_bwd(DescArgs a) {
+  pdl_wait();
+  extern __shared__ float sm[];
+  const int m1 = a.m1;
+  const int atom = blockIdx.x;
+  const int nn = a.nnei[atom];
+  const size_t base = (size_t)atom * NP;
+  const float* dTs = desc_dt(a, sm, atom);
   if constexpr (CQ) {
     // A thread per row: its dG row in column quads (consecutive threads ->
     // consecutive rows; live rows only: the fused layer kernels and the
@@ -1112,6 +1127,11 @@ void launch_desc_bwd(const DescArgs& a, cudaStream_t st) {
   if (a.n == 0) return;
   size_t sm = sizeof(float) * (8 * a.m1 + 2 * a.m1 * a.axis);
   launch_pdl(a.cq ? k_desc_bwd<true> : k_desc_bwd<false>, a.n, 128, sm, st, a);
+  note_launch();
+}
+void launch_desc_dt(const DescArgs& a, cudaStream_t st) {
+  if (a.n == 0) return;
+  launch_pdl(k_desc_dt, a.n, 128, sizeof(float) * (8 * a.m1 + 2 * a.m1 * a.axis), st, a);
   note_launch();
 }
 

@@ -929,6 +929,9 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
   ea.rowmap = ws.rowmap;
   ea.nrows = ws.row_off + n;
   const bool emb_tc = m->tcw.emb_W1_t != nullptr;
+  // without attention layers the SIMT net's adjoint takes the descriptor's in
+  const bool fold = !emb_tc && L == 0;
+  if (fold) ea.dT = ws.dG;
   if (emb_tc)
     tc_embed(m, n, atype, false, st);
   else
@@ -942,7 +945,7 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
     note_launch();
     prof_mark(m, "attn_fwd_tc", st);
   }
-  run_descriptor_fitting(m, n, atype, st);
+  run_descriptor_fitting(m, n, atype, st, fold);
   for (int l = L - 1; l >= 0 && n > 0; --l) {
     if (f16)
       launch_pdl(k_layer_bwd_tc<true>, grid, NT, B_SMEM, st, largs(l));
