@@ -699,7 +699,7 @@ void run_force_tangent(dp_model* m, int n, const double* coord, const double* v,
   }
   const float* scales = m->d_scales;
   launch_head_grad(ws.H[m->nfit - 1], Hd[m->nfit - 1], a.atype, m->grad + m->off_wout, m->grad + m->off_bout,
-                   m->grad + m->off_ebias, fan, n, scales, (float)m->out_scale, st);
+                   m->grad + m->off_ebias, fan, n, m->nt, scales, (float)m->out_scale, st);
   // tangent of the fitting adjoint (dE/dH_last = out_scale w_out is constant)
   const float* dHdc = nullptr;
   int cur = 0;

@@ -207,7 +207,7 @@ void launch_tanh_bwd(const float* dH, const float* Hcur, const float* Hprev, flo
 void launch_fit_grad(const float* A, const float* Ad, const float* dZ, const float* dZd, float* C, float* c, int I,
                      int O, int N, const float* scales, cudaStream_t st);
 void launch_head_grad(const float* H, const float* Hd, const int* atype, float* g_wout, float* g_bout, float* g_ebias,
-                      int O, int N, const float* scales, float out_scale, cudaStream_t st);
+                      int O, int N, int ntypes, const float* scales, float out_scale, cudaStream_t st);
 // loss of one frame, the gradient scales (1, energy term, force term) and
 // the direction v = F - F_ref of the force term
 void launch_train_prep(int n, const double* energy, double e_ref, const double* force, const double* force_ref,

@@ -82,19 +82,34 @@ __global__ void __launch_bounds__(256) k_fit_grad(const float* __restrict__ A, c
 }
 
 // Gradient of the energy head, e_i = out_scale (H_i . w_out + b_out) + ebias[t_i]:
-// w_out[o] += out_scale sum_n s1 H[n][o] + s2 H'[n][o]; b_out and ebias, constant in
-// the forces, s1 out_scale and s1 an atom.
+// w_out[o] += out_scale sum_n s1 H[n][o] + s2 H'[n][o], over grid.y - 2 slices of the
+// rows; the biases, constant in the forces, are two blocks of their own: ebias[t] += s1
+// times the type's atoms (counted, so exact), b_out += s1 times out_scale added up atom
+// by atom in FP32.
 __global__ void k_head_grad(const float* __restrict__ H, const float* __restrict__ Hd, const int* __restrict__ atype,
                             float* __restrict__ g_wout, float* __restrict__ g_bout, float* __restrict__ g_ebias, int O,
-                            int N, int chunk, const float* __restrict__ scales, float out_scale) {
+                            int N, int ntypes, int chunk, const float* __restrict__ scales, float out_scale) {
   pdl_wait();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n_begin = blockIdx.y * chunk, n_end = min(N, n_begin + chunk);
   const float s1 = scales[1], s2 = scales[2];
-  if (blockIdx.x == 0) {
-    for (int n = n_begin + threadIdx.x; n < n_end; n += blockDim.x) atomicAdd(&g_ebias[atype[n]], s1);
-    if (threadIdx.x == 0 && n_end > n_begin) atomicAdd(g_bout, s1 * out_scale * (float)(n_end - n_begin));
+  if (blockIdx.y >= gridDim.y - 2) {
+    if (blockIdx.x > 0) return;
+    if (blockIdx.y == gridDim.y - 1) {
+      for (int t = 0; t < ntypes; ++t) {
+        int count = 0;
+        for (int n = threadIdx.x; n - (int)threadIdx.x < N; n += blockDim.x)
+          count += __syncthreads_count(n < N && atype[n] == t);
+        if (threadIdx.x == 0) g_ebias[t] += s1 * (float)count;
+      }
+    } else if (threadIdx.x == 0) {
+      float b = 0.f;
+#pragma unroll 8
+      for (int n = 0; n < N; ++n) b += out_scale;
+      *g_bout += s1 * b;
+    }
+    return;
   }
+  const int n_begin = blockIdx.y * chunk, n_end = min(N, n_begin + chunk);
   if (o >= O) return;
   float s = 0.f, sd = 0.f;
 #pragma unroll 8
@@ -757,12 +772,12 @@ void launch_fit_grad(const float* A, const float* Ad, const float* dZ, const flo
 }
 
 void launch_head_grad(const float* H, const float* Hd, const int* atype, float* g_wout, float* g_bout, float* g_ebias,
-                      int O, int N, const float* scales, float out_scale, cudaStream_t st) {
+                      int O, int N, int ntypes, const float* scales, float out_scale, cudaStream_t st) {
   if (N <= 0 || O <= 0) return;
   const int splits = std::min(128, std::max(1, N / 32));
   const int chunk = (N + splits - 1) / splits;
-  launch_pdl(k_head_grad, dim3(blocks(O, 128), splits), 128, 0, st, H, Hd, atype, g_wout, g_bout, g_ebias, O, N, chunk,
-             scales, out_scale);
+  launch_pdl(k_head_grad, dim3(blocks(O, 128), splits + 2), 128, 0, st, H, Hd, atype, g_wout, g_bout, g_ebias, O, N,
+             ntypes, chunk, scales, out_scale);
   note_launch();
 }
 

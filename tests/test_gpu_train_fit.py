@@ -43,3 +43,30 @@ def test_fitting_gradient(fitting, natoms):
     assert np.linalg.norm(got - 2 * g) <= 1e-5 * np.linalg.norm(2 * g)
     assert abs(float(loss[0]) - L) <= 1e-5 * abs(L)
     m.close()
+
+
+def test_bias_gradients():
+    """The energy biases' own gradients (small against the others): every type's and
+    b_out's within 1e-5 of the oracle's."""
+    import torch
+
+    import paper_2604_07276_gb300 as p
+
+    cfg = synth.STUDENT_CONFIG
+    w = synth.make_weights(cfg, seed=9, bias_scale=0.1, stats=True)
+    coord, atype, box = synth.lattice_system(1100, seed=6, density=0.05)
+    n = len(atype)
+    f_ref = np.zeros((n, 3))
+    _, _, _, g = loss_and_grad(OracleModel.from_numpy(cfg, w), coord, box, atype, 5e3, f_ref)
+    m = p.DPA1(weight_file(cfg, w, "trainbias"), precision="fp32")
+    m.reserve(n)
+    dev = lambda a, t: torch.tensor(np.asarray(a), dtype=t, device="cuda")
+    loss = torch.zeros(3, dtype=torch.float64, device="cuda")
+    m.zero_grad()
+    m.train_frame(dev(coord, torch.float64), dev(p.box9(box), torch.float64), dev(atype, torch.int32), 5e3,
+                  dev(f_ref, torch.float64), loss)
+    got = m.get_grad()
+    m.close()
+    k = 1 + cfg.ntypes  # b_out, then a bias per type
+    assert np.abs(g[-k:]).min() > 0
+    assert (np.abs(got[-k:] - g[-k:]) <= 1e-5 * np.abs(g[-k:])).all()
