@@ -24,19 +24,24 @@ from .binding import DPA1, box_gradient as _box_gradient_device
 
 def box_gradient(coord: torch.Tensor, box: torch.Tensor, force: torch.Tensor, virial: torch.Tensor) -> torch.Tensor:
     """dE/dh [9] (row-major, h = box.view(3, 3)) from the coordinates the
-    call was given, its forces and its virial (all float64).
-
-    CUDA tensors that need no derivative of the result go through the library
-    (two launches instead of about ten); anything else through PyTorch."""
-    ts = (coord, box, force, virial)
-    if all(t.is_cuda and t.dtype == torch.float64 and t.is_contiguous() and t.device == coord.device for t in ts) and \
-            not (torch.is_grad_enabled() and any(t.requires_grad for t in ts)) and \
-            coord.dim() == 2 and coord.shape[1] == 3 and force.shape == coord.shape and box.numel() == 9 and \
-            virial.numel() == 9:
-        return _box_gradient_device(coord, box, force, virial)
+    call was given, its forces and its virial (all float64).  PyTorch operations, on
+    any device: differentiable in both modes, and open to ``torch.func`` and tracing."""
     h = box.reshape(3, 3).to(torch.float64)
     xf = coord.to(torch.float64).transpose(0, 1) @ force.to(torch.float64)
     return torch.linalg.solve(h.transpose(0, 1), xf - virial.reshape(3, 3).to(torch.float64)).reshape(9)
+
+
+def _saved_box_gradient(coord, box, force, virial):
+    """The same of tensors saved by a forward pass, which carry no derivative and no
+    transform (the forward pass has neither a forward-mode rule nor a vmap rule): by the
+    library's two kernels, if a saved-tensor hook has not changed what they are."""
+    ts = (coord, box, force, virial)
+    if all(type(t) is torch.Tensor and not t.requires_grad and t.is_cuda and t.dtype == torch.float64 and
+           t.is_contiguous() and t.device == coord.device for t in ts) and \
+            coord.dim() == 2 and coord.shape[1] == 3 and force.shape == coord.shape and box.numel() == 9 and \
+            virial.numel() == 9:
+        return _box_gradient_device(coord, box, force, virial)
+    return box_gradient(coord, box, force, virial)
 
 
 class DPA1Energy(torch.autograd.Function):
@@ -59,7 +64,7 @@ class DPA1Energy(torch.autograd.Function):
         g_coord = (-grad_e * force).to(grad_e.dtype)
         g_box = None
         if ctx.needs_input_grad[2]:
-            g_box = (grad_e * box_gradient(c, b, force, virial)).to(ctx.box_dtype)
+            g_box = (grad_e * _saved_box_gradient(c, b, force, virial)).to(ctx.box_dtype)
         return g_coord, None, g_box, None
 
 
