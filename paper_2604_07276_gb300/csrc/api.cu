@@ -208,8 +208,8 @@ std::vector<float> transpose_f(const std::vector<double>& v, int rows, int cols)
   return t;
 }
 
-// Transposed fitting weights and the output layer scaled by out_scale, from
-// the parameter vector.
+// Everything derived from the parameter vector: transposed fitting weights, the output
+// layer scaled by out_scale, the tensor-core images.
 void refresh_derived(dp_model* m, cudaStream_t st) {
   int fan = m->fit_in;
   for (int l = 0; l < m->nfit; ++l) {
@@ -221,7 +221,9 @@ void refresh_derived(dp_model* m, cudaStream_t st) {
   // concat mode: the first-layer bias per type pair follows em_b0 (entries E0 .. 2 E0 of the vector)
   if (m->concat && m->b0t_type)
     launch_add_rows(m->b0t_type, m->theta + m->emb[0], m->nt * m->nt, m->emb[0], m->b0t, st);
-  fit_tc_refresh(m, st);  // tensor-core weight images of the 16-bit paths, if built
+  // tensor-core weight images, if built
+  tc_embed_refresh(m, st);
+  fit_tc_refresh(m, st);
   if (m->xw.ready) bf16x_refresh(m, st);
 }
 

@@ -14,7 +14,8 @@ namespace dpa1 {
 // waits until the preceding kernel of the stream has finished and its writes are
 // visible.  A kernel launched with launch_pdl calls it, in every thread that goes
 // on, before it reads or writes anything that another kernel of the stream writes
-// or reads (before it: barriers, TMEM, weights fixed at dp_init).  192 atoms: 484
+// or reads (before it: barriers, TMEM, weights, which are written by ordinary launches
+// ahead of the evaluation's first kernel only).  192 atoms: 484
 // -> 426 us, 16 training frames of 582 atoms 14.3 -> 12.5 ms, 15,668 atoms 6.82 ->
 // 6.75 ms.  An explicit early trigger (griddepcontrol.launch_dependents after the
 // wait) made the waiting blocks compete with the running kernel: 15.6 ms for those

@@ -53,9 +53,6 @@ struct TcWeights {
     float beta[128] = {};
   };
   std::vector<Vectors> vectors;  // per attention layer, host copies passed as kernel parameters
-  struct EmbVectors {
-    float W0[32] = {}, b0[32] = {}, b1[64] = {}, b2[128] = {};
-  } emb_vec;  // the tensor-core embedding net's 1 -> E0 layer and biases
 };
 
 // BF16 two-term-split image of one GEMM operand B [K][N] (bf16x.cu).
@@ -223,6 +220,7 @@ using HostArrays = std::vector<std::pair<std::string, std::vector<double>>>;
 int tc_init_weights(dp_model* m, const HostArrays& arrays, std::string& msg);
 // tensor-core embedding net, tc_embed.cu
 int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg);
+void tc_embed_refresh(dp_model* m, cudaStream_t st);
 void tc_embed(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st);
 void tc_plan_buffers(dp_model* m, Arena& a, int cap);
 void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st);

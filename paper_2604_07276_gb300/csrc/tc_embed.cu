@@ -39,6 +39,10 @@ constexpr int EMB_TA = 128 * 64 * 2;    // activation tile: 128 rows x 64 cols
 constexpr int EMB_TD = 128 * 128 * 2;   // dZ3 tile: 128 rows x 128 cols
 constexpr int EMB_MAXT = 8;             // atom types (their type-pair table stays in L1)
 constexpr int EMB_THREADS = 256;
+// The first layer's weights and the later biases in shared memory (floats): W0 [32],
+// b1 [64], b2 [128], the first E0 / E1 / E2 of each used.  (With b0 as well, two CTAs of
+// the 32-64-128 net no longer fit on an SM.)
+constexpr int V_W0 = 0, V_B1 = 32, V_B2 = 96, EMB_VEC = 224;
 static_assert(2 * EMB_TD == 4 * EMB_TA, "the dZ3 hi / lo tiles fill the activation tiles");
 
 template <int E0_, int E1_, int E2_>
@@ -49,10 +53,10 @@ struct EmbShape {
   static constexpr int T1 = 64 * 64 * 2;               // W1 tile: 64 (E1 padded) rows x 64 cols
   static constexpr int T2 = E2P * 64 * 2;              // W2 tile: E2P rows x 64 cols
   static constexpr int WIMG = 2 * T1 + 2 * T2;         // W1 hi, W1 lo, W2 hi, W2 lo
-  static constexpr int F_SMEM = WIMG + 4 * EMB_TA + 64;
-  // the adjoint's dZ3 tiles reuse the four activation tiles; 512 bytes for one
-  // partial dE/dx per row
-  static constexpr int B_SMEM = WIMG + 4 * EMB_TA + 512 + 64;
+  static constexpr int VEC = WIMG + 4 * EMB_TA;        // the net's vectors
+  static constexpr int SMEM = VEC + EMB_VEC * 4 + 64;
+  // the trained vector: W0 b0 W1 b1 W2 b2
+  static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2;
   static constexpr int SPLIT = (E1 / 2) & ~7;          // first layer-2 unit of half 1 (24 / 32)
   static constexpr int G2 = (E1 + 7) / 8;              // 8-column groups of layer 2
   static constexpr int G3 = (E2 + 7) / 8;              // 8-column groups of layer 3
@@ -60,7 +64,7 @@ struct EmbShape {
   static constexpr int NK3 = E2P / 16;                 // 16-column chunks of Z3
   static constexpr int TM_H1 = 64 + E2P;               // TMEM columns of the layer-1 exchange (32)
   // CTAs per SM the shared memory allows (228 KB per SM, 1 KB of it reserved per CTA)
-  static constexpr int MIN_CTAS = 2 * ((F_SMEM > B_SMEM ? F_SMEM : B_SMEM) + 1024) <= 228 * 1024 ? 2 : 1;
+  static constexpr int MIN_CTAS = 2 * (SMEM + 1024) <= 228 * 1024 ? 2 : 1;
   static_assert(TM_H1 + 32 <= 256, "TMEM columns");
 };
 using EmbS100 = EmbShape<25, 50, 100>;
@@ -69,14 +73,13 @@ using EmbS128 = EmbShape<32, 64, 128>;
 struct EmbedTcArgs {
   const float* R;
   const int* nlist;
-  const int* nnei;
   const int* atype;
   const float* Gt;        // [ntypes][ntypes][E2]
   float* G0;              // fwd out, column-quad interleaved per atom (rm: packed rows [rows][E2])
   const float* dG0;       // bwd in, same layout as G0
   float* dR;              // bwd: dR[:,0] +=
   const float* b0t;       // concat type-embedding mode: first-layer bias per (centre,
-                          // neighbour) type [ntypes][ntypes][E0]; null: b0 below
+                          // neighbour) type [ntypes][ntypes][E0]; null: the net's b0
   float* H12;             // [tile][E0 + E1 units][128 rows]: layers 1 and 2 of the net,
                           // written by the forward, read by the adjoint
   const uint4* wimg;      // W1/W2 hi/lo tiles (FP16 or BF16, as the kernel's operands)
@@ -84,8 +87,8 @@ struct EmbedTcArgs {
   int rm;                 // G0 and dG0 packed rows (the modular layer layout) instead of interleaved
   const int* rowmap;      // the live rows (atom * NP + slot) in tile order
   const int* nrows;       // their number (device)
+  const float* w;         // the net's weights W0 b0 W1 b1 W2 b2 (its vectors are read from here)
   int* err;
-  float W0[32], b0[32], b1[64], b2[128];  // the net's first layer and biases (first E0 / E1 / E2 used)
 };
 
 // Thread layout (256 threads): warp w owns TMEM lane quadrant w % 4 (rows
@@ -140,6 +143,7 @@ __device__ __forceinline__ void embed_tc_front(const EmbedTcArgs& a, uint8_t* sm
   uint8_t* sH1l = sH1h + EMB_TA;
   uint8_t* sH2h = sH1l + EMB_TA;
   uint8_t* sH2l = sH2h + EMB_TA;
+  const float* vec = reinterpret_cast<const float*>(sm + S::VEC);
   const bool issuer = threadIdx.x == 0;
   // layer 1: half 0 evaluates units 0-15, half 1 units 16 .. E0 - 1; each
   // stores the hi and lo parts of its 8-column groups of H1 (K = E0, read as
@@ -147,7 +151,7 @@ __device__ __forceinline__ void embed_tc_front(const EmbedTcArgs& a, uint8_t* sm
   // both kernels), where the other half reads them after the hand-off
   constexpr int p0 = H == 0 ? 0 : 16, np = H == 0 ? 16 : S::E0 - 16;
 #pragma unroll
-  for (int p = p0; p < p0 + np; ++p) h1[p] = rv ? tanhf(fmaf(x, a.W0[p], b0row ? b0row[p] : a.b0[p])) : 0.f;
+  for (int p = p0; p < p0 + np; ++p) h1[p] = rv ? tanhf(fmaf(x, vec[V_W0 + p], b0row[p])) : 0.f;
   {
     float v[16];
 #pragma unroll
@@ -184,7 +188,7 @@ __device__ __forceinline__ void embed_tc_front(const EmbedTcArgs& a, uint8_t* sm
       for (int i = 0; i < 8; ++i) {
         const int b = 8 * g + i;
         float hb = 0.f;
-        if (b < S::E1 && rv) hb = h1[b % S::E0] + tanhf(z[8 * gg + i] + a.b1[b]);
+        if (b < S::E1 && rv) hb = h1[b % S::E0] + tanhf(z[8 * gg + i] + vec[V_B1 + b]);
         if (O::owns_b(b)) h2[b - O::b0] = hb;
         v[i] = hb;
       }
@@ -241,12 +245,17 @@ __device__ __forceinline__ void embed_bwd_front(const EmbedTcArgs& a, uint8_t* s
 }
 
 template <class S>
-__device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm, uint64_t*& bar, uint32_t*& s_tmem,
-                                               int smem_bytes) {
-  bar = reinterpret_cast<uint64_t*>(sm + smem_bytes - 64);
+__device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm, uint64_t*& bar, uint32_t*& s_tmem) {
+  bar = reinterpret_cast<uint64_t*>(sm + S::SMEM - 64);
   s_tmem = reinterpret_cast<uint32_t*>(bar + 1);
   uint4* d = reinterpret_cast<uint4*>(sm);
   for (int i = threadIdx.x; i < S::WIMG / 16; i += blockDim.x) d[i] = a.wimg[i];
+  float* vec = reinterpret_cast<float*>(sm + S::VEC);
+  for (int i = threadIdx.x; i < S::E2; i += blockDim.x) {
+    if (i < S::E0) vec[V_W0 + i] = a.w[i];
+    if (i < S::E1) vec[V_B1 + i] = a.w[S::gB1 + i];
+    vec[V_B2 + i] = a.w[S::gB2 + i];
+  }
   // activation tiles start at zero: columns never written later are read
   // only against zero weight rows, which needs finite values there
   for (int i = threadIdx.x; i < 4 * EMB_TA / 16; i += blockDim.x) d[S::WIMG / 16 + i] = make_uint4(0u, 0u, 0u, 0u);
@@ -260,8 +269,8 @@ __device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm
 
 // Layer 3 forward of the owned outputs: G0[c] = (h2[c % E1] + tanh(z3 + b2)) (1 + Gt[t_i][t_j][c]).
 template <class S, int H>
-__device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, uint32_t taddr, const float* gt, const float* h2,
-                                              bool rv, float* out_blk, int slot) {
+__device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, const float* b2, uint32_t taddr, const float* gt,
+                                              const float* h2, bool rv, float* out_blk, int slot) {
   using O = EmbOwn<S, H>;
 #pragma unroll
   for (int k = 0; k < S::NK3; ++k) {
@@ -277,8 +286,8 @@ __device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, uint32_t tad
       if (!O::owns_c(c)) continue;  // pairs never straddle an ownership boundary (SPLIT, E1, E1 + SPLIT even)
       const float2 g2 = *reinterpret_cast<const float2*>(gt + c);
       float2 o;
-      o.x = rv ? (h2[c % S::E1 - O::b0] + tanhf(z[i] + a.b2[c])) * (1.f + g2.x) : 0.f;
-      o.y = rv ? (h2[(c + 1) % S::E1 - O::b0] + tanhf(z[i + 1] + a.b2[c + 1])) * (1.f + g2.y) : 0.f;
+      o.x = rv ? (h2[c % S::E1 - O::b0] + tanhf(z[i] + b2[c])) * (1.f + g2.x) : 0.f;
+      o.y = rv ? (h2[(c + 1) % S::E1 - O::b0] + tanhf(z[i + 1] + b2[c + 1])) * (1.f + g2.y) : 0.f;
       if (rv) __stcs(reinterpret_cast<float2*>(out_blk + (a.rm ? (size_t)slot * S::E2 + c : cq_off(slot, c))), o);
     }
   }
@@ -334,7 +343,7 @@ __device__ __forceinline__ void embed_bwd_prefetch16(const float4* dg, bool rm, 
 // before it waits for Z3; chunk k + 1 is brought into L1 while chunk k is
 // processed.
 template <class S, bool F16, int H>
-__device__ __forceinline__ void embed_bwd_dz3(const EmbedTcArgs& a, uint32_t taddr, const float* gt, const float4* dg,
+__device__ __forceinline__ void embed_bwd_dz3(const EmbedTcArgs& a, const float* b2, uint32_t taddr, const float* gt, const float4* dg,
                                               bool rv, int row, int slot, uint8_t* sDZ3h, uint8_t* sDZ3l, float* dh2,
                                               float4* dcur) {
   using O = EmbOwn<S, H>;
@@ -370,7 +379,7 @@ __device__ __forceinline__ void embed_bwd_dz3(const EmbedTcArgs& a, uint32_t tad
           if (O::owns_c(c)) dh2[c % S::E1 - O::b0] += gq[t];
           float d = 0.f;
           if (store && c < S::E2 && rv) {
-            const float th = tanhf(z[8 * gg + 4 * q + t] + a.b2[c]);
+            const float th = tanhf(z[8 * gg + 4 * q + t] + b2[c]);
             d = gq[t] * (1.f - th * th);
           }
           dz[4 * q + t] = d;
@@ -428,6 +437,7 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
                                                const float4* dg, int slot, float* xch, Pre pre) {
   using O = EmbOwn<S, H>;
   const bool issuer = threadIdx.x == 0;
+  const float* vec = reinterpret_cast<const float*>(sm + S::VEC);
   uint8_t* sW1h = sm;
   uint8_t* sW1l = sW1h + S::T1;
   uint8_t* sW2h = sW1l + S::T1;
@@ -448,7 +458,7 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
   float dh2[O::nb];
 #pragma unroll
   for (int b = 0; b < O::nb; ++b) dh2[b] = 0.f;
-  embed_bwd_dz3<S, F16, H>(a, tm + lane_off, gt, dg, rv, row, slot, sDZ3h, sDZ3l, dh2, d0);
+  embed_bwd_dz3<S, F16, H>(a, vec + V_B2, tm + lane_off, gt, dg, rv, row, slot, sDZ3h, sDZ3l, dh2, d0);
   handoff();
   // dH2 (product part) = dZ3 W2^T -> TMEM [0, 64)
   if (issuer)
@@ -470,7 +480,7 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
   float dx = 0.f;
   if (rv) {
 #pragma unroll
-    for (int p = 0; p < S::E0; ++p) dx = fmaf(a.W0[p] * (1.f - h1[p] * h1[p]), dh1[p] + (H == 0 ? v[p] : 0.f), dx);
+    for (int p = 0; p < S::E0; ++p) dx = fmaf(vec[V_W0 + p] * (1.f - h1[p] * h1[p]), dh1[p] + (H == 0 ? v[p] : 0.f), dx);
   }
   // half 1 hands its part to half 0, which owns the row's dR update
   if (H == 1) xch[row] = dx;
@@ -531,7 +541,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
   }
   uint64_t* bar;
   uint32_t* s_tmem;
-  embed_tc_setup<S>(a, sm, bar, s_tmem, S::F_SMEM);
+  embed_tc_setup<S>(a, sm, bar, s_tmem);
   pdl_wait();
   const uint32_t tm = *s_tmem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
@@ -550,7 +560,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
     const bool rv = cur.rg >= 0;
     in.map(a, nrows, tile + gridDim.x, row);
     auto rows_next = [&] { in.rows(a, true); };
-    const float* b0row = a.b0t && rv ? a.b0t + ((size_t)cur.ti * a.ntypes + cur.tj) * S::E0 : nullptr;
+    const float* b0row = a.b0t ? a.b0t + ((size_t)cur.ti * a.ntypes + cur.tj) * S::E0 : a.w + S::gB0;
     if (half == 0)
       embed_tc_front<S, F16, 0>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
     else
@@ -571,10 +581,11 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
     }
     float* out = a.G0 + (size_t)(a.rm ? tile : cur.atom) * NP * S::E2;
     const int slot = a.rm ? row : cur.slot;
+    const float* b2 = reinterpret_cast<const float*>(sm + S::VEC) + V_B2;
     if (half == 0)
-      embed_fwd_out<S, 0>(a, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
+      embed_fwd_out<S, 0>(a, b2, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
     else
-      embed_fwd_out<S, 1>(a, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
+      embed_fwd_out<S, 1>(a, b2, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
     in.type(a);
     fence_before_sync();
     __syncthreads();
@@ -594,13 +605,15 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(
   }
   uint64_t* bar;
   uint32_t* s_tmem;
-  embed_tc_setup<S>(a, sm, bar, s_tmem, S::B_SMEM);
+  embed_tc_setup<S>(a, sm, bar, s_tmem);
   pdl_wait();
   const uint32_t tm = *s_tmem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
   const int row = quad * 32 + lane;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-  float* xch = reinterpret_cast<float*>(sm + S::WIMG + 4 * EMB_TA);  // [128] half 1's dE/dx
+  // [128] half 1's dE/dx, over the dZ2 tile once its product is done (rows that the
+  // next tile's dZ3 writes in full)
+  float* xch = reinterpret_cast<float*>(sm + S::WIMG);
   Sync sy{bar, 0u, a.err};
   const int nrows = *a.nrows;
   const int ntiles = (nrows + 127) / 128;
@@ -678,12 +691,35 @@ std::vector<uint8_t> emb_image(const std::vector<double>& W1, const std::vector<
   return img;
 }
 
+// The same from the trained vector w, element by element of W1, then W2 (the images'
+// padding stays as it was).
+template <class S, bool F16>
+__global__ void k_emb_image(const float* __restrict__ w, uint8_t* __restrict__ img) {
+  constexpr int N1 = S::E0 * S::E1, N2 = S::E1 * S::E2;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= N1 + N2) return;
+  const bool first = t < N1;
+  const float x = first ? w[S::gW1 + t] : w[S::gW2 + t - N1];
+  const int k = first ? t / S::E1 : (t - N1) / S::E2, n = first ? t % S::E1 : (t - N1) % S::E2;
+  uint8_t* hi = img + (first ? 0 : 2 * S::T1) + sw128_offset(n, k, first ? 64 : S::E2P);
+  *reinterpret_cast<uint16_t*>(hi) = (uint16_t)pack16<F16>(x, 0.f);
+  *reinterpret_cast<uint16_t*>(hi + (first ? S::T1 : S::T2)) = (uint16_t)pack16<F16>(x - round16<F16>(x), 0.f);
+}
+
+template <class S>
+void emb_refresh(dp_model* m, cudaStream_t st) {
+  const int blocks = (S::E0 * S::E1 + S::E1 * S::E2 + 255) / 256;
+  k_emb_image<S, true><<<blocks, 256, 0, st>>>(m->emb_packed, reinterpret_cast<uint8_t*>(m->tcw.emb_W1_t));
+  k_emb_image<S, false><<<blocks, 256, 0, st>>>(m->emb_packed, reinterpret_cast<uint8_t*>(m->tcw.emb_W2_t));
+  note_launch(2);
+}
+
 template <class S>
 void emb_set_smem() {
-  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
-  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
-  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
-  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
+  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
+  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
+  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
 }
 
 template <class S>
@@ -694,8 +730,8 @@ bool emb_is(const dp_model* m) {
 
 // Weight images of the tensor-core embedding net (the 25-50-100 and
 // 32-64-128 nets with at most EMB_MAXT types): the hi and lo parts of W1 and
-// W2 in FP16 (the fused 16-bit paths) and in BF16 (the bf16x mode), and its
-// per-unit vectors.  Other nets keep both images null (FP32 SIMT kernels).
+// W2 in FP16 (the fused 16-bit paths) and in BF16 (the bf16x mode).  Other nets
+// keep both images null (FP32 SIMT kernels).
 int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg) {
   auto get = [&](const std::string& name) -> const std::vector<double>& {
     for (auto& kv : arrays)
@@ -721,13 +757,6 @@ int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg) {
     w.allocations.push_back(d);
     (f16 ? w.emb_W1_t : w.emb_W2_t) = d;
   }
-  const std::vector<double>& W0 = get("em_W0");
-  const std::vector<double>& b0 = get("em_b0");
-  const std::vector<double>& b1 = get("em_b1");
-  const std::vector<double>& b2 = get("em_b2");
-  for (int q = 0; q < m->emb[0]; ++q) { w.emb_vec.W0[q] = (float)W0[q]; w.emb_vec.b0[q] = (float)b0[q]; }
-  for (int q = 0; q < m->emb[1]; ++q) w.emb_vec.b1[q] = (float)b1[q];
-  for (int q = 0; q < m->emb[2]; ++q) w.emb_vec.b2[q] = (float)b2[q];
   if (s100)
     emb_set_smem<EmbS100>();
   else
@@ -735,13 +764,22 @@ int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg) {
   return DP_OK;
 }
 
+// The images of changed weights (dp_set_params, dp_adam_step).
+void tc_embed_refresh(dp_model* m, cudaStream_t st) {
+  if (!m->tcw.emb_W1_t) return;
+  if (emb_is<EmbS100>(m))
+    emb_refresh<EmbS100>(m, st);
+  else
+    emb_refresh<EmbS128>(m, st);
+}
+
 namespace {
 // One launch of the tensor-core embedding net, forward or adjoint, with FP16
 // (the fused 16-bit paths) or BF16 (bf16x) operand splits.
 template <class S, bool F16>
 void tc_embed_launch_s(int grid, const EmbedTcArgs& et, bool bwd, cudaStream_t st) {
-  if (!bwd) launch_pdl(k_embed_tc_fwd_live<S, F16>, grid, EMB_THREADS, S::F_SMEM, st, et);
-  if (bwd) launch_pdl(k_embed_tc_bwd_live<S, F16>, grid, EMB_THREADS, S::B_SMEM, st, et);
+  if (!bwd) launch_pdl(k_embed_tc_fwd_live<S, F16>, grid, EMB_THREADS, S::SMEM, st, et);
+  if (bwd) launch_pdl(k_embed_tc_bwd_live<S, F16>, grid, EMB_THREADS, S::SMEM, st, et);
 }
 
 }  // namespace
@@ -754,12 +792,9 @@ void tc_embed(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st) {
   Workspace& ws = m->ws;
   const bool f16 = fused_tc_precision(m->precision);
   EmbedTcArgs et{};
-  et.R = ws.R; et.nlist = ws.nlist; et.nnei = ws.nnei; et.atype = atype; et.Gt = m->Gt;
+  et.R = ws.R; et.nlist = ws.nlist; et.atype = atype; et.Gt = m->Gt;
   et.n = n; et.ntypes = m->nt; et.err = m->d_err; et.b0t = m->b0t;
-  memcpy(et.W0, m->tcw.emb_vec.W0, sizeof(et.W0));
-  memcpy(et.b0, m->tcw.emb_vec.b0, sizeof(et.b0));
-  memcpy(et.b1, m->tcw.emb_vec.b1, sizeof(et.b1));
-  memcpy(et.b2, m->tcw.emb_vec.b2, sizeof(et.b2));
+  et.w = m->emb_packed;
   et.G0 = ws.G[0]; et.dG0 = ws.dG; et.dR = ws.dR; et.rm = f16 ? 0 : 1;
   et.rowmap = ws.rowmap;
   et.nrows = ws.row_off + n;
