@@ -44,11 +44,23 @@ __global__ void k_cell_setup(const double* __restrict__ box, double rcut, int ca
   if (threadIdx.x < 32 && blockIdx.x == 0) make_grid(box, rcut, cap_dim, cg, err);
 }
 
-// A coordinate inside the box needs no division (its floor is 0).
+// A coordinate's image inside the box: itself, without a division, if it is inside
+// (0 <= x < L, compared by the bits: negative values and NaN have larger ones).
+__device__ __forceinline__ double wrap_coord(double x, double L) {
+  const bool inside = (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(L);
+  return inside ? x : x - L * floor(x / L);
+}
+
 __device__ __forceinline__ int cell_coord(double x, double L, double scale, int nc) {
-  double w = x >= 0.0 && x < L ? x : x - L * floor(x / L);
-  int c = (int)(w * scale);
+  int c = (int)(wrap_coord(x, L) * scale);
   return c < 0 ? 0 : (c >= nc ? nc - 1 : c);
+}
+
+// An atom's entry of the list by cells: FP32 coordinates for the candidate screen, of
+// its image inside the box (far from the origin FP32 is too coarse), the index in w.
+__device__ __forceinline__ float4 cell_entry(double x, double y, double z, const double* L, int i) {
+  return make_float4((float)wrap_coord(x, L[0]), (float)wrap_coord(y, L[1]), (float)wrap_coord(z, L[2]),
+                     __int_as_float(i));
 }
 
 // The cell of atom i, its type checked into atype_c.
@@ -129,9 +141,10 @@ __global__ void k_cell_scan(const int* __restrict__ cell_count, int* __restrict_
   if (threadIdx.x == 0) cell_start[ncells] = carry;
 }
 
-// The atoms cell by cell: FP32 coordinates for the candidate screen, the index in w.
+// The atoms cell by cell.
 __global__ void k_cell_fill(const double* __restrict__ coord, const int* __restrict__ cell_of,
                             const int* __restrict__ cell_rank, int n, const int* __restrict__ cell_start,
+                            const CellGrid* __restrict__ cgp, const int* __restrict__ frame,
                             float4* __restrict__ cell_pos) {
   pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -139,7 +152,7 @@ __global__ void k_cell_fill(const double* __restrict__ coord, const int* __restr
   int c = cell_of[i];
   if (c < 0) return;  // padding of a packed batch
   cell_pos[cell_start[c] + cell_rank[i]] =
-      make_float4((float)coord[3 * i], (float)coord[3 * i + 1], (float)coord[3 * i + 2], __int_as_float(i));
+      cell_entry(coord[3 * i], coord[3 * i + 1], coord[3 * i + 2], cgp[frame ? frame[i] : 0].L, i);
 }
 
 // The four kernels above in one block, for up to SMALL_ATOMS atoms: each of them is a
@@ -225,7 +238,7 @@ __global__ void __launch_bounds__(SMALL_T) k_cells_small(const double* __restric
     const int i = tid + u * SMALL_T;
     if (i < n)
       cell_pos[(sh ? s_cnt[cell[u]] : __ldcg(cell_start + cell[u])) + rank[u]] =
-          make_float4((float)x[u][0], (float)x[u][1], (float)x[u][2], __int_as_float(i));
+          cell_entry(x[u][0], x[u][1], x[u][2], s_g.L, i);
   }
 }
 
@@ -303,7 +316,7 @@ __device__ __forceinline__ void sort_candidates(NbrShared& sh, int cnt, int hi_r
 __global__ void __launch_bounds__(32 * NBR_WARPS, 8)
 k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const CellGrid* __restrict__ cgp,
             const int* __restrict__ cell_of, const int* __restrict__ cell_start,
-            const float4* __restrict__ cell_pos, double rc2, int sel, int* __restrict__ nlist,
+            const float4* __restrict__ cell_pos, double rc2, float rc, int sel, int* __restrict__ nlist,
             int* __restrict__ nnei, int* __restrict__ ncand, int* __restrict__ atype_c, int* __restrict__ err,
             const int* __restrict__ frame, const int* __restrict__ cell_base, int cb0, int* __restrict__ rev_cnt,
             int* __restrict__ rev_rows) {
@@ -328,7 +341,7 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
   NbrShared& sh = s_sh[warp];
   const CellGrid* g = cgp + (frame ? fi : 0);
   const double xi = coord[3 * i], yi = coord[3 * i + 1], zi = coord[3 * i + 2];
-  const float fxi = (float)xi, fyi = (float)yi, fzi = (float)zi;
+  const float4 fi4 = cell_entry(xi, yi, zi, g->L, i);
   const float Lx = (float)g->L[0], Ly = (float)g->L[1], Lz = (float)g->L[2];
   const float iLx = 1.0f / Lx, iLy = 1.0f / Ly, iLz = 1.0f / Lz;
   // The cells of a row along x follow each other in cell_pos: a lane finds one
@@ -373,12 +386,15 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
   // pass 1: FP32 screen of the candidates, all lanes busy and NBR_U loads under way;
   // survivors are compacted into idx[] so that the FP64 decision below runs on full
   // warps (this part's FP64 rate is low, and a divergent FP64 branch costs the whole
-  // warp).  A component of the FP32 difference is off by at most ~1e-5 A and the
-  // squared distance near rc^2 by ~1.3e-4 A^2, far inside the margin, so a pair
-  // rejected here is never a neighbour (where FP32 and FP64 pick different images,
-  // both distances exceed L/2 > rcut).
+  // warp).  No neighbour may fail it.  With the coordinates in [0, L] and u = 2^-24,
+  // the two roundings, those of the difference and the edge make a component of the
+  // FP32 difference wrong by at most 4.5 u L, and, where the division by L tips to
+  // the other image within 5 u L of half an edge, by 14.5 u L; e = 16 u L per
+  // component lengthens a neighbour's distance to rc + sqrt(3) e at most.  The
+  // fixed margin is wider for edges up to 180 A (rc = 6 A).
   constexpr int NBR_U = 4;
-  const float rc2_screen = (float)rc2 * 1.0001f + 1e-4f;
+  const float far = rc + 1.7320509f * (16.f / 16777216.f) * fmaxf(Lx, fmaxf(Ly, Lz));
+  const float rc2_screen = fmaxf((float)rc2 * 1.0001f + 1e-4f, far * far * 1.000002f);
   constexpr float RINT = 12582912.f;  // 1.5 * 2^23: x + RINT - RINT rounds x to an integer
   int cur = 0;
   int2 seg = sh.seg[0];
@@ -398,7 +414,7 @@ k_neighbors(const double* __restrict__ coord, int n, int n_out, int base, const 
       const int j = __float_as_int(p[u].w);
       bool pass = false;
       if (j != i) {
-        float fx = p[u].x - fxi, fy = p[u].y - fyi, fz = p[u].z - fzi;
+        float fx = p[u].x - fi4.x, fy = p[u].y - fi4.y, fz = p[u].z - fi4.z;
         fx -= Lx * (__fmaf_rn(fx, iLx, RINT) - RINT);
         fy -= Ly * (__fmaf_rn(fy, iLy, RINT) - RINT);
         fz -= Lz * (__fmaf_rn(fz, iLz, RINT) - RINT);
@@ -486,11 +502,11 @@ void launch_neighbors(const NbrArgs& a, cudaStream_t st) {
     launch_pdl(k_cell_scan, 1, 1024, 0, st, a.cell_count, a.cell_start, a.grid, -1);
     note_launch();
     launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.cell_of, a.cell_rank, a.n, a.cell_start,
-               a.cell_pos);
+               a.grid, nullptr, a.cell_pos);
     note_launch();
   }
   launch_pdl(k_neighbors, (n_out + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st,
-             a.coord, a.n, n_out, a.base, a.grid, a.cell_of, a.cell_start, a.cell_pos, a.rcut * a.rcut, a.sel, a.nlist,
+             a.coord, a.n, n_out, a.base, a.grid, a.cell_of, a.cell_start, a.cell_pos, a.rcut * a.rcut, (float)a.rcut, a.sel, a.nlist,
              a.nnei, a.ncand, a.atype_c, a.err, nullptr, nullptr, 0, a.rev_cnt, a.rev_rows);
   note_launch();
 }
@@ -506,10 +522,10 @@ void launch_neighbors_packed(const NbrArgs& a, const int* frame, const int* cell
   launch_pdl(k_cell_scan, 1, 1024, 0, st, a.cell_count, a.cell_start, a.grid, ncells_total);
   note_launch();
   launch_pdl(k_cell_fill, (a.n + tb - 1) / tb, tb, 0, st, a.coord, a.cell_of, a.cell_rank, a.n, a.cell_start,
-             a.cell_pos);
+             a.grid, frame, a.cell_pos);
   note_launch();
   launch_pdl(k_neighbors, (a.n + NBR_WARPS - 1) / NBR_WARPS, 32 * NBR_WARPS, 0, st,
-             a.coord, a.n, a.n, 0, a.grid, a.cell_of, a.cell_start, a.cell_pos, a.rcut * a.rcut, a.sel, a.nlist, a.nnei,
+             a.coord, a.n, a.n, 0, a.grid, a.cell_of, a.cell_start, a.cell_pos, a.rcut * a.rcut, (float)a.rcut, a.sel, a.nlist, a.nnei,
              a.ncand, a.atype_c, a.err, frame, cell_base, cb0, a.rev_cnt, a.rev_rows);
   note_launch();
 }
