@@ -39,10 +39,24 @@ constexpr int EMB_TA = 128 * 64 * 2;    // activation tile: 128 rows x 64 cols
 constexpr int EMB_TD = 128 * 128 * 2;   // dZ3 tile: 128 rows x 128 cols
 constexpr int EMB_MAXT = 8;             // atom types (their type-pair table stays in L1)
 constexpr int EMB_THREADS = 256;
-// The first layer's weights and the later biases in shared memory (floats): W0 [32],
-// b1 [64], b2 [128], the first E0 / E1 / E2 of each used.  (With b0 as well, two CTAs of
-// the 32-64-128 net no longer fit on an SM.)
-constexpr int V_W0 = 0, V_B1 = 32, V_B2 = 96, EMB_VEC = 224;
+// The first layer's weights and the biases, as floats: W0 [32], b0 [32], b1 [64], b2
+// [128], the first E0 / E1 / E2 of each used.  They ride in the W1 tile, whose columns
+// from 32 on no product reads (shared memory of their own would leave one CTA of the
+// 32-64-128 net on an SM): float q lies in the upper half of the row's 128 bytes, 16 a
+// row, in the rows whose swizzle keeps columns 32 - 63 there (r % 8 < 4).  The adjoint
+// reads b2 one by one: four at a time spill (15,668 atoms: 540 us each; as constants of
+// the launch, which later weights do not reach, 523).
+constexpr int V_W0 = 0, V_B0 = 32, V_B1 = 64, V_B2 = 128, EMB_VEC = 256;
+__host__ __device__ constexpr int emb_vec_off(int q) { return ((q >> 6) * 8 + ((q >> 4) & 3)) * 128 + 64 + (q & 15) * 4; }
+// four of them, q % 4 == 0
+__device__ __forceinline__ float4 emb_vec4(const uint8_t* sm, int q) {
+  return *reinterpret_cast<const float4*>(sm + emb_vec_off(q));
+}
+__device__ __forceinline__ void emb_vec8(const uint8_t* sm, int q, float* v) {
+  const float4 a = emb_vec4(sm, q), b = emb_vec4(sm, q + 4);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
 static_assert(2 * EMB_TD == 4 * EMB_TA, "the dZ3 hi / lo tiles fill the activation tiles");
 
 template <int E0_, int E1_, int E2_>
@@ -53,8 +67,10 @@ struct EmbShape {
   static constexpr int T1 = 64 * 64 * 2;               // W1 tile: 64 (E1 padded) rows x 64 cols
   static constexpr int T2 = E2P * 64 * 2;              // W2 tile: E2P rows x 64 cols
   static constexpr int WIMG = 2 * T1 + 2 * T2;         // W1 hi, W1 lo, W2 hi, W2 lo
-  static constexpr int VEC = WIMG + 4 * EMB_TA;        // the net's vectors
-  static constexpr int SMEM = VEC + EMB_VEC * 4 + 64;
+  static constexpr int F_SMEM = WIMG + 4 * EMB_TA + 64;
+  // the adjoint's dZ3 tiles reuse the four activation tiles; 512 bytes for one
+  // partial dE/dx per row
+  static constexpr int B_SMEM = WIMG + 4 * EMB_TA + 512 + 64;
   // the trained vector: W0 b0 W1 b1 W2 b2
   static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2;
   static constexpr int SPLIT = (E1 / 2) & ~7;          // first layer-2 unit of half 1 (24 / 32)
@@ -64,7 +80,7 @@ struct EmbShape {
   static constexpr int NK3 = E2P / 16;                 // 16-column chunks of Z3
   static constexpr int TM_H1 = 64 + E2P;               // TMEM columns of the layer-1 exchange (32)
   // CTAs per SM the shared memory allows (228 KB per SM, 1 KB of it reserved per CTA)
-  static constexpr int MIN_CTAS = 2 * (SMEM + 1024) <= 228 * 1024 ? 2 : 1;
+  static constexpr int MIN_CTAS = 2 * (B_SMEM + 1024) <= 228 * 1024 ? 2 : 1;
   static_assert(TM_H1 + 32 <= 256, "TMEM columns");
 };
 using EmbS100 = EmbShape<25, 50, 100>;
@@ -82,12 +98,12 @@ struct EmbedTcArgs {
                           // neighbour) type [ntypes][ntypes][E0]; null: the net's b0
   float* H12;             // [tile][E0 + E1 units][128 rows]: layers 1 and 2 of the net,
                           // written by the forward, read by the adjoint
-  const uint4* wimg;      // W1/W2 hi/lo tiles (FP16 or BF16, as the kernel's operands)
+  const uint4* wimg;      // W1/W2 hi/lo tiles (FP16 or BF16, as the kernel's operands), the
+                          // vectors in the first
   int n, ntypes;
   int rm;                 // G0 and dG0 packed rows (the modular layer layout) instead of interleaved
   const int* rowmap;      // the live rows (atom * NP + slot) in tile order
   const int* nrows;       // their number (device)
-  const float* w;         // the net's weights W0 b0 W1 b1 W2 b2 (its vectors are read from here)
   int* err;
 };
 
@@ -143,15 +159,20 @@ __device__ __forceinline__ void embed_tc_front(const EmbedTcArgs& a, uint8_t* sm
   uint8_t* sH1l = sH1h + EMB_TA;
   uint8_t* sH2h = sH1l + EMB_TA;
   uint8_t* sH2l = sH2h + EMB_TA;
-  const float* vec = reinterpret_cast<const float*>(sm + S::VEC);
   const bool issuer = threadIdx.x == 0;
   // layer 1: half 0 evaluates units 0-15, half 1 units 16 .. E0 - 1; each
   // stores the hi and lo parts of its 8-column groups of H1 (K = E0, read as
   // 32) and leaves its units in TMEM columns [TM_H1, TM_H1 + 32) (free in
   // both kernels), where the other half reads them after the hand-off
   constexpr int p0 = H == 0 ? 0 : 16, np = H == 0 ? 16 : S::E0 - 16;
+  float w0[16], b0[16];
 #pragma unroll
-  for (int p = p0; p < p0 + np; ++p) h1[p] = rv ? tanhf(fmaf(x, vec[V_W0 + p], b0row[p])) : 0.f;
+  for (int i = 0; i < 16; i += 8) {
+    emb_vec8(sm, V_W0 + p0 + i, w0 + i);
+    emb_vec8(sm, V_B0 + p0 + i, b0 + i);
+  }
+#pragma unroll
+  for (int p = p0; p < p0 + np; ++p) h1[p] = rv ? tanhf(fmaf(x, w0[p - p0], b0row ? b0row[p] : b0[p - p0])) : 0.f;
   {
     float v[16];
 #pragma unroll
@@ -183,12 +204,13 @@ __device__ __forceinline__ void embed_tc_front(const EmbedTcArgs& a, uint8_t* sm
     for (int gg = 0; gg < 2; ++gg) {
       const int g = 2 * k + gg;
       if (g < O::g_lo || g >= O::g_hi) continue;
-      float v[8];
+      float v[8], b1[8];
+      emb_vec8(sm, V_B1 + 8 * g, b1);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int b = 8 * g + i;
         float hb = 0.f;
-        if (b < S::E1 && rv) hb = h1[b % S::E0] + tanhf(z[8 * gg + i] + vec[V_B1 + b]);
+        if (b < S::E1 && rv) hb = h1[b % S::E0] + tanhf(z[8 * gg + i] + b1[i]);
         if (O::owns_b(b)) h2[b - O::b0] = hb;
         v[i] = hb;
       }
@@ -245,17 +267,12 @@ __device__ __forceinline__ void embed_bwd_front(const EmbedTcArgs& a, uint8_t* s
 }
 
 template <class S>
-__device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm, uint64_t*& bar, uint32_t*& s_tmem) {
-  bar = reinterpret_cast<uint64_t*>(sm + S::SMEM - 64);
+__device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm, uint64_t*& bar, uint32_t*& s_tmem,
+                                               int smem_bytes) {
+  bar = reinterpret_cast<uint64_t*>(sm + smem_bytes - 64);
   s_tmem = reinterpret_cast<uint32_t*>(bar + 1);
   uint4* d = reinterpret_cast<uint4*>(sm);
   for (int i = threadIdx.x; i < S::WIMG / 16; i += blockDim.x) d[i] = a.wimg[i];
-  float* vec = reinterpret_cast<float*>(sm + S::VEC);
-  for (int i = threadIdx.x; i < S::E2; i += blockDim.x) {
-    if (i < S::E0) vec[V_W0 + i] = a.w[i];
-    if (i < S::E1) vec[V_B1 + i] = a.w[S::gB1 + i];
-    vec[V_B2 + i] = a.w[S::gB2 + i];
-  }
   // activation tiles start at zero: columns never written later are read
   // only against zero weight rows, which needs finite values there
   for (int i = threadIdx.x; i < 4 * EMB_TA / 16; i += blockDim.x) d[S::WIMG / 16 + i] = make_uint4(0u, 0u, 0u, 0u);
@@ -269,7 +286,7 @@ __device__ __forceinline__ void embed_tc_setup(const EmbedTcArgs& a, uint8_t* sm
 
 // Layer 3 forward of the owned outputs: G0[c] = (h2[c % E1] + tanh(z3 + b2)) (1 + Gt[t_i][t_j][c]).
 template <class S, int H>
-__device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, const float* b2, uint32_t taddr, const float* gt,
+__device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, const uint8_t* sm, uint32_t taddr, const float* gt,
                                               const float* h2, bool rv, float* out_blk, int slot) {
   using O = EmbOwn<S, H>;
 #pragma unroll
@@ -285,9 +302,10 @@ __device__ __forceinline__ void embed_fwd_out(const EmbedTcArgs& a, const float*
       const int c = 16 * k + i;
       if (!O::owns_c(c)) continue;  // pairs never straddle an ownership boundary (SPLIT, E1, E1 + SPLIT even)
       const float2 g2 = *reinterpret_cast<const float2*>(gt + c);
+      const float2 b2 = *reinterpret_cast<const float2*>(sm + emb_vec_off(V_B2 + c));
       float2 o;
-      o.x = rv ? (h2[c % S::E1 - O::b0] + tanhf(z[i] + b2[c])) * (1.f + g2.x) : 0.f;
-      o.y = rv ? (h2[(c + 1) % S::E1 - O::b0] + tanhf(z[i + 1] + b2[c + 1])) * (1.f + g2.y) : 0.f;
+      o.x = rv ? (h2[c % S::E1 - O::b0] + tanhf(z[i] + b2.x)) * (1.f + g2.x) : 0.f;
+      o.y = rv ? (h2[(c + 1) % S::E1 - O::b0] + tanhf(z[i + 1] + b2.y)) * (1.f + g2.y) : 0.f;
       if (rv) __stcs(reinterpret_cast<float2*>(out_blk + (a.rm ? (size_t)slot * S::E2 + c : cq_off(slot, c))), o);
     }
   }
@@ -343,8 +361,8 @@ __device__ __forceinline__ void embed_bwd_prefetch16(const float4* dg, bool rm, 
 // before it waits for Z3; chunk k + 1 is brought into L1 while chunk k is
 // processed.
 template <class S, bool F16, int H>
-__device__ __forceinline__ void embed_bwd_dz3(const EmbedTcArgs& a, const float* b2, uint32_t taddr, const float* gt, const float4* dg,
-                                              bool rv, int row, int slot, uint8_t* sDZ3h, uint8_t* sDZ3l, float* dh2,
+__device__ __forceinline__ void embed_bwd_dz3(const EmbedTcArgs& a, const uint8_t* sm, uint32_t taddr,
+                                              const float* gt, const float4* dg, bool rv, int row, int slot, uint8_t* sDZ3h, uint8_t* sDZ3l, float* dh2,
                                               float4* dcur) {
   using O = EmbOwn<S, H>;
   using D = EmbDz3<S, H>;
@@ -379,7 +397,7 @@ __device__ __forceinline__ void embed_bwd_dz3(const EmbedTcArgs& a, const float*
           if (O::owns_c(c)) dh2[c % S::E1 - O::b0] += gq[t];
           float d = 0.f;
           if (store && c < S::E2 && rv) {
-            const float th = tanhf(z[8 * gg + 4 * q + t] + b2[c]);
+            const float th = tanhf(z[8 * gg + 4 * q + t] + *reinterpret_cast<const float*>(sm + emb_vec_off(V_B2 + c)));
             d = gq[t] * (1.f - th * th);
           }
           dz[4 * q + t] = d;
@@ -437,7 +455,6 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
                                                const float4* dg, int slot, float* xch, Pre pre) {
   using O = EmbOwn<S, H>;
   const bool issuer = threadIdx.x == 0;
-  const float* vec = reinterpret_cast<const float*>(sm + S::VEC);
   uint8_t* sW1h = sm;
   uint8_t* sW1l = sW1h + S::T1;
   uint8_t* sW2h = sW1l + S::T1;
@@ -458,7 +475,7 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
   float dh2[O::nb];
 #pragma unroll
   for (int b = 0; b < O::nb; ++b) dh2[b] = 0.f;
-  embed_bwd_dz3<S, F16, H>(a, vec + V_B2, tm + lane_off, gt, dg, rv, row, slot, sDZ3h, sDZ3l, dh2, d0);
+  embed_bwd_dz3<S, F16, H>(a, sm, tm + lane_off, gt, dg, rv, row, slot, sDZ3h, sDZ3l, dh2, d0);
   handoff();
   // dH2 (product part) = dZ3 W2^T -> TMEM [0, 64)
   if (issuer)
@@ -479,8 +496,11 @@ __device__ __forceinline__ void embed_bwd_tail(const EmbedTcArgs& a, uint8_t* sm
   tmem_ld16(tm + lane_off + 80, v + 16);
   float dx = 0.f;
   if (rv) {
+    float w0[32];
 #pragma unroll
-    for (int p = 0; p < S::E0; ++p) dx = fmaf(vec[V_W0 + p] * (1.f - h1[p] * h1[p]), dh1[p] + (H == 0 ? v[p] : 0.f), dx);
+    for (int p = 0; p < S::E0; p += 8) emb_vec8(sm, V_W0 + p, w0 + p);
+#pragma unroll
+    for (int p = 0; p < S::E0; ++p) dx = fmaf(w0[p] * (1.f - h1[p] * h1[p]), dh1[p] + (H == 0 ? v[p] : 0.f), dx);
   }
   // half 1 hands its part to half 0, which owns the row's dR update
   if (H == 1) xch[row] = dx;
@@ -541,7 +561,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
   }
   uint64_t* bar;
   uint32_t* s_tmem;
-  embed_tc_setup<S>(a, sm, bar, s_tmem);
+  embed_tc_setup<S>(a, sm, bar, s_tmem, S::F_SMEM);
   pdl_wait();
   const uint32_t tm = *s_tmem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
@@ -560,7 +580,7 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
     const bool rv = cur.rg >= 0;
     in.map(a, nrows, tile + gridDim.x, row);
     auto rows_next = [&] { in.rows(a, true); };
-    const float* b0row = a.b0t ? a.b0t + ((size_t)cur.ti * a.ntypes + cur.tj) * S::E0 : a.w + S::gB0;
+    const float* b0row = a.b0t && rv ? a.b0t + ((size_t)cur.ti * a.ntypes + cur.tj) * S::E0 : nullptr;
     if (half == 0)
       embed_tc_front<S, F16, 0>(a, sm, tm, lane_off, sy, row, rv, cur.x, b0row, h1, h2, rows_next);
     else
@@ -581,11 +601,10 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_fwd_live(
     }
     float* out = a.G0 + (size_t)(a.rm ? tile : cur.atom) * NP * S::E2;
     const int slot = a.rm ? row : cur.slot;
-    const float* b2 = reinterpret_cast<const float*>(sm + S::VEC) + V_B2;
     if (half == 0)
-      embed_fwd_out<S, 0>(a, b2, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
+      embed_fwd_out<S, 0>(a, sm, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
     else
-      embed_fwd_out<S, 1>(a, b2, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
+      embed_fwd_out<S, 1>(a, sm, tm + lane_off, cur.gt(a, S::E2), h2, rv, out, slot);
     in.type(a);
     fence_before_sync();
     __syncthreads();
@@ -605,15 +624,13 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(
   }
   uint64_t* bar;
   uint32_t* s_tmem;
-  embed_tc_setup<S>(a, sm, bar, s_tmem);
+  embed_tc_setup<S>(a, sm, bar, s_tmem, S::B_SMEM);
   pdl_wait();
   const uint32_t tm = *s_tmem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quad = warp & 3, half = warp >> 2;
   const int row = quad * 32 + lane;
   const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-  // [128] half 1's dE/dx, over the dZ2 tile once its product is done (rows that the
-  // next tile's dZ3 writes in full)
-  float* xch = reinterpret_cast<float*>(sm + S::WIMG);
+  float* xch = reinterpret_cast<float*>(sm + S::WIMG + 4 * EMB_TA);  // [128] half 1's dE/dx
   Sync sy{bar, 0u, a.err};
   const int nrows = *a.nrows;
   const int ntiles = (nrows + 127) / 128;
@@ -663,9 +680,9 @@ __global__ void __launch_bounds__(EMB_THREADS, S::MIN_CTAS) k_embed_tc_bwd_live(
 namespace {
 // The hi and lo parts of W1 and W2 of a net of shape S as swizzled K-major
 // tiles (W1 as [E1 (64 rows)][E0 (K)], W2 as [E2P rows][E1 (K)]), in FP16
-// (f16) or BF16.
+// (f16) or BF16, and the vectors v (EMB_VEC floats) in the first.
 template <class S>
-std::vector<uint8_t> emb_image(const std::vector<double>& W1, const std::vector<double>& W2, bool f16) {
+std::vector<uint8_t> emb_image(const std::vector<double>& W1, const std::vector<double>& W2, const float* v, bool f16) {
   std::vector<uint8_t> img(S::WIMG, 0);
   auto put = [&](int off, int r, int c, int R, double x, bool lo) {
     if (f16) {
@@ -688,16 +705,23 @@ std::vector<uint8_t> emb_image(const std::vector<double>& W1, const std::vector<
       put(2 * S::T1, c, b, S::E2P, W2[(size_t)b * S::E2 + c], false);
       put(2 * S::T1 + S::T2, c, b, S::E2P, W2[(size_t)b * S::E2 + c], true);
     }
+  for (int q = 0; q < EMB_VEC; ++q) memcpy(img.data() + emb_vec_off(q), v + q, sizeof(float));
   return img;
 }
 
-// The same from the trained vector w, element by element of W1, then W2 (the images'
-// padding stays as it was).
+// The same from the trained vector w, element by element of W1, then W2, then the
+// vectors (the images' padding stays as it was).
 template <class S, bool F16>
 __global__ void k_emb_image(const float* __restrict__ w, uint8_t* __restrict__ img) {
   constexpr int N1 = S::E0 * S::E1, N2 = S::E1 * S::E2;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= N1 + N2) return;
+  if (t >= N1 + N2) {
+    const int q = t - N1 - N2, V[4] = {V_W0, V_B0, V_B1, V_B2}, E[4] = {S::E0, S::E0, S::E1, S::E2};
+    const int g[4] = {0, S::gB0, S::gB1, S::gB2};
+    for (int k = 0; k < 4; ++k)
+      if (q < EMB_VEC && q >= V[k] && q < V[k] + E[k]) *reinterpret_cast<float*>(img + emb_vec_off(q)) = w[g[k] + q - V[k]];
+    return;
+  }
   const bool first = t < N1;
   const float x = first ? w[S::gW1 + t] : w[S::gW2 + t - N1];
   const int k = first ? t / S::E1 : (t - N1) / S::E2, n = first ? t % S::E1 : (t - N1) % S::E2;
@@ -708,7 +732,7 @@ __global__ void k_emb_image(const float* __restrict__ w, uint8_t* __restrict__ i
 
 template <class S>
 void emb_refresh(dp_model* m, cudaStream_t st) {
-  const int blocks = (S::E0 * S::E1 + S::E1 * S::E2 + 255) / 256;
+  const int blocks = (S::E0 * S::E1 + S::E1 * S::E2 + EMB_VEC + 255) / 256;
   k_emb_image<S, true><<<blocks, 256, 0, st>>>(m->emb_packed, reinterpret_cast<uint8_t*>(m->tcw.emb_W1_t));
   k_emb_image<S, false><<<blocks, 256, 0, st>>>(m->emb_packed, reinterpret_cast<uint8_t*>(m->tcw.emb_W2_t));
   note_launch(2);
@@ -716,10 +740,10 @@ void emb_refresh(dp_model* m, cudaStream_t st) {
 
 template <class S>
 void emb_set_smem() {
-  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
-  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
-  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
-  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
+  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_fwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::F_SMEM);
+  cudaFuncSetAttribute(k_embed_tc_bwd_live<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::B_SMEM);
 }
 
 template <class S>
@@ -730,8 +754,8 @@ bool emb_is(const dp_model* m) {
 
 // Weight images of the tensor-core embedding net (the 25-50-100 and
 // 32-64-128 nets with at most EMB_MAXT types): the hi and lo parts of W1 and
-// W2 in FP16 (the fused 16-bit paths) and in BF16 (the bf16x mode).  Other nets
-// keep both images null (FP32 SIMT kernels).
+// W2 in FP16 (the fused 16-bit paths) and in BF16 (the bf16x mode), with its per-unit
+// vectors.  Other nets keep both images null (FP32 SIMT kernels).
 int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg) {
   auto get = [&](const std::string& name) -> const std::vector<double>& {
     for (auto& kv : arrays)
@@ -746,8 +770,17 @@ int tc_init_embedding(dp_model* m, const HostArrays& arrays, std::string& msg) {
   if (!(s100 || s128) || m->nt > EMB_MAXT) return DP_OK;
   const std::vector<double>& W1 = get("em_W1");  // [E0][E1]
   const std::vector<double>& W2 = get("em_W2");  // [E1][E2]
+  float v[EMB_VEC] = {};
+  auto vec = [&](const char* name, int at, int count) {
+    const std::vector<double>& x = get(name);
+    for (int q = 0; q < count; ++q) v[at + q] = (float)x[q];
+  };
+  vec("em_W0", V_W0, m->emb[0]);
+  vec("em_b0", V_B0, m->emb[0]);
+  vec("em_b1", V_B1, m->emb[1]);
+  vec("em_b2", V_B2, m->emb[2]);
   for (int f16 = 1; f16 >= 0; --f16) {  // FP16 image (fused paths), BF16 image (bf16x)
-    const std::vector<uint8_t> img = s100 ? emb_image<EmbS100>(W1, W2, f16 != 0) : emb_image<EmbS128>(W1, W2, f16 != 0);
+    const std::vector<uint8_t> img = s100 ? emb_image<EmbS100>(W1, W2, v, f16 != 0) : emb_image<EmbS128>(W1, W2, v, f16 != 0);
     void* d = nullptr;
     if (cudaMalloc(&d, img.size()) != cudaSuccess ||
         cudaMemcpy(d, img.data(), img.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -778,8 +811,8 @@ namespace {
 // (the fused 16-bit paths) or BF16 (bf16x) operand splits.
 template <class S, bool F16>
 void tc_embed_launch_s(int grid, const EmbedTcArgs& et, bool bwd, cudaStream_t st) {
-  if (!bwd) launch_pdl(k_embed_tc_fwd_live<S, F16>, grid, EMB_THREADS, S::SMEM, st, et);
-  if (bwd) launch_pdl(k_embed_tc_bwd_live<S, F16>, grid, EMB_THREADS, S::SMEM, st, et);
+  if (!bwd) launch_pdl(k_embed_tc_fwd_live<S, F16>, grid, EMB_THREADS, S::F_SMEM, st, et);
+  if (bwd) launch_pdl(k_embed_tc_bwd_live<S, F16>, grid, EMB_THREADS, S::B_SMEM, st, et);
 }
 
 }  // namespace
@@ -794,7 +827,6 @@ void tc_embed(dp_model* m, int n, const int* atype, bool bwd, cudaStream_t st) {
   EmbedTcArgs et{};
   et.R = ws.R; et.nlist = ws.nlist; et.atype = atype; et.Gt = m->Gt;
   et.n = n; et.ntypes = m->nt; et.err = m->d_err; et.b0t = m->b0t;
-  et.w = m->emb_packed;
   et.G0 = ws.G[0]; et.dG0 = ws.dG; et.dR = ws.dR; et.rm = f16 ? 0 : 1;
   et.rowmap = ws.rowmap;
   et.nrows = ws.row_off + n;
