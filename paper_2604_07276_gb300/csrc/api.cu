@@ -1355,8 +1355,8 @@ long long dp_debug_copy(dp_model* m, const char* name, void* host_dst, size_t by
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(DP_ERR_CUDA, "sync failed");
   if (s[0] == 'G') {
     // the fused paths keep G column-quad interleaved per atom, the others packed
-    // over the live rows: return it row-major per atom, packed layouts with zeros
-    // past the last neighbour
+    // over the live rows; either way only live rows are written: return it
+    // row-major per atom with zeros past the last neighbour
     const size_t m1 = (size_t)m->m1, full = rows * m1;
     const bool cq = fused_tc_precision(m->precision);
     std::vector<float> raw(full), out(full, 0.f);
@@ -1366,14 +1366,14 @@ long long dp_debug_copy(dp_model* m, const char* name, void* host_dst, size_t by
          cudaMemcpy(off.data(), ws.row_off, off.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess))
       return fail(DP_ERR_CUDA, "copy failed");
     for (size_t atom = 0; atom < (size_t)m->call_nlocal; ++atom) {
+      const int o = off[atom], k = off[atom + 1] - o;
+      if (o < 0 || k < 0 || k > NP || (size_t)(o + k) > rows) continue;  // no evaluation has run
+      float* dst = &out[atom * NP * m1];
       if (cq) {
-        for (int r = 0; r < NP; ++r)
-          for (size_t c = 0; c < m1; ++c)
-            out[(atom * NP + r) * m1 + c] = raw[atom * NP * m1 + cq_off(r, (int)c)];
+        for (int r = 0; r < k; ++r)
+          for (size_t c = 0; c < m1; ++c) dst[r * m1 + c] = raw[atom * NP * m1 + cq_off(r, (int)c)];
       } else {
-        const int o = off[atom], k = off[atom + 1] - o;
-        if (o < 0 || k < 0 || k > NP || (size_t)(o + k) > rows) continue;  // no evaluation has run
-        memcpy(&out[atom * NP * m1], &raw[(size_t)o * m1], sizeof(float) * k * m1);
+        memcpy(dst, &raw[(size_t)o * m1], sizeof(float) * k * m1);
       }
     }
     memcpy(host_dst, out.data(), sz);
