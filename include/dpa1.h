@@ -84,7 +84,9 @@ DP_API int dp_init(dp_model** out, const char* weights_path, const char* const* 
 
 /* Energy, forces and virial of one frame from HOST arrays (Sec. IV-A,
  * deepmd::compute()).  Copies inputs to the device, runs the whole path on
- * the model's stream, copies results back and synchronises.  Grows the
+ * the model's stream, copies results back and synchronises.  Waits first for
+ * the device calls of this model that are still under way, whatever their
+ * streams (as every call on the model's own stream does).  Grows the
  * workspace when natoms exceeds the reserved size.  natoms == 0 gives
  * zero energy and virial. */
 DP_API int dp_compute(dp_model* m, int natoms, const double* coord, const double* box, const int* atype,
@@ -96,7 +98,9 @@ DP_API int dp_compute(dp_model* m, int natoms, const double* coord, const double
  * CUDA graph.  natoms must not exceed the size reserved with dp_reserve
  * (DP_ERR_CAPACITY otherwise, nothing launched).  Device-side failures (box
  * check, buffer overflow) are recorded in a device flag read by
- * dp_get_status; the outputs are then unspecified. */
+ * dp_get_status; the outputs are then unspecified.  A model has one
+ * workspace: its device calls on different streams are for the caller to
+ * order. */
 DP_API int dp_compute_device(dp_model* m, int natoms, const double* d_coord, const double* d_box,
                       const int* d_atype, double* d_energy, double* d_force, double* d_virial,
                       double* d_atom_energy, void* cuda_stream);

@@ -344,6 +344,23 @@ int translate_err(int bits) {
   return DP_OK;
 }
 
+// A device call, or a change of the weights, was queued on the caller's stream st.
+void note_device_call(dp_model* m, cudaStream_t st) {
+  m->pending = true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+  if (cs != cudaStreamCaptureStatusNone) m->captured = true;
+}
+
+// Before a call on the model's own stream: its workspace and weights may be in use by a
+// device call on another.  The caller's streams may be gone by now, hence the device.
+int wait_device_calls(dp_model* m) {
+  if (!m->pending) return DP_OK;
+  CUDA_TRY(cudaDeviceSynchronize());
+  m->pending = m->captured;
+  return DP_OK;
+}
+
 // Stages a1-a2 on the stream.
 // Neighbour-stage arguments for n atoms at coord, with the list, counts,
 // clamped types and reverse list written from workspace slot rel on.
@@ -1015,8 +1032,9 @@ int dp_compute_device_local(dp_model* m, int natoms, int nlocal, const double* d
     return fail(DP_ERR_ARG, "null device pointer");
   if (natoms > m->ws.cap) return fail(DP_ERR_CAPACITY, "natoms exceeds the reserved workspace (call dp_reserve)");
   CUDA_TRY(cudaSetDevice(m->device));
-  return run_device(m, natoms, nlocal, d_coord, d_box, d_atype, d_energy, d_force, d_virial, d_atom_energy,
-                    reinterpret_cast<cudaStream_t>(stream));
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  note_device_call(m, st);
+  return run_device(m, natoms, nlocal, d_coord, d_box, d_atype, d_energy, d_force, d_virial, d_atom_energy, st);
 }
 
 int dp_compute_device(dp_model* m, int natoms, const double* d_coord, const double* d_box, const int* d_atype,
@@ -1039,6 +1057,7 @@ int dp_compute_local(dp_model* m, int natoms, int nlocal, const double* coord, c
   for (long long i = 0; i < 3LL * natoms; ++i)
     if (!std::isfinite(coord[i])) return fail(DP_ERR_NAN, "non-finite coordinate");
   CUDA_TRY(cudaSetDevice(m->device));
+  if ((rc = wait_device_calls(m)) != DP_OK) return rc;
   if (natoms > m->ws.cap && (rc = dp_reserve(m, natoms)) != DP_OK) return rc;
   Workspace& ws = m->ws;
   cudaStream_t st = m->stream;
@@ -1133,7 +1152,8 @@ int dp_compute_batch(dp_model* m, int nframes, const int* off, const double* coo
   // min(P, BATCH_PACK_ATOMS) slots (at least the largest frame), and a larger
   // batch runs as several passes of consecutive frames.
   const long long want = std::max(padded(maxn), std::min(P, (long long)BATCH_PACK_ATOMS));
-  int rc;
+  int rc = wait_device_calls(m);
+  if (rc != DP_OK) return rc;
   if (want > m->ws.cap && (rc = dp_reserve(m, (int)want)) != DP_OK) {
     if (want == padded(maxn) || (rc = dp_reserve(m, (int)padded(maxn))) != DP_OK) return rc;
   }
@@ -1292,6 +1312,7 @@ int dp_nlist_device(dp_model* m, int natoms, const double* d_coord, const double
   if (natoms > m->ws.cap) return fail(DP_ERR_CAPACITY, "natoms exceeds the reserved workspace (call dp_reserve)");
   CUDA_TRY(cudaSetDevice(m->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  note_device_call(m, st);
   // types are not needed for the list: pass a zero-type buffer of the workspace
   CUDA_TRY(cudaMemsetAsync(m->ws.atype, 0, sizeof(int) * (size_t)(natoms > 0 ? natoms : 1), st));
   run_neighbors(m, natoms, d_coord, d_box, m->ws.atype, st);
@@ -1522,6 +1543,7 @@ int dp_train_frame(dp_model* m, int natoms, const double* d_coord, const double*
   if (natoms > m->ws.cap) return fail(DP_ERR_CAPACITY, "natoms exceeds the reserved workspace (call dp_reserve)");
   CUDA_TRY(cudaSetDevice(m->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  note_device_call(m, st);
   const int cap = m->ws.cap, m1 = m->m1, nfit = m->nfit;
   const size_t rows = (size_t)cap * NP;
   int fmax = m->fit_in;
@@ -1593,6 +1615,7 @@ int dp_adam_step(dp_model* m, double lr, double beta1, double beta2, double eps,
     return fail(DP_ERR_ARG, "dp_adam_step: bad hyper-parameters");
   CUDA_TRY(cudaSetDevice(m->device));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  note_device_call(m, st);
   const int t = ++m->adam_t;
   const float bc1 = (float)(1.0 - std::pow(beta1, t)), bc2 = (float)(1.0 - std::pow(beta2, t));
   launch_adam(m->theta, m->grad, m->adam_m, m->adam_v, m->ntheta, (float)lr, (float)beta1, (float)beta2, (float)eps,
@@ -1612,6 +1635,11 @@ int dp_md_run(dp_model* m, int natoms, double* d_coord, double* d_vel, const dou
   if (natoms > m->ws.cap) return fail(DP_ERR_CAPACITY, "natoms exceeds the reserved workspace (call dp_reserve)");
   CUDA_TRY(cudaSetDevice(m->device));
   cudaStream_t st = stream ? reinterpret_cast<cudaStream_t>(stream) : m->stream;
+  if (stream) {
+    note_device_call(m, st);
+  } else if (int w = wait_device_calls(m)) {
+    return w;
+  }
   if (!m->d_md_counter) {
     void* p = nullptr;
     CUDA_TRY(cudaMalloc(&p, sizeof(int)));

@@ -193,6 +193,9 @@ struct dp_model {
   char* d_io = nullptr;
   cudaStream_t stream = nullptr;  // own stream of the host API
   cudaStream_t last_stream = nullptr;
+  // device calls queued on the caller's streams that no host call has waited for, and
+  // whether one of them was captured (its replays are not seen here)
+  bool pending = false, captured = false;
   int last_natoms = 0;
   dpa1::Profiler prof;
   // velocity-Verlet: step counter, the kick's per-block kinetic energies and
