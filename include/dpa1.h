@@ -184,8 +184,8 @@ DP_API int dp_nlist_device(dp_model* m, int natoms, const double* d_coord, const
  * Forces are first evaluated at the starting coordinates.  With
  * use_graph != 0 one step is captured once into a CUDA graph (cached in the
  * model for the same pointers, sizes, dt and precision) and replayed nsteps
- * times.  Runs on cuda_stream (NULL: the model's own stream, then
- * synchronised).  natoms must not exceed the reserved size. */
+ * times.  Runs on cuda_stream (NULL: the model's own stream, behind the work
+ * queued on the default stream, then synchronised).  natoms must not exceed the reserved size. */
 DP_API int dp_md_run(dp_model* m, int natoms, double* d_coord, double* d_vel, const double* d_mass,
                      const double* d_box, const int* d_atype, double dt, int nsteps, double* d_force,
                      double* d_energy, double* d_virial, double* d_thermo, int use_graph, void* cuda_stream);

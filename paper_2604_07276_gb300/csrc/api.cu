@@ -991,6 +991,8 @@ int dp_init(dp_model** out, const char* weights_path, const char* const* type_ma
   }
   if (cudaStreamCreateWithFlags(&m->stream, cudaStreamNonBlocking) != cudaSuccess)
     return fail_free(fail(DP_ERR_CUDA, "stream creation failed"));
+  if (cudaEventCreateWithFlags(&m->order, cudaEventDisableTiming) != cudaSuccess)
+    return fail_free(fail(DP_ERR_CUDA, "event creation failed"));
   if (cudaHostAlloc(reinterpret_cast<void**>(&m->h_io), IO_BYTES, cudaHostAllocDefault) != cudaSuccess ||
       cudaMalloc(reinterpret_cast<void**>(&m->d_io), IO_BYTES) != cudaSuccess)
     return fail_free(fail(DP_ERR_CUDA, "allocation of the host-call staging failed"));
@@ -1637,8 +1639,17 @@ int dp_md_run(dp_model* m, int natoms, double* d_coord, double* d_vel, const dou
   cudaStream_t st = stream ? reinterpret_cast<cudaStream_t>(stream) : m->stream;
   if (stream) {
     note_device_call(m, st);
-  } else if (int w = wait_device_calls(m)) {
-    return w;
+  } else {
+    if (int w = wait_device_calls(m)) return w;
+    // the caller has filled the arrays on the default stream, which this one is not
+    // tied to (while a blocking stream is being captured, the default one takes no work)
+    cudaStreamCaptureStatus cs;
+    if (cudaStreamIsCapturing(nullptr, &cs) == cudaSuccess) {
+      CUDA_TRY(cudaEventRecord(m->order, nullptr));
+      CUDA_TRY(cudaStreamWaitEvent(st, m->order, 0));
+    } else {
+      cudaGetLastError();
+    }
   }
   if (!m->d_md_counter) {
     void* p = nullptr;
@@ -1712,6 +1723,7 @@ void dp_free(dp_model* m) {
   if (m->h_io) cudaFreeHost(m->h_io);
   if (m->d_io) cudaFree(m->d_io);
   if (m->stream) cudaStreamDestroy(m->stream);
+  if (m->order) cudaEventDestroy(m->order);
   for (auto& e : m->prof.ev)
     if (e) cudaEventDestroy(e);
   if (m->md_exec) cudaGraphExecDestroy(m->md_exec);

@@ -192,6 +192,7 @@ struct dp_model {
   char* h_io = nullptr;
   char* d_io = nullptr;
   cudaStream_t stream = nullptr;  // own stream of the host API
+  cudaEvent_t order = nullptr;    // places that stream behind the default stream (dp_md_run)
   cudaStream_t last_stream = nullptr;
   // device calls queued on the caller's streams that no host call has waited for, and
   // whether one of them was captured (its replays are not seen here)

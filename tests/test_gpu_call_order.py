@@ -103,3 +103,34 @@ def test_host_call_after_training_step():
     again = m.compute(coord, box, atype)
     assert got[0] == again[0] != before[0] and np.array_equal(got[1], again[1])
     m.close()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_md_behind_the_default_stream(default_model, graph):
+    """The arrays of a run are filled by copies that wait behind other work of the default stream."""
+    import torch
+
+    import paper_2604_07276_gb300 as p
+    from paper_2604_07276_gb300 import md
+
+    cfg, w, _ = default_model
+    coord, atype, box = synth.water_box(0)
+    vel = synth.maxwell_boltzmann(atype, 50.0, seed=11)
+    m = p.DPA1(weight_file(cfg, w, "default"), precision="fp16x")
+    state = md.MDState(coord, vel, synth.MASSES[atype], box, atype)
+    x0, v0 = state.coord.clone(), state.vel.clone()
+    big = torch.zeros(1 << 28, device="cuda")
+    runs = []
+    for busy in (False, True):
+        state.coord.zero_().add_(torch.arange(3 * len(atype), device="cuda").reshape(-1, 3) * 0.01)
+        torch.cuda.synchronize()
+        if busy:
+            for _ in range(60):  # some milliseconds
+                big.add_(1.0)
+        state.coord.copy_(x0)
+        state.vel.copy_(v0)
+        thermo = md.run(m, state, dt=0.1, nsteps=2, graph=graph)
+        runs.append((thermo.clone(), state.coord.clone(), state.vel.clone()))
+    for a, b in zip(*runs):
+        assert torch.equal(a, b)
+    m.close()
