@@ -279,8 +279,14 @@ class DPA1:
         _check(self.lib.dp_get_grad(self.h, out.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), len(out)))
         return out
 
+    def _stream(self, stream):
+        """The stream given, or PyTorch's current one, as for the calls that take tensors."""
+        import torch
+
+        return stream if stream is not None else torch.cuda.current_stream(self.device).cuda_stream
+
     def zero_grad(self, stream=None) -> None:
-        _check(self.lib.dp_zero_grad(self.h, stream))
+        _check(self.lib.dp_zero_grad(self.h, self._stream(stream)))
 
     def train_frame(self, coord, box, atype, e_ref: float, force_ref, loss, pe=1.0, pf=1.0, stream=None):
         """``dp_train_frame`` on CUDA tensors; ``loss`` is a float64 [3] tensor."""
@@ -292,7 +298,8 @@ class DPA1:
                                        loss.data_ptr(), st))
 
     def adam_step(self, lr: float, beta1: float = 0.9, beta2: float = 0.999, eps: float = 1e-8, stream=None) -> None:
-        _check(self.lib.dp_adam_step(self.h, float(lr), float(beta1), float(beta2), float(eps), stream))
+        _check(self.lib.dp_adam_step(self.h, float(lr), float(beta1), float(beta2), float(eps),
+                                     self._stream(stream)))
 
     def set_profiling(self, on: bool) -> None:
         _check(self.lib.dp_set_profiling(self.h, 1 if on else 0))

@@ -134,3 +134,36 @@ def test_md_behind_the_default_stream(default_model, graph):
     for a, b in zip(*runs):
         assert torch.equal(a, b)
     m.close()
+
+
+def test_training_calls_on_the_current_stream():
+    """zero_grad and adam_step without a stream follow train_frame, which runs on PyTorch's current one."""
+    import torch
+
+    import paper_2604_07276_gb300 as p
+
+    cfg = synth.STUDENT_CONFIG
+    m = p.DPA1(weight_file(cfg, synth.make_weights(cfg, seed=12, bias_scale=0.1), "order_student"), precision="fp32")
+    frame = synth.lattice_system(300, seed=3, density=0.06)
+    m.reserve(300)
+    c, b, t = _device_args(p, frame)[:3]
+    loss = torch.zeros(3, dtype=torch.float64, device="cuda")
+    f_ref = torch.zeros((300, 3), dtype=torch.float64, device="cuda")
+    big = torch.zeros(1 << 28, device="cuda")
+    m.zero_grad()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for _ in range(40):  # some milliseconds
+            big.add_(1.0)
+        m.train_frame(c, b, t, 1.0, f_ref, loss)
+        m.zero_grad()
+        assert not m.get_grad().any()
+        before = m.get_params()
+        for _ in range(40):
+            big.add_(1.0)
+        m.train_frame(c, b, t, 1.0, f_ref, loss)
+        m.adam_step(0.02)
+        after = m.get_params()
+    assert np.mean(after != before) > 0.9
+    assert not m.get_grad().any()  # the step clears it
+    m.close()
