@@ -509,7 +509,7 @@ void run_network_f32(dp_model* m, int n, const int* atype, cudaStream_t st) {
   const int* nrows = ws.row_off + n;  // the live rows (device)
   // a5: embedding
   EmbedArgs ea{};
-  ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
+  ea.R = ws.R; ea.nlist = ws.nlist; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0];
   ea.dG0 = ws.dG; ea.dR = ws.dR; ea.rowmap = ws.rowmap; ea.nrows = ws.row_off + n; ea.packed = 1;
   launch_embed_rows(ea, m->emb, false, st);
@@ -570,7 +570,7 @@ void run_network_bf16x(dp_model* m, int n, const int* atype, cudaStream_t st) {
   // other nets, and any net while its weight gradient is wanted, in FP32
   const bool emb_tc = m->tcw.emb_W2_t != nullptr && !m->fit_keep;
   EmbedArgs ea{};
-  ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
+  ea.R = ws.R; ea.nlist = ws.nlist; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0];
   ea.dG0 = ws.dG; ea.dR = ws.dR; ea.rowmap = ws.rowmap; ea.nrows = ws.row_off + n; ea.packed = 1;
   if (emb_tc)
@@ -682,7 +682,7 @@ int run_device(dp_model* m, int n, int nlocal, const double* coord, const double
 // The weight gradients of both loss terms of the evaluation that just ran (no
 // attention layer, its intermediates still in the workspace, the fitting adjoint in
 // keep): grad += s1 dE/dtheta + s2 (dE/dtheta)', ' being the tangent along the atom
-// displacement field v and s1, s2 = d_scales[1], [2].
+// displacement field v and s1, s2 = d_scales[0], [1].
 void run_force_tangent(dp_model* m, int n, const double* coord, const double* v, float* Rd, float* Gd, float* dGd,
                        float* Td, float* Xd, float* dXd, const std::vector<float*>& Hd, const FitKeep& keep,
                        float* const* dHd, float* dZd, float* Zd, cudaStream_t st) {
@@ -956,7 +956,7 @@ int dp_init(dp_model** out, const char* weights_path, const char* const* type_ma
     if ((rc = dev_upload(m, &m->grad, zeros)) != DP_OK) return fail_free(rc);
     if ((rc = dev_upload(m, &m->adam_m, zeros)) != DP_OK) return fail_free(rc);
     if ((rc = dev_upload(m, &m->adam_v, zeros)) != DP_OK) return fail_free(rc);
-    std::vector<float> sc = {1.f, 0.f, 0.f, 0.f};
+    std::vector<float> sc = {0.f, 0.f};
     if ((rc = dev_upload(m, &m->d_scales, sc)) != DP_OK) return fail_free(rc);
     m->emb_packed = m->theta;
     m->ebias = m->theta + m->off_ebias;

@@ -123,7 +123,6 @@ void gemm_f32(const float* A, int lda, const float* B, int ldb, const float* bia
 struct EmbedArgs {
   const float* R;
   const int* nlist;
-  const int* nnei;
   const int* atype;
   int n, ntypes, m1;
   const float* w;   // packed embedding-net weights (W0 b0 W1 b1 W2 b2)
@@ -203,12 +202,12 @@ void launch_tanh_bwd(const float* dH, const float* Hcur, const float* Hprev, flo
 
 // --- training of the student (train.cu, simt.cu)
 // A fitting layer's weight and bias gradients: C[I][O] += A'^T (s2 dZ) + A^T (s2 dZ' + s1
-// dZ), c[O] += column sums of s2 dZ' + s1 dZ, with s1, s2 = scales[1], scales[2].
+// dZ), c[O] += column sums of s2 dZ' + s1 dZ, with s1, s2 = scales[0], scales[1].
 void launch_fit_grad(const float* A, const float* Ad, const float* dZ, const float* dZd, float* C, float* c, int I,
                      int O, int N, const float* scales, cudaStream_t st);
 void launch_head_grad(const float* H, const float* Hd, const int* atype, float* g_wout, float* g_bout, float* g_ebias,
                       int O, int N, int ntypes, const float* scales, float out_scale, cudaStream_t st);
-// loss of one frame, the gradient scales (1, energy term, force term) and
+// loss of one frame, the gradient scales (energy term, force term) and
 // the direction v = F - F_ref of the force term
 void launch_train_prep(int n, const double* energy, double e_ref, const double* force, const double* force_ref,
                        double pe, double pf, double* v, double* loss, float* scales, cudaStream_t st);
@@ -245,7 +244,7 @@ struct JvpArgs {
 void launch_env_jvp(const JvpArgs& a, cudaStream_t st);
 // G'.
 bool launch_embed_jvp(const JvpArgs& a, const int* widths, cudaStream_t st);
-// grad += scales[1] dE/d(embedding weights) + scales[2] (dE/d(embedding weights))'.
+// grad += scales[0] dE/d(embedding weights) + scales[1] (dE/d(embedding weights))'.
 bool launch_embed_grad(const JvpArgs& a, const int* widths, float* grad, const float* scales, cudaStream_t st);
 void launch_desc_jvp_fwd(const JvpArgs& a, cudaStream_t st);
 void launch_desc_jvp_bwd(const JvpArgs& a, cudaStream_t st);

@@ -171,7 +171,7 @@ struct dp_model {
   // non-null: the next evaluation leaves every fitting layer's dE/dH and dE/dZ there,
   // layer by layer, and runs the embedding net in FP32
   const dpa1::FitKeep* fit_keep = nullptr;
-  float* d_scales = nullptr;          // [4]: 1, energy-loss scale, force-loss scale, 0
+  float* d_scales = nullptr;          // [2]: energy-loss scale, force-loss scale
   void* t_buf = nullptr;              // training scratch: energy, virial, forces, the direction
                                       // v = F - F_ref, the fitting adjoint and the tangents of the evaluation
   int t_cap = 0;                      // atoms t_buf is laid out for

@@ -291,17 +291,6 @@ __device__ __forceinline__ float2 smooth_logit(float t, float S, float2 wj, floa
   return make_float2(hh, hl);
 }
 
-// the largest pair (ordered by h, then l) over the warp; every lane gets the same
-__device__ __forceinline__ float2 warp_max_pair(float2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, v.x, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, v.y, o);
-    if (oh > v.x || (oh == v.x && ol > v.y)) v = make_float2(oh, ol);
-  }
-  return v;
-}
-
 __device__ __forceinline__ float pair_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
 
 // Forward, register-tiled, 512 threads.  The products (S, then each 128-column
@@ -1155,7 +1144,7 @@ __global__ void k_energy_head(const float* __restrict__ H, const float* __restri
     dZ[i] = d * (1.f - t * t);
   }
   s = warp_sum(s);
-  if (lane == 0) e[atom] = 1.0f * (s + *bptr) + ebias[atype[atom]];
+  if (lane == 0) e[atom] = (s + *bptr) + ebias[atype[atom]];
 }
 
 void launch_energy_head(const float* H, const float* Hprev, int n, int nlocal, int width, const float* w_out,

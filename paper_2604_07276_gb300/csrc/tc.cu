@@ -883,7 +883,6 @@ void tc_plan_buffers(dp_model* m, Arena& a, int cap) {
   ws.tc.p[0] = a.take<__nv_bfloat16>(rows * yhat_ld(m->m1) * (size_t)std::max(1, m->nattn));  // yhat per layer
   ws.tc.p[1] = a.take<float>(rows * (size_t)std::max(1, m->nattn));                // rstd per layer
   ws.tc.p[4] = a.take<float2>(rows * (size_t)std::max(1, m->nattn));               // softmax stats per layer
-  ws.tc.p[2] = nullptr;
   // layers 1 and 2 of the tensor-core embedding net, for its adjoint
   ws.tc.p[5] = m->tcw.emb_W1_t ? a.take<float>(rows * (size_t)(m->emb[0] + m->emb[1])) : nullptr;
 }
@@ -923,7 +922,7 @@ void tc_run_network(dp_model* m, int n, const int* atype, cudaStream_t st) {
   // embedding (nets without tensor-core tiles: FP32 SIMT), then the attention
   // layers forward
   EmbedArgs ea{};
-  ea.R = ws.R; ea.nlist = ws.nlist; ea.nnei = ws.nnei; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m->m1;
+  ea.R = ws.R; ea.nlist = ws.nlist; ea.atype = atype; ea.n = n; ea.ntypes = m->nt; ea.m1 = m->m1;
   ea.w = m->emb_packed; ea.Gt = m->Gt; ea.b0t = m->b0t; ea.G0 = ws.G[0]; ea.dG0 = ws.dG;
   ea.dR = ws.dR;
   ea.rowmap = ws.rowmap;

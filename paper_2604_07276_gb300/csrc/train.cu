@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(256) k_fit_grad(const float* __restrict__ A, c
   const int i0 = blockIdx.x * 64, o0 = blockIdx.y * 64;
   const int n_begin = blockIdx.z * chunk;
   const int n_end = min(N, n_begin + chunk);
-  const float s1 = scales[1], s2 = scales[2];
+  const float s1 = scales[0], s2 = scales[1];
   float acc[4][4] = {}, bias = 0.f;
   for (int n0 = n_begin; n0 < n_end; n0 += WG_ROWS) {
 #pragma unroll
@@ -91,7 +91,7 @@ __global__ void k_head_grad(const float* __restrict__ H, const float* __restrict
                             int N, int ntypes, int chunk, const float* __restrict__ scales, float out_scale) {
   pdl_wait();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  const float s1 = scales[1], s2 = scales[2];
+  const float s1 = scales[0], s2 = scales[1];
   if (blockIdx.y >= gridDim.y - 2) {
     if (blockIdx.x > 0) return;
     if (blockIdx.y == gridDim.y - 1) {
@@ -147,10 +147,8 @@ __global__ void k_train_prep(int n, const double* __restrict__ energy, double e_
     loss[0] = lE + lF;
     loss[1] = lE;
     loss[2] = lF;
-    scales[0] = 1.0f;
-    scales[1] = (float)(2.0 * pe * de / (nn * nn));
-    scales[2] = (float)(-2.0 * pf / (3.0 * nn));
-    scales[3] = 0.f;
+    scales[0] = (float)(2.0 * pe * de / (nn * nn));
+    scales[1] = (float)(-2.0 * pf / (3.0 * nn));
   }
 }
 
@@ -227,7 +225,7 @@ struct JvpEmbedSmem {
   static constexpr int pad4(int x) { return (x + 3) / 4 * 4; }
   static constexpr int L1 = pad4(E1), L2 = pad4(E2), L0 = pad4(E0);
   // packed weights in the parameter vector
-  static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2, NW = gB2 + E2;
+  static constexpr int gB0 = E0, gW1 = 2 * E0, gB1 = gW1 + E0 * E1, gW2 = gB1 + E1, gB2 = gW2 + E1 * E2;
   // shared memory (floats)
   static constexpr int W1 = 0, W2 = W1 + E0 * L1, W0 = W2 + E1 * L2, B0 = W0 + L0, B1 = B0 + L0, B2 = B1 + L1,
                        X = B2 + L2, XD = X + JROWS, TP = XD + JROWS;  // TP: the rows' type pairs (int)
@@ -327,8 +325,8 @@ __global__ void __launch_bounds__(JTHREADS) k_embed_jvp(JvpArgs a, float* __rest
   for (int t = tid; t < E2; t += JTHREADS) sm[S::B2 + t] = a.w[S::gB2 + t];
   float s1 = 0.f, s2 = 1.f;
   if (MODE == 1) {
-    s1 = scales[1];
-    s2 = scales[2];
+    s1 = scales[0];
+    s2 = scales[1];
     for (int t = tid; t < E1 * E2; t += JTHREADS) sm[S::W2T + (t % E2) * S::L1 + t / E2] = a.w[S::gW2 + t];
     for (int t = tid; t < E0 * E1; t += JTHREADS) sm[S::W1T + (t % E1) * S::L0 + t / E1] = a.w[S::gW1 + t];
   }
