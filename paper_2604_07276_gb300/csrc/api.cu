@@ -465,24 +465,23 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
       dZn = keep->dZ[l - 1];
     }
     float* dst = l > 0 ? dHn : ws.dX;
-    // the layer below: its dZ = dH (1 - t^2), t = H - its skip input, with the product
+    // the layer below: its dZ = dH (1 - t^2), t = H - its skip input.  fit_gemm_tc forms
+    // it with the product, in all its warps.  In gemm_bf16x's epilogue, four warps
+    // for all the tiles of a CTA, it takes longer than a launch of its own at every
+    // size (fitting stage of 582 atoms 88.1 us against 87.0, of 4,096 149.5 against
+    // 138.2, of 15,668 346 against 276).
     const float* Hc = l > 0 ? ws.H[l - 1] : nullptr;
     const float* Hp = l > 1 && m->fit[l - 1] == m->fit[l - 2] ? ws.H[l - 2] : nullptr;
     float* Z = l > 0 ? dZn : nullptr;
-    if (fit_x) {
-      // the persistent GEMM's four epilogue warps bind once a CTA walks many tiles:
-      // dZ is formed there for small boxes only (3,001 atoms: 171 -> 137 us for the
-      // fitting stage, with the narrower N blocks; 15,668: 308 -> 359 us)
-      const bool with = n <= 4096;
-      gemm_bf16x(m, m->xw.fitT[l], dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st,
-                 nullptr, Hc, Hp, with ? Z : nullptr);
-      if (!with && l > 0) launch_tanh_bwd(dst, Hc, Hp, Z, (long long)n * in, st);
-    } else if (fit_tc) {
+    if (fit_tc) {
       fit_gemm_tc(m, l, true, dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, Hc, Hp, Z,
                   st);
     } else {
-      gemm_f32(dZ, out, m->fitWT[l], in, nullptr, res ? dH : nullptr, out, dst, in, n, in, out,
-               res ? EPI_RES : EPI_BIAS, st);
+      if (fit_x)
+        gemm_bf16x(m, m->xw.fitT[l], dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st);
+      else
+        gemm_f32(dZ, out, m->fitWT[l], in, nullptr, res ? dH : nullptr, out, dst, in, n, in, out,
+                 res ? EPI_RES : EPI_BIAS, st);
       if (l > 0) launch_tanh_bwd(dst, Hc, Hp, Z, (long long)n * in, st);
     }
     std::swap(dH, dHn);

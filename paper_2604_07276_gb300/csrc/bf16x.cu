@@ -82,10 +82,6 @@ struct XGemmArgs {
   int M, N, nkb, bn_max, epi;
   int bn, stages;    // columns per CTA (see x_bn), depth of the ring
   const int* m_dev;  // non-null: the rows are *m_dev (device, <= M)
-  // fitting adjoint: Z = C (1 - t^2) with t = Hc - Hp (Hp null: Hc), all [M][ldc]; null: none
-  const float* Hc;
-  const float* Hp;
-  float* Z;
   int* err;
 };
 
@@ -110,7 +106,6 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo) {
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-template <bool ZOUT>
 __global__ void __launch_bounds__(XTHREADS, 1)
 k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XGemmArgs a) {
   pdl_wait();
@@ -285,19 +280,7 @@ k_gemm_bf16x(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ XG
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const long long m = m0 + 4 * (k0 + k) + (lane >> 3);
-              if (m < M) {
-                *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o[k];
-                if (ZOUT) {
-                  float4 t = *reinterpret_cast<const float4*>(a.Hc + m * a.ldc + n);
-                  if (a.Hp) {
-                    const float4 p = *reinterpret_cast<const float4*>(a.Hp + m * a.ldc + n);
-                    t.x -= p.x; t.y -= p.y; t.z -= p.z; t.w -= p.w;
-                  }
-                  *reinterpret_cast<float4*>(a.Z + m * a.ldc + n) =
-                      make_float4(o[k].x * (1.f - t.x * t.x), o[k].y * (1.f - t.y * t.y), o[k].z * (1.f - t.z * t.z),
-                                  o[k].w * (1.f - t.w * t.w));
-                }
-              }
+              if (m < M) *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o[k];
             }
           }
         }
@@ -1090,8 +1073,7 @@ int bf16x_init_weights(dp_model* m, std::string& msg) {
     fan = m->fit[l];
   }
   bf16x_refresh(m, nullptr);
-  for (auto k : {k_gemm_bf16x<false>, k_gemm_bf16x<true>})
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(x_smem(XBN), x_smem(16)));
+  cudaFuncSetAttribute(k_gemm_bf16x, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(x_smem(XBN), x_smem(16)));
   cudaFuncSetAttribute(k_attn_core_fwd_bf16x<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, XF_SMEM);
   cudaFuncSetAttribute(k_attn_core_fwd_bf16x<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, XF_SMEM);
   cudaFuncSetAttribute(k_attn_core_bwd_bf16x<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
@@ -1120,8 +1102,7 @@ void bf16x_free(dp_model* m) {
 }
 
 int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const float* bias, const float* R, int ldr,
-               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev, const float* Hc, const float* Hp,
-               float* Z) {
+               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev) {
   if (M <= 0) return DP_OK;
   CUtensorMap map;
   const cuuint64_t dims[2] = {(cuuint64_t)im.K, (cuuint64_t)M};
@@ -1145,9 +1126,6 @@ int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const flo
   a.bn_max = im.bn_max;
   a.epi = epi;
   a.m_dev = m_dev;
-  a.Hc = Hc;
-  a.Hp = Hp;
-  a.Z = Z;
   a.err = m->d_err;
   // persistent: about one CTA per SM over the N blocks
   const int mt = (M + XBM - 1) / XBM, sms = x_sm_count(m->device);
@@ -1155,10 +1133,7 @@ int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const flo
   a.stages = x_stages(a.bn);
   const int nnb = (im.N + a.bn - 1) / a.bn;
   dim3 grid((unsigned)std::min(mt, std::max(1, sms / nnb)), (unsigned)nnb);
-  if (Z)
-    launch_pdl(k_gemm_bf16x<true>, grid, XTHREADS, x_smem(a.bn), st, map, a);
-  else
-    launch_pdl(k_gemm_bf16x<false>, grid, XTHREADS, x_smem(a.bn), st, map, a);
+  launch_pdl(k_gemm_bf16x, grid, XTHREADS, x_smem(a.bn), st, map, a);
   note_launch();
   return DP_OK;
 }

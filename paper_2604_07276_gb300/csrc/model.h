@@ -239,8 +239,7 @@ int bf16x_init_weights(dp_model* m, std::string& msg);
 void bf16x_refresh(dp_model* m, cudaStream_t st);
 void bf16x_free(dp_model* m);
 int gemm_bf16x(dp_model* m, const XImage& im, const float* A, int lda, const float* bias, const float* R, int ldr,
-               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev = nullptr, const float* Hc = nullptr,
-               const float* Hp = nullptr, float* Z = nullptr);
+               float* C, int ldc, int M, int epi, cudaStream_t st, const int* m_dev = nullptr);
 void attn_core_fwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 void attn_core_bwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 // the fused 16-bit layer kernels (tc.cu) serve DP_PREC_BF16 and DP_PREC_FP16X;
