@@ -346,18 +346,38 @@ int translate_err(int bits) {
 
 // A device call, or a change of the weights, was queued on the caller's stream st.
 void note_device_call(dp_model* m, cudaStream_t st) {
-  m->pending = true;
+  (st == nullptr || st == cudaStreamLegacy ? m->default_pending : m->other_pending) = true;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
   if (cs != cudaStreamCaptureStatusNone) m->captured = true;
 }
 
+// Places the model's own stream, which is not tied to the default one, behind the work
+// queued there; done is false if the default stream takes no event (while a blocking
+// stream is being captured).
+int behind_default(dp_model* m, bool* done) {
+  cudaStreamCaptureStatus cs;
+  *done = cudaStreamIsCapturing(nullptr, &cs) == cudaSuccess;
+  if (!*done) {
+    cudaGetLastError();
+    return DP_OK;
+  }
+  CUDA_TRY(cudaEventRecord(m->order, nullptr));
+  CUDA_TRY(cudaStreamWaitEvent(m->stream, m->order, 0));
+  return DP_OK;
+}
+
 // Before a call on the model's own stream: its workspace and weights may be in use by a
-// device call on another.  The caller's streams may be gone by now, hence the device.
+// device call on another.  A caller's stream may be gone by now: the device is waited
+// for then, as after captured calls, whose replays are not seen here.
 int wait_device_calls(dp_model* m) {
-  if (!m->pending) return DP_OK;
-  CUDA_TRY(cudaDeviceSynchronize());
-  m->pending = m->captured;
+  bool all = m->other_pending || m->captured;
+  if (m->default_pending && !all) {
+    if (int rc = behind_default(m, &all)) return rc;
+    all = !all;
+  }
+  if (all) CUDA_TRY(cudaDeviceSynchronize());
+  m->default_pending = m->other_pending = false;
   return DP_OK;
 }
 
@@ -1640,15 +1660,8 @@ int dp_md_run(dp_model* m, int natoms, double* d_coord, double* d_vel, const dou
     note_device_call(m, st);
   } else {
     if (int w = wait_device_calls(m)) return w;
-    // the caller has filled the arrays on the default stream, which this one is not
-    // tied to (while a blocking stream is being captured, the default one takes no work)
-    cudaStreamCaptureStatus cs;
-    if (cudaStreamIsCapturing(nullptr, &cs) == cudaSuccess) {
-      CUDA_TRY(cudaEventRecord(m->order, nullptr));
-      CUDA_TRY(cudaStreamWaitEvent(st, m->order, 0));
-    } else {
-      cudaGetLastError();
-    }
+    bool done;  // the caller has filled the arrays on the default stream
+    if (int w = behind_default(m, &done)) return w;
   }
   if (!m->d_md_counter) {
     void* p = nullptr;

@@ -192,11 +192,11 @@ struct dp_model {
   char* h_io = nullptr;
   char* d_io = nullptr;
   cudaStream_t stream = nullptr;  // own stream of the host API
-  cudaEvent_t order = nullptr;    // places that stream behind the default stream (dp_md_run)
+  cudaEvent_t order = nullptr;    // places that stream behind the default one
   cudaStream_t last_stream = nullptr;
-  // device calls queued on the caller's streams that no host call has waited for, and
-  // whether one of them was captured (its replays are not seen here)
-  bool pending = false, captured = false;
+  // device calls queued on the default stream and on others that no host call has waited
+  // for, and whether a device call was ever captured
+  bool default_pending = false, other_pending = false, captured = false;
   int last_natoms = 0;
   dpa1::Profiler prof;
   // velocity-Verlet: step counter, the kick's per-block kinetic energies and
