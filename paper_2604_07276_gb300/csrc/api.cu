@@ -461,7 +461,7 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
                  res ? EPI_RES_TANH : EPI_TANH, st);
     else if (fit_tc)
       fit_gemm_tc(m, l, false, hin, fan, m->fitb[l], res ? hin : nullptr, fan, ws.H[l], out, n,
-                  res ? EPI_RES_TANH : EPI_TANH, nullptr, nullptr, nullptr, st);
+                  res ? EPI_RES_TANH : EPI_TANH, st);
     else
       gemm_f32(hin, fan, m->fitW[l], out, m->fitb[l], res ? hin : nullptr, fan, ws.H[l], out, n, out, fan,
                res ? EPI_RES_TANH : EPI_TANH, st);
@@ -485,25 +485,20 @@ void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t s
       dZn = keep->dZ[l - 1];
     }
     float* dst = l > 0 ? dHn : ws.dX;
-    // the layer below: its dZ = dH (1 - t^2), t = H - its skip input.  fit_gemm_tc forms
-    // it with the product, in all its warps.  In gemm_bf16x's epilogue, four warps
-    // for all the tiles of a CTA, it takes longer than a launch of its own at every
-    // size (fitting stage of 582 atoms 88.1 us against 87.0, of 4,096 149.5 against
-    // 138.2, of 15,668 346 against 276).
-    const float* Hc = l > 0 ? ws.H[l - 1] : nullptr;
-    const float* Hp = l > 1 && m->fit[l - 1] == m->fit[l - 2] ? ws.H[l - 2] : nullptr;
-    float* Z = l > 0 ? dZn : nullptr;
-    if (fit_tc) {
-      fit_gemm_tc(m, l, true, dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, Hc, Hp, Z,
-                  st);
-    } else {
-      if (fit_x)
-        gemm_bf16x(m, m->xw.fitT[l], dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st);
-      else
-        gemm_f32(dZ, out, m->fitWT[l], in, nullptr, res ? dH : nullptr, out, dst, in, n, in, out,
-                 res ? EPI_RES : EPI_BIAS, st);
-      if (l > 0) launch_tanh_bwd(dst, Hc, Hp, Z, (long long)n * in, st);
-    }
+    if (fit_x)
+      gemm_bf16x(m, m->xw.fitT[l], dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st);
+    else if (fit_tc)
+      fit_gemm_tc(m, l, true, dZ, out, nullptr, res ? dH : nullptr, out, dst, in, n, res ? EPI_RES : EPI_BIAS, st);
+    else
+      gemm_f32(dZ, out, m->fitWT[l], in, nullptr, res ? dH : nullptr, out, dst, in, n, in, out,
+               res ? EPI_RES : EPI_BIAS, st);
+    // the layer below: its dZ = dH (1 - t^2), t = H - its skip input.  In the products'
+    // epilogues it takes longer than by a launch of its own: fitting stage of 4,096
+    // atoms 149.5 us against 138.2 (bf16x) and 135.4 against 133.3 (fp16x), of 15,668
+    // 346 against 276 and 295 against 286, of 582 the same within a microsecond.
+    if (l > 0)
+      launch_tanh_bwd(dst, ws.H[l - 1], l > 1 && m->fit[l - 1] == m->fit[l - 2] ? ws.H[l - 2] : nullptr, dZn,
+                      (long long)n * in, st);
     std::swap(dH, dHn);
     std::swap(dZ, dZn);
   }

@@ -14,17 +14,16 @@
 //   warps 4-11  : split each A tile in place (A_hi) and into its A_lo tile.
 //   warp 1      : issues the MMAs (one thread), accumulator in TMEM.
 //   warp 2      : allocates / frees TMEM.
-//   all warps   : the epilogue (TMEM -> bias, tanh, residual -> global; in the
-//                 backward pass also the next layer's dZ = dH (1 - t^2)); warp
+//   all warps   : the epilogue (TMEM -> bias, tanh, residual -> global); warp
 //                 w reads TMEM lane quadrant w % 4 and every third 16-column
 //                 chunk, starting at chunk w / 4.
 // BN: the widest tile (256 columns) reads A the fewest times, but a small box
 // has few 128-row tiles, and each CTA walks the whole K alone: BN shrinks until
 // the tiles fill the SMs once (192 atoms, K = 1608, N = 240: 2 CTAs -> 30), and
 // the ring deepens with the room that leaves.  A tile's sums do not depend on
-// BN.  With the dZ epilogue and the energy head's seed (7 launches, were 12) the
-// fitting stage of 192 atoms took 192 -> 107 us, of 582 208 -> 111, of 15,668
-// (one tile per SM row, BN = 240) 326 -> 310.
+// BN.  With the energy head's seed (9 launches, were 12) the fitting stage of 192
+// atoms took 192 -> 91 us, of 582 208 -> 96, of 15,668 (one tile per SM row, BN =
+// 240) 326 -> 288.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -63,10 +62,6 @@ struct FitGemmArgs {
   int bn;               // columns per CTA (multiple of 16; 256 is a multiple of it or it is N)
   int stages;
   int epi;
-  // backward: Z = C (1 - t^2) with t = Hc - Hp (Hp null: Hc), all [M][ldc]; null: none
-  const float* Hc;
-  const float* Hp;
-  float* Z;
   int* err;
 };
 
@@ -243,15 +238,6 @@ k_fit_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ FitG
           o.x += rr.x; o.y += rr.y; o.z += rr.z; o.w += rr.w;
         }
         *reinterpret_cast<float4*>(a.C + m * a.ldc + n) = o;
-        if (a.Z) {
-          float4 t = *reinterpret_cast<const float4*>(a.Hc + m * a.ldc + n);
-          if (a.Hp) {
-            const float4 p = *reinterpret_cast<const float4*>(a.Hp + m * a.ldc + n);
-            t.x -= p.x; t.y -= p.y; t.z -= p.z; t.w -= p.w;
-          }
-          *reinterpret_cast<float4*>(a.Z + m * a.ldc + n) =
-              make_float4(o.x * (1.f - t.x * t.x), o.y * (1.f - t.y * t.y), o.z * (1.f - t.z * t.z), o.w * (1.f - t.w * t.w));
-        }
       }
     }
   }
@@ -391,8 +377,7 @@ void fit_tc_refresh(dp_model* m, cudaStream_t st) {
 }
 
 int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, const float* bias, const float* R,
-                int ldr, float* C, int ldc, int M, int epi, const float* Hc, const float* Hp, float* Z,
-                cudaStream_t st) {
+                int ldr, float* C, int ldc, int M, int epi, cudaStream_t st) {
   if (M <= 0) return DP_OK;
   const int fan = layer == 0 ? m->fit_in : m->fit[layer - 1];
   const int out = m->fit[layer];
@@ -423,9 +408,6 @@ int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, 
   a.bn = fit_bn(mt, s.N, sms);
   a.stages = fit_stages(a.bn);
   a.epi = epi;
-  a.Hc = Hc;
-  a.Hp = Hp;
-  a.Z = Z;
   a.err = m->d_err;
   dim3 grid((unsigned)mt, (unsigned)((s.N + a.bn - 1) / a.bn));
   launch_pdl(k_fit_gemm, grid, FTHREADS, fit_smem(a.bn), st, map, a);

@@ -247,8 +247,7 @@ void attn_core_bwd_bf16x(dp_model* m, int n, int l, cudaStream_t st);
 // stored Q | K and [P G, rowsum P], LayerNorm kernels)
 inline bool fused_tc_precision(int p) { return p == DP_PREC_BF16 || p == DP_PREC_FP16X; }
 int fit_gemm_tc(dp_model* m, int layer, bool backward, const float* A, int lda, const float* bias, const float* R,
-                int ldr, float* C, int ldc, int M, int epi, const float* Hc, const float* Hp, float* Z,
-                cudaStream_t st);
+                int ldr, float* C, int ldc, int M, int epi, cudaStream_t st);
 // stages a7-a11 (descriptor, fitting forward / backward, descriptor backward)
 void run_descriptor_fitting(dp_model* m, int n, const int* atype, cudaStream_t st, bool fold = false);
 }  // namespace dpa1
